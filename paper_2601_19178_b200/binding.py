@@ -86,6 +86,12 @@ def _load() -> ctypes.CDLL:
 
 
 lib = _load()
+try:
+    from . import _pycall
+except ImportError as e:
+    raise ImportError(f"{e}: build it with `python paper_2601_19178_b200/build.py`") from e
+_ATTEND, _ATTEND_VISIBLE, _ATTEND_STATIC = (
+    ctypes.cast(f, ctypes.c_void_p).value for f in (lib.ckv_attend, lib.ckv_attend_visible, lib.ckv_attend_static))
 
 
 def _ptr(x) -> Optional[int]:
@@ -113,10 +119,25 @@ def _host_i32(a) -> np.ndarray:
     return np.ascontiguousarray(a, dtype=np.int32)
 
 
+def _current_stream() -> int:
+    """Handle of torch's current stream on the current device."""
+    # (the handle alone: torch.cuda.current_stream() builds a Stream object around it, 3 us)
+    global _current_stream
+    import torch
+    torch.cuda.init()
+    raw, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+    if raw is None or device is None:
+        def _current_stream():
+            return torch.cuda.current_stream().cuda_stream
+    else:
+        def _current_stream():
+            return raw(device())
+    return _current_stream()
+
+
 def _stream(stream) -> Optional[int]:
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return _current_stream()
     return getattr(stream, "cuda_stream", stream)
 
 
@@ -180,6 +201,12 @@ def ckv_cache_clear(ctx) -> None:
 
 def ckv_attend(ctx, users, q_off, queries, out, stream=None) -> None:
     """users: host int64 [n]; q_off: host int32 [n+1]; queries/out: device (or host) buffers."""
+    stream = _stream(stream)
+    st = _pycall.attend(_ATTEND, ctx or 0, users, q_off, None, queries, out, stream or 0)
+    if st == CKV_OK:
+        return
+    if st is not None:
+        _check(ctx, st, "ckv_attend")
     users, q_off = _host_i64(users), _host_i32(q_off)
     if q_off.shape[0] != users.shape[0] + 1:
         raise ValueError("q_off must have len(users) + 1 entries")
@@ -189,6 +216,13 @@ def ckv_attend(ctx, users, q_off, queries, out, stream=None) -> None:
 
 def ckv_attend_visible(ctx, users, q_off, vis, queries, out, stream=None) -> None:
     """ckv_attend with a visible length per query row: vis int32 [q_off[n]] (host array or device tensor)."""
+    stream = _stream(stream)
+    if vis is not None:
+        st = _pycall.attend(_ATTEND_VISIBLE, ctx or 0, users, q_off, vis, queries, out, stream or 0)
+        if st == CKV_OK:
+            return
+        if st is not None:
+            _check(ctx, st, "ckv_attend_visible")
     users, q_off = _host_i64(users), _host_i32(q_off)
     if q_off.shape[0] != users.shape[0] + 1:
         raise ValueError("q_off must have len(users) + 1 entries")
@@ -205,6 +239,12 @@ def ckv_attend_static(ctx, users, q_off, queries, out, stream=None) -> None:
     library.  queries/out must be device buffers; raises CkvError(CKV_ERR_TOO_LARGE) beyond
     256 users per call or when the partial results do not fit.  Calls that may overlap on the
     GPU race on that array."""
+    stream = _stream(stream)
+    st = _pycall.attend(_ATTEND_STATIC, ctx or 0, users, q_off, None, queries, out, stream or 0)
+    if st == CKV_OK:
+        return
+    if st is not None:
+        _check(ctx, st, "ckv_attend_static")
     users, q_off = _host_i64(users), _host_i32(q_off)
     if q_off.shape[0] != users.shape[0] + 1:
         raise ValueError("q_off must have len(users) + 1 entries")

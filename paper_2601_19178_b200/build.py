@@ -1,4 +1,5 @@
-"""Builds libckv.so (sm_100a) next to this file with nvcc.  No GPU is needed to build.
+"""Builds libckv.so (sm_100a) next to this file with nvcc, and with the host compiler the CPython helper _pycall.so
+of the binding.  No GPU is needed to build.
 
     python paper_2601_19178_b200/build.py [--force] [--verbose] [--bounds]     (or: python __graft_entry__.py)
 """
@@ -9,12 +10,14 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 OBJ = os.path.join(ROOT, "_build")
 LIB = os.path.join(PKG, "libckv.so")
+PYCALL = os.path.join(PKG, "_pycall.so")
 LIB_BOUNDS = os.path.join(PKG, "libckv_bounds.so")
 
 NVCC_FLAGS = [
@@ -35,6 +38,20 @@ def _newest(paths) -> float:
     return max(os.path.getmtime(p) for p in paths)
 
 
+def build_pycall(force: bool = False) -> str:
+    src = os.path.join(CSRC, "pycall.c")
+    if force or not os.path.exists(PYCALL) or os.path.getmtime(PYCALL) < os.path.getmtime(src):
+        tmp = PYCALL + f".tmp{os.getpid()}"
+        cmd = [os.environ.get("CC") or "gcc", "-O2", "-Wall", "-shared", "-fPIC", "-fvisibility=hidden",
+               "-I", sysconfig.get_paths()["include"], src, "-o", tmp]
+        r = subprocess.run(cmd, capture_output=True, text=True)
+        if r.returncode != 0:
+            sys.stderr.write(r.stdout + r.stderr)
+            raise RuntimeError("the host compiler failed on " + src)
+        os.replace(tmp, PYCALL)
+    return PYCALL
+
+
 def build(force: bool = False, verbose: bool = False, bounds: bool = False) -> str:
     """bounds=True builds libckv_bounds.so instead: the same library with every index, row and shared-memory
     offset the kernels compute range-checked into the context's error word (-DCKV_BOUNDS)."""
@@ -46,6 +63,7 @@ def build(force: bool = False, verbose: bool = False, bounds: bool = False) -> s
     obj_dir = OBJ + ("_bounds" if bounds else "")
     lib = LIB_BOUNDS if bounds else LIB
     os.makedirs(obj_dir, exist_ok=True)
+    build_pycall(force)
     nvcc = _nvcc()
     extra = (["-Xptxas", "-v"] if verbose else []) + (["-DCKV_BOUNDS"] if bounds else [])
     hdr_time = _newest(headers) if headers else 0.0

@@ -149,6 +149,7 @@ struct Plan {
     int32_t* d_split = nullptr;
     Work* d_works = nullptr;
     int32_t n_items = 0, n_split = 0, split_items = 0, max_M = 0, max_L = 0, n_req = 0, family = 1, n_vblocks = 0;
+    int32_t parts = 1;       // family 2: warps that share a unit
     int64_t part_rows = 0;
     uint64_t last_use = 0;
 };
@@ -210,11 +211,12 @@ struct ckv_ctx {
     cudaStream_t pipe_stream[kMaxRanges] = {};
     cudaEvent_t pipe_start = nullptr, pipe_plan = nullptr, pipe_h2d[kMaxRanges] = {}, pipe_done[kMaxRanges] = {};
     bool pipe_ready = false;
-    // L2 residency of the pool: an access-policy window over the pool allocation is put on the caller's
-    // stream around the kernels of a decode call and taken off again before the call returns
+    // L2 residency of the pool: the kernels of a decode call are launched with an access-policy window over the pool
+    // allocation (a launch attribute: the caller's stream is left alone)
+    SmemGrants grants;
     bool l2_ready = false;       // the persisting-L2 carve-out of this device was raised for this context
     size_t l2_window = 0;        // bytes of the window (0: not available)
-    float l2_ratio = 1.f;
+    cudaAccessPolicyWindow window{};
     // statistics of the last attend
     int64_t st_launches = 0, st_items = 0, st_split = 0, st_kernel = 0, st_ws = 0, st_hit = 0, st_loader = 0,
             st_allocs = 0, st_l2 = 0, st_ranges = 1;
@@ -420,8 +422,69 @@ void arena_give(ckv_ctx* ctx, int64_t base, int64_t units)
 
 int64_t units_of_len(const ckv_ctx* ctx, int64_t L) { return (int64_t)ctx->cfg.n_groups * ((L + 31) / 32 * 32); }
 
-int64_t auto_split_len(const ckv_ctx* ctx, int64_t total_positions, int family, int max_M)
+// The kernel family of a request list (0: the forced one cannot take it).
+int choose_family(const ckv_ctx* ctx, bool with_vis, int32_t n, int64_t n_active, int64_t total_pos, int32_t max_M,
+                  int32_t max_L, bool all_single)
 {
+    const bool can_mma = ctx->has_mma;
+    // visible lengths and sides that are not shared are served by every gathering kernel, not by the pool-side
+    // factorisation
+    const bool plain = !with_vis && !ctx->full_k && !ctx->full_v;
+    const bool can_umma = ctx->has_umma;
+    // tcgen05 from three 16-query blocks on, else the warp-level tensor-core kernel (faster than the CUDA-core
+    // kernel from a single query on); the CUDA-core kernel serves what neither supports
+    // One query per user: the pool-side factorisation trades the row gathers for two tables per (user, group) in
+    // HBM (n_entries floats per request and group: not beyond 2 GiB of workspace).
+    const bool can_fact = plain && all_single && n_active > 0 &&
+                          fact_max_history(ctx->cfg.dtype, ctx->cfg.head_dim, ctx->d_user, ctx->n_entries) >= max_L &&
+                          (int64_t)n * ctx->cfg.n_groups * (fact_row_floats(ctx->n_entries) + fact_aux_floats()) *
+                                  (int64_t)sizeof(float) <= ((int64_t)2 << 30);
+    // It pays when histories are long against the pool and there are enough (user, group) pairs to fill the SMs
+    // (one CTA holds a whole pair; the gathering kernel splits long histories over CTAs).  Cost lines fitted to
+    // B200 measurements, in microseconds of one SM: a pair costs a + b n_entries + c L on the factorised path,
+    // a position d on the gathering path.
+    bool fact_pays = false;
+    if (can_fact) {
+        const bool wide = ctx->cfg.head_dim == 64;
+        const double a = wide ? 4.8 : 4.7, b = wide ? 0.00032 : 0.00024, c = wide ? 0.0010 : 0.0008,
+                     d = wide ? 0.0047 : 0.0025;
+        const double pairs = (double)n_active * ctx->cfg.n_groups, mean_L = (double)total_pos / (double)n_active;
+        const double waves = std::ceil(pairs / ctx->n_sms);
+        const double t_fact = waves * (a + b * ctx->n_entries + c * mean_L);
+        const double t_gather = d * (double)total_pos * ctx->cfg.n_groups / ctx->n_sms;
+        fact_pays = t_fact < t_gather;
+    }
+    switch (ctx->opt_kernel) {
+        case 0: return can_umma && max_M >= 48 ? 3 : fact_pays ? 4 : can_mma ? 2 : 1;
+        case 1: return 1;
+        case 2: return can_mma ? 2 : 0;
+        case 3: return can_umma ? 3 : 0;
+        case 4: return can_fact ? 4 : 0;
+    }
+    return 0;
+}
+
+// Warps that share one unit of the warp-level tensor-core kernel: `tiles` 32-position tiles of all query blocks of
+// one group in all, the longest history `max_tiles` of them.  The longest unit must not keep a warp busy longer than
+// the resident warps are with everything.
+int mma_parts(const ckv_ctx* ctx, int64_t tiles, int64_t max_tiles, int max_M)
+{
+    const int64_t warps = (int64_t)ctx->n_sms * mma_warps_per_sm(ctx->cfg.head_dim, max_M);
+    const int64_t share = std::max<int64_t>(tiles * ctx->cfg.n_groups / warps, 1);
+    int parts = 1;
+    while (parts < kMmaMaxParts && max_tiles > parts * share) parts *= 2;
+    return parts;
+}
+
+// Block size of the CUDA-core kernel: blocks of more warps when there are fewer blocks than SMs.
+bool simt_wide(const ckv_ctx* ctx, int64_t n_items) { return n_items * ctx->cfg.n_groups <= ctx->n_sms; }
+
+int64_t auto_split_len(const ckv_ctx* ctx, int64_t total_positions, int family, int max_M, int max_L)
+{
+    if (family == 4) return INT32_MAX;  // one CTA holds a whole history
+    // up to 64 Ki positions the warps that share a unit of the warp-level tensor-core kernel are enough (64 tiles
+    // for each of them), up to 4096 the 16 warps of a CUDA-core block are
+    if ((family == 2 && max_L <= 65536) || (family == 1 && max_L <= 4096)) return INT32_MAX;
     // Enough (chunk, group) blocks to fill the SMs several times over, but chunks long
     // enough that the merge of partial results stays a small fraction of the work.
     int64_t c;
@@ -496,44 +559,17 @@ ckv_status build_plan(ckv_ctx* ctx, Plan& pl, int32_t n, const int64_t* users, c
     pl.max_M = max_M;
     pl.max_L = max_L;
     pl.n_req = n;
-    const bool can_mma = ctx->has_mma;
-    // visible lengths and sides that are not shared are served by every gathering kernel, not by the pool-side
-    // factorisation
-    const bool plain = !with_vis && !ctx->full_k && !ctx->full_v;
-    const bool can_umma = ctx->has_umma;
-    // tcgen05 from three 16-query blocks on, else the warp-level tensor-core kernel (faster than the CUDA-core
-    // kernel from a single query on); the CUDA-core kernel serves what neither supports
-    // One query per user: the pool-side factorisation trades the row gathers for two tables per (user, group) in
-    // HBM (n_entries floats per request and group: not beyond 2 GiB of workspace).
-    const bool can_fact = plain && all_single && n_active > 0 &&
-                          fact_max_history(ctx->cfg.dtype, ctx->cfg.head_dim, ctx->d_user, ctx->n_entries) >= max_L &&
-                          (int64_t)n * ctx->cfg.n_groups * (fact_row_floats(ctx->n_entries) + fact_aux_floats()) *
-                                  (int64_t)sizeof(float) <= ((int64_t)2 << 30);
-    // It pays when histories are long against the pool and there are enough (user, group) pairs to fill the SMs
-    // (one CTA holds a whole pair; the gathering kernel splits long histories over CTAs).  Cost lines fitted to
-    // B200 measurements, in microseconds of one SM: a pair costs a + b n_entries + c L on the factorised path,
-    // a position d on the gathering path.
-    bool fact_pays = false;
-    if (can_fact) {
-        const bool wide = ctx->cfg.head_dim == 64;
-        const double a = wide ? 4.8 : 4.7, b = wide ? 0.00032 : 0.00024, c = wide ? 0.0010 : 0.0008,
-                     d = wide ? 0.0047 : 0.0025;
-        const double pairs = (double)n_active * ctx->cfg.n_groups, mean_L = (double)total_pos / (double)n_active;
-        const double waves = std::ceil(pairs / ctx->n_sms);
-        const double t_fact = waves * (a + b * ctx->n_entries + c * mean_L);
-        const double t_gather = d * (double)total_pos * ctx->cfg.n_groups / ctx->n_sms;
-        fact_pays = t_fact < t_gather;
+    pl.family = choose_family(ctx, with_vis, n, n_active, total_pos, max_M, max_L, all_single);
+    if (pl.family == 0) return CKV_ERR_UNSUPPORTED;
+    const int64_t C = ctx->opt_split > 0 && pl.family != 4 ? ctx->opt_split
+                                                           : auto_split_len(ctx, total_pos, pl.family, max_M, max_L);
+    pl.parts = 1;
+    if (pl.family == 2 && ctx->opt_split == 0) {
+        int64_t tiles = 0;
+        const int qpw = mma_queries_per_warp(ctx->cfg.head_dim, max_M);
+        for (const Req& r : reqs) tiles += (int64_t)((r.L + 31) / 32) * ((r.M + qpw - 1) / qpw);
+        pl.parts = mma_parts(ctx, tiles, (std::min<int64_t>(C, max_L) + 31) / 32, max_M);
     }
-    if (ctx->opt_kernel == 0)
-        pl.family = can_umma && max_M >= 48 ? 3 : fact_pays ? 4 : can_mma ? 2 : 1;
-    else if (ctx->opt_kernel == 4 && can_fact) pl.family = 4;
-    else if (ctx->opt_kernel == 1) pl.family = 1;
-    else if (ctx->opt_kernel == 2 && can_mma) pl.family = 2;
-    else if (ctx->opt_kernel == 3 && can_umma) pl.family = 3;
-    else return CKV_ERR_UNSUPPORTED;
-    const int64_t C = pl.family == 4         ? (int64_t)INT32_MAX  // one CTA holds a whole history
-                      : ctx->opt_split > 0 ? ctx->opt_split
-                                           : auto_split_len(ctx, total_pos, pl.family, max_M);
     std::vector<Item> items;
     std::vector<int32_t> split;
     items.reserve((size_t)n);
@@ -663,9 +699,9 @@ ckv_status get_plan(ckv_ctx* ctx, int32_t n, const int64_t* users, const int32_t
 // ---- L2 residency of the pool ------------------------------------------------------------------------
 // The pool is read by every work item of every decode call while the compressed caches stream through L2
 // once.  The device's persisting-L2 carve-out is raised to the pool's size (a per-process setting that ends
-// with the process; the previous value comes back when the last context on the device goes away), and each
-// decode call puts an access-policy window over the pool on the caller's stream while it enqueues its
-// kernels: pool lines are then kept in the carve-out and the streaming data cannot evict them.
+// with the process; the previous value comes back when the last context on the device goes away), and the
+// kernels of a decode call carry an access-policy window over the pool as a launch attribute: pool lines are
+// then kept in the carve-out and the streaming data cannot evict them.
 std::mutex g_l2_mu;
 int g_l2_users[64];
 size_t g_l2_prev[64];
@@ -701,7 +737,11 @@ void l2_prepare(ckv_ctx* ctx)
     }
     if (cur < want) cur = want;
     ctx->l2_window = std::min(pool_bytes, (size_t)max_window);
-    ctx->l2_ratio = ctx->l2_window <= cur ? 1.0f : (float)((double)cur / (double)ctx->l2_window);
+    ctx->window.base_ptr = ctx->pool;
+    ctx->window.num_bytes = ctx->l2_window;
+    ctx->window.hitRatio = ctx->l2_window <= cur ? 1.0f : (float)((double)cur / (double)ctx->l2_window);
+    ctx->window.hitProp = cudaAccessPropertyPersisting;
+    ctx->window.missProp = cudaAccessPropertyStreaming;
 }
 
 void l2_release(ckv_ctx* ctx)
@@ -717,39 +757,12 @@ void l2_release(ckv_ctx* ctx)
     ctx->l2_ready = false;
 }
 
-// Puts the pool's window on a stream for the lifetime of the object and restores what the stream had.
-struct L2Window {
-    cudaStream_t s;
-    cudaStreamAttrValue prev;
-    bool on = false;
-    L2Window(ckv_ctx* ctx, cudaStream_t stream) : s(stream)
-    {
-        ctx->st_l2 = 0;
-        if (!ctx->opt_l2 || ctx->l2_window == 0) return;
-        if (cudaStreamGetAttribute(s, cudaStreamAttributeAccessPolicyWindow, &prev) != cudaSuccess) {
-            cudaGetLastError();
-            return;
-        }
-        cudaStreamAttrValue v;
-        std::memset(&v, 0, sizeof v);
-        v.accessPolicyWindow.base_ptr = ctx->pool;
-        v.accessPolicyWindow.num_bytes = ctx->l2_window;
-        v.accessPolicyWindow.hitRatio = ctx->l2_ratio;
-        v.accessPolicyWindow.hitProp = cudaAccessPropertyPersisting;
-        v.accessPolicyWindow.missProp = cudaAccessPropertyStreaming;
-        if (cudaStreamSetAttribute(s, cudaStreamAttributeAccessPolicyWindow, &v) != cudaSuccess) {
-            cudaGetLastError();
-            return;
-        }
-        on = true;
-        ctx->st_l2 = 1;
-    }
-    ~L2Window()
-    {
-        if (on && cudaStreamSetAttribute(s, cudaStreamAttributeAccessPolicyWindow, &prev) != cudaSuccess)
-            cudaGetLastError();
-    }
-};
+Launch launch_on(ckv_ctx* ctx, cudaStream_t s)
+{
+    const bool window = ctx->opt_l2 && ctx->l2_window > 0;
+    ctx->st_l2 = window;
+    return Launch{s, window ? &ctx->window : nullptr, &ctx->grants};
+}
 
 bool offsets_ok32(const int32_t* off, int32_t n)
 {
@@ -1170,13 +1183,14 @@ namespace {
 // on B200 a warp spends about 100 clocks per TMA gather instruction it issues, so with the compute warps doing
 // their own gathers the TMA loader measured slower (cfg4: 607 against 522 us; cfg5, Zipf indices that profit
 // from L1, which TMA bypasses: 5.07 against 2.37 ms).  Both loaders give the same bits.
-ckv_status run_mma(ckv_ctx* ctx, int D, int max_M, const AttendArgs& a, cudaStream_t s)
+ckv_status run_mma(ckv_ctx* ctx, int D, int max_M, int parts, const AttendArgs& a, const InlineTable* tab,
+                   const Launch& l)
 {
     const int loader = ctx->opt_loader == 2 ? 2 : 1;
     // the TMA loader serves the plain form only (both sides shared, no visible lengths)
     if (loader == 2 && (!ctx->has_tma || a.cv.full_k || a.cv.full_v || a.vis)) return CKV_ERR_UNSUPPORTED;
     ctx->st_loader = loader;
-    CK(launch_attend_mma(D, max_M, a, loader == 2 ? ctx->tmaps : nullptr, ctx->d_err, s));
+    CK(launch_attend_mma(D, max_M, parts, a, tab, loader == 2 ? ctx->tmaps : nullptr, ctx->d_err, l));
     return CKV_OK;
 }
 
@@ -1204,6 +1218,66 @@ cudaError_t pipe_prepare(ckv_ctx* ctx)
     return e;
 }
 
+// A short request list as kernel arguments: nothing is planned, uploaded or kept for it.
+struct InlineList {
+    InlineTable tab;
+    int32_t n = 0, max_M = 0, parts = 1, family = 0;
+};
+
+// Fills `x`; x.family stays 0 if the list has to go through a plan (too long, or a kernel family or a chunking that
+// works from tables in device memory).
+ckv_status inline_list(ckv_ctx* ctx, int32_t n, const int64_t* users, const int32_t* q_off, bool with_vis, InlineList& x)
+{
+    if (n > kInlineReqs || ctx->opt_split > 0 || ctx->opt_kernel > 2 || ctx->opt_loader == 2) return CKV_OK;
+    int64_t total_pos = 0;
+    int32_t max_L = 0, min_L = INT32_MAX;
+    bool all_single = true;
+    for (int32_t k = 0; k < n; ++k) {
+        const UserEntry* f = ctx->users.find(users[k]);
+        if (!f) return CKV_ERR_UNKNOWN_USER;
+        const int32_t M = q_off[k + 1] - q_off[k];
+        if (M <= 0) continue;
+        x.tab.r[x.n++] = InlineReq{(uint32_t)(f->base >> 5), f->L, q_off[k], M};
+        total_pos += f->L;
+        max_L = std::max(max_L, f->L);
+        min_L = std::min(min_L, f->L);
+        x.max_M = std::max(x.max_M, M);
+        all_single = all_single && M == 1;
+    }
+    const int family = choose_family(ctx, with_vis, n, x.n, total_pos, x.max_M, max_L, all_single);
+    if ((family != 1 && family != 2) || auto_split_len(ctx, total_pos, family, x.max_M, max_L) < max_L) return CKV_OK;
+    if (family == 2) {
+        int64_t tiles = 0;
+        const int qpw = mma_queries_per_warp(ctx->cfg.head_dim, x.max_M);
+        for (int32_t k = 0; k < x.n; ++k)
+            tiles += (int64_t)((x.tab.r[k].L + 31) / 32) * ((x.tab.r[k].M + qpw - 1) / qpw);
+        x.parts = mma_parts(ctx, tiles, (max_L + 31) / 32, x.max_M);
+    }
+    // longest first, as in a plan: the tail of the grid is made of short ones
+    if (max_L != min_L && (int64_t)x.n * ctx->cfg.n_groups > ctx->n_sms)
+        std::sort(x.tab.r, x.tab.r + x.n, [](const InlineReq& a, const InlineReq& b) { return a.L > b.L; });
+    x.family = family;
+    return CKV_OK;
+}
+
+// The launches between two optional timing events.
+template <typename F>
+ckv_status timed(ckv_ctx* ctx, bool time_it, cudaStream_t s, F&& attend)
+{
+    ctx->ev_valid = false;
+    if (time_it) {
+        for (auto& e : ctx->ev)
+            if (!e) CK(cudaEventCreate(&e));
+        CK(cudaEventRecord(ctx->ev[0], s));
+    }
+    const ckv_status st = attend();
+    if (st != CKV_OK || !time_it) return st;
+    CK(cudaEventRecord(ctx->ev[1], s));
+    CK(cudaEventRecord(ctx->ev[2], s));
+    ctx->ev_valid = true;
+    return CKV_OK;
+}
+
 // The kernels of one slice of a plan (items [i0, i1), split requests [s0, s1)) on stream s.
 ckv_status launch_slice(ckv_ctx* ctx, const Plan* pl, AttendArgs a, int i0, int i1, int s0, int s1, bool time_it,
                         cudaStream_t s)
@@ -1212,26 +1286,27 @@ ckv_status launch_slice(ckv_ctx* ctx, const Plan* pl, AttendArgs a, int i0, int 
     a.items = pl->d_items + i0;
     a.works = pl->d_works ? pl->d_works + i0 : nullptr;
     a.n_items = i1 - i0;
-    L2Window l2(ctx, s);
+    a.inl = 0;
+    const Launch l = launch_on(ctx, s);
     if (time_it) CK(cudaEventRecord(ctx->ev[0], s));
     if (a.n_items > 0) {
         if (pl->family == 4) {
             float* tw = (float*)ctx->partials.p;
             CK(launch_attend_fact(D, a, pl->n_req, pl->max_L, ctx->n_sms, tw,
-                                  tw + (size_t)pl->n_req * G * fact_row_floats(ctx->n_entries), s));
+                                  tw + (size_t)pl->n_req * G * fact_row_floats(ctx->n_entries), l));
             ctx->st_launches += 2;
         } else if (pl->family == 3)
-            CK(launch_attend_umma(pl->max_M, a, ctx->n_sms, ctx->d_err, s));
+            CK(launch_attend_umma(pl->max_M, a, ctx->n_sms, ctx->d_err, l));
         else if (pl->family == 2) {
-            ckv_status st2 = run_mma(ctx, D, pl->max_M, a, s);
+            ckv_status st2 = run_mma(ctx, D, pl->max_M, pl->parts, a, nullptr, l);
             if (st2 != CKV_OK) return st2;
         } else
-            CK(launch_attend_simt(ctx->cfg.dtype, D, pl->max_M, a, s));
+            CK(launch_attend_simt(ctx->cfg.dtype, D, pl->max_M, simt_wide(ctx, a.n_items), a, nullptr, l));
         ctx->st_launches++;
     }
     if (time_it) CK(cudaEventRecord(ctx->ev[1], s));
     if (s1 > s0) {
-        CK(launch_combine(D, a, pl->d_split + s0, s1 - s0, s));
+        CK(launch_combine(D, a, pl->d_split + s0, s1 - s0, l));
         ctx->st_launches++;
     }
     if (time_it) CK(cudaEventRecord(ctx->ev[2], s));
@@ -1315,6 +1390,51 @@ ckv_status attend_impl(ckv_ctx* ctx, int32_t n, const int64_t* users, const int3
         CK(cudaMemcpyAsync(ctx->stage_q.p, queries, q_bytes, cudaMemcpyHostToDevice, s));
     }
 
+    const auto fill_args = [&](AttendArgs& a) {
+        a.cv = view_of(ctx);
+        a.reqs = nullptr;
+        a.items = nullptr;
+        a.works = nullptr;
+        a.n_items = a.inl = 0;
+        a.queries = d_q;
+        a.vis = d_vis;
+        a.vmax = nullptr;
+        a.out = d_out;
+        a.partials = nullptr;
+        a.out_dtype = ctx->cfg.out_dtype;
+        a.mode = ctx->cfg.mode;
+        a.scale = ctx->scale;
+        a.arena_units = ctx->cap_units;
+        a.q_rows = Q;
+        a.part_rows = 0;
+        a.err = ctx->d_err;
+    };
+    if (n_ranges == 1) {
+        InlineList x;
+        ckv_status st = inline_list(ctx, n, users, q_off, vis != nullptr, x);
+        if (st != CKV_OK) return st;
+        if (x.family != 0) {
+            ctx->st_items = x.n;
+            ctx->st_split = ctx->st_ws = ctx->st_hit = 0;
+            ctx->st_kernel = x.family;
+            if (Q == 0) return CKV_OK;
+            AttendArgs a;
+            fill_args(a);
+            a.n_items = x.n;
+            a.inl = 1;
+            const Launch l = launch_on(ctx, s);
+            st = timed(ctx, ctx->opt_time != 0, s, [&]() -> ckv_status {
+                if (x.family == 2) return run_mma(ctx, D, x.max_M, x.parts, a, &x.tab, l);
+                CK(launch_attend_simt(ctx->cfg.dtype, D, x.max_M, simt_wide(ctx, x.n), a, &x.tab, l));
+                return CKV_OK;
+            });
+            if (st != CKV_OK) return st;
+            ctx->st_launches = 1;
+            if (o_host) CK(cudaMemcpyAsync(out, d_out, o_bytes, cudaMemcpyDeviceToHost, s));
+            return CKV_OK;
+        }
+    }
+
     Plan* pl = nullptr;
     ckv_status st = get_plan(ctx, n, users, q_off, vis != nullptr, n_ranges, r_user, s, &pl);
     if (st != CKV_OK) {
@@ -1339,23 +1459,13 @@ ckv_status attend_impl(ckv_ctx* ctx, int32_t n, const int64_t* users, const int3
     ctx->st_ws = (int64_t)ws;
 
     AttendArgs a;
-    a.cv = view_of(ctx);
+    fill_args(a);
     a.reqs = pl->d_reqs;
     a.items = pl->d_items;
-    a.works = pl->d_works;
     a.n_items = pl->n_items;
-    a.queries = d_q;
-    a.vis = d_vis;
-    a.vmax = nullptr;
-    a.out = d_out;
     a.partials = (float*)ctx->partials.p;
-    a.out_dtype = ctx->cfg.out_dtype;
-    a.mode = ctx->cfg.mode;
-    a.scale = ctx->scale;
-    a.arena_units = ctx->cap_units;
-    a.q_rows = Q;
+    a.works = pl->d_works;
     a.part_rows = pl->family == 4 ? 0 : pl->part_rows;
-    a.err = ctx->d_err;
     ctx->ev_valid = false;
     if (d_vis && pl->family == 3 && pl->n_items > 0) {
         // the tcgen05 kernel's roles skip what lies behind every row's limit: the largest limit per block of queries
@@ -1775,7 +1885,7 @@ extern "C" ckv_status ckv_attend_static(ckv_ctx* ctx, int32_t n, const int64_t* 
     else if (ctx->opt_kernel == 1) family = 1;
     else if (ctx->opt_kernel == 2 && ctx->has_mma) family = 2;
     else return CKV_ERR_UNSUPPORTED;
-    const int64_t C = ctx->opt_split > 0 ? ctx->opt_split : auto_split_len(ctx, total_pos, family, max_M);
+    const int64_t C = ctx->opt_split > 0 ? ctx->opt_split : auto_split_len(ctx, total_pos, family, max_M, INT32_MAX);
     const int64_t row_floats = (int64_t)G * (D + 2);
     const int64_t cap_rows = (int64_t)((kStaticBytes - kOffPartials) / sizeof(float)) / row_floats;
     int32_t n_items = 0, n_split = 0;
@@ -1814,6 +1924,7 @@ extern "C" ckv_status ckv_attend_static(ckv_ctx* ctx, int32_t n, const int64_t* 
     a.items = (const Item*)(base + kOffItems);
     a.works = nullptr;
     a.n_items = n_items;
+    a.inl = 0;
     a.queries = queries;
     a.vis = nullptr;
     a.vmax = nullptr;
@@ -1826,12 +1937,13 @@ extern "C" ckv_status ckv_attend_static(ckv_ctx* ctx, int32_t n, const int64_t* 
     a.q_rows = Q;
     a.part_rows = part_rows;
     a.err = ctx->d_err;
+    const Launch l{s, nullptr, &ctx->grants};
     if (n_items > 0) {
         if (family == 2)
-            CK(launch_attend_mma(D, max_M, a, nullptr, ctx->d_err, s));
+            CK(launch_attend_mma(D, max_M, 1, a, nullptr, nullptr, ctx->d_err, l));
         else
-            CK(launch_attend_simt(ctx->cfg.dtype, D, max_M, a, s));
+            CK(launch_attend_simt(ctx->cfg.dtype, D, max_M, simt_wide(ctx, n_items), a, nullptr, l));
     }
-    if (n_split > 0) CK(launch_combine(D, a, (const int32_t*)(base + kOffSplit), n_split, s));
+    if (n_split > 0) CK(launch_combine(D, a, (const int32_t*)(base + kOffSplit), n_split, l));
     return CKV_OK;
 }

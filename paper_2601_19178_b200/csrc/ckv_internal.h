@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <utility>
+
 #include "ckv.h"
 
 namespace ckv {
@@ -26,6 +28,17 @@ struct Item {
     int32_t begin;     // first position of the chunk
     int32_t len;       // positions in the chunk (0 only for an empty history)
     int32_t part_row;  // first row of this chunk's partial results, or -1: write `out`
+};
+
+// A whole request as a kernel argument: short request lists travel with the launch instead of through tables in
+// device memory (no upload, nothing to wait for).  Arena units are handed out in multiples of 32, Lpad is L rounded up.
+struct InlineReq {
+    uint32_t base32;   // Req::base / 32
+    int32_t L, q0, M;
+};
+constexpr int kInlineReqs = 224;  // with AttendArgs just under the 4 KB of kernel arguments that every launch can take
+struct InlineTable {
+    InlineReq r[kInlineReqs];
 };
 
 // An Item merged with its request row, for kernels that read their work list once per unit
@@ -62,6 +75,7 @@ struct AttendArgs {
     const Item* items;
     const Work* works;     // one per item, same order (tcgen05 family only, else null)
     int32_t n_items;
+    int32_t inl;           // the requests are kernel arguments (InlineTable), one unsplit item each; reqs and items are null
     const void* queries;   // [Q][G][D]
     const int32_t* vis;    // null, or per query row the number of leading history positions it attends [Q]
     const int32_t* vmax;   // tcgen05 family with visible lengths: largest limit per (request, block of 128 queries)
@@ -76,6 +90,63 @@ struct AttendArgs {
     int64_t part_rows;     // rows of `partials`
     int* err;              // device error word (the context's)
 };
+
+// How a launcher launches: stream, the access-policy window over the pool (null: none) as a launch attribute, and the
+// context's record of which kernels have been allowed how much dynamic shared memory (the permission belongs to the
+// device the context sits on, so it is asked for once per context and kernel, not once per launch).
+struct SmemGrants {
+    static constexpr int kMax = 48;
+    const void* fn[kMax];
+    size_t bytes[kMax];
+    int n = 0;
+};
+struct Launch {
+    cudaStream_t s;
+    const cudaAccessPolicyWindow* window;
+    SmemGrants* grants;
+};
+inline cudaError_t grant_smem(SmemGrants* g, const void* fn, size_t bytes)
+{
+    if (bytes <= 48 * 1024) return cudaSuccess;
+    int i = 0;
+    if (g) {
+        while (i < g->n && g->fn[i] != fn) ++i;
+        if (i < g->n && g->bytes[i] >= bytes) return cudaSuccess;
+    }
+    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess && g && i < SmemGrants::kMax) {
+        g->fn[i] = fn;
+        g->bytes[i] = bytes;
+        if (i == g->n) ++g->n;
+    }
+    return e;
+}
+// cluster: thread blocks per cluster along x (1: none)
+template <typename... P, typename... A>
+cudaError_t launch_kernel(const Launch& l, void (*fn)(P...), dim3 grid, int threads, size_t smem, int cluster, A&&... args)
+{
+    cudaError_t e = grant_smem(l.grants, (const void*)fn, smem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute at[2];
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = dim3((unsigned)threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = l.s;
+    c.attrs = at;
+    if (cluster > 1) {
+        at[c.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        at[c.numAttrs].val.clusterDim.x = (unsigned)cluster;
+        at[c.numAttrs].val.clusterDim.y = at[c.numAttrs].val.clusterDim.z = 1;
+        ++c.numAttrs;
+    }
+    if (l.window) {
+        at[c.numAttrs].id = cudaLaunchAttributeAccessPolicyWindow;
+        at[c.numAttrs].val.accessPolicyWindow = *l.window;
+        ++c.numAttrs;
+    }
+    return cudaLaunchKernelEx(&c, fn, std::forward<A>(args)...);
+}
 
 // ---- kernels_pack.cu
 cudaError_t launch_pool_layout(int dtype, int G, int m, int d_shared, int D, const void* src,
@@ -103,18 +174,23 @@ cudaError_t launch_check_indices(int idx_bytes, int n_entries, const void* idxK,
                                  int* bad_flag, cudaStream_t s);
 
 // ---- kernels_simt.cu : CUDA-core family (any number of queries, best for few)
-cudaError_t launch_attend_simt(int dtype, int D, int max_M, const AttendArgs& a, cudaStream_t s);
+// tab: the requests when a.inl is set.  wide: blocks of more warps (few blocks, each with a history to itself)
+cudaError_t launch_attend_simt(int dtype, int D, int max_M, bool wide, const AttendArgs& a, const InlineTable* tab,
+                               const Launch& l);
 // Merges the partial results of split requests into `out`.
-cudaError_t launch_combine(int D, const AttendArgs& a, const int32_t* split_reqs, int n_split,
-                           cudaStream_t s);
+cudaError_t launch_combine(int D, const AttendArgs& a, const int32_t* split_reqs, int n_split, const Launch& l);
 
 // ---- kernels_mma.cu : warp-level tensor-core family (bf16, head_dim 32 or 64, d_user <= 8)
 bool mma_supported(int dtype, int head_dim, int d_user);  // d_user of the shared side(s)
 int mma_queries_per_warp(int head_dim, int max_M);
 // tensor_maps: null = fill the staging ring with cp.async copies; else the two maps of make_pool_tensor_maps =
 // fill it with TMA gathers (err_flag: device int, OR-ed with a code if a bounded wait for a tile ran out).
-cudaError_t launch_attend_mma(int head_dim, int max_M, const AttendArgs& a, const void* tensor_maps, int* err_flag,
-                              cudaStream_t s);
+// parts: warps that share one (item, group, query block), a power of two up to kMmaMaxParts; more than four lie in a
+// cluster of thread blocks.  tab: the requests when a.inl is set (cp.async loader only).
+constexpr int kMmaMaxParts = 32;
+cudaError_t launch_attend_mma(int head_dim, int max_M, int parts, const AttendArgs& a, const InlineTable* tab,
+                              const void* tensor_maps, int* err_flag, const Launch& l);
+int mma_warps_per_sm(int head_dim, int max_M);
 bool make_pool_tensor_maps(int head_dim, int64_t rows, const void* poolK, const void* poolV, void* maps_out);
 
 // ---- kernels_fact.cu : pool-side factorisation for one query per user (bf16, head_dim 32 or 64, d_user <= 8)
@@ -126,7 +202,7 @@ int fact_row_floats(int n_entries);
 // a.items: one unsplit item per request with a query.  tw: [n_req][G][fact_row_floats(n_entries)] floats,
 // aux: [n_req][G][fact_aux_floats()].
 cudaError_t launch_attend_fact(int head_dim, const AttendArgs& a, int n_req, int max_L, int n_sms, float* tw,
-                               float* aux, cudaStream_t s);
+                               float* aux, const Launch& l);
 
 // ---- kernels_route.cu : prefill router, fused scores + row arg-max (bf16, d_in 32 / 64 / 128)
 bool route_supported(int d_in);
@@ -149,7 +225,7 @@ cudaError_t launch_project(int d_in, int d_out, int G, const void* x, const void
 bool umma_supported(int dtype, int head_dim, int d_user, int idx_bytes);
 // err_flag: device int, OR-ed with a non-zero code if a bounded wait inside the kernel ran out.
 // Persistent: one CTA per SM (n_sms of them at most).
-cudaError_t launch_attend_umma(int max_M, const AttendArgs& a, int n_sms, int* err_flag, cudaStream_t s);
+cudaError_t launch_attend_umma(int max_M, const AttendArgs& a, int n_sms, int* err_flag, const Launch& l);
 // Fills vmax (one int per request and block of 128 queries, at Work::pad[0] + block) from a.vis; a.works as for the attend.
 cudaError_t launch_vis_block_max(const AttendArgs& a, int32_t* vmax, cudaStream_t s);
 

@@ -465,45 +465,27 @@ __global__ void __launch_bounds__(kOutWarps * 32, 1)
     }
 }
 
-// Opt-in to large dynamic shared memory (per launch: the attribute belongs to the current device).
-template <typename K>
-cudaError_t set_smem(K kernel, size_t bytes)
-{
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 template <int D>
-cudaError_t launch_fact(const AttendArgs& a, int n_req, int max_L, int n_sms, float* tw, float* aux, cudaStream_t s)
+cudaError_t launch_fact(const AttendArgs& a, int n_req, int max_L, int n_sms, float* tw, float* aux, const Launch& l)
 {
     const int m = a.cv.n_entries, G = a.cv.n_groups;
     const bool i16 = a.cv.idx_bytes == 2, soft = a.mode == CKV_SOFTMAX;
-    fact_table_kernel<D><<<dim3((m + 255) / 256, (n_req + 16 * kTableMT - 1) / (16 * kTableMT), G), 128, 0, s>>>(
-        a, n_req, tw);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_kernel(l, fact_table_kernel<D>,
+                                  dim3((m + 255) / 256, (n_req + 16 * kTableMT - 1) / (16 * kTableMT), G), 128, 0, 1, a, n_req, tw);
     if (e != cudaSuccess) return e;
     const int s_cap = std::max((max_L + 31) / 32 * 32, 9 * (kMainThreads / 32));  // scores; later the warps' sums
     const size_t smem_main = (2 * (size_t)m + s_cap + 32) * sizeof(float);
     const int n_pairs = a.n_items * G;
     const dim3 grid(n_pairs < n_sms ? n_pairs : n_sms);
-#define CKV_FACT_MAIN(MODE, I16)                                                       \
-    do {                                                                               \
-        e = set_smem(fact_main_kernel<D, MODE, I16>, smem_main);                       \
-        if (e != cudaSuccess) return e;                                                \
-        fact_main_kernel<D, MODE, I16><<<grid, kMainThreads, smem_main, s>>>(a, tw, aux, s_cap); \
-    } while (0)
-    if (soft) {
-        if (i16) CKV_FACT_MAIN(CKV_SOFTMAX, true); else CKV_FACT_MAIN(CKV_SOFTMAX, false);
-    } else {
-        if (i16) CKV_FACT_MAIN(CKV_SILU_OVER_L, true); else CKV_FACT_MAIN(CKV_SILU_OVER_L, false);
-    }
+#define CKV_FACT_MAIN(MODE, I16) \
+    launch_kernel(l, fact_main_kernel<D, MODE, I16>, grid, kMainThreads, smem_main, 1, a, tw, aux, s_cap)
+    if (soft) e = i16 ? CKV_FACT_MAIN(CKV_SOFTMAX, true) : CKV_FACT_MAIN(CKV_SOFTMAX, false);
+    else e = i16 ? CKV_FACT_MAIN(CKV_SILU_OVER_L, true) : CKV_FACT_MAIN(CKV_SILU_OVER_L, false);
 #undef CKV_FACT_MAIN
-    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const size_t smem_out = std::max((size_t)kOutWarps * 2 * 32 * D * 2, (size_t)kOutWarps * 16 * D * sizeof(float));
-    e = set_smem(fact_out_kernel<D>, smem_out);
-    if (e != cudaSuccess) return e;
-    fact_out_kernel<D><<<dim3((n_req + 15) / 16, G), kOutWarps * 32, smem_out, s>>>(a, n_req, tw, aux);
-    return cudaGetLastError();
+    return launch_kernel(l, fact_out_kernel<D>, dim3((n_req + 15) / 16, G), kOutWarps * 32, smem_out, 1, a, n_req,
+                         (const float*)tw, (const float*)aux);
 }
 
 }  // namespace
@@ -523,11 +505,11 @@ int fact_row_floats(int n_entries) { return row_floats(n_entries); }
 // Three launches; a.items holds one unsplit item per request with a query; tw: [n_req][G][fact_row_floats()] floats,
 // aux: [n_req][G][fact_aux_floats()] floats.
 cudaError_t launch_attend_fact(int D, const AttendArgs& a, int n_req, int max_L, int n_sms, float* tw, float* aux,
-                               cudaStream_t s)
+                               const Launch& l)
 {
     if (a.n_items == 0) return cudaSuccess;
-    return D == 64 ? launch_fact<64>(a, n_req, max_L, n_sms, tw, aux, s)
-                   : launch_fact<32>(a, n_req, max_L, n_sms, tw, aux, s);
+    return D == 64 ? launch_fact<64>(a, n_req, max_L, n_sms, tw, aux, l)
+                   : launch_fact<32>(a, n_req, max_L, n_sms, tw, aux, l);
 }
 
 }  // namespace ckv

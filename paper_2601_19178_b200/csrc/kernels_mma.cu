@@ -13,6 +13,12 @@
 // arena; they are copied into the ring in place of pool rows (cp.async loader only) and nothing is
 // patched.  With visible lengths a query row only takes the positions before its own limit.
 //
+// Several warps may share one (item, group, query block): `parts` of them, a power of two, take its 32-position
+// tiles in turn and merge their (m, l, O) at the end, through shared memory inside a block and through distributed
+// shared memory between the blocks of a cluster.  What bounds a small call is the chain index -> row -> product of
+// one warp times the tiles it walks, so the tiles are spread until every SM has warps; a call needs no second launch
+// and no partial results in device memory for it.
+//
 // Two ways to fill the ring (template parameter TMA), same results bit for bit:
 //   - 16-byte cp.async copies through L1 (hot rows of skewed index distributions stay in L1, but every
 //     row crosses the L1 / shared-memory data pipe on the way in and again on the way out);
@@ -21,6 +27,8 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <math_constants.h>
+
+#include <type_traits>
 
 #include "ckv_internal.h"
 #include "ptx_helpers.cuh"
@@ -131,23 +139,62 @@ __device__ __forceinline__ int swz(int r)
     return D == 64 ? (r & 7) : ((r >> 1) & 3);
 }
 
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// a 32-bit word of another block of the cluster, at this block's shared-memory address `addr`
+__device__ __forceinline__ float ld_cluster(uint32_t addr, uint32_t rank)
+{
+    uint32_t remote;
+    float v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(remote) : "memory");
+    return v;
+}
+
+struct TmaMaps {
+    CUtensorMap K, V;
+};
+
 // VAR = false: both sides shared and no visible lengths (the hot configurations); the code for the variants is
-// compiled out.
-template <int D, int MT, int MODE, bool IDX16, bool TMA, bool VAR>
+// compiled out.  SHARED = false: one warp per unit.
+template <int D, int MT, int MODE, bool IDX16, bool TMA, bool VAR, bool SHARED>
 __global__ void __launch_bounds__(128, MmaCfg<D, MT, TMA>::MIN_BLOCKS)
-    attend_mma_kernel(const AttendArgs a, int n_mb, const __grid_constant__ CUtensorMap tmK,
-                      const __grid_constant__ CUtensorMap tmV, int* err_flag)
+    attend_mma_kernel(const __grid_constant__ AttendArgs a, int n_mb, int log_wpu, int n_cta, int* err_flag,
+                      const __grid_constant__ std::conditional_t<TMA, TmaMaps, InlineTable> tab)
 {
     using C = MmaCfg<D, MT, TMA>;
     constexpr int NTD = D / 8, KS = D / 16, ROWB = C::ROWB, CPR = C::CPR, RPI = C::RPI, NST = C::NST;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, t = lane & 3;
-    const int64_t wid = (int64_t)blockIdx.x * C::WARPS + warp;
-    if (wid >= (int64_t)a.n_items * n_mb) return;
-    const Item it = a.items[wid / n_mb];
-    const int mb = (int)(wid % n_mb);
-    const Req rq = a.reqs[it.req];
+    // 2^log_wpu warps of a block and the n_cta blocks of its cluster share a unit; this warp is number `part` of
+    // `parts` and takes tiles part, part + parts, ... of the chunk
+    if constexpr (!SHARED) {
+        log_wpu = 0;
+        n_cta = 1;
+    }
+    const int wpu = 1 << log_wpu, sub = warp & (wpu - 1), parts = wpu * n_cta;
+    const uint32_t rank = n_cta > 1 ? blockIdx.x % (uint32_t)n_cta : 0;
+    const int part = (int)rank * wpu + sub;
+    const int64_t uid = ((int64_t)(n_cta > 1 ? blockIdx.x / (uint32_t)n_cta : blockIdx.x) * C::WARPS + warp) >> log_wpu;
+    if (uid >= (int64_t)a.n_items * n_mb) return;
+    const int item = (int)(uid / n_mb), mb = (int)(uid - (int64_t)item * n_mb);
+    Item it;
+    Req rq;
+    bool from_table = false;
+    if constexpr (!TMA) from_table = a.inl != 0;
+    if (from_table) {
+        if constexpr (!TMA) {
+            const InlineReq& r = tab.r[item];
+            rq = Req{(int64_t)r.base32 * 32, r.L, (r.L + 31) & ~31, r.q0, r.M, -1, 1};
+            it = Item{item, 0, r.L, -1};
+        }
+    } else {
+        it = a.items[item];
+        rq = a.reqs[it.req];
+    }
     const int row0 = mb * 16 * MT;
     if (row0 >= rq.M) return;
     const int grp = blockIdx.y, G = a.cv.n_groups, d_user = a.cv.d_user;
@@ -213,17 +260,20 @@ __global__ void __launch_bounds__(128, MmaCfg<D, MT, TMA>::MIN_BLOCKS)
     const int cr = lane / CPR, cc = lane % CPR;  // this lane's row within a copy instruction and its chunk
     const char* pK = reinterpret_cast<const char*>(a.cv.poolK) + (int64_t)grp * a.cv.n_entries * ROWB + cc * 16;
     const char* pV = reinterpret_cast<const char*>(a.cv.poolV) + (int64_t)grp * a.cv.n_entries * ROWB + cc * 16;
-    const int64_t unit0 = rq.base + (int64_t)grp * rq.Lpad + it.begin + lane;  // this lane's position of step 0
-    (void)CKV_CLAMP(unit0 - lane + ((it.len + 31) & ~31) - 1, a.arena_units, err_flag);  // the chunk's last (padded) unit
+    const int64_t chunk0 = rq.base + (int64_t)grp * rq.Lpad + it.begin;  // the chunk's first unit
+    (void)CKV_CLAMP(chunk0 + ((it.len + 31) & ~31) - 1, a.arena_units, err_flag);  // the chunk's last (padded) unit
+    const int64_t unit0 = chunk0 + 32 * part + lane;  // this lane's position of step 0
+    const int stride = 32 * parts;                    // positions between two of this warp's steps
     const uint16_t* uK = reinterpret_cast<const uint16_t*>(a.cv.userK);
     const uint16_t* uV = reinterpret_cast<const uint16_t*>(a.cv.userV);
     const int end = VAR ? min(it.begin + it.len, lim_max) : it.begin + it.len;  // nothing behind the last visible position is touched
-    const int nsteps = VAR ? (end > it.begin ? (end - it.begin + 31) >> 5 : 0) : (it.len + 31) >> 5;
+    const int n_tiles = VAR ? (end > it.begin ? (end - it.begin + 31) >> 5 : 0) : (it.len + 31) >> 5;
+    const int nsteps = n_tiles > part ? (n_tiles - part + parts - 1) >> (log_wpu + (31 - __clz(n_cta))) : 0;
     const int full_end = VAR ? min(end, lim_min) : end;  // up to here every row of this warp sees every position
     // A side that is not shared: its rows are the chunk's own units in the arena, and what stands in for the pool
-    // index of the position in lane l of tile `step` is its offset 32 step + l from the chunk's first unit.
-    if (full_k) pK = reinterpret_cast<const char*>(a.cv.userK) + (unit0 - lane) * ROWB + cc * 16;
-    if (full_v) pV = reinterpret_cast<const char*>(a.cv.userV) + (unit0 - lane) * ROWB + cc * 16;
+    // index of the position in lane l of a tile is its offset from the chunk's first unit.
+    if (full_k) pK = reinterpret_cast<const char*>(a.cv.userK) + chunk0 * ROWB + cc * 16;
+    if (full_v) pV = reinterpret_cast<const char*>(a.cv.userV) + chunk0 * ROWB + cc * 16;
     const float sc = a.scale * (MODE == CKV_SOFTMAX ? kLog2e : 0.5f);
 
     uint32_t smem0 = smem_u32(smem_raw);
@@ -276,7 +326,7 @@ __global__ void __launch_bounds__(128, MmaCfg<D, MT, TMA>::MIN_BLOCKS)
                 }
             }
             if (lane < 16) {
-                const CUtensorMap* tm = lane < 8 ? &tmK : &tmV;
+                const CUtensorMap* tm = lane < 8 ? &tab.K : &tab.V;
                 const uint32_t dst = (lane < 8 ? kt : vt) + j4 * ROWB;
                 asm volatile(
                     "cp.async.bulk.tensor.2d.shared::cluster.global.tile::gather4.mbarrier::complete_tx::bytes "
@@ -301,16 +351,16 @@ __global__ void __launch_bounds__(128, MmaCfg<D, MT, TMA>::MIN_BLOCKS)
     };
     auto fetch_idx = [&](int step, int& idx_k, int& idx_v) {
         if (step < nsteps) {
-            idx_k = full_k ? 32 * step + lane : load_index<IDX16>(a.cv.idxK, unit0 + 32 * step);
-            idx_v = full_v ? 32 * step + lane : load_index<IDX16>(a.cv.idxV, unit0 + 32 * step);
+            idx_k = full_k ? 32 * part + stride * step + lane : load_index<IDX16>(a.cv.idxK, unit0 + stride * step);
+            idx_v = full_v ? 32 * part + stride * step + lane : load_index<IDX16>(a.cv.idxV, unit0 + stride * step);
         } else {
             idx_k = idx_v = 0;
         }
     };
     auto fetch_user = [&](int step, uint4& k, uint4& v) {
         if (wide_user && step < nsteps) {
-            if (!full_k) k = load_user_part(uK, unit0 + 32 * step, d_user);
-            if (!full_v) v = load_user_part(uV, unit0 + 32 * step, d_user);
+            if (!full_k) k = load_user_part(uK, unit0 + stride * step, d_user);
+            if (!full_v) v = load_user_part(uV, unit0 + stride * step, d_user);
         }
     };
 
@@ -332,7 +382,7 @@ __global__ void __launch_bounds__(128, MmaCfg<D, MT, TMA>::MIN_BLOCKS)
 
     bool ok = true;
     for (int step = 0; step < nsteps; ++step) {
-        const int p0 = it.begin + 32 * step;
+        const int p0 = it.begin + 32 * part + stride * step;
         if (step + NST - 1 < nsteps) issue(step + NST - 1, ikA, ivA);
         if constexpr (!TMA) cp_async_commit();
         ikA = ikB; ivA = ivB; ikB = ikC; ivB = ivC;
@@ -364,11 +414,11 @@ __global__ void __launch_bounds__(128, MmaCfg<D, MT, TMA>::MIN_BLOCKS)
         } else if (d_user > 0 && !(full_k && full_v)) {
             for (int e = 0; e < d_user; ++e) {
                 if (!full_k) {
-                    const uint16_t xk = __ldg(uK + (unit0 + 32 * step) * d_user + e);
+                    const uint16_t xk = __ldg(uK + (unit0 + stride * step) * d_user + e);
                     asm volatile("st.shared.u16 [%0], %1;" ::"r"(kt + offU + 2 * e), "h"(xk) : "memory");
                 }
                 if (!full_v) {
-                    const uint16_t xv = __ldg(uV + (unit0 + 32 * step) * d_user + e);
+                    const uint16_t xv = __ldg(uV + (unit0 + stride * step) * d_user + e);
                     asm volatile("st.shared.u16 [%0], %1;" ::"r"(vt + offU + 2 * e), "h"(xv) : "memory");
                 }
             }
@@ -500,12 +550,85 @@ __global__ void __launch_bounds__(128, MmaCfg<D, MT, TMA>::MIN_BLOCKS)
         __syncwarp();
     }
     if constexpr (TMA) {
-        if (!ok) {
-            if (lane == 0) atomicOr(err_flag, ERR_MMA_LOAD);
-            return;
-        }
+        // (a warp that gave up still takes part in the merge: the error word says that the outputs are not valid)
+        if (!ok && lane == 0) atomicOr(err_flag, ERR_MMA_LOAD);
     } else {
         cp_async_wait<0>();
+    }
+
+    // merge the parts of the unit: registers as they are, value i of lane l at [i][l] of the giving warp's own ring
+    if constexpr (SHARED) {
+        constexpr int FR = NTD * 4 + 4;
+        static_assert(FR * 128 <= NST * 2 * C::TILE_B, "a fragment fits the warp's ring");
+        auto give = [&](int mt) {
+            const uint32_t p = ring + lane * 4;
+            auto put = [&](int i, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(p + i * 128), "f"(v) : "memory"); };
+            put(0, m_run[mt][0]);
+            put(1, m_run[mt][1]);
+            put(2, l_run[mt][0]);
+            put(3, l_run[mt][1]);
+#pragma unroll
+            for (int i = 0; i < NTD * 4; ++i) put(4 + i, o[mt][i >> 2][i & 3]);
+        };
+        auto take = [&](int mt, auto&& get) {
+            if constexpr (MODE == CKV_SOFTMAX) {
+                float ca[2], cb[2];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const float m2 = get(h), mn = fmaxf(m_run[mt][h], m2), ms = mn == -CUDART_INF_F ? 0.f : mn;
+                    ca[h] = ex2(m_run[mt][h] - ms);
+                    cb[h] = ex2(m2 - ms);
+                    m_run[mt][h] = mn;
+                    l_run[mt][h] = l_run[mt][h] * ca[h] + get(2 + h) * cb[h];
+                }
+#pragma unroll
+                for (int i = 0; i < NTD * 4; ++i) {
+                    float& x = o[mt][i >> 2][i & 3];
+                    x = x * ca[(i >> 1) & 1] + get(4 + i) * cb[(i >> 1) & 1];
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < NTD * 4; ++i) o[mt][i >> 2][i & 3] += get(4 + i);
+            }
+        };
+        auto unit_sync = [&]() {
+            if (log_wpu == 2) asm volatile("bar.sync 1, 128;" ::: "memory");
+            else if (log_wpu == 1) asm volatile("bar.sync %0, 64;" ::"r"(2 + (warp >> 1)) : "memory");
+        };
+        constexpr uint32_t RING_B = NST * 2 * C::TILE_B;
+        for (int mt = 0; mt < MT; ++mt) {
+#pragma unroll
+            for (int x = 0; x < MT; ++x)  // (constant indices keep the fragments in registers)
+                if (x == mt && sub != 0) give(x);
+            unit_sync();
+            if (sub == 0)
+#pragma unroll
+                for (int x = 0; x < MT; ++x)
+                    if (x == mt)
+                        for (int w = 1; w < wpu; ++w)
+                            take(x, [&](int i) {
+                                float v;
+                                asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(ring + w * RING_B + lane * 4 + i * 128) : "memory");
+                                return v;
+                            });
+            unit_sync();
+        }
+        if (n_cta > 1) {
+            for (int mt = 0; mt < MT; ++mt) {
+#pragma unroll
+                for (int x = 0; x < MT; ++x)
+                    if (x == mt && sub == 0 && rank != 0) give(x);
+                cluster_sync();
+                if (sub == 0 && rank == 0)
+#pragma unroll
+                    for (int x = 0; x < MT; ++x)
+                        if (x == mt)
+                            for (int r = 1; r < n_cta; ++r)
+                                take(x, [&](int i) { return ld_cluster(ring + lane * 4 + i * 128, (uint32_t)r); });
+                cluster_sync();  // the other blocks' shared memory has been read
+            }
+        }
+        if (part != 0) return;
     }
 
     // epilogue: finish the row sums over the quad, then store outputs or partials
@@ -548,35 +671,43 @@ __global__ void __launch_bounds__(128, MmaCfg<D, MT, TMA>::MIN_BLOCKS)
     }
 }
 
-template <int D, int MT, int MODE, bool IDX16, bool TMA, bool VAR>
-cudaError_t launch_mma_one(const AttendArgs& a, int n_mb, dim3 grid, const CUtensorMap* maps, int* err_flag,
-                           cudaStream_t s)
+template <int D, int MT, int MODE, bool IDX16, bool TMA, bool VAR, bool SHARED>
+cudaError_t launch_mma_one(const AttendArgs& a, int n_mb, int parts, const InlineTable* tab, const CUtensorMap* maps,
+                           int* err_flag, const Launch& l)
 {
     using C = MmaCfg<D, MT, TMA>;
-    // per launch: the attribute belongs to the current device, and a context may sit on any of them
-    cudaError_t e = cudaFuncSetAttribute(attend_mma_kernel<D, MT, MODE, IDX16, TMA, VAR>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-    if (e != cudaSuccess) return e;
-    static const CUtensorMap none{};
-    attend_mma_kernel<D, MT, MODE, IDX16, TMA, VAR>
-        <<<grid, 128, C::SMEM, s>>>(a, n_mb, TMA ? maps[0] : none, TMA ? maps[1] : none, err_flag);
-    return cudaGetLastError();
+    int log_wpu = 0;
+    while (log_wpu < 2 && (1 << log_wpu) < parts) ++log_wpu;
+    const int n_cta = parts >> log_wpu;
+    const int64_t units = (int64_t)a.n_items * n_mb, upb = C::WARPS >> log_wpu;
+    const dim3 grid((unsigned)((units + upb - 1) / upb * n_cta), a.cv.n_groups);
+    if constexpr (TMA) {
+        return launch_kernel(l, attend_mma_kernel<D, MT, MODE, IDX16, true, VAR, SHARED>, grid, 128, C::SMEM, n_cta, a, n_mb,
+                             log_wpu, n_cta, err_flag, TmaMaps{maps[0], maps[1]});
+    } else {
+        static const InlineTable none{};
+        return launch_kernel(l, attend_mma_kernel<D, MT, MODE, IDX16, false, VAR, SHARED>, grid, 128, C::SMEM, n_cta, a, n_mb,
+                             log_wpu, n_cta, err_flag, tab ? *tab : none);
+    }
 }
 
 template <int D, int MT>
-cudaError_t launch_mma(const AttendArgs& a, int n_mb, const CUtensorMap* maps, int* err_flag, cudaStream_t s)
+cudaError_t launch_mma(const AttendArgs& a, int n_mb, int parts, const InlineTable* tab, const CUtensorMap* maps,
+                       int* err_flag, const Launch& l)
 {
-    const int64_t warps = (int64_t)a.n_items * n_mb;
-    const dim3 grid((unsigned)((warps + 3) / 4), a.cv.n_groups);
     const bool i16 = a.cv.idx_bytes == 2;
     const bool var = a.vis != nullptr || a.cv.full_k || a.cv.full_v;  // the TMA loader is never asked for with these
-#define CKV_MMA_GO(MODE, I16)                                                                        \
-    (maps  ? launch_mma_one<D, MT, MODE, I16, true, false>(a, n_mb, grid, maps, err_flag, s)         \
-     : var ? launch_mma_one<D, MT, MODE, I16, false, true>(a, n_mb, grid, maps, err_flag, s)         \
-           : launch_mma_one<D, MT, MODE, I16, false, false>(a, n_mb, grid, maps, err_flag, s))
+#define CKV_MMA_ONE(MODE, I16, TMA, VAR)                                                                   \
+    (parts > 1 ? launch_mma_one<D, MT, MODE, I16, TMA, VAR, true>(a, n_mb, parts, tab, maps, err_flag, l)  \
+               : launch_mma_one<D, MT, MODE, I16, TMA, VAR, false>(a, n_mb, parts, tab, maps, err_flag, l))
+#define CKV_MMA_GO(MODE, I16)                                                                              \
+    (maps  ? CKV_MMA_ONE(MODE, I16, true, false)                                                           \
+     : var ? CKV_MMA_ONE(MODE, I16, false, true)                                                           \
+           : CKV_MMA_ONE(MODE, I16, false, false))
     if (a.mode == CKV_SOFTMAX) return i16 ? CKV_MMA_GO(CKV_SOFTMAX, true) : CKV_MMA_GO(CKV_SOFTMAX, false);
     return i16 ? CKV_MMA_GO(CKV_SILU_OVER_L, true) : CKV_MMA_GO(CKV_SILU_OVER_L, false);
 #undef CKV_MMA_GO
+#undef CKV_MMA_ONE
 }
 
 }  // namespace
@@ -589,18 +720,25 @@ bool mma_supported(int dtype, int head_dim, int d_user)
 // head_dim 64 rows keep a warp busy with one 16-query tile; 32-wide heads take up to four
 int mma_queries_per_warp(int D, int max_M) { return (D == 64 || max_M <= 16) ? 16 : (max_M <= 32 ? 32 : 64); }
 
-cudaError_t launch_attend_mma(int D, int max_M, const AttendArgs& a, const void* tensor_maps, int* err_flag,
-                              cudaStream_t s)
+// warps of the kernel that are resident on an SM
+int mma_warps_per_sm(int D, int max_M)
+{
+    if (D == 64) return 4 * MmaCfg<64, 1, false>::MIN_BLOCKS;
+    return mma_queries_per_warp(D, max_M) == 16 ? 4 * MmaCfg<32, 1, false>::MIN_BLOCKS : 8;
+}
+
+cudaError_t launch_attend_mma(int D, int max_M, int parts, const AttendArgs& a, const InlineTable* tab,
+                              const void* tensor_maps, int* err_flag, const Launch& l)
 {
     if (a.n_items == 0) return cudaSuccess;
     const CUtensorMap* maps = reinterpret_cast<const CUtensorMap*>(tensor_maps);
     const int qpw = mma_queries_per_warp(D, max_M);
     const int n_mb = (max_M + qpw - 1) / qpw;
-    if (D == 64) return launch_mma<64, 1>(a, n_mb, maps, err_flag, s);
+    if (D == 64) return launch_mma<64, 1>(a, n_mb, parts, tab, maps, err_flag, l);
     switch (qpw) {
-        case 16: return launch_mma<32, 1>(a, n_mb, maps, err_flag, s);
-        case 32: return launch_mma<32, 2>(a, n_mb, maps, err_flag, s);
-        default: return launch_mma<32, 4>(a, n_mb, maps, err_flag, s);
+        case 16: return launch_mma<32, 1>(a, n_mb, parts, tab, maps, err_flag, l);
+        case 32: return launch_mma<32, 2>(a, n_mb, parts, tab, maps, err_flag, l);
+        default: return launch_mma<32, 4>(a, n_mb, parts, tab, maps, err_flag, l);
     }
 }
 

@@ -8,6 +8,8 @@
 // rows therefore only ever exist in registers.  Scores are reduced over the LPR lanes
 // with shuffles, the softmax is the running-max form, and partial results of the
 // sub-warps / warps / history chunks are merged with the usual (m, l, acc) rule.
+// Two block sizes: 4 warps when there are blocks enough for every SM, 16 (8 with several queries per user) when there
+// are not: a small call is a chain of dependent loads per step, so it wants few steps per warp.
 // A side that is not shared (sharing only keys or only values) has its full-width rows in the
 // arena: they are read in place of the pool rows, coalesced, and nothing is patched.  With
 // visible lengths a query row only takes the positions before its own limit.
@@ -20,7 +22,6 @@
 namespace ckv {
 namespace {
 
-constexpr int kWarps = 4;
 constexpr float kLog2e = 1.4426950408889634f;
 
 __device__ __forceinline__ uint4 ldg16(const void* p)
@@ -80,8 +81,9 @@ __device__ __forceinline__ void store_out(void* out, int64_t i, float v, int out
         reinterpret_cast<float*>(out)[i] = v;
 }
 
-template <bool BF16, int D, int QB, int MODE>
-__global__ void __launch_bounds__(kWarps * 32, QB == 1 ? 5 : 1) attend_simt_kernel(const AttendArgs a)
+template <bool BF16, int D, int QB, int MODE, int kWarps>
+__global__ void __launch_bounds__(kWarps * 32, QB == 1 && kWarps == 4 ? 5 : 1)
+    attend_simt_kernel(const __grid_constant__ AttendArgs a, const __grid_constant__ InlineTable tab)
 {
     constexpr int ES = BF16 ? 2 : 4;
     constexpr int EPL = 16 / ES;         // elements per lane
@@ -93,9 +95,17 @@ __global__ void __launch_bounds__(kWarps * 32, QB == 1 ? 5 : 1) attend_simt_kern
     __shared__ float sm_m[kWarps][QB], sm_l[kWarps][QB];
     __shared__ float sm_acc[kWarps][QB][D];
 
-    const Item it = a.items[blockIdx.x];
+    Item it;
+    Req rq;
+    if (a.inl) {
+        const InlineReq& r = tab.r[blockIdx.x];
+        rq = Req{(int64_t)r.base32 * 32, r.L, (r.L + 31) & ~31, r.q0, r.M, -1, 1};
+        it = Item{(int)blockIdx.x, 0, r.L, -1};
+    } else {
+        it = a.items[blockIdx.x];
+        rq = a.reqs[it.req];
+    }
     const int g = blockIdx.y;
-    const Req rq = a.reqs[it.req];
     const CacheView& cv = a.cv;
     const int G = cv.n_groups, d_user = cv.d_user, idx_bytes = cv.idx_bytes;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -387,43 +397,43 @@ __global__ void __launch_bounds__(128) combine_kernel(const AttendArgs a, const 
 }
 
 template <bool BF16, int D>
-cudaError_t launch_simt_d(const AttendArgs& a, int max_M, cudaStream_t s)
+cudaError_t launch_simt_d(const AttendArgs& a, int max_M, bool wide, const InlineTable& tab, const Launch& l)
 {
-    const dim3 grid(a.n_items, a.cv.n_groups), block(kWarps * 32);
-    const bool sm = a.mode == CKV_SOFTMAX;
-    if (max_M <= 1) {
-        if (sm) attend_simt_kernel<BF16, D, 1, CKV_SOFTMAX><<<grid, block, 0, s>>>(a);
-        else attend_simt_kernel<BF16, D, 1, CKV_SILU_OVER_L><<<grid, block, 0, s>>>(a);
-    } else {
-        if (sm) attend_simt_kernel<BF16, D, 4, CKV_SOFTMAX><<<grid, block, 0, s>>>(a);
-        else attend_simt_kernel<BF16, D, 4, CKV_SILU_OVER_L><<<grid, block, 0, s>>>(a);
+    const dim3 grid(a.n_items, a.cv.n_groups);
+#define CKV_SIMT_GO(QB, MODE, W) launch_kernel(l, attend_simt_kernel<BF16, D, QB, MODE, W>, grid, W * 32, 0, 1, a, tab)
+    if (a.mode == CKV_SOFTMAX) {
+        if (max_M <= 1) return wide ? CKV_SIMT_GO(1, CKV_SOFTMAX, 16) : CKV_SIMT_GO(1, CKV_SOFTMAX, 4);
+        return wide ? CKV_SIMT_GO(4, CKV_SOFTMAX, 8) : CKV_SIMT_GO(4, CKV_SOFTMAX, 4);
     }
-    return cudaGetLastError();
+    if (max_M <= 1) return wide ? CKV_SIMT_GO(1, CKV_SILU_OVER_L, 16) : CKV_SIMT_GO(1, CKV_SILU_OVER_L, 4);
+    return wide ? CKV_SIMT_GO(4, CKV_SILU_OVER_L, 8) : CKV_SIMT_GO(4, CKV_SILU_OVER_L, 4);
+#undef CKV_SIMT_GO
 }
 
 }  // namespace
 
-cudaError_t launch_attend_simt(int dtype, int D, int max_M, const AttendArgs& a, cudaStream_t s)
+cudaError_t launch_attend_simt(int dtype, int D, int max_M, bool wide, const AttendArgs& a, const InlineTable* tab,
+                               const Launch& l)
 {
     if (a.n_items == 0) return cudaSuccess;
+    static const InlineTable none{};
+    const InlineTable& t = tab ? *tab : none;
     const bool bf = dtype == CKV_BF16;
     switch (D) {
-        case 16: return bf ? launch_simt_d<true, 16>(a, max_M, s) : launch_simt_d<false, 16>(a, max_M, s);
-        case 32: return bf ? launch_simt_d<true, 32>(a, max_M, s) : launch_simt_d<false, 32>(a, max_M, s);
-        case 64: return bf ? launch_simt_d<true, 64>(a, max_M, s) : launch_simt_d<false, 64>(a, max_M, s);
-        case 128: return bf ? launch_simt_d<true, 128>(a, max_M, s) : launch_simt_d<false, 128>(a, max_M, s);
+        case 16: return bf ? launch_simt_d<true, 16>(a, max_M, wide, t, l) : launch_simt_d<false, 16>(a, max_M, wide, t, l);
+        case 32: return bf ? launch_simt_d<true, 32>(a, max_M, wide, t, l) : launch_simt_d<false, 32>(a, max_M, wide, t, l);
+        case 64: return bf ? launch_simt_d<true, 64>(a, max_M, wide, t, l) : launch_simt_d<false, 64>(a, max_M, wide, t, l);
+        case 128: return bf ? launch_simt_d<true, 128>(a, max_M, wide, t, l) : launch_simt_d<false, 128>(a, max_M, wide, t, l);
     }
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_combine(int D, const AttendArgs& a, const int32_t* split_reqs, int n_split,
-                           cudaStream_t s)
+cudaError_t launch_combine(int D, const AttendArgs& a, const int32_t* split_reqs, int n_split, const Launch& l)
 {
     if (n_split == 0) return cudaSuccess;
     const dim3 grid(n_split, a.cv.n_groups);
-    if (a.mode == CKV_SOFTMAX) combine_kernel<CKV_SOFTMAX><<<grid, 128, 0, s>>>(a, split_reqs, D);
-    else combine_kernel<CKV_SILU_OVER_L><<<grid, 128, 0, s>>>(a, split_reqs, D);
-    return cudaGetLastError();
+    return a.mode == CKV_SOFTMAX ? launch_kernel(l, combine_kernel<CKV_SOFTMAX>, grid, 128, 0, 1, a, split_reqs, D)
+                                 : launch_kernel(l, combine_kernel<CKV_SILU_OVER_L>, grid, 128, 0, 1, a, split_reqs, D);
 }
 
 }  // namespace ckv

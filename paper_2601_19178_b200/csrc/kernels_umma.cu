@@ -1221,7 +1221,7 @@ cudaError_t launch_vis_block_max(const AttendArgs& a, int32_t* vmax, cudaStream_
     return cudaGetLastError();
 }
 
-cudaError_t launch_attend_umma(int max_M, const AttendArgs& a, int n_sms, int* err_flag, cudaStream_t s)
+cudaError_t launch_attend_umma(int max_M, const AttendArgs& a, int n_sms, int* err_flag, const Launch& l)
 {
     if (a.n_items == 0) return cudaSuccess;
     const int n_mb = (max_M + 127) / 128;
@@ -1229,10 +1229,7 @@ cudaError_t launch_attend_umma(int max_M, const AttendArgs& a, int n_sms, int* e
     if (n_work + n_sms >= (int64_t)1 << 32) return cudaErrorInvalidValue;  // the kernel counts units in 32 bits
     const unsigned grid = (unsigned)(n_work < n_sms ? n_work : n_sms);
     auto go = [&](auto kernel) {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-        if (e != cudaSuccess) return e;
-        kernel<<<grid, kThreads, kSmemBytes, s>>>(a, n_mb, n_work, err_flag);
-        return cudaGetLastError();
+        return launch_kernel(l, kernel, grid, kThreads, kSmemBytes, 1, a, n_mb, n_work, err_flag);
     };
     const bool sm = a.mode == CKV_SOFTMAX, vis = a.vis != nullptr;
     if (vis && a.vmax == nullptr) return cudaErrorInvalidValue;

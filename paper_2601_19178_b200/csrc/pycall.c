@@ -1,0 +1,93 @@
+/*
+ * CPython helper of binding.py: marshals the arguments of the decode calls.  A decode call of a few users takes the
+ * GPU about 6 us; taking two array addresses, two tensor addresses and going through ctypes took Python another 4.
+ * Marshalling only: the call itself is the C-ABI function whose address is passed in.
+ */
+#define PY_SSIZE_T_CLEAN
+#include <Python.h>
+#include <stdint.h>
+
+static PyObject *s_data_ptr, *s_is_contiguous;
+
+/* Address and length of a C-contiguous host array of whole numbers of `size` bytes; 0 if `o` is something else. */
+static int host_array(PyObject* o, Py_ssize_t size, Py_buffer* b)
+{
+    if (PyObject_GetBuffer(o, b, PyBUF_C_CONTIGUOUS | PyBUF_FORMAT) != 0) {
+        PyErr_Clear();
+        return 0;
+    }
+    const char* f = b->format ? b->format : "B";
+    if (b->ndim == 1 && b->itemsize == size && (f[0] == 'l' || f[0] == 'i' || f[0] == 'q') && f[1] == 0) return 1;
+    PyBuffer_Release(b);
+    return 0;
+}
+
+/* Address of a contiguous tensor; 0 if `o` is something else (an exception of the tensor's own stays set). */
+static int tensor_address(PyObject* o, void** p)
+{
+    PyObject* c = PyObject_CallMethodNoArgs(o, s_is_contiguous);
+    if (!c) {
+        if (PyErr_ExceptionMatches(PyExc_AttributeError)) PyErr_Clear();
+        return 0;
+    }
+    const int yes = c == Py_True;
+    Py_DECREF(c);
+    if (!yes) return 0;
+    PyObject* a = PyObject_CallMethodNoArgs(o, s_data_ptr);
+    if (!a) return 0;
+    *p = PyLong_AsVoidPtr(a);
+    Py_DECREF(a);
+    return !PyErr_Occurred();
+}
+
+typedef int32_t (*attend_fn)(void*, int32_t, const void*, const void*, const void*, void*, void*);
+typedef int32_t (*attend_visible_fn)(void*, int32_t, const void*, const void*, const void*, const void*, void*, void*);
+
+/* attend(function address, context, users int64[n], q_off int32[n + 1], vis tensor | None, queries, out, stream):
+ * the status of the call, or None if an argument is not of the plain kind (binding.py then converts it). */
+static PyObject* attend(PyObject* self, PyObject* const* args, Py_ssize_t n_args)
+{
+    (void)self;
+    if (n_args != 8) {
+        PyErr_SetString(PyExc_TypeError, "attend takes 8 arguments");
+        return NULL;
+    }
+    void* fn = PyLong_AsVoidPtr(args[0]);
+    void* ctx = PyLong_AsVoidPtr(args[1]);
+    void* stream = PyLong_AsVoidPtr(args[7]);
+    if (PyErr_Occurred()) return NULL;
+    Py_buffer users, q_off;
+    if (!host_array(args[2], 8, &users)) Py_RETURN_NONE;
+    if (!host_array(args[3], 4, &q_off)) {
+        PyBuffer_Release(&users);
+        Py_RETURN_NONE;
+    }
+    const Py_ssize_t n = users.len / 8;
+    void *vis = NULL, *q = NULL, *out = NULL;
+    const int with_vis = args[4] != Py_None;
+    int32_t status = 0;
+    const int plain = q_off.len / 4 == n + 1 && n <= INT32_MAX && (!with_vis || tensor_address(args[4], &vis)) &&
+                      tensor_address(args[5], &q) && tensor_address(args[6], &out);
+    if (plain) {
+        Py_BEGIN_ALLOW_THREADS;
+        status = with_vis ? ((attend_visible_fn)fn)(ctx, (int32_t)n, users.buf, q_off.buf, vis, q, out, stream)
+                          : ((attend_fn)fn)(ctx, (int32_t)n, users.buf, q_off.buf, q, out, stream);
+        Py_END_ALLOW_THREADS;
+    }
+    PyBuffer_Release(&users);
+    PyBuffer_Release(&q_off);
+    if (PyErr_Occurred()) return NULL;
+    if (!plain) Py_RETURN_NONE;
+    return PyLong_FromLong(status);
+}
+
+static PyMethodDef methods[] = {{"attend", (PyCFunction)(void (*)(void))attend, METH_FASTCALL, "one decode call"},
+                                {NULL, NULL, 0, NULL}};
+static struct PyModuleDef module = {PyModuleDef_HEAD_INIT, "_pycall", NULL, -1, methods, NULL, NULL, NULL, NULL};
+
+PyMODINIT_FUNC PyInit__pycall(void)
+{
+    s_data_ptr = PyUnicode_InternFromString("data_ptr");
+    s_is_contiguous = PyUnicode_InternFromString("is_contiguous");
+    return s_data_ptr && s_is_contiguous ? PyModule_Create(&module) : NULL;
+}

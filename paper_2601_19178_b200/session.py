@@ -62,16 +62,21 @@ class CollectiveKV:
     def cache_put_batch(self, users, hist_off, idx_K, idx_V, user_K, user_V):
         B.ckv_cache_put_batch(self.ctx, users, hist_off, idx_K, idx_V, user_K, user_V, self.d_user)
 
+    def _out_for(self, queries: torch.Tensor) -> torch.Tensor:
+        if queries.dtype == self.out_dtype and queries.is_contiguous():
+            return torch.empty_like(queries)  # (half the host time of spelling out shape, dtype and device)
+        return torch.empty(queries.shape, dtype=self.out_dtype, device=queries.device)
+
     def attend(self, users, q_off, queries: torch.Tensor, out: Optional[torch.Tensor] = None) -> torch.Tensor:
         if out is None:
-            out = torch.empty(queries.shape, dtype=self.out_dtype, device=queries.device)
+            out = self._out_for(queries)
         B.ckv_attend(self.ctx, users, q_off, queries, out)
         return out
 
     def attend_visible(self, users, q_off, vis, queries: torch.Tensor, out: Optional[torch.Tensor] = None) -> torch.Tensor:
         """attend with a visible length per query row (self-attention over the cached sequence)."""
         if out is None:
-            out = torch.empty(queries.shape, dtype=self.out_dtype, device=queries.device)
+            out = self._out_for(queries)
         B.ckv_attend_visible(self.ctx, users, q_off, vis, queries, out)
         return out
 
