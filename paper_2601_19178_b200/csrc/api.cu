@@ -1422,7 +1422,8 @@ ckv_status attend_impl(ckv_ctx* ctx, int32_t n, const int64_t* users, const int3
             fill_args(a);
             a.n_items = x.n;
             a.inl = 1;
-            const Launch l = launch_on(ctx, s);
+            Launch l = launch_on(ctx, s);
+            l.early = true;
             st = timed(ctx, ctx->opt_time != 0, s, [&]() -> ckv_status {
                 if (x.family == 2) return run_mma(ctx, D, x.max_M, x.parts, a, &x.tab, l);
                 CK(launch_attend_simt(ctx->cfg.dtype, D, x.max_M, simt_wide(ctx, x.n), a, &x.tab, l));

@@ -104,6 +104,8 @@ struct Launch {
     cudaStream_t s;
     const cudaAccessPolicyWindow* window;
     SmemGrants* grants;
+    bool early = false;  // programmatic launch: the blocks may be set up while the stream's previous kernel still runs
+                         // (the kernel waits for that one's memory itself, grid_dependency_wait)
 };
 inline cudaError_t grant_smem(SmemGrants* g, const void* fn, size_t bytes)
 {
@@ -127,7 +129,7 @@ cudaError_t launch_kernel(const Launch& l, void (*fn)(P...), dim3 grid, int thre
 {
     cudaError_t e = grant_smem(l.grants, (const void*)fn, smem);
     if (e != cudaSuccess) return e;
-    cudaLaunchAttribute at[2];
+    cudaLaunchAttribute at[3];
     cudaLaunchConfig_t c{};
     c.gridDim = grid;
     c.blockDim = dim3((unsigned)threads);
@@ -143,6 +145,11 @@ cudaError_t launch_kernel(const Launch& l, void (*fn)(P...), dim3 grid, int thre
     if (l.window) {
         at[c.numAttrs].id = cudaLaunchAttributeAccessPolicyWindow;
         at[c.numAttrs].val.accessPolicyWindow = *l.window;
+        ++c.numAttrs;
+    }
+    if (l.early) {
+        at[c.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[c.numAttrs].val.programmaticStreamSerializationAllowed = 1;
         ++c.numAttrs;
     }
     return cudaLaunchKernelEx(&c, fn, std::forward<A>(args)...);

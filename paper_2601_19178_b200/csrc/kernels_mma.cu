@@ -169,6 +169,7 @@ __global__ void __launch_bounds__(128, MmaCfg<D, MT, TMA>::MIN_BLOCKS)
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, t = lane & 3;
+    grid_dependency_wait();
     // 2^log_wpu warps of a block and the n_cta blocks of its cluster share a unit; this warp is number `part` of
     // `parts` and takes tiles part, part + parts, ... of the chunk
     if constexpr (!SHARED) {

@@ -95,6 +95,7 @@ __global__ void __launch_bounds__(kWarps * 32, QB == 1 && kWarps == 4 ? 5 : 1)
     __shared__ float sm_m[kWarps][QB], sm_l[kWarps][QB];
     __shared__ float sm_acc[kWarps][QB][D];
 
+    grid_dependency_wait();
     Item it;
     Req rq;
     if (a.inl) {

@@ -40,6 +40,13 @@ __device__ __forceinline__ float tanh_fast(float x)
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// Programmatic launch (Launch::early): lets the stream's next kernel be set up, then waits until the previous one
+// has finished and its memory is visible.  Without that launch attribute both are no-ops.
+__device__ __forceinline__ void grid_dependency_wait()
+{
+    asm volatile("griddepcontrol.launch_dependents;\ngriddepcontrol.wait;" ::: "memory");
+}
+
 // Range checks of the debug build (-DCKV_BOUNDS, the stand-in for a memory checker where none can run): every
 // index taken from the compressed cache, every unit, query / output / partial row and shared-memory offset a
 // kernel computes is compared with its bound; a violation ORs kErrBounds into the context's error word
