@@ -199,7 +199,10 @@ struct ckv_ctx {
     uint64_t generation = 1;
     // scratch
     DevBuf stage_q, stage_out, stage_vis, vmax, partials;
-    int* d_flag = nullptr;
+    int* h_flag = nullptr;     // pinned, mapped: a kernel that checks indices raises it, the host reads it behind a synchronise
+    void* put_host = nullptr;  // pinned table of a put of many users
+    size_t put_host_cap = 0;
+    DevBuf put_dev, put_in[4];  // its device copy; staged host inputs up to kKeepStaged bytes each
     Plan plans[kMaxPlans];
     uint64_t tick = 0;
     // options
@@ -248,27 +251,6 @@ bool is_device_ptr(const void* p)
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
-// A temporary device copy of host input, freed by the destructor.
-struct Staged {
-    const void* dev = nullptr;
-    void* owned = nullptr;
-    ~Staged()
-    {
-        if (owned) cudaFree(owned);
-    }
-    cudaError_t init(const void* src, size_t bytes, cudaStream_t s)
-    {
-        if (bytes == 0 || src == nullptr || is_device_ptr(src)) {
-            dev = src;
-            return cudaSuccess;
-        }
-        cudaError_t e = cudaMalloc(&owned, bytes);
-        if (e != cudaSuccess) return e;
-        dev = owned;
-        return cudaMemcpyAsync(owned, src, bytes, cudaMemcpyHostToDevice, s);
-    }
-};
-
 cudaError_t grow(DevBuf& b, size_t bytes, int64_t* allocs = nullptr)
 {
     if (bytes <= b.cap) return cudaSuccess;
@@ -290,6 +272,38 @@ cudaError_t grow(DevBuf& b, size_t bytes, int64_t* allocs = nullptr)
     b.cap = want;
     return cudaSuccess;
 }
+
+constexpr size_t kKeepStaged = size_t(16) << 20;
+
+// A device copy of host input: in `keep` up to kKeepStaged bytes (the context's, for calls that wait for the stream
+// before they return), else in memory that the destructor frees.
+struct Staged {
+    const void* dev = nullptr;
+    void* owned = nullptr;
+    ~Staged()
+    {
+        if (owned) cudaFree(owned);
+    }
+    cudaError_t init(const void* src, size_t bytes, cudaStream_t s, DevBuf* keep = nullptr)
+    {
+        if (bytes == 0 || src == nullptr || is_device_ptr(src)) {
+            dev = src;
+            return cudaSuccess;
+        }
+        void* p;
+        if (keep && bytes <= kKeepStaged) {
+            cudaError_t e = grow(*keep, bytes);
+            if (e != cudaSuccess) return e;
+            p = keep->p;
+        } else {
+            cudaError_t e = cudaMalloc(&owned, bytes);
+            if (e != cudaSuccess) return e;
+            p = owned;
+        }
+        dev = p;
+        return cudaMemcpyAsync(p, src, bytes, cudaMemcpyHostToDevice, s);
+    }
+};
 
 void free_plan(Plan& p)
 {
@@ -799,13 +813,15 @@ ckv_status ckv_create(const ckv_config* cfg, ckv_ctx** out)
     ctx->scale = cfg->scale > 0.f ? cfg->scale
                                   : (cfg->mode == CKV_SOFTMAX ? 1.0f / std::sqrt((float)cfg->head_dim) : 1.0f);
     DeviceGuard dg(cfg->device);
-    if (!dg.ok || cudaMalloc((void**)&ctx->d_flag, 2 * sizeof(int)) != cudaSuccess ||
-        cudaMemset(ctx->d_flag, 0, 2 * sizeof(int)) != cudaSuccess) {
+    if (!dg.ok || cudaMalloc((void**)&ctx->d_err, sizeof(int)) != cudaSuccess ||
+        cudaMemset(ctx->d_err, 0, sizeof(int)) != cudaSuccess ||
+        cudaHostAlloc((void**)&ctx->h_flag, sizeof(int), cudaHostAllocMapped) != cudaSuccess) {
         cudaGetLastError();
+        if (ctx->d_err) cudaFree(ctx->d_err);
         delete ctx;
         return CKV_ERR_CUDA;
     }
-    ctx->d_err = ctx->d_flag + 1;
+    *ctx->h_flag = 0;
     if (cudaDeviceGetAttribute(&ctx->n_sms, cudaDevAttrMultiProcessorCount, cfg->device) != cudaSuccess || ctx->n_sms < 1) {
         cudaGetLastError();
         ctx->n_sms = 148;
@@ -820,9 +836,12 @@ ckv_status ckv_destroy(ckv_ctx* ctx)
     DeviceGuard dg(ctx->cfg.device);
     drop_plans(ctx);
     void* bufs[] = {ctx->pool,    ctx->a_idxK,     ctx->a_idxV,      ctx->a_userK,   ctx->a_userV,
-                    ctx->d_flag,  ctx->stage_q.p,  ctx->stage_out.p, ctx->partials.p, ctx->stage_vis.p, ctx->vmax.p};
+                    ctx->d_err,   ctx->stage_q.p,  ctx->stage_out.p, ctx->partials.p, ctx->stage_vis.p, ctx->vmax.p,
+                    ctx->put_dev.p, ctx->put_in[0].p, ctx->put_in[1].p, ctx->put_in[2].p, ctx->put_in[3].p};
     for (void* b : bufs)
         if (b) cudaFree(b);
+    if (ctx->h_flag) cudaFreeHost(ctx->h_flag);
+    if (ctx->put_host) cudaFreeHost(ctx->put_host);
     for (auto& e : ctx->ev)
         if (e) cudaEventDestroy(e);
     for (int r = 0; r < kMaxRanges; ++r) {
@@ -938,26 +957,43 @@ ckv_status ckv_cache_put_batch(ckv_ctx* ctx, int32_t n, const int64_t* users, co
     }
     int64_t base = 0;
     if (total_units > 0) {
-        Staged sik, siv, suk, suv, sho, suo;
+        Staged sik, siv, suk, suv;
         const size_t ib = (size_t)P * G * sizeof(int32_t);
-        if (eb[0]) CK(sik.init(idx_K, ib, s));
+        if (eb[0]) CK(sik.init(idx_K, ib, s, &ctx->put_in[0]));
         if (eb[1]) {
-            if (idx_V == idx_K && eb[0]) siv.dev = sik.dev; else CK(siv.init(idx_V, ib, s));
+            if (idx_V == idx_K && eb[0]) siv.dev = sik.dev; else CK(siv.init(idx_V, ib, s, &ctx->put_in[1]));
         }
-        CK(suk.init(user_K, (size_t)P * G * eb[2], s));
-        CK(suv.init(user_V, (size_t)P * G * eb[3], s));
-        CK(sho.init(hist_off, sizeof(int64_t) * ((size_t)n + 1), s));
-        CK(suo.init(unit_off.data(), sizeof(int64_t) * ((size_t)n + 1), s));
+        CK(suk.init(user_K, (size_t)P * G * eb[2], s, &ctx->put_in[2]));
+        CK(suv.init(user_V, (size_t)P * G * eb[3], s, &ctx->put_in[3]));
+        // the users' table: a kernel argument, or, for many users, uploaded from pinned memory
+        PutTable inl;
+        PutUser* tab = inl.u;
+        if (n > kInlinePuts) {
+            const size_t bytes = sizeof(PutUser) * (size_t)n;
+            CK(grow(ctx->put_dev, bytes));
+            if (bytes > ctx->put_host_cap) {
+                if (ctx->put_host) cudaFreeHost(ctx->put_host);
+                ctx->put_host = nullptr;
+                ctx->put_host_cap = 0;
+                CK(cudaMallocHost(&ctx->put_host, bytes));
+                ctx->put_host_cap = bytes;
+            }
+            tab = (PutUser*)ctx->put_host;
+        }
+        for (int32_t k = 0; k < n; ++k)
+            tab[k] = PutUser{hist_off[k], (int32_t)(unit_off[k] / (32 * (int64_t)G)), (int32_t)(hist_off[k + 1] - hist_off[k])};
+        if (n > kInlinePuts)
+            CK(cudaMemcpyAsync(ctx->put_dev.p, tab, sizeof(PutUser) * (size_t)n, cudaMemcpyHostToDevice, s));
         ckv_status st = arena_take(ctx, total_units, s, &base);
         if (st != CKV_OK) return st;
-        cudaError_t e = cudaMemsetAsync(ctx->d_flag, 0, sizeof(int), s);
-        if (e == cudaSuccess)
-            e = launch_pack(ctx->cfg.dtype, G, ctx->n_entries, ctx->idx_bytes, n, (const int64_t*)sho.dev,
-                            (const int64_t*)suo.dev, total_units, base, (const int32_t*)sik.dev,
-                            (const int32_t*)siv.dev, suk.dev, suv.dev, view_of(ctx), ctx->cfg.head_dim, ctx->d_flag, s);
-        int bad = 0;
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&bad, ctx->d_flag, sizeof(int), cudaMemcpyDeviceToHost, s);
+        volatile int* const flag = ctx->h_flag;
+        *flag = 0;
+        cudaError_t e = launch_pack(ctx->cfg.dtype, G, ctx->n_entries, ctx->idx_bytes, n,
+                                    n > kInlinePuts ? (const PutUser*)ctx->put_dev.p : nullptr, &inl,
+                                    total_units / (32 * (int64_t)G), base, (const int32_t*)sik.dev, (const int32_t*)siv.dev,
+                                    suk.dev, suv.dev, view_of(ctx), ctx->cfg.head_dim, ctx->h_flag, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        const bool bad = *flag != 0;
         if (e != cudaSuccess || bad) {  // nothing was stored: the units go back
             arena_give(ctx, base, total_units);
             return e != cudaSuccess ? ctx->fail(e) : CKV_ERR_INDEX_RANGE;
@@ -1003,30 +1039,36 @@ ckv_status ckv_cache_append(ckv_ctx* ctx, int64_t user, int32_t L_new, const int
     cudaStream_t s = (cudaStream_t)stream;
     Staged sik, siv, suk, suv;
     const size_t ib = (size_t)L_new * G * sizeof(int32_t);
-    if (eb[0]) CK(sik.init(idx_K, ib, s));
+    if (eb[0]) CK(sik.init(idx_K, ib, s, &ctx->put_in[0]));
     if (eb[1]) {
-        if (idx_V == idx_K && eb[0]) siv.dev = sik.dev; else CK(siv.init(idx_V, ib, s));
+        if (idx_V == idx_K && eb[0]) siv.dev = sik.dev; else CK(siv.init(idx_V, ib, s, &ctx->put_in[1]));
     }
-    CK(suk.init(user_K, (size_t)L_new * G * eb[2], s));
-    CK(suv.init(user_V, (size_t)L_new * G * eb[3], s));
-    // the longer history is written to a run of its own (the old units are read while it is written) and the
-    // old run is given back afterwards
-    int64_t base = 0;
-    ckv_status st = arena_take(ctx, units, s, &base);
-    if (st != CKV_OK) return st;
-    cudaError_t e = cudaMemsetAsync(ctx->d_flag, 0, sizeof(int), s);
-    if (e == cudaSuccess)
-        e = launch_append(ctx->cfg.dtype, G, ctx->n_entries, ctx->idx_bytes, old.base, old.L, old.Lpad, base,
-                          L_new, Lpad_tot, (const int32_t*)sik.dev, (const int32_t*)siv.dev, suk.dev, suv.dev,
-                          view_of(ctx), ctx->cfg.head_dim, ctx->d_flag, s);
-    int bad = 0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&bad, ctx->d_flag, sizeof(int), cudaMemcpyDeviceToHost, s);
+    CK(suk.init(user_K, (size_t)L_new * G * eb[2], s, &ctx->put_in[2]));
+    CK(suv.init(user_V, (size_t)L_new * G * eb[3], s, &ctx->put_in[3]));
+    // New positions that fit the padding of the old history are written behind it (nothing enqueued before reads
+    // there).  Otherwise the longer history is written to a run of its own (the old units are read while it is
+    // written) and the old run is given back afterwards.
+    const bool in_place = Lpad_tot == old.Lpad;
+    int64_t base = old.base;
+    if (!in_place) {
+        ckv_status st = arena_take(ctx, units, s, &base);
+        if (st != CKV_OK) return st;
+    }
+    volatile int* const flag = ctx->h_flag;
+    *flag = 0;
+    auto append = [&](int32_t n_new) {
+        return launch_append(ctx->cfg.dtype, G, ctx->n_entries, ctx->idx_bytes, old.base, old.L, old.Lpad, base, n_new,
+                             Lpad_tot, (const int32_t*)sik.dev, (const int32_t*)siv.dev, suk.dev, suv.dev, view_of(ctx),
+                             ctx->cfg.head_dim, ctx->h_flag, s);
+    };
+    cudaError_t e = append(L_new);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess || bad) {  // the user keeps the old history
-        arena_give(ctx, base, units);
+    if (e != cudaSuccess || *flag) {  // the user keeps the old history
+        if (!in_place) arena_give(ctx, base, units);
+        else if (e == cudaSuccess) e = append(0);  // padding again
         return e != cudaSuccess ? ctx->fail(e) : CKV_ERR_INDEX_RANGE;
     }
-    arena_give(ctx, old.base, (int64_t)G * old.Lpad);
+    if (!in_place) arena_give(ctx, old.base, (int64_t)G * old.Lpad);
     *f = UserEntry{base, L_tot, Lpad_tot};
     ctx->live_positions += L_new;
     ctx->generation++;
@@ -1131,13 +1173,13 @@ ckv_status ckv_cache_import(ckv_ctx* ctx, int32_t n, const int64_t* users, const
             if (eb[i] > 0)
                 e = cudaMemcpyAsync(dst[i] + base * eb[i], (const char*)blob + off[i], (size_t)(total * eb[i]),
                                     cudaMemcpyDefault, s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_flag, 0, sizeof(int), s);
+        volatile int* const flag = ctx->h_flag;
+        *flag = 0;
         if (e == cudaSuccess)
             e = launch_check_indices(ctx->idx_bytes, ctx->n_entries, eb[0] ? dst[0] + base * eb[0] : nullptr,
-                                     eb[1] ? dst[1] + base * eb[1] : nullptr, total, ctx->d_flag, s);
-        int bad = 0;
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&bad, ctx->d_flag, sizeof(int), cudaMemcpyDeviceToHost, s);
+                                     eb[1] ? dst[1] + base * eb[1] : nullptr, total, ctx->h_flag, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        const bool bad = *flag != 0;
         if (e != cudaSuccess || bad) {  // nothing was stored: the units go back
             arena_give(ctx, base, total);
             return e != cudaSuccess ? ctx->fail(e) : CKV_ERR_INDEX_RANGE;
@@ -1199,6 +1241,56 @@ ckv_status run_mma(ckv_ctx* ctx, int D, int max_M, int parts, const AttendArgs& 
 }  // extern "C"
 
 namespace {
+
+// An error word in pinned host memory for one call of the context-free router: 64 of them for the process, handed out
+// and given back under a lock (a call beyond that many at the same time gets one of its own).
+class HostFlag {
+    static constexpr int kSlots = 64, kStride = 16;  // a cache line each
+    static std::mutex mu_;
+    static int* pool_;
+    static uint64_t used_;
+    int slot_ = -1;
+
+public:
+    int* p = nullptr;
+    HostFlag()
+    {
+        {
+            std::lock_guard<std::mutex> lock(mu_);
+            if (!pool_ && cudaHostAlloc((void**)&pool_, kSlots * kStride * sizeof(int),
+                                        cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
+                cudaGetLastError();
+                pool_ = nullptr;
+                return;
+            }
+            for (int i = 0; i < kSlots && slot_ < 0; ++i)
+                if (!(used_ >> i & 1)) slot_ = i;
+            if (slot_ >= 0) {
+                used_ |= 1ull << slot_;
+                p = pool_ + slot_ * kStride;
+            }
+        }
+        if (!p && cudaHostAlloc((void**)&p, sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
+            cudaGetLastError();
+            p = nullptr;
+        }
+        if (p) *p = 0;
+    }
+    ~HostFlag()
+    {
+        if (slot_ < 0) {
+            if (p) cudaFreeHost(p);
+            return;
+        }
+        std::lock_guard<std::mutex> lock(mu_);
+        used_ &= ~(1ull << slot_);
+    }
+    HostFlag(const HostFlag&) = delete;
+    HostFlag& operator=(const HostFlag&) = delete;
+};
+std::mutex HostFlag::mu_;
+int* HostFlag::pool_ = nullptr;
+uint64_t HostFlag::used_ = 0;
 
 constexpr size_t kPipeMinBytes = size_t(4) << 20;  // host query buffers below this are not worth pipelining
 constexpr size_t kPipeManyBytes = size_t(96) << 20;  // from here on: eight ranges instead of four
@@ -1599,28 +1691,6 @@ ckv_status ckv_cache_bytes(ckv_ctx* ctx, int64_t* compressed, int64_t* full_widt
     return CKV_OK;
 }
 
-namespace {
-
-// one error word per device for the context-free tcgen05 router (allocated on first use, never freed)
-int* route_err_word(int device)
-{
-    static std::mutex mu;
-    static int* words[64] = {};
-    std::lock_guard<std::mutex> lock(mu);
-    if (device >= 64) return nullptr;
-    if (!words[device]) {
-        int* p = nullptr;
-        if (cudaMalloc(&p, sizeof(int)) != cudaSuccess || cudaMemset(p, 0, sizeof(int)) != cudaSuccess) {
-            cudaGetLastError();
-            return nullptr;
-        }
-        words[device] = p;
-    }
-    return words[device];
-}
-
-}  // namespace
-
 ckv_status ckv_route(int32_t device, int32_t n, int32_t n_groups, int32_t d_in, int32_t n_entries, const void* x,
                      const void* W, const float* bias, int32_t* idx_out, int32_t variant, void* stream)
 {
@@ -1637,16 +1707,12 @@ ckv_status ckv_route(int32_t device, int32_t n, int32_t n_groups, int32_t d_in, 
     if (variant == 1) {
         e = launch_route(d_in, x, W, bias, n, n_entries, n_groups, idx_out, s);
     } else {
-        int* word = route_err_word(device);
-        if (!word) return CKV_ERR_OOM;
-        e = launch_route_umma(d_in, x, W, bias, n, n_entries, n_groups, idx_out, word, s);
-        int bad = 0;
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&bad, word, sizeof(int), cudaMemcpyDeviceToHost, s);
+        HostFlag flag;
+        if (!flag.p) return CKV_ERR_OOM;
+        e = launch_route_umma(d_in, x, W, bias, n, n_entries, n_groups, idx_out, flag.p, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e == cudaSuccess && bad) {  // a bounded wait inside the kernel ran out: the output is not valid
-            cudaMemsetAsync(word, 0, sizeof(int), s);
-            return CKV_ERR_CUDA;
-        }
+        // a bounded wait inside the kernel ran out: the output is not valid
+        if (e == cudaSuccess && *(volatile int*)flag.p) return CKV_ERR_CUDA;
     }
     if (e != cudaSuccess) {
         cudaGetLastError();

@@ -158,16 +158,25 @@ cudaError_t launch_kernel(const Launch& l, void (*fn)(P...), dim3 grid, int thre
 // ---- kernels_pack.cu
 cudaError_t launch_pool_layout(int dtype, int G, int m, int d_shared, int D, const void* src,
                                void* dst, cudaStream_t s);
-// Packs n users' [P][G] indices and [P][G][d_user] user parts into arena units and
-// validates index range; *bad_flag (device int) is OR-ed with 1 on a bad index.
-// The arena arrays and the sides' widths come from `cv` (head_dim D).
-cudaError_t launch_pack(int dtype, int G, int n_entries, int idx_bytes, int n_users,
-                        const int64_t* hist_off_dev, const int64_t* unit_off_dev,
-                        int64_t total_units, int64_t arena_base, const int32_t* idxK,
+// One user of a put: where its positions start in the [P][G] inputs and its 32-position tiles among those of the batch.
+struct PutUser {
+    int64_t pos0;
+    int32_t tile0, L;
+};
+constexpr int kInlinePuts = 224;  // users whose table travels as a kernel argument
+struct PutTable {
+    PutUser u[kInlinePuts];
+};
+// Packs n users' [P][G] indices and [P][G][d_user] user parts into arena units and validates the index range;
+// *bad_flag (host-mapped int) becomes 1 on a bad index.  The users come from `table` (device memory) or, if that is
+// null, from *inl.  The arena arrays and the sides' widths come from `cv` (head_dim D).
+cudaError_t launch_pack(int dtype, int G, int n_entries, int idx_bytes, int n_users, const PutUser* table,
+                        const PutTable* inl, int64_t total_tiles, int64_t arena_base, const int32_t* idxK,
                         const int32_t* idxV, const void* userK, const void* userV, const CacheView& cv, int D,
                         int* bad_flag, cudaStream_t s);
 // Writes a user's units for L_old + L_new positions at arena unit dst_base: the first L_old positions copied from
-// the units at old_base (same arena), the rest packed from the new [L_new][G] indices and [L_new][G][d_user] parts.
+// the units at old_base (same arena), the rest packed from the new [L_new][G] indices and [L_new][G][d_user] parts.  dst_base = old_base (and
+// Lpad_tot = Lpad_old): the new positions are written behind the old ones, in place.
 cudaError_t launch_append(int dtype, int G, int n_entries, int idx_bytes, int64_t old_base, int L_old,
                           int Lpad_old, int64_t dst_base, int L_new, int Lpad_tot, const int32_t* idxK,
                           const int32_t* idxV, const void* userK, const void* userV, const CacheView& cv, int D,
@@ -175,7 +184,7 @@ cudaError_t launch_append(int dtype, int G, int n_entries, int idx_bytes, int64_
 cudaError_t launch_materialize(int dtype, int D, const CacheView& cv, int64_t base, int L, int Lpad,
                                void* K_out, void* V_out, cudaStream_t s);
 
-// ORs 1 into *bad_flag (device int) if any of the n_units stored K or V indices is >= n_entries (idxK or idxV may be
+// *bad_flag (host-mapped int) becomes 1 if any of the n_units stored K or V indices is >= n_entries (idxK or idxV may be
 // null: that side is not checked).
 cudaError_t launch_check_indices(int idx_bytes, int n_entries, const void* idxK, const void* idxV, int64_t n_units,
                                  int* bad_flag, cudaStream_t s);
@@ -219,7 +228,7 @@ cudaError_t launch_route(int d_in, const void* x, const void* W, const float* bi
                          int32_t* out, cudaStream_t s);
 
 // ---- kernels_route_umma.cu : the same router on tcgen05 (TMEM accumulators, warp-specialised)
-// err_flag: device int, OR-ed with a non-zero code if a bounded wait inside the kernel ran out (nothing is written then).
+// err_flag: host-mapped int, set to a non-zero code if a bounded wait inside the kernel ran out (nothing is written then).
 cudaError_t launch_route_umma(int d_in, const void* x, const void* W, const float* bias, int n, int n_entries, int G,
                               int32_t* out, int* err_flag, cudaStream_t s);
 

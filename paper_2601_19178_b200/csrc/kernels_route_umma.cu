@@ -304,7 +304,7 @@ __global__ void __launch_bounds__(kThreadsRU, 1)
     tc_after();
     if (warp == kIssueWarp)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
-    if (tid == 0 && *abort_flag) atomicOr(err_flag, ERR_ROUTE);
+    if (tid == 0 && *abort_flag) *reinterpret_cast<volatile int*>(err_flag) = ERR_ROUTE;
 }
 
 template <int DIN>
@@ -321,7 +321,7 @@ cudaError_t launch_t(const void* x, const void* W, const float* bias, int n, int
 
 }  // namespace
 
-// err_flag: device int, OR-ed with a non-zero code if a bounded wait inside the kernel ran out (nothing is written then).
+// err_flag: host-mapped int, set to a non-zero code if a bounded wait inside the kernel ran out (nothing is written then).
 cudaError_t launch_route_umma(int d_in, const void* x, const void* W, const float* bias, int n, int n_entries, int G,
                               int32_t* out, int* err_flag, cudaStream_t s)
 {
