@@ -1,14 +1,20 @@
 // Prefill router (Sec. 4.3) on the tcgen05 tensor cores: I[i][g] = lowest j maximising x_i . W_g[j] + b_g[j].
 //
-// One CTA owns 256 positions of one group, as two blocks of 128.  Their inputs sit in shared memory once (A operand,
-// K-major core-matrix layout); the group's weight rows stream through a four-stage ring in tiles of 128 entries
-// (B operand, same layout, 16-byte cp.async by four producer warps, each bound to one stage), and every tile is
-// multiplied with both blocks, which halves the weight traffic out of L2 per product.  One thread issues the two
-// 128 x 128 x d_in products of a tile into the tile's two TMEM accumulators (two per block, alternating: all 512
-// columns); two groups of four warps, one per block (thread = position = TMEM lane), read their accumulator, add
-// the bias, and keep a running (best score, entry) in registers, so the score matrix never leaves the SM.
+// One CTA owns 256 positions of one group, as two blocks of 128, and every S-th share of the group's entries (S CTAs in
+// a cluster share the positions when there are too few of them to fill the SMs).  The positions' inputs sit in TMEM
+// (A operand, lane = position); the group's weight rows stream through a ring of shared-memory stages in tiles of 128
+// entries (B operand, one swizzled TMA box per tile), and every tile is multiplied with both blocks.  The bias is one
+// more K = 16 step of the product, ones times the bias cut into three bf16 parts whose sum is the fp32 bias exactly, so
+// the read-out touches no shared memory.  One thread issues the products into three 128-column TMEM accumulators in
+// turn; two groups of four warps, one per block (thread = position = TMEM lane), fetch their accumulator into registers,
+// release it at once, and keep a running (best score, entry); the score matrix never leaves the SM.
+// What bounds it: the 128 x 128 x 16 products (64 clocks each, five per block and tile at d_in = 64) and, behind them,
+// the hand-offs between the issuing thread and the read-out.  Keeping shared memory to the B operand is what matters:
+// with A in shared memory too the operand fetch takes all of its 128 bytes per clock, and the bias loads and weight
+// stores that compete with it held the previous form of this kernel at 2100 clocks per tile.
 // Every wait is bounded: a time-out raises the CTA's abort flag, the CTA drains, frees its TMEM, reports through
 // the error word and writes nothing.
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <math_constants.h>
 
@@ -17,14 +23,15 @@
 namespace ckv {
 namespace {
 
-constexpr int kRows = 256, kTileN = 128, kMaxStages = 4, kBiasSlots = 8;
-constexpr int kEpiWarps = 8, kIssueWarp = 8, kProdWarp0 = 9, kProdWarps = 4;
-constexpr int kThreadsRU = (kProdWarp0 + kProdWarps) * 32;
+constexpr int kRows = 256, kTileN = 128, kAcc = 3;
+constexpr int kEpiWarps = 8, kIssueWarp = 8, kLoadWarp = 9, kBiasWarp = 10;
+constexpr int kThreadsRU = (kBiasWarp + 1) * 32;
+constexpr int kMaxClusterRU = 8;
 constexpr uint32_t kSpin = 1u << 18, kSuspend = 4000;
 enum { ERR_ROUTE = 64 };
 
-// B_AFULL / B_AEMPTY: [2 * block + buffer]
-enum Bar { B_FULL = 0, B_EMPTY = kMaxStages, B_AFULL = 2 * kMaxStages, B_AEMPTY = 2 * kMaxStages + 4, B_DRAIN = 2 * kMaxStages + 8, B_COUNT };
+constexpr int kMaxStages = 8;
+enum Bar { B_FULL = 0, B_EMPTY = kMaxStages, B_AFULL = 2 * kMaxStages, B_AEMPTY = B_AFULL + kAcc, B_DRAIN = B_AEMPTY + kAcc, B_COUNT };
 
 __device__ __forceinline__ uint32_t s_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void bar_init(uint32_t bar, uint32_t count)
@@ -66,6 +73,14 @@ __device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_
         "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(acc)
         : "memory");
 }
+__device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t acc)
+{
+    asm volatile(
+        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
+        "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(acc)
+        : "memory");
+}
 // shared-memory matrix descriptor, no swizzle: start address, leading / stride byte offsets (16-byte units), version 1
 __device__ __forceinline__ uint64_t mat_desc(uint32_t addr, uint32_t lbo_bytes, uint32_t sbo_bytes)
 {
@@ -101,42 +116,52 @@ __device__ __forceinline__ void wait_ld32(uint32_t (&r)[32])
                  :
                  : "memory");
 }
+// 16 / 32 consecutive columns of this thread's lane
+__device__ __forceinline__ void st16(uint32_t taddr, const uint32_t* r)
+{
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(
+            taddr),
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+        "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+        : "memory");
+}
 __device__ __forceinline__ float max3f(float a, float b, float c)
 {
     float r;
     asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
     return r;
 }
-// 16-byte copy global -> shared; src_bytes = 0 fills the destination with zeros instead
-__device__ __forceinline__ void cp16(uint32_t dst, const void* src, uint32_t src_bytes)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
-}
-
 template <int DIN>
 struct RU {
-    static constexpr int CPR = DIN / 8;              // 16-byte chunks per row
-    static constexpr int SBO = CPR * 128;            // bytes per group of 8 rows
-    static constexpr int XTILE = kRows * DIN * 2;    // bytes of the positions' tile
-    static constexpr int TILE = kTileN * DIN * 2;    // bytes of a weight tile
-    static constexpr int STAGES = 4;
-    static constexpr int PPT = kProdWarps / STAGES;  // producer warps that share one tile (each stage has its own warps)
-    static constexpr int OFF_X = 0, OFF_W = XTILE, OFF_BIAS = OFF_W + STAGES * TILE,
-                         OFF_BAR = OFF_BIAS + kBiasSlots * kTileN * 4,
-                         OFF_ABORT = OFF_BAR + 24 * 8, SMEM = OFF_ABORT + 16;
+    static constexpr int ROWB = DIN >= 64 ? 128 : 64;      // bytes of a row inside a TMA box = its swizzle span
+    static constexpr int BOXES = DIN == 128 ? 2 : 1;       // boxes (of 64 inputs) per tile
+    static constexpr int BOX = kTileN * ROWB;              // bytes of a box
+    static constexpr int TILE = BOXES * BOX;               // bytes of a weight tile
+    static constexpr int STAGES = DIN == 128 ? 5 : 8;
+    static constexpr int BIAS = kTileN * 32;               // bytes of a tile's bias step (16 bf16 per entry)
+    static constexpr int OFF_W = 0, OFF_BIAS = STAGES * TILE, OFF_ONES = OFF_BIAS + STAGES * BIAS,
+                         OFF_BEST = OFF_ONES + 128 * 32,   // [kRows] (score, entry): read by the cluster's first CTA
+                         OFF_BAR = OFF_BEST + kRows * 8, OFF_ABORT = OFF_BAR + B_COUNT * 8, SMEM = OFF_ABORT + 16;
+    static_assert(STAGES <= kMaxStages && SMEM <= 227 * 1024, "shared memory");
+    static constexpr uint32_t COL_A = kAcc * kTileN;       // TMEM columns of the inputs, DIN / 2 per block
+    static_assert(COL_A + 2 * (DIN / 2) <= 512, "TMEM columns");
 };
-// byte offset of (row r, 16-byte chunk c) in the K-major core-matrix layout: 8 x 16-byte core matrices, chunks of a
-// row group 128 bytes apart, row groups SBO apart
+// Swizzled K-major operand (TMA box of ROWB-byte rows, groups of eight rows ROWB * 8 bytes apart).
 template <int DIN>
-__device__ __forceinline__ uint32_t tile_off(int r, int c)
+__device__ __forceinline__ uint64_t swz_desc(uint32_t addr)
 {
-    return (uint32_t)((r >> 3) * RU<DIN>::SBO + c * 128 + (r & 7) * 16);
+    constexpr uint64_t layout = RU<DIN>::ROWB == 128 ? 2 : 4;  // 128-byte / 64-byte swizzle
+    return (uint64_t)((addr & 0x3ffffu) >> 4) | (1ull << 16) | ((uint64_t)(RU<DIN>::ROWB * 8 >> 4) << 32) | (1ull << 46) |
+           (layout << 61);
 }
+// K-major core matrices of 16 bf16 per row, no swizzle: row r, 16-byte chunk c
+__device__ __forceinline__ uint32_t step_off(int r, int c) { return (uint32_t)((r >> 3) * 256 + c * 128 + (r & 7) * 16); }
 
 template <int DIN>
 __global__ void __launch_bounds__(kThreadsRU, 1)
-    route_umma_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ W, const float* __restrict__ bias, int n,
-                      int m, int G, int32_t* __restrict__ out, int* __restrict__ err_flag)
+    route_umma_kernel(const uint16_t* __restrict__ x, const __grid_constant__ CUtensorMap tmW, const float* __restrict__ bias,
+                      int n, int m, int G, int32_t* __restrict__ out, int* err_flag, int n_split)
 {
     using L = RU<DIN>;
     extern __shared__ __align__(1024) unsigned char usm[];
@@ -145,18 +170,22 @@ __global__ void __launch_bounds__(kThreadsRU, 1)
     const uint32_t sb = s_u32(usm);
     auto bar = [&](int i) { return sb + L::OFF_BAR + 8u * (uint32_t)i; };
     volatile int* abort_flag = reinterpret_cast<volatile int*>(usm + L::OFF_ABORT);
-    const int grp = blockIdx.y;
-    const int64_t row0 = (int64_t)blockIdx.x * kRows;
-    const uint16_t* Wg = W + (int64_t)grp * m * DIN;
+    const int grp = blockIdx.y, split = (int)(blockIdx.x % (uint32_t)n_split);
+    const int64_t row0 = (int64_t)(blockIdx.x / (uint32_t)n_split) * kRows;
+    const int n_blocks = n - row0 > 128 ? 2 : 1;
     const float* bg = bias ? bias + (int64_t)grp * m : nullptr;
-    const int n_tiles = (m + kTileN - 1) / kTileN;
+    // this CTA's tiles of the group's entries
+    const int all_tiles = (m + kTileN - 1) / kTileN;
+    const int tile0 = (int)((int64_t)all_tiles * split / n_split), n_tiles = (int)((int64_t)all_tiles * (split + 1) / n_split) - tile0;
+    // a tile needs the bias step if there is a bias, or entries past the last one to rule out
+    auto biased = [&](int t) { return bg != nullptr || (tile0 + t + 1) * kTileN > m; };
 
     if (tid == 0) {
         for (int s = 0; s < L::STAGES; ++s) {
-            bar_init(bar(B_FULL + s), L::PPT);
+            bar_init(bar(B_FULL + s), 2);  // the loading thread (with the box's bytes) and the bias warp
             bar_init(bar(B_EMPTY + s), 1);
         }
-        for (int e = 0; e < 4; ++e) {
+        for (int e = 0; e < kAcc; ++e) {
             bar_init(bar(B_AFULL + e), 1);
             bar_init(bar(B_AEMPTY + e), 128);
         }
@@ -169,98 +198,122 @@ __global__ void __launch_bounds__(kThreadsRU, 1)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    // the positions' inputs, once: row r of the tile is position row0 + r (zero rows past the end)
-    for (int q = tid; q < kRows * L::CPR; q += kThreadsRU) {
-        const int r = (q & 7) + 8 * (q / (8 * L::CPR)), c = (q >> 3) % L::CPR;
-        const bool in = row0 + r < n;
-        cp16(sb + L::OFF_X + tile_off<DIN>(r, c), x + (in ? (row0 + r) * DIN + c * 8 : 0), in ? 16u : 0u);
+    if (warp == kBiasWarp) {
+        // A operand of the bias step: three ones per position; and the second chunk of every bias slot stays zero
+        for (int r = lane; r < 128; r += 32) {
+            *reinterpret_cast<uint4*>(usm + L::OFF_ONES + step_off(r, 0)) = make_uint4(0x3f803f80u, 0x3f80u, 0, 0);
+            *reinterpret_cast<uint4*>(usm + L::OFF_ONES + step_off(r, 1)) = make_uint4(0, 0, 0, 0);
+            for (int s = 0; s < L::STAGES; ++s)
+                *reinterpret_cast<uint4*>(usm + L::OFF_BIAS + s * L::BIAS + step_off(r, 1)) = make_uint4(0, 0, 0, 0);
+        }
+        fence_async();
     }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    fence_async();
     tc_before();
     __syncthreads();
     tc_after();
     const uint32_t tmem = tmem_slot;
     bool ok = true;
+    float best = -CUDART_INF_F;
+    int arg = 0;
+
+    const int e = warp >> 2;  // block of a read-out warp
+    const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
+    const int row = 128 * e + (warp & 3) * 32 + lane;  // its thread's position
+    if (warp < kEpiWarps && e < n_blocks) {
+        // the positions' inputs, once: two bf16 per column (zero rows past the end)
+        const uint4* xr = reinterpret_cast<const uint4*>(x + (row0 + row) * DIN);
+        const bool in = row0 + row < n;
+#pragma unroll
+        for (int h = 0; h < DIN / 32; ++h) {
+            uint32_t v[16];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint4 w = in ? __ldg(xr + 4 * h + q) : make_uint4(0, 0, 0, 0);
+                v[4 * q] = w.x; v[4 * q + 1] = w.y; v[4 * q + 2] = w.z; v[4 * q + 3] = w.w;
+            }
+            st16(tmem + lane_base + L::COL_A + e * (DIN / 2) + 16 * h, v);
+        }
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    }
+    tc_before();
+    __syncthreads();
+    tc_after();
 
     if (warp < kEpiWarps) {
         // ------------------------------------------------------------ running arg-max, thread = position
-        const int e = warp >> 2, row = 128 * e + (warp & 3) * 32 + lane;  // block e, position row of the CTA
-        const uint32_t tacc0 = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(2 * kTileN * e);
-        float best = -CUDART_INF_F;
-        int arg = 0;
-        for (int t = 0; t < n_tiles && ok; ++t) {
-            const int a = t & 1;
-            ok = bar_wait(bar(B_AFULL + 2 * e + a), (t >> 1) & 1, abort_flag);
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
-            tc_after();
-            const uint32_t tacc = tacc0 + (uint32_t)(kTileN * a);
-            const float4* bs = reinterpret_cast<const float4*>(usm + L::OFF_BIAS) + (t % kBiasSlots) * (kTileN / 4);
-            const int j0 = t * kTileN;
-            // 32 columns at a time, the next 32 already on their way out of TMEM.  Only the maximum of a block is
-            // compared with the running best (a new best gets rare quickly); the block is searched for its first
-            // maximal column only then.  Entries come in increasing order and the comparison is strict, so the
-            // lowest entry wins among equals; past the last entry the bias slot holds -inf.
-            uint32_t va[32], vb[32];
-            ld32(tacc, va);
-            auto block = [&](uint32_t (&v)[32], int c4) {
-                float f[32];
+        if (e < n_blocks) {
+            for (int t = 0; t < n_tiles; ++t) {
+                const int k = n_blocks * t + e, a = k % kAcc;
+                ok = bar_wait(bar(B_AFULL + a), (k / kAcc) & 1, abort_flag);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                tc_after();
+                const uint32_t tacc = tmem + lane_base + (uint32_t)(kTileN * a);
+                const int j0 = (tile0 + t) * kTileN;
+                // the whole accumulator into registers, so that it is free again before it is looked at
+                uint32_t v[4][32];
 #pragma unroll
-                for (int k = 0; k < 32; k += 4) {
-                    const float4 b4 = bs[8 * c4 + (k >> 2)];
-                    f[k] = __uint_as_float(v[k]) + b4.x;
-                    f[k + 1] = __uint_as_float(v[k + 1]) + b4.y;
-                    f[k + 2] = __uint_as_float(v[k + 2]) + b4.z;
-                    f[k + 3] = __uint_as_float(v[k + 3]) + b4.w;
+                for (int c = 0; c < 4; ++c) ld32(tacc + 32 * c, v[c]);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) wait_ld32(v[c]);
+                tc_before();
+                bar_arrive(bar(B_AEMPTY + a));
+                // Only the maximum of 32 columns is compared with the running best (a new best gets rare quickly); they
+                // are searched for their first maximal column only then.  Entries come in increasing order and the
+                // comparison is strict, so the lowest entry wins among equals; past the last entry the bias is -inf.
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    float m0 = __uint_as_float(v[c][0]), m1 = __uint_as_float(v[c][1]);
+#pragma unroll
+                    for (int q = 2; q < 30; q += 4) {
+                        m0 = max3f(m0, __uint_as_float(v[c][q]), __uint_as_float(v[c][q + 1]));
+                        m1 = max3f(m1, __uint_as_float(v[c][q + 2]), __uint_as_float(v[c][q + 3]));
+                    }
+                    const float mx = max3f(fmaxf(m0, m1), __uint_as_float(v[c][30]), __uint_as_float(v[c][31]));
+                    if (mx > best) {
+                        best = mx;
+                        int first = 31;
+#pragma unroll
+                        for (int q = 30; q >= 0; --q) first = __uint_as_float(v[c][q]) == mx ? q : first;
+                        arg = j0 + 32 * c + first;
+                    }
                 }
-                float mx = f[0];
-#pragma unroll
-                for (int k = 1; k + 1 < 32; k += 2) mx = max3f(mx, f[k], f[k + 1]);
-                mx = fmaxf(mx, f[31]);
-                if (mx > best) {
-                    best = mx;
-                    int first = 31;
-#pragma unroll
-                    for (int k = 30; k >= 0; --k) first = f[k] == mx ? k : first;
-                    arg = j0 + 32 * c4 + first;
-                }
-            };
-#pragma unroll 1
-            for (int c4 = 0; c4 < kTileN / 32; c4 += 2) {
-                wait_ld32(va);
-                ld32(tacc + 32 * (c4 + 1), vb);
-                block(va, c4);
-                wait_ld32(vb);
-                if (c4 + 2 < kTileN / 32) ld32(tacc + 32 * (c4 + 2), va);
-                block(vb, c4 + 1);
             }
-            tc_before();
-            bar_arrive(bar(B_AEMPTY + 2 * e + a));
         }
-        if (ok && !*abort_flag && row0 + row < n) out[(row0 + row) * G + grp] = arg;
         if (!ok) *abort_flag = 1;
     } else if (warp == kIssueWarp) {
         // ------------------------------------------------------------ MMA issue
         if (lane == 0) {
             constexpr uint32_t idesc = idesc_bf16(128, kTileN);
+            const uint64_t ones = mat_desc(sb + L::OFF_ONES, 128, 256);
+            int s = 0, a = 0;
+            uint32_t ps = 0, pa = 1;  // parities: stage full; accumulator free (the first round passes)
             for (int t = 0; t < n_tiles && ok; ++t) {
-                const int s = t % L::STAGES, a = t & 1;
-                ok = bar_wait(bar(B_FULL + s), (t / L::STAGES) & 1, abort_flag);
-                for (int e = 0; e < 2 && ok; ++e) {
-                    if (t >= 2) ok = bar_wait(bar(B_AEMPTY + 2 * e + a), ((t >> 1) - 1) & 1, abort_flag);
+                ok = bar_wait(bar(B_FULL + s), ps, abort_flag);
+                const uint64_t w = swz_desc<DIN>(sb + L::OFF_W + s * L::TILE),
+                               b = mat_desc(sb + L::OFF_BIAS + s * L::BIAS, 128, 256);
+                const bool bt = biased(t);
+                for (int blk = 0; blk < n_blocks && ok; ++blk) {
+                    ok = bar_wait(bar(B_AEMPTY + a), pa, abort_flag);
                     if (!ok) break;
                     tc_after();
+                    const uint32_t d = tmem + (uint32_t)(kTileN * a), at = tmem + L::COL_A + blk * (DIN / 2);
 #pragma unroll
                     for (int ks = 0; ks < DIN / 16; ++ks)
-                        mma_ss(tmem + (uint32_t)(kTileN * (2 * e + a)),
-                               mat_desc(sb + L::OFF_X + e * 16 * L::SBO + ks * 256, 128, L::SBO),
-                               mat_desc(sb + L::OFF_W + s * L::TILE + ks * 256, 128, L::SBO), idesc, ks > 0 ? 1u : 0u);
-                    tc_commit_to(bar(B_AFULL + 2 * e + a));
+                        mma_ts(d, at + 8 * ks, w + (uint64_t)(((ks & 3) * 32 + (ks >> 2) * L::BOX) >> 4), idesc, ks > 0);
+                    if (bt) mma_ss(d, ones, b, idesc, 1u);
+                    tc_commit_to(bar(B_AFULL + a));
+                    if (++a == kAcc) {
+                        a = 0;
+                        pa ^= 1;
+                    }
                 }
                 if (!ok) break;
                 tc_commit_to(bar(B_EMPTY + s));
+                if (++s == L::STAGES) {
+                    s = 0;
+                    ps ^= 1;
+                }
             }
             if (!ok) *abort_flag = 1;
             // nothing of this CTA may still run on the tensor core at teardown
@@ -269,54 +322,150 @@ __global__ void __launch_bounds__(kThreadsRU, 1)
             if (!bar_wait(bar(B_DRAIN), 0, &never)) *abort_flag = 1;
         }
         __syncwarp();
+    } else if (warp == kLoadWarp) {
+        // ------------------------------------------------------------ weight tiles
+        if (lane == 0) {
+            int s = 0, issued = 0;
+            uint32_t pe = 1;
+            for (int t = 0; t < n_tiles; ++t) {
+                ok = bar_wait(bar(B_EMPTY + s), pe, abort_flag);
+                if (!ok) break;
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar(B_FULL + s)), "r"(L::TILE)
+                             : "memory");
+#pragma unroll
+                for (int h = 0; h < L::BOXES; ++h)
+                    asm volatile(
+                        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
+                        "[%4];" ::"r"(sb + L::OFF_W + s * L::TILE + h * L::BOX),
+                        "l"(&tmW), "r"(64 * h), "r"(grp * m + (tile0 + t) * kTileN), "r"(bar(B_FULL + s))
+                        : "memory");
+                ++issued;
+                if (++s == L::STAGES) {
+                    s = 0;
+                    pe ^= 1;
+                }
+            }
+            if (!ok) {
+                *abort_flag = 1;
+                // the copies in flight land before the CTA ends: every stage's last fill has its bytes (a stage whose
+                // bias arrival is missing times out here, with its bytes long there)
+                volatile int never = 0;
+                for (int k = issued > L::STAGES ? issued - L::STAGES : 0; k < issued; ++k)
+                    bar_wait(bar(B_FULL + k % L::STAGES), (k / L::STAGES) & 1, &never);
+            }
+        }
+        __syncwarp();
     } else {
-        // ------------------------------------------------------------ producers
-        // warp p works for stage p % STAGES only (its waits on that stage's barriers are then in phase order) and
-        // copies part p / STAGES of each of that stage's tiles
-        const int p = warp - kProdWarp0, part = p / L::STAGES;
-        constexpr int kPartRows = kTileN / L::PPT;
-        float* bias_s = reinterpret_cast<float*>(usm + L::OFF_BIAS);
-        for (int t = p % L::STAGES; t < n_tiles && ok; t += L::STAGES) {
-            const int s = t % L::STAGES, j0 = t * kTileN;
-            if (t >= L::STAGES) ok = bar_wait(bar(B_EMPTY + s), ((t / L::STAGES) - 1) & 1, abort_flag);
+        // ------------------------------------------------------------ bias steps: b = hi + mid + lo, bf16 each, exactly
+        int s = 0;
+        uint32_t pe = 1;
+        for (int t = 0; t < n_tiles; ++t) {
+            ok = bar_wait(bar(B_EMPTY + s), pe, abort_flag);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
-            const uint32_t dst = sb + L::OFF_W + s * L::TILE;
-            for (int q = lane; q < kPartRows * L::CPR; q += 32) {
-                const int r = part * kPartRows + (q & 7) + 8 * (q / (8 * L::CPR)), c = (q >> 3) % L::CPR;
-                const int j = min(j0 + r, m - 1);
-                cp16(dst + tile_off<DIN>(r, c), Wg + (int64_t)j * DIN + c * 8, 16u);
+            if (biased(t)) {
+#pragma unroll
+                for (int i = 0; i < kTileN / 32; ++i) {
+                    const int r = 32 * i + lane, j = (tile0 + t) * kTileN + r;
+                    const float b = j < m ? (bg ? __ldg(bg + j) : 0.f) : -CUDART_INF_F;
+                    const uint32_t hi = __float_as_uint(b) & 0xffff0000u;
+                    const float r1 = isfinite(b) ? b - __uint_as_float(hi) : 0.f;
+                    const uint32_t mid = __float_as_uint(r1) & 0xffff0000u, lo = __float_as_uint(r1 - __uint_as_float(mid));
+                    *reinterpret_cast<uint4*>(usm + L::OFF_BIAS + s * L::BIAS + step_off(r, 0)) =
+                        make_uint4((hi >> 16) | mid, lo >> 16, 0, 0);
+                }
+                fence_async();
             }
-            asm volatile("cp.async.commit_group;" ::: "memory");
-            for (int k = part * kPartRows + lane; k < (part + 1) * kPartRows; k += 32) {
-                const int j = j0 + k;
-                bias_s[(t % kBiasSlots) * kTileN + k] = j < m ? (bg ? __ldg(bg + j) : 0.f) : -CUDART_INF_F;
-            }
-            asm volatile("cp.async.wait_group 0;" ::: "memory");
-            fence_async();  // the copies of this lane are visible to the tensor core's proxy
             __syncwarp();
             if (lane == 0) bar_arrive(bar(B_FULL + s));
+            if (++s == L::STAGES) {
+                s = 0;
+                pe ^= 1;
+            }
         }
         if (!ok) *abort_flag = 1;
     }
+
     tc_before();
     __syncthreads();
     tc_after();
+    // (the TMEM goes back before the CTA waits for the others of its cluster: two clusters that had each other's SMs
+    // to wait for could otherwise block each other)
     if (warp == kIssueWarp)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+    // the CTAs of a cluster looked at different entries: the first of them, in the order of the entries, takes the best
+    if (n_split > 1) {
+        if (warp < kEpiWarps) {
+            float* mine = reinterpret_cast<float*>(usm + L::OFF_BEST) + 2 * row;
+            mine[0] = best;
+            mine[1] = __int_as_float(arg);
+        }
+        __syncwarp();
+        asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (split == 0 && warp < kEpiWarps) {
+            for (int r = 1; r < n_split; ++r) {
+                uint32_t remote;
+                float b2, a2;
+                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(sb + L::OFF_BEST + 8 * row), "r"(r));
+                asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(b2), "=f"(a2) : "r"(remote) : "memory");
+                if (b2 > best) {
+                    best = b2;
+                    arg = __float_as_int(a2);
+                }
+            }
+        }
+        __syncwarp();
+        asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+    if (warp < kEpiWarps && split == 0 && !*abort_flag && row0 + row < n) out[(row0 + row) * G + grp] = arg;
     if (tid == 0 && *abort_flag) *reinterpret_cast<volatile int*>(err_flag) = ERR_ROUTE;
+}
+
+// The weights as rows of `d_in` inputs, boxes of 128 rows and at most 64 inputs.
+bool make_weight_map(int d_in, int64_t rows, const void* W, CUtensorMap* map)
+{
+    typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                 const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                                 CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+    static const EncodeFn encode = [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        const bool ok = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q) == cudaSuccess &&
+                        q == cudaDriverEntryPointSuccess;
+        return ok ? reinterpret_cast<EncodeFn>(fn) : nullptr;
+    }();
+    if (!encode) return false;
+    const cuuint64_t dims[2] = {(cuuint64_t)d_in, (cuuint64_t)rows}, strides[1] = {(cuuint64_t)d_in * 2};
+    const cuuint32_t box[2] = {(cuuint32_t)(d_in < 64 ? d_in : 64), (cuuint32_t)kTileN}, estr[2] = {1, 1};
+    return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(W), dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, d_in < 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                  CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 template <int DIN>
 cudaError_t launch_t(const void* x, const void* W, const float* bias, int n, int m, int G, int32_t* out, int* err_flag,
                      cudaStream_t s)
 {
-    cudaError_t e = cudaFuncSetAttribute(route_umma_kernel<DIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, RU<DIN>::SMEM);
-    if (e != cudaSuccess) return e;
-    const dim3 grid((unsigned)((n + kRows - 1) / kRows), (unsigned)G);
-    route_umma_kernel<DIN><<<grid, kThreadsRU, RU<DIN>::SMEM, s>>>((const uint16_t*)x, (const uint16_t*)W, bias, n, m, G,
-                                                                   out, err_flag);
-    return cudaGetLastError();
+    CUtensorMap map;
+    if (!make_weight_map(DIN, (int64_t)G * m, W, &map)) return cudaErrorInvalidValue;
+    // CTAs per position block: as many as shorten the run most, counting whole waves of CTAs over the SMs and about
+    // four tiles' time for setting one up
+    int dev = 0, sms = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int64_t ctas = (int64_t)((n + kRows - 1) / kRows) * G, tiles = (m + kTileN - 1) / kTileN;
+    int split = 1;
+    int64_t best = INT64_MAX;
+    for (int sp = 1; sp <= kMaxClusterRU && sp <= tiles; sp *= 2) {
+        const int64_t cost = (ctas * sp + sms - 1) / sms * ((tiles + sp - 1) / sp + 4);
+        if (cost < best) {
+            best = cost;
+            split = sp;
+        }
+    }
+    const dim3 grid((unsigned)((n + kRows - 1) / kRows * split), (unsigned)G);
+    return launch_kernel(Launch{s, nullptr, nullptr}, route_umma_kernel<DIN>, grid, kThreadsRU, RU<DIN>::SMEM, split,
+                         (const uint16_t*)x, map, bias, n, m, G, out, err_flag, split);
 }
 
 }  // namespace
