@@ -24,14 +24,16 @@ namespace ckv {
 namespace {
 
 constexpr int kRows = 256, kTileN = 128, kAcc = 3;
-constexpr int kEpiWarps = 8, kIssueWarp = 8, kLoadWarp = 9, kBiasWarp = 10;
-constexpr int kThreadsRU = (kBiasWarp + 1) * 32;
+constexpr int kEpiWarps = 8, kIssueWarp = kEpiWarps, kIssuers = 2, kLoadWarp = kIssueWarp + kIssuers, kBiasWarp = kLoadWarp + 1;
+constexpr int kThreadsRU = (kBiasWarp + 1) * 32;  // twelve warps: 168 registers for a read-out thread's 128 columns
 constexpr int kMaxClusterRU = 8;
 constexpr uint32_t kSpin = 1u << 18, kSuspend = 4000;
 enum { ERR_ROUTE = 64 };
 
-constexpr int kMaxStages = 8;
-enum Bar { B_FULL = 0, B_EMPTY = kMaxStages, B_AFULL = 2 * kMaxStages, B_AEMPTY = B_AFULL + kAcc, B_DRAIN = B_AEMPTY + kAcc, B_COUNT };
+// A step k is (tile, block); it uses accumulator k mod 3.  With two blocks an accumulator goes from one block to the
+// other, so that its uses are told apart by barriers per step mod 6: each has one waiting role, which meets every phase.
+constexpr int kMaxStages = 8, kAccBars = 2 * kAcc;
+enum Bar { B_FULL = 0, B_EMPTY = kMaxStages, B_AFULL = 2 * kMaxStages, B_AEMPTY = B_AFULL + kAccBars, B_DRAIN = B_AEMPTY + kAccBars, B_COUNT };
 
 __device__ __forceinline__ uint32_t s_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void bar_init(uint32_t bar, uint32_t count)
@@ -141,9 +143,9 @@ struct RU {
     static constexpr int STAGES = DIN == 128 ? 5 : 8;
     static constexpr int BIAS = kTileN * 32;               // bytes of a tile's bias step (16 bf16 per entry)
     static constexpr int OFF_W = 0, OFF_BIAS = STAGES * TILE, OFF_ONES = OFF_BIAS + STAGES * BIAS,
-                         OFF_BEST = OFF_ONES + 128 * 32,   // [kRows] (score, entry): read by the cluster's first CTA
+                         OFF_BEST = OFF_ONES + 128 * 32,   // [kRows] (score, entry), read by the cluster's first CTA
                          OFF_BAR = OFF_BEST + kRows * 8, OFF_ABORT = OFF_BAR + B_COUNT * 8, SMEM = OFF_ABORT + 16;
-    static_assert(STAGES <= kMaxStages && SMEM <= 227 * 1024, "shared memory");
+    static_assert(STAGES <= kMaxStages && SMEM <= 226 * 1024, "shared memory");
     static constexpr uint32_t COL_A = kAcc * kTileN;       // TMEM columns of the inputs, DIN / 2 per block
     static_assert(COL_A + 2 * (DIN / 2) <= 512, "TMEM columns");
 };
@@ -183,13 +185,13 @@ __global__ void __launch_bounds__(kThreadsRU, 1)
     if (tid == 0) {
         for (int s = 0; s < L::STAGES; ++s) {
             bar_init(bar(B_FULL + s), 2);  // the loading thread (with the box's bytes) and the bias warp
-            bar_init(bar(B_EMPTY + s), 1);
+            bar_init(bar(B_EMPTY + s), (uint32_t)n_blocks);
         }
-        for (int e = 0; e < kAcc; ++e) {
+        for (int e = 0; e < kAccBars; ++e) {
             bar_init(bar(B_AFULL + e), 1);
             bar_init(bar(B_AEMPTY + e), 128);
         }
-        bar_init(bar(B_DRAIN), 1);
+        bar_init(bar(B_DRAIN), kIssuers);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -203,9 +205,9 @@ __global__ void __launch_bounds__(kThreadsRU, 1)
         for (int r = lane; r < 128; r += 32) {
             *reinterpret_cast<uint4*>(usm + L::OFF_ONES + step_off(r, 0)) = make_uint4(0x3f803f80u, 0x3f80u, 0, 0);
             *reinterpret_cast<uint4*>(usm + L::OFF_ONES + step_off(r, 1)) = make_uint4(0, 0, 0, 0);
-            for (int s = 0; s < L::STAGES; ++s)
-                *reinterpret_cast<uint4*>(usm + L::OFF_BIAS + s * L::BIAS + step_off(r, 1)) = make_uint4(0, 0, 0, 0);
         }
+        for (int r = lane; r < kTileN * L::STAGES; r += 32)  // (slots are whole groups of eight rows, one behind the other)
+            *reinterpret_cast<uint4*>(usm + L::OFF_BIAS + step_off(r, 1)) = make_uint4(0, 0, 0, 0);
         fence_async();
     }
     tc_before();
@@ -216,10 +218,11 @@ __global__ void __launch_bounds__(kThreadsRU, 1)
     float best = -CUDART_INF_F;
     int arg = 0;
 
-    const int e = warp >> 2;  // block of a read-out warp
+    // four read-out warps and one issuing thread per block of positions
+    const int e = warp >> 2;
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-    const int row = 128 * e + (warp & 3) * 32 + lane;  // its thread's position
-    if (warp < kEpiWarps && e < n_blocks) {
+    const int row = 128 * e + (warp & 3) * 32 + lane;  // this read-out thread's position
+    if (warp < 4 * n_blocks) {
         // the positions' inputs, once: two bf16 per column (zero rows past the end)
         const uint4* xr = reinterpret_cast<const uint4*>(x + (row0 + row) * DIN);
         const bool in = row0 + row < n;
@@ -241,79 +244,64 @@ __global__ void __launch_bounds__(kThreadsRU, 1)
 
     if (warp < kEpiWarps) {
         // ------------------------------------------------------------ running arg-max, thread = position
-        if (e < n_blocks) {
-            for (int t = 0; t < n_tiles; ++t) {
-                const int k = n_blocks * t + e, a = k % kAcc;
-                ok = bar_wait(bar(B_AFULL + a), (k / kAcc) & 1, abort_flag);
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok) break;
-                tc_after();
-                const uint32_t tacc = tmem + lane_base + (uint32_t)(kTileN * a);
-                const int j0 = (tile0 + t) * kTileN;
-                // the whole accumulator into registers, so that it is free again before it is looked at
-                uint32_t v[4][32];
+        for (int t = 0; e < n_blocks && t < n_tiles; ++t) {
+            const int k = n_blocks * t + e, b = k % kAccBars;
+            ok = bar_wait(bar(B_AFULL + b), (k / kAccBars) & 1, abort_flag);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            tc_after();
+            const uint32_t tacc = tmem + lane_base + (uint32_t)(kTileN * (k % kAcc));
+            const int j0 = (tile0 + t) * kTileN;
+            // the whole accumulator into registers, so that it is free again before it is looked at
+            uint32_t v[kTileN / 32][32];
 #pragma unroll
-                for (int c = 0; c < 4; ++c) ld32(tacc + 32 * c, v[c]);
+            for (int c = 0; c < kTileN / 32; ++c) ld32(tacc + 32 * c, v[c]);
 #pragma unroll
-                for (int c = 0; c < 4; ++c) wait_ld32(v[c]);
-                tc_before();
-                bar_arrive(bar(B_AEMPTY + a));
-                // Only the maximum of 32 columns is compared with the running best (a new best gets rare quickly); they
-                // are searched for their first maximal column only then.  Entries come in increasing order and the
-                // comparison is strict, so the lowest entry wins among equals; past the last entry the bias is -inf.
+            for (int c = 0; c < kTileN / 32; ++c) wait_ld32(v[c]);
+            tc_before();
+            bar_arrive(bar(B_AEMPTY + b));
+            // Only the maximum of 32 columns is compared with the running best (a new best gets rare quickly); they are
+            // searched for their first maximal column only then.  Entries come in increasing order and the comparison
+            // is strict, so the lowest entry wins among equals; past the last entry the bias is -inf.
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    float m0 = __uint_as_float(v[c][0]), m1 = __uint_as_float(v[c][1]);
+            for (int c = 0; c < kTileN / 32; ++c) {
+                float m0 = __uint_as_float(v[c][0]), m1 = __uint_as_float(v[c][1]);
 #pragma unroll
-                    for (int q = 2; q < 30; q += 4) {
-                        m0 = max3f(m0, __uint_as_float(v[c][q]), __uint_as_float(v[c][q + 1]));
-                        m1 = max3f(m1, __uint_as_float(v[c][q + 2]), __uint_as_float(v[c][q + 3]));
-                    }
-                    const float mx = max3f(fmaxf(m0, m1), __uint_as_float(v[c][30]), __uint_as_float(v[c][31]));
-                    if (mx > best) {
-                        best = mx;
-                        int first = 31;
+                for (int q = 2; q < 30; q += 4) {
+                    m0 = max3f(m0, __uint_as_float(v[c][q]), __uint_as_float(v[c][q + 1]));
+                    m1 = max3f(m1, __uint_as_float(v[c][q + 2]), __uint_as_float(v[c][q + 3]));
+                }
+                const float mx = max3f(fmaxf(m0, m1), __uint_as_float(v[c][30]), __uint_as_float(v[c][31]));
+                if (mx > best) {
+                    best = mx;
+                    int first = 31;
 #pragma unroll
-                        for (int q = 30; q >= 0; --q) first = __uint_as_float(v[c][q]) == mx ? q : first;
-                        arg = j0 + 32 * c + first;
-                    }
+                    for (int q = 30; q >= 0; --q) first = __uint_as_float(v[c][q]) == mx ? q : first;
+                    arg = j0 + 32 * c + first;
                 }
             }
         }
         if (!ok) *abort_flag = 1;
-    } else if (warp == kIssueWarp) {
-        // ------------------------------------------------------------ MMA issue
+    } else if (warp < kIssueWarp + kIssuers) {
+        // ------------------------------------------------------------ MMA issue, one thread per block
         if (lane == 0) {
             constexpr uint32_t idesc = idesc_bf16(128, kTileN);
             const uint64_t ones = mat_desc(sb + L::OFF_ONES, 128, 256);
-            int s = 0, a = 0;
-            uint32_t ps = 0, pa = 1;  // parities: stage full; accumulator free (the first round passes)
-            for (int t = 0; t < n_tiles && ok; ++t) {
-                ok = bar_wait(bar(B_FULL + s), ps, abort_flag);
-                const uint64_t w = swz_desc<DIN>(sb + L::OFF_W + s * L::TILE),
-                               b = mat_desc(sb + L::OFF_BIAS + s * L::BIAS, 128, 256);
-                const bool bt = biased(t);
-                for (int blk = 0; blk < n_blocks && ok; ++blk) {
-                    ok = bar_wait(bar(B_AEMPTY + a), pa, abort_flag);
-                    if (!ok) break;
-                    tc_after();
-                    const uint32_t d = tmem + (uint32_t)(kTileN * a), at = tmem + L::COL_A + blk * (DIN / 2);
-#pragma unroll
-                    for (int ks = 0; ks < DIN / 16; ++ks)
-                        mma_ts(d, at + 8 * ks, w + (uint64_t)(((ks & 3) * 32 + (ks >> 2) * L::BOX) >> 4), idesc, ks > 0);
-                    if (bt) mma_ss(d, ones, b, idesc, 1u);
-                    tc_commit_to(bar(B_AFULL + a));
-                    if (++a == kAcc) {
-                        a = 0;
-                        pa ^= 1;
-                    }
-                }
+            const int blk = warp - kIssueWarp;
+            for (int t = 0; blk < n_blocks && t < n_tiles; ++t) {
+                const int k = n_blocks * t + blk, s = t % L::STAGES, kp = k - kAcc;  // kp: the accumulator's use before
+                ok = bar_wait(bar(B_FULL + s), (t / L::STAGES) & 1, abort_flag) &&
+                     (kp < 0 || bar_wait(bar(B_AEMPTY + kp % kAccBars), (kp / kAccBars) & 1, abort_flag));
                 if (!ok) break;
+                tc_after();
+                const uint64_t w = swz_desc<DIN>(sb + L::OFF_W + s * L::TILE);
+                const uint32_t d = tmem + (uint32_t)(kTileN * (k % kAcc)), at = tmem + L::COL_A + blk * (DIN / 2);
+#pragma unroll
+                for (int ks = 0; ks < DIN / 16; ++ks)
+                    mma_ts(d, at + 8 * ks, w + (uint64_t)(((ks & 3) * 32 + (ks >> 2) * L::BOX) >> 4), idesc, ks > 0);
+                if (biased(t)) mma_ss(d, ones, mat_desc(sb + L::OFF_BIAS + s * L::BIAS, 128, 256), idesc, 1u);
+                tc_commit_to(bar(B_AFULL + k % kAccBars));
                 tc_commit_to(bar(B_EMPTY + s));
-                if (++s == L::STAGES) {
-                    s = 0;
-                    ps ^= 1;
-                }
             }
             if (!ok) *abort_flag = 1;
             // nothing of this CTA may still run on the tensor core at teardown
@@ -357,31 +345,42 @@ __global__ void __launch_bounds__(kThreadsRU, 1)
         __syncwarp();
     } else {
         // ------------------------------------------------------------ bias steps: b = hi + mid + lo, bf16 each, exactly
-        int s = 0;
-        uint32_t pe = 1;
-        for (int t = 0; t < n_tiles; ++t) {
-            ok = bar_wait(bar(B_EMPTY + s), pe, abort_flag);
+        // two tiles at a time: the wait, the fence and the hand-over are a chain, and one per tile would set the pace
+        constexpr int kPer = kTileN / 32;
+        auto load_bias = [&](int t, float (&b)[2 * kPer]) {
+#pragma unroll
+            for (int i = 0; i < 2 * kPer; ++i) {
+                const int j = (tile0 + t) * kTileN + 32 * i + lane;
+                b[i] = j < m ? (bg ? __ldg(bg + j) : 0.f) : -CUDART_INF_F;
+            }
+        };
+        float nxt[2 * kPer];
+        load_bias(0, nxt);
+        for (int t = 0; t < n_tiles; t += 2) {
+            float cur[2 * kPer];
+#pragma unroll
+            for (int i = 0; i < 2 * kPer; ++i) cur[i] = nxt[i];
+            load_bias(t + 2, nxt);
+            const int n_t = min(2, n_tiles - t);
+            for (int h = 0; h < n_t; ++h)
+                ok = ok && bar_wait(bar(B_EMPTY + (t + h) % L::STAGES), (((t + h) / L::STAGES) & 1) ^ 1, abort_flag);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
-            if (biased(t)) {
+            if (biased(t + n_t - 1)) {
 #pragma unroll
-                for (int i = 0; i < kTileN / 32; ++i) {
-                    const int r = 32 * i + lane, j = (tile0 + t) * kTileN + r;
-                    const float b = j < m ? (bg ? __ldg(bg + j) : 0.f) : -CUDART_INF_F;
+                for (int i = 0; i < 2 * kPer; ++i) {
+                    if (i >= kPer && n_t < 2) break;
+                    const float b = cur[i];
                     const uint32_t hi = __float_as_uint(b) & 0xffff0000u;
                     const float r1 = isfinite(b) ? b - __uint_as_float(hi) : 0.f;
                     const uint32_t mid = __float_as_uint(r1) & 0xffff0000u, lo = __float_as_uint(r1 - __uint_as_float(mid));
-                    *reinterpret_cast<uint4*>(usm + L::OFF_BIAS + s * L::BIAS + step_off(r, 0)) =
-                        make_uint4((hi >> 16) | mid, lo >> 16, 0, 0);
+                    *reinterpret_cast<uint4*>(usm + L::OFF_BIAS + (t + i / kPer) % L::STAGES * L::BIAS +
+                                              step_off(32 * (i % kPer) + lane, 0)) = make_uint4((hi >> 16) | mid, lo >> 16, 0, 0);
                 }
                 fence_async();
             }
             __syncwarp();
-            if (lane == 0) bar_arrive(bar(B_FULL + s));
-            if (++s == L::STAGES) {
-                s = 0;
-                pe ^= 1;
-            }
+            if (lane < n_t) bar_arrive(bar(B_FULL + (t + lane) % L::STAGES));
         }
         if (!ok) *abort_flag = 1;
     }
