@@ -222,6 +222,7 @@ __global__ void __launch_bounds__(128, MmaCfg<D, MT, TMA>::MIN_BLOCKS)
     }
     // rows 8..15 of the only query tile are all padding when the user has at most 8 queries
     const bool has_hi = MT > 1 || row0 + 8 < rq.M;
+    const int n_mt = (min(rq.M - row0, 16 * MT) + 15) >> 4;  // query tiles that hold queries
     // positions a query row attends: [0, lim); rows beyond the user's queries take none
     int lim[MT][2], lim_max = rq.L, lim_min = rq.L;
     if constexpr (VAR) {
@@ -427,37 +428,19 @@ __global__ void __launch_bounds__(128, MmaCfg<D, MT, TMA>::MIN_BLOCKS)
         __syncwarp();
         const bool tail = p0 + 32 > full_end;  // some (row, position) pair of this tile is not attended
 
-        uint32_t kf[4][2 * KS];
+        auto load_k = [&](int nt, uint32_t (&kf)[2 * KS]) {
 #pragma unroll
-        for (int nt = 0; nt < 4; ++nt) {
-            if constexpr (D == 64) {
-#pragma unroll
-                for (int kp = 0; kp < 2; ++kp)
-                    ldsm4(kf[nt][4 * kp], kf[nt][4 * kp + 1], kf[nt][4 * kp + 2], kf[nt][4 * kp + 3],
-                          kt + nt * (8 * ROWB) + offK[kp]);
-            } else {
-                ldsm4(kf[nt][0], kf[nt][1], kf[nt][2], kf[nt][3], kt + nt * (8 * ROWB) + offK[0]);
-            }
-        }
-        uint32_t vb[2][NTD][2];
-#pragma unroll
-        for (int b = 0; b < 2; ++b)
+            for (int kp = 0; kp < (D == 64 ? 2 : 1); ++kp)
+                ldsm4(kf[4 * kp], kf[4 * kp + 1], kf[4 * kp + 2], kf[4 * kp + 3], kt + nt * (8 * ROWB) + offK[kp]);
+        };
+        auto load_v = [&](int b, uint32_t (&vb)[NTD][2]) {
 #pragma unroll
             for (int jp = 0; jp < NTD / 2; ++jp)
-                ldsm4_trans(vb[b][2 * jp][0], vb[b][2 * jp][1], vb[b][2 * jp + 1][0], vb[b][2 * jp + 1][1],
-                            vt + b * (16 * ROWB) + offV[jp]);
-
-#pragma unroll
-        for (int mt = 0; mt < MT; ++mt) {
-            float s[4][4];
-#pragma unroll
-            for (int nt = 0; nt < 4; ++nt) {
-                s[nt][0] = s[nt][1] = s[nt][2] = s[nt][3] = 0.f;
-#pragma unroll
-                for (int ks = 0; ks < KS; ++ks) mma_bf16(s[nt], qa[mt][ks], kf[nt][2 * ks], kf[nt][2 * ks + 1]);
-            }
+                ldsm4_trans(vb[2 * jp][0], vb[2 * jp][1], vb[2 * jp + 1][0], vb[2 * jp + 1][1], vt + b * (16 * ROWB) + offV[jp]);
+        };
+        // weights of query tile mt from its scores
+        auto normalise = [&](int mt, float (&s)[4][4], uint32_t (&pa)[2][4]) {
             // element (nt, e): position p0 + 8 nt + 2t + (e & 1), query row g (e < 2) or g + 8
-            uint32_t pa[2][4];
             if constexpr (MODE == CKV_SOFTMAX) {
                 if (tail) {
                     const int e_lo = VAR ? min(end, lim[mt][0]) : end, e_hi = VAR ? min(end, lim[mt][1]) : end;
@@ -540,10 +523,53 @@ __global__ void __launch_bounds__(128, MmaCfg<D, MT, TMA>::MIN_BLOCKS)
                     pa[nt >> 1][(nt & 1) * 2 + 1] = pack_bf16(w[2], w[3]);
                 }
             }
+        };
+        if constexpr (MT == 1) {  // every fragment requested up front
+            uint32_t kf[4][2 * KS], vb[2][NTD][2], pa[2][4];
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt) load_k(nt, kf[nt]);
+#pragma unroll
+            for (int b = 0; b < 2; ++b) load_v(b, vb[b]);
+            float s[4][4];
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt) {
+                s[nt][0] = s[nt][1] = s[nt][2] = s[nt][3] = 0.f;
+#pragma unroll
+                for (int ks = 0; ks < KS; ++ks) mma_bf16(s[nt], qa[0][ks], kf[nt][2 * ks], kf[nt][2 * ks + 1]);
+            }
+            normalise(0, s, pa);
 #pragma unroll
             for (int b = 0; b < 2; ++b)
 #pragma unroll
-                for (int j = 0; j < NTD; ++j) mma_bf16(o[mt][j], pa[b], vb[b][j][0], vb[b][j][1]);
+                for (int j = 0; j < NTD; ++j) mma_bf16(o[0][j], pa[b], vb[b][j][0], vb[b][j][1]);
+        } else {  // a fragment serves all query tiles and is gone again: their accumulators need the registers
+            float s[MT][4][4];
+            uint32_t pa[MT][2][4];
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt) {
+                uint32_t kf[2 * KS];
+                load_k(nt, kf);
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt) {
+                    s[mt][nt][0] = s[mt][nt][1] = s[mt][nt][2] = s[mt][nt][3] = 0.f;
+                    if (mt < n_mt)
+#pragma unroll
+                        for (int ks = 0; ks < KS; ++ks) mma_bf16(s[mt][nt], qa[mt][ks], kf[2 * ks], kf[2 * ks + 1]);
+                }
+            }
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt)
+                if (mt < n_mt) normalise(mt, s[mt], pa[mt]);
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                uint32_t vb[NTD][2];
+                load_v(b, vb);
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt)
+                    if (mt < n_mt)
+#pragma unroll
+                        for (int j = 0; j < NTD; ++j) mma_bf16(o[mt][j], pa[mt][b], vb[j][0], vb[j][1]);
+            }
         }
         // every lane is done with this tile before the ring slot is refilled (TMA: its ordinary stores
         // and loads are ordered before the asynchronous-proxy writes of the refill)
@@ -718,13 +744,14 @@ bool mma_supported(int dtype, int head_dim, int d_user)
     return dtype == CKV_BF16 && (head_dim == 32 || head_dim == 64) && d_user <= 8;
 }
 
-// head_dim 64 rows keep a warp busy with one 16-query tile; 32-wide heads take up to four
-int mma_queries_per_warp(int D, int max_M) { return (D == 64 || max_M <= 16) ? 16 : (max_M <= 32 ? 32 : 64); }
+// Every gathered row serves all the queries a warp holds, so it holds as many as there are, up to what its registers
+// take: four 16-query tiles of 32-wide heads, three of 64-wide ones.
+int mma_queries_per_warp(int D, int max_M) { return max_M <= 16 ? 16 : max_M <= 32 ? 32 : D == 64 || max_M <= 48 ? 48 : 64; }
 
 // warps of the kernel that are resident on an SM
 int mma_warps_per_sm(int D, int max_M)
 {
-    if (D == 64) return 4 * MmaCfg<64, 1, false>::MIN_BLOCKS;
+    if (D == 64) return 8;
     return mma_queries_per_warp(D, max_M) == 16 ? 4 * MmaCfg<32, 1, false>::MIN_BLOCKS : 8;
 }
 
@@ -735,10 +762,17 @@ cudaError_t launch_attend_mma(int D, int max_M, int parts, const AttendArgs& a, 
     const CUtensorMap* maps = reinterpret_cast<const CUtensorMap*>(tensor_maps);
     const int qpw = mma_queries_per_warp(D, max_M);
     const int n_mb = (max_M + qpw - 1) / qpw;
-    if (D == 64) return launch_mma<64, 1>(a, n_mb, parts, tab, maps, err_flag, l);
+    if (D == 64) {
+        switch (qpw) {
+            case 16: return launch_mma<64, 1>(a, n_mb, parts, tab, maps, err_flag, l);
+            case 32: return launch_mma<64, 2>(a, n_mb, parts, tab, maps, err_flag, l);
+            default: return launch_mma<64, 3>(a, n_mb, parts, tab, maps, err_flag, l);
+        }
+    }
     switch (qpw) {
         case 16: return launch_mma<32, 1>(a, n_mb, parts, tab, maps, err_flag, l);
         case 32: return launch_mma<32, 2>(a, n_mb, parts, tab, maps, err_flag, l);
+        case 48: return launch_mma<32, 3>(a, n_mb, parts, tab, maps, err_flag, l);
         default: return launch_mma<32, 4>(a, n_mb, parts, tab, maps, err_flag, l);
     }
 }

@@ -1,33 +1,33 @@
 // tcgen05 gather-concat-attention kernel (bf16, head_dim 32) for many queries per user.
 //
-// Persistent: one CTA per SM walks a static round-robin share of the work units, where a unit
-// is (work item = history chunk of one user, group, block of up to 128 queries).  The history
-// chunk is processed in tiles of 128 positions, each split into two halves of 64 positions.
-// Roles (warp-specialised, 20 warps):
-//   warps 0-11  three normalisation groups of four warps: thread i of a group owns query row i = TMEM lane i
-//   warps 12-14 one issuing thread per group: the score MMAs and the weighted-sum MMAs of that group's halves;
-//               warp 12 owns the TMEM allocation
-//   warps 15-19 producers, one tile each in turn: gather pool rows into shared memory with
-//               16-byte cp.async, patch the user-specific leading elements (Eq. K), publish the
-//               tile; the owner of a unit's first tile also stages Q.  (A side that is not shared --
-//               sharing only keys or only values -- is copied from the user's full-width rows instead.)
+// Persistent: one CTA per SM holds three workers, and every worker walks its own static round-robin share of the work
+// units, where a unit is (work item = history chunk of one user, group, block of up to 128 queries).  The history chunk
+// is processed in tiles of 64 positions.  A worker is (warp-specialised, 6 warps of the CTA's 18)
+//   four normalisation warps: thread i owns query row i = TMEM lane i
+//   one issuing thread: the score MMAs and the weighted-sum MMAs
+//   one producer warp: gathers pool rows into the worker's ring of shared-memory stages with 16-byte cp.async, patches
+//     the user-specific leading elements (Eq. K), publishes the tile one tile later, and stages Q with a unit's first
+//     tile.  (A side that is not shared -- sharing only keys or only values -- is copied from the user's full-width
+//     rows instead.)
+// Workers share nothing but the SM: no merge between them, no hand-over, every barrier has one waiting role that meets
+// its phases in order.
 //
-// The halves of the CTA's tile stream go to the groups in turn (half h to group h mod 3).  A group has two score
-// buffers in TMEM; the weights of a half are written over the head of the scores they were computed from (32
-// columns of bf16 pairs over 64 columns of fp32):
-//   S_bi  = Q K_half^T                UMMA 128 x 64 x 32, A = Q smem, B = half K tile smem (K-major)
-//   P_bi  = exp2(S_bi c - m) | silu   group b: tcgen05.ld -> math -> bf16 -> tcgen05.st, in place
-//   O_b  += P_bi V_half               UMMA 128 x 32 x 64, A = P from TMEM, B = half V tile (MN-major)
-// One thread issues both kinds of MMA of its group, in the order weighted sum of step t, scores of step t + 2
-// (into the buffer the weighted sum has just read): the tensor core runs one thread's instructions in order, so
-// the buffer needs no completion hand-off in between, and the scores of step t + 1 are there while the group
-// normalises step t.  Why three groups: the normalisation of a half is a chain of dependent work for its warp
-// (wait for the scores, TMEM load, arithmetic, TMEM store, publish; at a unit's end the accumulator read-out and
-// the merge) during most of which the special-function unit of the warp's sub-partition is idle; measured on a
-// stripped-down pipeline, two groups keep that unit 70 % busy, three 85 %, and registers (65536 / 640 threads =
-// 96 each, enough for one 32-column chunk of scores at a time) and TMEM (3 x (2 x 64 + 32) = 480 columns) admit
-// no fourth.  The groups keep separate accumulators O_b with separate reference maxima and row sums and merge
-// them through shared memory when a unit ends; nothing drains between work units.
+// A worker has two score buffers in TMEM; the weights of a tile are written over the head of the scores they were
+// computed from (32 columns of bf16 pairs over 64 columns of fp32):
+//   S_i  = Q K_tile^T                 UMMA 128 x 64 x 32, A = Q smem, B = K tile smem (K-major)
+//   P_i  = exp2(S_i c - m) | silu     tcgen05.ld -> math -> bf16 -> tcgen05.st, in place
+//   O   += P_i V_tile                 UMMA 128 x 32 x 64, A = P from TMEM, B = V tile (MN-major)
+// The issuing thread issues the weighted sum of step t, then the scores of step t + 2 (into the buffer the weighted sum
+// has just read): the tensor core runs one thread's instructions in order, so the buffer needs no completion hand-off in
+// between, and the scores of step t + 1 are there while the group normalises step t.
+//
+// What bounds it: the special-function unit (one ex2 or tanh per score, 16 per clock per SM).  The normalisation of a
+// tile is a chain of dependent work for its warp (wait for the scores, TMEM load, arithmetic, TMEM store, publish; at a
+// unit's end the last weighted sum, the accumulator read-out, the store) during most of which that unit is idle on the
+// warp's sub-partition; three workers fill each other's gaps.  Registers (65536 / 20 warps = 96 a thread, enough for one
+// 32-column chunk of scores at a time) and TMEM (3 x (2 x 64 + 32) = 480 columns) admit no fourth.  With the three groups
+// on one unit instead (its tiles dealt out in turn, accumulators merged through shared memory at its end) a unit cost
+// FIGURES
 //
 // Softmax bookkeeping.  The reference maximum m of a row is the largest of the first 32 scores of the group's
 // first half of the unit and stays fixed: later scores may exceed it by up to 2^64 (fp32 accumulators and bf16
@@ -51,55 +51,40 @@ namespace ckv {
 namespace {
 
 constexpr int D = 32;
-constexpr int TK = 128;                  // positions per tile (one shared-memory stage)
-constexpr int TH = 64;                   // positions per half tile = one MMA / normalisation step of a group
-constexpr int NG = 3;                    // normalisation groups
-constexpr int NS = 10;                   // K/V stages
-constexpr int NQ = 3;                    // Q buffers
-constexpr int kGroupThreads = 128;       // one normalisation group
-constexpr int kIssueWarp0 = 4 * NG;      // warps 12..14 issue the MMAs of group 0..2; warp 12 owns the TMEM allocation
-constexpr int kProducerWarp0 = kIssueWarp0 + NG;
-constexpr int kProducerWarps = 5;        // each owns every fifth tile of the stream
-constexpr int kThreads = (kProducerWarp0 + kProducerWarps) * 32;  // 640
-constexpr int kTileK = TK * D * 2;       // 8 KB, also the Q tile
+constexpr int TH = 64;                   // positions per tile = one step: one score MMA, normalisation, weighted sum
+constexpr int NW = 3;                    // workers
+constexpr int NS = 7;                    // K/V stages of a worker (at most)
+constexpr int kGroupThreads = 128;       // normalisation threads of a worker
+constexpr int kIssueWarp0 = 4 * NW;      // warps 12..14 issue the MMAs of worker 0..2; warp 12 owns the TMEM allocation
+constexpr int kProducerWarp0 = kIssueWarp0 + NW;
+constexpr int kThreads = (kProducerWarp0 + NW) * 32;  // 576
+constexpr int kTileQ = 128 * D * 2;      // 8 KB
+constexpr int kTileK = TH * D * 2;       // 4 KB
 constexpr int kVGroup = 512;             // bytes of one 8-row group of a V tile
-constexpr int kTileV = (TK / 8) * kVGroup;  // 8 KB
+constexpr int kTileV = (TH / 8) * kVGroup;  // 4 KB
 constexpr uint32_t kTmemCols = 512;
-constexpr int NB = 2;                    // score / weight buffers per group
-constexpr uint32_t kColGroup = 64 * NB + D;  // group b: S_bi (and P_bi over its head) at kColGroup b + 64 i, O_b behind them
-static_assert(kColGroup * NG <= kTmemCols, "TMEM columns");
+constexpr uint32_t kColWorker = 2 * TH + D;  // worker b: S_i (and P_i over its head) at kColWorker b + 64 i, O behind them
+static_assert(kColWorker * NW <= kTmemCols, "TMEM columns");
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kHeadroom = 64.0f;       // log2 units a score may exceed the reference maximum
 constexpr float kSumLimit = 1180591620717411303424.0f;  // 2^70: a chunk's sum beyond it gives the excess away
 constexpr uint32_t kSpinLimit = 1u << 18;  // polls of a wait before the CTA gives up
 constexpr uint32_t kSuspendNs = 4000;      // how long one poll may stay suspended in hardware (longer hints wake later)
-static_assert(NS > kProducerWarps, "every producer warp holds one stage while it copies");
-static_assert(NS % kProducerWarps == 0, "a stage is always filled by the same producer warp, one use after the other");
 
-// dynamic shared memory map
-constexpr int kOffQ = 0;
-constexpr int kOffK = kOffQ + NQ * kTileK;
-constexpr int kOffV = kOffK + NS * kTileK;
-constexpr int kOffX = kOffV + NS * kTileV;          // what the other groups hand to the merging one when a unit ends: [NG - 1][34][128] floats
-constexpr int kOffBar = kOffX + (NG - 1) * 34 * 128 * 4;
-constexpr int kOffAbort = kOffBar + 448;
-constexpr int kSmemBytes = kOffAbort + 32;
+// barrier slots (8 bytes each) of a worker
+enum { BAR_FULL = 0, BAR_EMPTY = NS, BAR_QEMPTY = 2 * NS, BAR_SFULL = BAR_QEMPTY + 2, BAR_PREADY = BAR_SFULL + 2,
+       BAR_DRAIN = BAR_PREADY + 2, BAR_COUNT };
 
-// barrier slots (8 bytes each) behind kOffBar
-enum {
-    BAR_FULL = 0, BAR_EMPTY = NS, BAR_QEMPTY = 2 * NS, BAR_QFULL = 2 * NS + NQ,
-    BAR_SFULL = 2 * NS + 2 * NQ,          // [NB b + i]
-    BAR_PREADY = BAR_SFULL + NG * NB,     // [NB b + i]
-    BAR_PFREE = BAR_PREADY + NG * NB,     // [NB b + i]
-    BAR_OFULL = BAR_PFREE + NG * NB,      // [b]
-    BAR_XFULL = BAR_OFULL + NG,           // [slot]
-    BAR_XEMPTY = BAR_XFULL + NG - 1,      // [slot]
-    BAR_DRAIN = BAR_XEMPTY + NG - 1,      // [b]
-    BAR_COUNT = BAR_DRAIN + NG
+// dynamic shared memory map, DUB = bytes of a user part: per worker two Q blocks, the K stages, the V stages, and a ring
+// of what the producer has requested from the compressed cache, tile by tile
+template <int DUB>
+struct Map {
+    static constexpr int STAGES = DUB >= 8 ? NS - 1 : NS;
+    static constexpr int META = 256 + 2 * TH * DUB, META_SLOTS = 4;  // K indices, V indices, K user parts, V user parts
+    static constexpr int Q = 0, K = 2 * kTileQ, V = K + STAGES * kTileK, M = V + STAGES * kTileV, WORKER = M + META_SLOTS * META;
+    static constexpr int BAR = NW * WORKER, ABORT = BAR + NW * BAR_COUNT * 8, BYTES = ABORT + 32;
+    static_assert(BYTES <= 231424, "shared memory of one CTA");
 };
-static_assert(BAR_COUNT * 8 <= 448, "barrier area");
-static_assert(kSmemBytes <= 232448, "shared memory of one CTA");
-
 
 // error codes OR-ed into the context's device error word: which role gave up (bits 0..3); bits 8..11 carry the
 // site code of the first wait that ran out (see SITE_*)
@@ -116,10 +101,7 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar)
 // Bounded wait on a phase parity.  Returns false on time-out or when the CTA is aborting.
 // A wait that runs out (rather than being ended by the abort flag) leaves its site code in the word behind the flag;
 // the first one stays, and the kernel reports it in bits 8.. of the error word.
-enum {
-    SITE_SFULL = 1, SITE_OFULL, SITE_XEMPTY, SITE_XFULL, SITE_PFREE, SITE_TILE, SITE_Q, SITE_PREADY, SITE_TAIL_TILE,
-    SITE_STAGE, SITE_QBUF, SITE_DRAIN, SITE_QTURN
-};
+enum { SITE_SFULL = 1, SITE_OFULL, SITE_PREV, SITE_TILE, SITE_PREADY, SITE_STAGE, SITE_QBUF, SITE_DRAIN };
 __device__ __forceinline__ void note_site(const volatile int* abort_flag, int site)
 {
     atomicCAS(const_cast<int*>(abort_flag) + 1, 0, site);
@@ -141,8 +123,8 @@ __device__ __noinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const vola
     note_site(abort_flag, site);
     return false;
 }
-// The bounded wait with its first poll inline: most waits of the issuing threads find their phase complete.
-__device__ __forceinline__ bool mbar_wait_fast(uint32_t bar, uint32_t parity, const volatile int* abort_flag, int site)
+// One poll, without waiting.
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity)
 {
     uint32_t ok;
     asm volatile(
@@ -152,7 +134,12 @@ __device__ __forceinline__ bool mbar_wait_fast(uint32_t bar, uint32_t parity, co
         : "=r"(ok)
         : "r"(bar), "r"(parity)
         : "memory");
-    return ok != 0 || mbar_wait(bar, parity, abort_flag, site);
+    return ok != 0;
+}
+// The bounded wait with its first poll inline: most waits of the issuing threads find their phase complete.
+__device__ __forceinline__ bool mbar_wait_fast(uint32_t bar, uint32_t parity, const volatile int* abort_flag, int site)
+{
+    return mbar_test(bar, parity) || mbar_wait(bar, parity, abort_flag, site);
 }
 // 16-byte copy global -> shared; src_bytes = 0 fills the destination with zeros instead.
 // Pool rows go through L1 (with skewed indices the hot rows then stop hammering a few L2 lines
@@ -317,14 +304,13 @@ __device__ __forceinline__ void mul2_scalar(float& d0, float& d1, float a0, floa
 __device__ __forceinline__ uint32_t k_off(int r, int c) { return (uint32_t)((r >> 3) * 512 + c * 128 + (r & 7) * 16); }
 __device__ __forceinline__ uint32_t v_off(int r, int c) { return (uint32_t)((r >> 3) * kVGroup + c * 128 + (r & 7) * 16); }
 
-// Inside a tile the producers place history position 32 c + 4 q + i (q < 8, i < 4) in row
-// 32 c + 8 i + q: a lane then reads the indices of four consecutive positions with one load and
-// its four 16-byte copies of an instruction still fall into different shared-memory banks.
+// Inside a tile the producer places position 32 c + 4 q + i (q < 8, i < 4) in row
+// 32 c + 8 i + q: a lane's four 16-byte copies of a 32-position block then fall into different shared-memory banks.
 // Attention does not depend on the order of positions; only the tail mask has to know which
 // position a score column belongs to.
 __device__ __forceinline__ int pos_of_col(int c, int e) { return 32 * c + 4 * (e & 7) + (e >> 3); }
 
-// ---- normalisation of one 128 x 64 score half tile by its group (thread = query row = TMEM lane) ----
+// ---- normalisation of one 128 x 64 score tile by its group (thread = query row = TMEM lane) ----
 
 // Multiplies this thread's row of O (32 columns) by f.
 __device__ __noinline__ void rescale_row(uint32_t tO, float f)
@@ -337,8 +323,7 @@ __device__ __noinline__ void rescale_row(uint32_t tO, float f)
     tmem_st32(tO, o);
 }
 
-// Multiplies the 32 weights (16 columns of bf16 pairs) this thread wrote for the first chunk of the current half
-// tile by f, a power of two: exact unless a weight drops below the smallest bf16.
+// Multiplies the 32 weights (16 columns of bf16 pairs) this thread wrote for the first chunk of the current tile by f, a power of two: exact unless a weight drops below the smallest bf16.
 __device__ __noinline__ void rescale_weights(uint32_t tP, float f)
 {
     for (int c = 0; c < 16; ++c) {
@@ -382,7 +367,7 @@ __device__ __noinline__ float chunk_max(const uint32_t* cur, float sc, float nm,
     return mx;
 }
 
-// Softmax weights of one 32-column chunk (c = 0, 1) of a 128 x 64 score half tile: p = exp2(s c - m) as bf16
+// Softmax weights of one 32-column chunk (c = 0, 1) of a 128 x 64 score tile: p = exp2(s c - m) as bf16
 // pairs written over the head of the scores (columns 0..31 of the buffer; chunk 1 of the scores, columns 32..63,
 // is still to be read when chunk 0's weights land on columns 0..15, and chunk 1's weights
 // land on columns 16..31, whose scores have been consumed).  The chunk's weights are added to the row sum l.  With `first` (chunk 0 of the group's first half
@@ -481,32 +466,31 @@ __device__ __forceinline__ void silu_chunk(const uint32_t (&cur)[32], int c, uin
     tmem_st16(tS + 16 * c, p);
 }
 
-// The user-specific leading elements of one row (DUB = 2 d_user bytes), as the producers carry
-// them from the compressed cache to a shared-memory tile.
+// The user-specific leading elements of one row (DUB = 2 d_user bytes), on their way from the request ring to a tile.
 template <int DUB> struct UserPart;
 template <> struct UserPart<0> {};
 template <> struct UserPart<2> {
     uint16_t v;
-    __device__ __forceinline__ void load(const char* p) { v = __ldg(reinterpret_cast<const uint16_t*>(p)); }
+    __device__ __forceinline__ void take(const unsigned char* p) { v = *reinterpret_cast<const uint16_t*>(p); }
     __device__ __forceinline__ void store(unsigned char* p) const { *reinterpret_cast<uint16_t*>(p) = v; }
 };
 template <> struct UserPart<4> {
     uint32_t v;
-    __device__ __forceinline__ void load(const char* p) { v = __ldg(reinterpret_cast<const uint32_t*>(p)); }
+    __device__ __forceinline__ void take(const unsigned char* p) { v = *reinterpret_cast<const uint32_t*>(p); }
     __device__ __forceinline__ void store(unsigned char* p) const { *reinterpret_cast<uint32_t*>(p) = v; }
 };
 template <> struct UserPart<8> {
     uint2 v;
-    __device__ __forceinline__ void load(const char* p) { v = __ldg(reinterpret_cast<const uint2*>(p)); }
+    __device__ __forceinline__ void take(const unsigned char* p) { v = *reinterpret_cast<const uint2*>(p); }
     __device__ __forceinline__ void store(unsigned char* p) const { *reinterpret_cast<uint2*>(p) = v; }
 };
 template <> struct UserPart<16> {
     uint4 v;
-    __device__ __forceinline__ void load(const char* p) { v = __ldg(reinterpret_cast<const uint4*>(p)); }
+    __device__ __forceinline__ void take(const unsigned char* p) { v = *reinterpret_cast<const uint4*>(p); }
     __device__ __forceinline__ void store(unsigned char* p) const { *reinterpret_cast<uint4*>(p) = v; }
 };
 
-// One work unit of the CTA's share, decoded from its Work record.
+// One work unit of a worker's share, decoded from its Work record.
 struct Unit {
     Work wk;
     int grp;
@@ -514,13 +498,6 @@ struct Unit {
     int n_tiles;     // > 0: tiles to process; 0: empty history (zero output rows); < 0: nothing at all
     int last_valid;  // real positions in the last tile
 };
-
-// Which group takes a unit's first half (half p goes to group (p + rotation) mod NG).  A function of the unit
-// alone -- not of its place in a CTA's stream -- so that results do not depend on what else a call processes.
-__device__ __forceinline__ int unit_rotation(const Unit& u)
-{
-    return (int)((uint32_t)(u.grp + (u.row0 >> 7) + (u.wk.begin >> 6)) % (uint32_t)NG);
-}
 
 __device__ __forceinline__ Work load_work(const Work* p)
 {
@@ -536,25 +513,21 @@ __device__ __forceinline__ Work load_work(const Work* p)
     return u.w;
 }
 
-// The CTA's tile stream: units blockIdx.x, blockIdx.x + gridDim.x, ... tile by tile.  Every role
-// walks an identical copy, so stage and buffer indices need no communication.  The record of
-// the following unit is always in flight while the current one is processed.  Unit w stands for
-// (item, group, query block) = (w / n_mb / G, w / n_mb % G, w % n_mb); the coordinates are
-// stepped with carries instead of divided out each time.
+// A worker's units: worker b of block x takes units x + gridDim.x b, then every (NW gridDim.x)-th.  Every role walks an
+// identical copy, so stage and buffer indices need no communication.  The record of the following unit is always in
+// flight while the current one is processed.  Unit w stands for (item, group, query block) = (w / n_mb / G,
+// w / n_mb % G, w % n_mb); the coordinates are stepped with carries instead of divided out each time.
 // KEEP_EMPTY: also stop at units with an empty history (the role that writes their zero rows).
 template <bool KEEP_EMPTY, bool VIS>
-struct Stream {
+struct Units {
     const Work* works;
     const int32_t* vmax;         // VIS: per (request, query block) the largest visible length of its rows
     uint32_t n_mb, n_groups;
-    uint32_t w, n_work;          // the host keeps n_work + gridDim.x below 2^32
+    uint32_t w, n_work, stride;  // the host keeps n_work + stride below 2^32
     uint32_t item, grp, mb;      // coordinates of unit w
-    uint32_t d_item, d_grp, d_mb;  // gridDim.x in the same mixed radix
+    uint32_t d_item, d_grp, d_mb;  // the stride in the same mixed radix
     Unit u;
-    Work nxt;    // record of unit w + gridDim.x (valid if that is < n_work)
-    int j;       // tile inside the unit
-    int g;       // tiles before this one in the stream
-    int useq;    // units with tiles before this one
+    Work nxt;    // record of unit w + stride (valid if that is < n_work)
     bool valid;
     __device__ __forceinline__ void step(uint32_t& it, uint32_t& gr, uint32_t& m) const
     {
@@ -577,7 +550,7 @@ struct Stream {
             u.wk = nxt;
             u.grp = (int)grp;
             u.row0 = (int)mb * 128;
-            const uint32_t wn = w + gridDim.x;
+            const uint32_t wn = w + stride;
             uint32_t ni = item, ng = grp, nm = mb;
             step(ni, ng, nm);
             if (wn < n_work) nxt = load_work(works + ni);
@@ -586,11 +559,10 @@ struct Stream {
             if constexpr (VIS) {
                 if (u.row0 < u.wk.M) len = min(len, max(__ldg(vmax + u.wk.pad[0] + mb) - u.wk.begin, 0));
             }
-            u.n_tiles = u.row0 < u.wk.M ? (len + TK - 1) / TK : -1;
-            u.last_valid = len - (u.n_tiles - 1) * TK;
+            u.n_tiles = u.row0 < u.wk.M ? (len + TH - 1) / TH : -1;
+            u.last_valid = len - (u.n_tiles - 1) * TH;
             if (u.n_tiles > 0 || (KEEP_EMPTY && u.n_tiles == 0)) {
                 valid = true;
-                j = 0;
                 return;
             }
             w = wn;
@@ -599,56 +571,29 @@ struct Stream {
             mb = nm;
         }
     }
-    __device__ __forceinline__ void to_next_unit()
+    __device__ __forceinline__ void next()
     {
-        w += gridDim.x;
+        w += stride;
         step(item, grp, mb);
         take();
     }
-    __device__ __forceinline__ void init(const AttendArgs& a, int n_mb_, int64_t n_work_)
+    __device__ __forceinline__ void init(const AttendArgs& a, int n_mb_, int64_t n_work_, int worker)
     {
         works = a.works;
         if constexpr (VIS) vmax = a.vmax;
         n_mb = (uint32_t)n_mb_;
         n_groups = (uint32_t)a.cv.n_groups;
         n_work = (uint32_t)n_work_;
-        w = blockIdx.x;
+        stride = NW * gridDim.x;
+        w = blockIdx.x + gridDim.x * (uint32_t)worker;
         mb = w % n_mb;
         grp = (w / n_mb) % n_groups;
         item = (w / n_mb) / n_groups;
-        d_mb = gridDim.x % n_mb;
-        d_grp = (gridDim.x / n_mb) % n_groups;
-        d_item = (gridDim.x / n_mb) / n_groups;
-        g = 0;
-        useq = 0;
+        d_mb = stride % n_mb;
+        d_grp = (stride / n_mb) % n_groups;
+        d_item = (stride / n_mb) / n_groups;
         if (w < n_work) nxt = load_work(works + item);
         take();
-    }
-    __device__ __forceinline__ void next_unit()
-    {
-        g += u.n_tiles > 0 ? u.n_tiles : 0;
-        useq += u.n_tiles > 0;
-        to_next_unit();
-    }
-    __device__ __forceinline__ void advance()
-    {
-        ++g;
-        if (++j == u.n_tiles) {
-            ++useq;
-            to_next_unit();
-        }
-    }
-    // n tiles on
-    __device__ __forceinline__ void advance_by(int n)
-    {
-        g += n;
-        j += n;
-        while (valid && j >= u.n_tiles) {
-            const int over = j - u.n_tiles;
-            ++useq;
-            to_next_unit();  // sets j = 0
-            j = over;
-        }
     }
 };
 
@@ -656,41 +601,24 @@ struct Stream {
 template <int MODE, int DUB, bool VIS>
 __global__ void __launch_bounds__(kThreads, 1) attend_umma_kernel(const AttendArgs a, int n_mb, int64_t n_work, int* err_flag)
 {
+    using L = Map<DUB>;
+    constexpr int NS = L::STAGES;
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ uint32_t tmem_base_slot;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t sbase = smem_u32(smem);
-    const uint32_t bar0 = sbase + kOffBar;
-    auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kOffAbort);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::ABORT);
     const int G = a.cv.n_groups;
 
     if (tid == 0) {
-        for (int s = 0; s < NS; ++s) {
-            mbar_init(bar(BAR_FULL + s), 1);   // lane 0 of the producer warp that owns the tile
-            mbar_init(bar(BAR_EMPTY + s), 2);  // one arrival per half
-        }
-        for (int q = 0; q < NQ; ++q) {
-            mbar_init(bar(BAR_QEMPTY + q), NG);  // every issuer
-            mbar_init(bar(BAR_QFULL + q), 1);    // lane 0 of the producer warp that staged the unit's Q block
-        }
-        for (int bi = 0; bi < NG * NB; ++bi) {
-            mbar_init(bar(BAR_SFULL + bi), 1);
-            mbar_init(bar(BAR_PREADY + bi), kGroupThreads);
-            mbar_init(bar(BAR_PFREE + bi), 1);
-        }
-        for (int b = 0; b < NG; ++b) {
-            mbar_init(bar(BAR_OFULL + b), 1);
-            mbar_init(bar(BAR_DRAIN + b), 1);
-        }
-        for (int b = 0; b < NG - 1; ++b) {
-            mbar_init(bar(BAR_XFULL + b), kGroupThreads);
-            mbar_init(bar(BAR_XEMPTY + b), kGroupThreads);
+        for (int b = 0; b < NW; ++b) {
+            const uint32_t bar0 = sbase + L::BAR + b * (BAR_COUNT * 8);
+            for (int i = 0; i < BAR_COUNT; ++i)  // (full: lane 0 of the producer; empty: the commit behind a weighted sum)
+                mbar_init(bar0 + 8 * i, i == BAR_PREADY || i == BAR_PREADY + 1 ? kGroupThreads : 1);
         }
         abort_flag[0] = 0;  // raised by the first role that gives up
         abort_flag[1] = 0;  // site of the first wait that ran out
-        abort_flag[4] = 0;  // units whose Q block has a producer at work on it (see the producers)
         abort_flag[2] = 0;  // never raised: the flag of the teardown wait, which must not be cut short
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -704,29 +632,30 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma_kernel(const AttendAr
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_base_slot;
+    const int b = warp < kIssueWarp0 ? warp >> 2 : warp < kProducerWarp0 ? warp - kIssueWarp0 : warp - kProducerWarp0;  // worker
+    const uint32_t bar0 = sbase + L::BAR + b * (BAR_COUNT * 8), wbase = sbase + b * L::WORKER;
+    auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
+    const uint32_t tS0 = tmem + kColWorker * b, tO0 = tS0 + 2u * TH;  // lane 0 of the score buffers and the accumulator
 
     if (warp < kIssueWarp0) {
-        // --------------------------------------------------------------- normalisation groups
-        const int b = warp >> 2;                    // group
+        // --------------------------------------------------------------- normalisation
         const int row = tid & (kGroupThreads - 1);  // query row inside the block = TMEM lane
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-        const uint32_t tS0 = tmem + lane_base + kColGroup * b, tO = tS0 + 64u * NB;
+        const uint32_t tSl = tS0 + lane_base, tO = tO0 + lane_base;
         const float sc = a.scale * (MODE == CKV_SOFTMAX ? kLog2e : 0.5f);
-        float* xch = reinterpret_cast<float*>(smem + kOffX);
-        int cnt = 0;    // halves this group has normalised
-        int ocnt = 0;   // units in which this group had halves
-        int xcnt = 0;   // units exchanged between the groups
+        int cnt = 0;    // tiles normalised
+        int stage = 0, sphase = 0;  // stage of the tile last normalised and the parity of its release: cnt - 1 in units of NS
         bool ok = true;
-        uint32_t sa[32];  // one 32-column chunk of a half's scores
-        Stream<true, VIS> sn;
-        sn.init(a, n_mb, n_work);
-        for (; sn.valid && ok; sn.next_unit()) {
-            const Unit& u = sn.u;
+        uint32_t sa[32];  // one 32-column chunk of a tile's scores
+        Units<true, VIS> un;
+        un.init(a, n_mb, n_work, b);
+        for (; un.valid && ok; un.next()) {
+            const Unit& u = un.u;
             const int r = u.row0 + row;
             if (r < u.wk.M) (void)CKV_CLAMP((int64_t)(u.wk.q0 + r), a.q_rows, err_flag);
             const int64_t out_base = ((int64_t)(u.wk.q0 + r) * G + u.grp) * D;
             if (u.n_tiles == 0) {  // empty history, or a chunk behind every row's visible length: zero rows
-                if (b == 0 && r < u.wk.M) {
+                if (r < u.wk.M) {
                     if (u.wk.part_row >= 0) {  // (only with visible lengths) an empty partial result
                         float* pr = a.partials + (CKV_CLAMP((int64_t)(u.wk.part_row + r), a.part_rows, err_flag) * G + u.grp) * (D + 2);
                         pr[0] = -CUDART_INF_F;
@@ -745,40 +674,35 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma_kernel(const AttendAr
             int lim = u.wk.L;
             if constexpr (VIS) lim = r < u.wk.M ? min(max(__ldg(a.vis + u.wk.q0 + r), 0), u.wk.L) : 0;
             float m_ref = -CUDART_INF_F, l = 0.f;
-            int mine = 0;  // halves of this unit normalised by this group
-            // The unit's non-empty halves are p = 2 j + half < n_half (only the second half of the last tile can be
-            // empty); half p goes to group (p + unit_rotation) mod NG.
-            const int n_half = 2 * u.n_tiles - (u.last_valid <= TH ? 1 : 0);
-            for (int p = (b + NG - unit_rotation(u)) % NG; p < n_half && ok; p += NG) {
-                const int j = p >> 1, half = p & 1;
-                const int valid = (j == u.n_tiles - 1 ? u.last_valid : TK) - TH * half;  // real positions of the half
-                const int i = cnt % NB;                                                   // buffer of this step
-                const uint32_t tS = tS0 + 64u * i;
-                ok = mbar_wait_fast(bar(BAR_SFULL + NB * b + i), (cnt / NB) & 1, abort_flag, SITE_SFULL);
+            for (int j = 0; j < u.n_tiles && ok; ++j) {
+                const int valid = j == u.n_tiles - 1 ? u.last_valid : TH;  // real positions of the tile
+                const int i = cnt & 1;                                     // buffer of this step
+                const uint32_t tS = tSl + (uint32_t)TH * i;
+                ok = mbar_wait_fast(bar(BAR_SFULL + i), (cnt >> 1) & 1, abort_flag, SITE_SFULL);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tc_fence_after();
-                // (softmax, only taken when a row leaves the headroom) the previous step's MMAs must have finished
-                // before O_b is rescaled
+                // (softmax, only taken when a row leaves the headroom) the previous step's weighted sum must have
+                // finished before O is rescaled: it is what releases that step's stage
                 auto wait_prev = [&]() {
-                    bool w = mbar_wait(bar(BAR_PFREE + NB * b + (cnt - 1) % NB), ((cnt - 1) / NB) & 1, abort_flag, SITE_PFREE);
+                    bool w = mbar_wait(bar(BAR_EMPTY + stage), sphase, abort_flag, SITE_PREV);
                     return __all_sync(0xffffffffu, w);
                 };
-                // real (and, with visible lengths, attended) positions of this thread's row in the half
+                // real (and, with visible lengths, attended) positions of this thread's row in the tile
                 int valid_r = valid;
                 bool tail = valid < TH;
                 if constexpr (VIS) {
-                    valid_r = min(valid, lim - (u.wk.begin + j * TK + TH * half));
+                    valid_r = min(valid, lim - (u.wk.begin + j * TH));
                     tail = __any_sync(0xffffffffu, valid_r < TH);
                 }
-                // One 32-column chunk at a time: the other groups' warps on this sub-partition cover the TMEM load.
+                // One 32-column chunk at a time: the other workers' warps on this sub-partition cover the TMEM load.
                 if (tail) {  // end of a history or of some row's visible positions: masked columns
 #pragma unroll 1
                     for (int c = 0; c < 2 && ok; ++c) {
                         tmem_ld32(tS + 32 * c, sa);
                         tmem_wait_ld32(sa);
                         if constexpr (MODE == CKV_SOFTMAX)
-                            ok = softmax_chunk<true, VIS>(sa, c, tS, tO, sc, valid_r, mine == 0, mine > 0, m_ref, l, wait_prev);
+                            ok = softmax_chunk<true, VIS>(sa, c, tS, tO, sc, valid_r, j == 0, j > 0, m_ref, l, wait_prev);
                         else
                             silu_chunk<true>(sa, c, tS, sc, valid_r);
                     }
@@ -788,7 +712,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma_kernel(const AttendAr
                         tmem_ld32(tS + 32 * c, sa);
                         tmem_wait_ld32(sa);
                         if constexpr (MODE == CKV_SOFTMAX)
-                            ok = softmax_chunk<false, VIS>(sa, c, tS, tO, sc, valid, mine == 0, mine > 0, m_ref, l, wait_prev);
+                            ok = softmax_chunk<false, VIS>(sa, c, tS, tO, sc, valid, j == 0, j > 0, m_ref, l, wait_prev);
                         else
                             silu_chunk<false>(sa, c, tS, sc, valid);
                     }
@@ -796,99 +720,52 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma_kernel(const AttendAr
                 if (!ok) break;
                 tc_wait_st();
                 tc_fence_before();
-                mbar_arrive(bar(BAR_PREADY + NB * b + i));
+                mbar_arrive(bar(BAR_PREADY + i));
+                if (cnt > 0 && ++stage == NS) {
+                    stage = 0;
+                    sphase ^= 1;
+                }
                 ++cnt;
-                ++mine;
             }
             if (!ok) break;
 
-            // ---- the unit's epilogue: fetch O_b, merge the groups, store
-            float o[32];
-            if (mine > 0) {
-                ok = mbar_wait(bar(BAR_OFULL + b), ocnt & 1, abort_flag, SITE_OFULL);
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok) break;
-                ++ocnt;
-                tc_fence_after();
-                uint32_t raw[32];
-                tmem_ld32(tO, raw);
-                tmem_wait_ld32(raw);
+            // ---- the unit's epilogue: O is complete with the last tile's weighted sum (its stage's release)
+            ok = mbar_wait(bar(BAR_EMPTY + stage), sphase, abort_flag, SITE_OFULL);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            tc_fence_after();
+            tmem_ld32(tO, sa);
+            tmem_wait_ld32(sa);
+            tc_fence_before();  // (the next unit overwrites O behind this group's next hand-over)
+            if (r < u.wk.M) {
+                auto o = [&](int e) { return __uint_as_float(sa[e]); };
+                if (u.wk.part_row < 0) {
+                    float inv;
+                    if constexpr (MODE == CKV_SOFTMAX) inv = l > 0.f ? 1.0f / l : 0.f;
+                    else inv = 1.0f / (float)u.wk.L;
+                    if (a.out_dtype == CKV_BF16) {
+                        uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(a.out) + out_base);
 #pragma unroll
-                for (int e = 0; e < 32; ++e) o[e] = __uint_as_float(raw[e]);
-                tc_fence_before();
-            } else {
-#pragma unroll
-                for (int e = 0; e < 32; ++e) o[e] = 0.f;
-            }
-            // Group 0 merges and stores, always: a barrier of the hand-over is then waited on by the same threads use
-            // after use.  (With the merging passed round -- to the group that has the unit's last half -- a group
-            // could come to wait for a use while the one before was still open, and a parity wait cannot tell.)
-            if (b != 0) {
-                const int slot = b - 1;
-                float* x = xch + slot * 34 * 128;
-                if (xcnt > 0) ok = mbar_wait(bar(BAR_XEMPTY + slot), (xcnt - 1) & 1, abort_flag, SITE_XEMPTY);
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok) break;
-                x[row] = m_ref;
-                x[128 + row] = l;
-#pragma unroll
-                for (int e = 0; e < 32; ++e) x[(2 + e) * 128 + row] = o[e];
-                mbar_arrive(bar(BAR_XFULL + slot));
-                ++xcnt;
-            } else {
-#pragma unroll 1
-                for (int slot = 0; slot < NG - 1 && ok; ++slot) {
-                    const float* x = xch + slot * 34 * 128;
-                    ok = mbar_wait(bar(BAR_XFULL + slot), xcnt & 1, abort_flag, SITE_XFULL);
-                    ok = __all_sync(0xffffffffu, ok);
-                    if (!ok) break;
-                    const float m1 = x[row], l1 = x[128 + row];
-                    if constexpr (MODE == CKV_SOFTMAX) {
-                        const float mt = fmaxf(m_ref, m1);
-                        const float ms = mt == -CUDART_INF_F ? 0.f : mt;
-                        const float c0 = ex2(m_ref - ms), c1 = ex2(m1 - ms);
-                        l = l * c0 + l1 * c1;
-#pragma unroll
-                        for (int e = 0; e < 32; ++e) o[e] = o[e] * c0 + x[(2 + e) * 128 + row] * c1;
-                        m_ref = mt;
-                    } else {
-#pragma unroll
-                        for (int e = 0; e < 32; ++e) o[e] += x[(2 + e) * 128 + row];
-                    }
-                    mbar_arrive(bar(BAR_XEMPTY + slot));
-                }
-                if (!ok) break;
-                ++xcnt;
-                if (r < u.wk.M) {
-                    if (u.wk.part_row < 0) {
-                        float inv;
-                        if constexpr (MODE == CKV_SOFTMAX) inv = l > 0.f ? 1.0f / l : 0.f;
-                        else inv = 1.0f / (float)u.wk.L;
-                        if (a.out_dtype == CKV_BF16) {
-                            uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(a.out) + out_base);
-#pragma unroll
-                            for (int q4 = 0; q4 < 4; ++q4) {
-                                uint4 v;
-                                v.x = pack_bf16(o[8 * q4 + 0] * inv, o[8 * q4 + 1] * inv);
-                                v.y = pack_bf16(o[8 * q4 + 2] * inv, o[8 * q4 + 3] * inv);
-                                v.z = pack_bf16(o[8 * q4 + 4] * inv, o[8 * q4 + 5] * inv);
-                                v.w = pack_bf16(o[8 * q4 + 6] * inv, o[8 * q4 + 7] * inv);
-                                dst[q4] = v;
-                            }
-                        } else {
-                            float4* dst = reinterpret_cast<float4*>(reinterpret_cast<float*>(a.out) + out_base);
-#pragma unroll
-                            for (int q4 = 0; q4 < 8; ++q4)
-                                dst[q4] = make_float4(o[4 * q4] * inv, o[4 * q4 + 1] * inv, o[4 * q4 + 2] * inv,
-                                                      o[4 * q4 + 3] * inv);
+                        for (int q4 = 0; q4 < 4; ++q4) {
+                            uint4 v;
+                            v.x = pack_bf16(o(8 * q4 + 0) * inv, o(8 * q4 + 1) * inv);
+                            v.y = pack_bf16(o(8 * q4 + 2) * inv, o(8 * q4 + 3) * inv);
+                            v.z = pack_bf16(o(8 * q4 + 4) * inv, o(8 * q4 + 5) * inv);
+                            v.w = pack_bf16(o(8 * q4 + 6) * inv, o(8 * q4 + 7) * inv);
+                            dst[q4] = v;
                         }
                     } else {
-                        float* pr = a.partials + (CKV_CLAMP((int64_t)(u.wk.part_row + r), a.part_rows, err_flag) * G + u.grp) * (D + 2);
-                        pr[0] = m_ref;
-                        pr[1] = l;
+                        float4* dst = reinterpret_cast<float4*>(reinterpret_cast<float*>(a.out) + out_base);
 #pragma unroll
-                        for (int e = 0; e < 32; ++e) pr[2 + e] = o[e];
+                        for (int q4 = 0; q4 < 8; ++q4)
+                            dst[q4] = make_float4(o(4 * q4) * inv, o(4 * q4 + 1) * inv, o(4 * q4 + 2) * inv, o(4 * q4 + 3) * inv);
                     }
+                } else {
+                    float* pr = a.partials + (CKV_CLAMP((int64_t)(u.wk.part_row + r), a.part_rows, err_flag) * G + u.grp) * (D + 2);
+                    pr[0] = m_ref;
+                    pr[1] = l;
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) pr[2 + e] = o(e);
                 }
             }
         }
@@ -898,139 +775,81 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma_kernel(const AttendAr
             if (lane == 0) atomicOr(err_flag, ERR_NORMALISE);
         }
     } else if (warp < kProducerWarp0) {
-        // --------------------------------------------------------------------- MMA issue for one group
-        // One thread per group, and its loop is the pipeline's pacemaker: it is a chain of dependent instructions
-        // of a single thread, so everything that can be kept out of it is (descriptors are a constant plus an
-        // offset, the two pending weighted sums live in named registers, waits poll once inline before they call).
+        // --------------------------------------------------------------------- MMA issue
+        // One thread, and its loop paces the worker: it is a chain of dependent instructions, so everything that can be
+        // kept out of it is (descriptors are a constant plus an offset, waits poll once inline before they call).
         if (lane == 0) {
-            const int b = warp - kIssueWarp0;
             constexpr uint32_t idesc_s = make_idesc(128, TH, false), idesc_pv = make_idesc(128, D, true);
-            const uint32_t tS0 = tmem + kColGroup * b, tO = tS0 + 64u * NB;
-            const uint64_t dq0 = smem_desc(sbase + kOffQ, 128, 512), dk0 = smem_desc(sbase + kOffK, 128, 512),
-                           dv0 = smem_desc(sbase + kOffV, kVGroup, 128);
+            const uint64_t dq0 = smem_desc(wbase + L::Q, 128, 512), dk0 = smem_desc(wbase + L::K, 128, 512),
+                           dv0 = smem_desc(wbase + L::V, kVGroup, 128);
             auto at = [](uint64_t d, uint32_t byte_off) { return d + (uint64_t)(byte_off >> 4); };  // no carry out of the address field
-            static_assert(NB == 2, "two pending weighted sums");
-            Stream<false, VIS> ss;
-            ss.init(a, n_mb, n_work);
-            int cnt = 0;   // steps whose scores have been issued
-            int done = 0;  // steps whose weighted sum has been issued
-            // what the weighted sums of the (at most two) steps in flight need, oldest first: byte offset of the half V
-            // tile, stage to release, flags (bit 0: O_b already holds the unit's earlier halves; bit 1: the group's
-            // last half of the unit)
-            uint32_t pv_off0 = 0, pv_off1 = 0;
-            int pv_s0 = 0, pv_s1 = 0, pv_f0 = 0, pv_f1 = 0;
-            int gs = 0, gp = 0;  // stage and phase parity of the unit's first tile: g % NS, (g / NS) & 1
+            Units<false, VIS> un;
+            un.init(a, n_mb, n_work, b);
+            int cnt = 0, done = 0;    // steps whose scores / weighted sum have been issued; at most two apart
+            int s = 0, par = 0;       // stage of step cnt and the phase parity of its tile
+            int pv_s = 0;             // stage of step `done`
+            uint32_t acc0 = 0, acc1 = 0;  // of the steps in flight, oldest first: O already holds earlier tiles of the unit
+            int useq = 0;             // units begun
             bool ok = true;
-            // O_b += P_bi V_half for step `done`, whose group has written P_bi
-            auto do_pv = [&]() {
+            // O += P_i V for step `done`, once the group has written P_i
+            auto issue_pv = [&]() {
                 const int i = done & 1;
+                if (!mbar_wait_fast(bar(BAR_PREADY + i), (done >> 1) & 1, abort_flag, SITE_PREADY)) return false;
                 tc_fence_after();
-                const uint64_t dv = at(dv0, pv_off0);
+                const uint64_t dv = at(dv0, (uint32_t)pv_s * kTileV);
 #pragma unroll
                 for (int kk = 0; kk < TH / 16; ++kk)  // sixteen positions per instruction
-                    umma_ts(tO, tS0 + 64u * i + 8 * kk, at(dv, kk * 2 * kVGroup), idesc_pv, ((pv_f0 & 1) || kk > 0) ? 1u : 0u);
-                tc_commit(bar(BAR_EMPTY + pv_s0));
-                tc_commit(bar(BAR_PFREE + NB * b + i));
-                if (pv_f0 & 2) tc_commit(bar(BAR_OFULL + b));
-                pv_off0 = pv_off1;
-                pv_s0 = pv_s1;
-                pv_f0 = pv_f1;
+                    umma_ts(tO0, tS0 + (uint32_t)TH * i + 8 * kk, at(dv, kk * 2 * kVGroup), idesc_pv, kk > 0 ? 1u : acc0);
+                tc_commit(bar(BAR_EMPTY + pv_s));
+                acc0 = acc1;
+                if (++pv_s == NS) pv_s = 0;
                 ++done;
-            };
-            // ... waiting for the weights first (used where the thread can do nothing else)
-            auto issue_pv = [&]() {
-                if (!mbar_wait_fast(bar(BAR_PREADY + NB * b + (done & 1)), (done >> 1) & 1, abort_flag, SITE_PREADY)) return false;
-                do_pv();
                 return true;
             };
-            for (; ok && ss.valid; ss.next_unit()) {
-                const Unit& u = ss.u;
-                const int n_half = 2 * u.n_tiles - (u.last_valid <= TH ? 1 : 0);
-                const int rot = unit_rotation(u);
-                const uint32_t q_off = (uint32_t)(ss.useq % NQ) * kTileK;
-                bool q_seen = false;  // this thread has seen the unit's Q block staged
-                for (int p = (b + NG - rot) % NG; p < n_half; p += NG) {
-                    const int t = gs + (p >> 1), half = p & 1;
-                    const int s = t % NS, par = gp ^ ((t / NS) & 1);
-                    // buffer i still holds the weights of step cnt - NB: its weighted sum goes first (and before the
-                    // wait for the tile: at a unit's end the group is waiting for exactly this weighted sum).  The tensor
+            for (; ok && un.valid; un.next(), ++useq) {
+                const uint64_t dq = at(dq0, (uint32_t)(useq & 1) * kTileQ);
+                for (int j = 0; j < un.u.n_tiles; ++j) {
+                    // buffer i still holds the weights of step cnt - 2: its weighted sum goes first (and before the wait
+                    // for the tile: at a unit's end the group is waiting for exactly this weighted sum).  The tensor
                     // core runs this thread's instructions in order, so the scores below need not wait for it to finish.
-                    if (ok && cnt - done == NB) ok = issue_pv();
+                    if (cnt - done == 2) ok = issue_pv();
                     if (ok) ok = mbar_wait_fast(bar(BAR_FULL + s), par, abort_flag, SITE_TILE);
-                    if (ok && !q_seen) {  // first scores of a unit: its Q block must have landed
-                        ok = mbar_wait_fast(bar(BAR_QFULL + ss.useq % NQ), (ss.useq / NQ) & 1, abort_flag, SITE_Q);
-                        q_seen = true;
-                    }
                     if (!ok) break;
                     tc_fence_after();
                     const int i = cnt & 1;
-                    const uint64_t dq = at(dq0, q_off), dk = at(dk0, (uint32_t)s * kTileK + half * (TH / 8) * 512);
+                    const uint64_t dk = at(dk0, (uint32_t)s * kTileK);
 #pragma unroll
                     for (int ks = 0; ks < D / 16; ++ks)
-                        umma_ss(tS0 + 64u * i, at(dq, ks * 256), at(dk, ks * 256), idesc_s, ks > 0 ? 1u : 0u);
-                    tc_commit(bar(BAR_SFULL + NB * b + i));
-                    const uint32_t off = (uint32_t)s * kTileV + half * (TH / 8) * kVGroup;
-                    const int f = (p >= NG ? 1 : 0) | (p + NG >= n_half ? 2 : 0);
-                    if (cnt == done) {
-                        pv_off0 = off;
-                        pv_s0 = s;
-                        pv_f0 = f;
-                    } else {
-                        pv_off1 = off;
-                        pv_s1 = s;
-                        pv_f1 = f;
+                        umma_ss(tS0 + (uint32_t)TH * i, at(dq, ks * 256), at(dk, ks * 256), idesc_s, ks > 0 ? 1u : 0u);
+                    tc_commit(bar(BAR_SFULL + i));
+                    (cnt == done ? acc0 : acc1) = j > 0 ? 1u : 0u;
+                    if (++s == NS) {
+                        s = 0;
+                        par ^= 1;
                     }
                     ++cnt;
                 }
-                if (!ok) break;
-                const int t_last = gs + u.n_tiles - 1;
-                const bool empty_tail = u.last_valid <= TH && (2 * u.n_tiles - 1 + rot) % NG == b;
-                // A weighted sum is normally issued when its buffer is wanted for the scores two steps on.  In a run of
-                // short units whose halves go to the other groups that could be many units on -- while the other groups
-                // wait, at the end of the unit it belongs to, for this group's accumulator, the issuing threads behind
-                // them stop releasing Q blocks and stages, and the tile or Q block this thread is waiting for never comes.
-                // So where this thread passes a unit in which it issued nothing (or has only the empty tail to release),
-                // whatever it still holds is issued first; waiting for the weights there cannot block on anything this
-                // thread does later.  Units in which the group has halves keep their lead of two steps.
-                if (!q_seen || empty_tail)
-                    while (ok && done < cnt) ok = issue_pv();
-                if (!ok) break;
-                if (empty_tail) {
-                    // the empty second half of the unit's last tile is this group's: nothing to compute, but the
-                    // stage needs this half's release
-                    ok = mbar_wait_fast(bar(BAR_FULL + t_last % NS), gp ^ ((t_last / NS) & 1), abort_flag, SITE_TAIL_TILE);
-                    if (!ok) break;
-                    mbar_arrive(bar(BAR_EMPTY + t_last % NS));
-                }
-                // This issuer no longer reads the unit's Q buffer.  It observes every staging of a buffer,
-                // whether it has halves in the unit or not: the buffer is staged again only after all
-                // issuers have released it, so no issuer can run a use ahead of another on these barriers.
-                if (!q_seen) ok = mbar_wait_fast(bar(BAR_QFULL + ss.useq % NQ), (ss.useq / NQ) & 1, abort_flag, SITE_Q);
-                if (!ok) break;
-                tc_commit(bar(BAR_QEMPTY + ss.useq % NQ));
-                gp ^= ((t_last + 1) / NS) & 1;
-                gs = (t_last + 1) % NS;
+                if (ok) tc_commit(bar(BAR_QEMPTY + (useq & 1)));
             }
             while (ok && done < cnt) ok = issue_pv();
             if (!ok) {
                 *abort_flag = 1;
                 atomicOr(err_flag, ERR_MMA);
             }
-            // nothing of this CTA may still be running on the tensor core at teardown
-            tc_commit(bar(BAR_DRAIN + b));
-            if (!mbar_wait(bar(BAR_DRAIN + b), 0, abort_flag + 2, SITE_DRAIN)) atomicOr(err_flag, ERR_DRAIN);
+            // nothing of this worker may still be running on the tensor core at teardown
+            tc_commit(bar(BAR_DRAIN));
+            if (!mbar_wait(bar(BAR_DRAIN), 0, abort_flag + 2, SITE_DRAIN)) atomicOr(err_flag, ERR_DRAIN);
         }
         __syncwarp();
     } else {
-        // --------------------------------------------------------------------- producers
-        // Producer warp pw owns every kProducerWarps-th tile of the stream and does all of its
-        // copies, so the per-tile bookkeeping is paid by one warp while the others work on their own
-        // tiles.  Lane (q = lane / 4, chunk = lane % 4) copies chunk `chunk` of the pool rows of
-        // positions 32 rb + 4 q + i (rb, i < 4) into tile rows 32 rb + 8 i + q, and patches the
-        // user-specific leading elements of tile rows 32 rb + lane.  A producer is one warp running a chain of
-        // dependent instructions per tile: five of them keep the stage ring ahead of three groups only because a
-        // tile's 32 copies per lane are issued back to back, with nothing that waits between them.
-        const int pw = warp - kProducerWarp0, q = lane >> 2, chunk = lane & 3;
+        // --------------------------------------------------------------------- producer
+        // Lane (q = lane / 4, chunk = lane % 4) copies chunk `chunk` of the pool rows of positions 32 rb + 4 q + i
+        // (rb < 2, i < 4) into tile rows 32 rb + 8 i + q, and patches the user-specific leading elements of tile rows
+        // 32 rb + lane.  A tile is published one tile later, when its copies have had time to land (or as soon as there
+        // is no free stage to copy into).  Its indices and user parts are contiguous streams of the arena: they come
+        // into shared memory with asynchronous copies of their own, two tiles ahead (held in registers instead they
+        // cost the warp a stall of a memory latency per tile, wherever the compiler moves a register).
+        const int q = lane >> 2, chunk = lane & 3;
         const int patch_pos = 4 * (lane & 7) + (lane >> 3);  // position (inside a 32-block) held by row `lane`
         const uint32_t kv_lane = (uint32_t)(chunk * 128 + q * 16);
         const int64_t pool_stride = (int64_t)a.cv.n_entries * (D * 2);
@@ -1042,133 +861,158 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma_kernel(const AttendAr
         const bool full_k = a.cv.full_k != 0, full_v = a.cv.full_v != 0;
         const char* rowsK0 = reinterpret_cast<const char*>(a.cv.userK) + chunk * 16;
         const char* rowsV0 = reinterpret_cast<const char*>(a.cv.userV) + chunk * 16;
-        Stream<false, VIS> st;
-        st.init(a, n_mb, n_work);
-        for (int i = 0; i < pw && st.valid; ++i) st.advance();
+        Units<false, VIS> un;
+        un.init(a, n_mb, n_work, b);
         bool ok = true;
-        // Everything a tile needs from the compressed cache is requested one tile of this warp ahead:
-        uint2 xk, xv;                     // pool rows of positions 4 lane .. 4 lane + 3
-        UserPart<DUB> uk_n[4], uv_n[4];   // user-specific leading elements (Eq. K: dims [0, d_user)) of tile rows 32 rb + lane
-        auto fetch = [&]() {
-            if (!st.valid) return;
-            const int pos0 = st.u.wk.begin + st.j * TK;
-            const int64_t unit0 = st.u.wk.base + (int64_t)st.u.grp * st.u.wk.Lpad + pos0;  // arena unit of the tile's position 0
-            (void)CKV_CLAMP(unit0, a.arena_units, err_flag);
-            const int valid = st.j == st.u.n_tiles - 1 ? st.u.last_valid : TK;
-            xk = xv = make_uint2(0, 0);
-            if (pos0 + 4 * lane < st.u.wk.Lpad) {  // the arena is padded to 32 positions per user
-                if (!full_k) xk = __ldg(reinterpret_cast<const uint2*>(reinterpret_cast<const uint16_t*>(a.cv.idxK) + unit0 + 4 * lane));
-                if (!full_v) xv = __ldg(reinterpret_cast<const uint2*>(reinterpret_cast<const uint16_t*>(a.cv.idxV) + unit0 + 4 * lane));
-            }
-            if (full_k) xk = make_uint2((4 * lane) | ((4 * lane + 1) << 16), (4 * lane + 2) | ((4 * lane + 3) << 16));
-            if (full_v) xv = make_uint2((4 * lane) | ((4 * lane + 1) << 16), (4 * lane + 2) | ((4 * lane + 3) << 16));
-            if constexpr (DUB > 0) {
-#pragma unroll
-                for (int rb = 0; rb < 4; ++rb) {
-                    if (32 * rb + patch_pos < valid) {
-                        if (!full_k) uk_n[rb].load(reinterpret_cast<const char*>(a.cv.userK) + (unit0 + 32 * rb + patch_pos) * DUB);
-                        if (!full_v) uv_n[rb].load(reinterpret_cast<const char*>(a.cv.userV) + (unit0 + 32 * rb + patch_pos) * DUB);
-                    }
-                }
-            }
+        struct Tile {
+            int valid;               // real positions; 0: no tile
+            int grp, q_rows;         // q_rows >= 0: first tile of a unit with that many query rows in its block
+            int64_t q_row, unit0;    // first query row; arena unit of the tile's position 0
         };
-        fetch();
-        while (st.valid && ok) {
-            const int s = st.g % NS;
-            UserPart<DUB> uk[4], uv[4];
+        int j = 0, mslot = 0;  // tile of the unit that is requested next, and its slot of the request ring
+        const uint32_t meta0 = wbase + L::M;
+        unsigned char* const metap = smem + b * L::WORKER + L::M;
+        auto request = [&]() {
+            Tile t;
+            t.valid = t.grp = 0;
+            t.q_rows = -1;
+            t.q_row = t.unit0 = 0;
+            if (un.valid) {
+                const Unit& u = un.u;
+                const int pos0 = u.wk.begin + j * TH, room = u.wk.Lpad - pos0;  // (the arena is padded to 32 positions per user)
+                t.grp = u.grp;
+                t.unit0 = u.wk.base + (int64_t)u.grp * u.wk.Lpad + pos0;
+                (void)CKV_CLAMP(t.unit0, a.arena_units, err_flag);
+                t.valid = j == u.n_tiles - 1 ? u.last_valid : TH;
+                if (j == 0) {
+                    t.q_rows = u.wk.M - u.row0;
+                    t.q_row = u.wk.q0 + u.row0;
+                }
+                const uint32_t dst = meta0 + mslot * L::META;
 #pragma unroll
-            for (int rb = 0; rb < 4; ++rb) {
-                uk[rb] = uk_n[rb];
-                uv[rb] = uv_n[rb];
-            }
-            const uint2 xk_cur = xk, xv_cur = xv;  // this tile's indices (fetch() below refills xk, xv for the next)
-            if (st.g >= NS) {
-                if (lane == 0) ok = mbar_wait(bar(BAR_EMPTY + s), ((st.g / NS) - 1) & 1, abort_flag, SITE_STAGE);
-                ok = __all_sync(0xffffffffu, ok);
-            }
-            if (!ok) break;
-            const int q_slot = st.j == 0 ? st.useq % NQ : -1;
-            if (st.j == 0) {  // a new unit: stage its Q block (rows beyond M are zero)
-                // Q blocks are taken up in unit order.  A parity wait cannot tell "this buffer's previous use has been
-                // released" from "not even the use before that has": with short units the producers work on five
-                // consecutive units at once, so the warp staging unit u could otherwise overtake the one still
-                // waiting to stage unit u - NQ.
-                if (lane == 0) {
-                    ok = false;
-                    for (uint32_t it = 0; it < (kSpinLimit << 3); ++it) {
-                        if (abort_flag[4] == st.useq) {
-                            ok = true;
-                            break;
-                        }
-                        if ((it & 63u) == 63u && *abort_flag) break;
-                        __nanosleep(64);
+                for (int k = 0; k < (16 + 8 * DUB + 31) / 32; ++k) {
+                    const int c = lane + 32 * k;  // 16-byte chunk of the slot
+                    const char* src;
+                    int pos;
+                    bool want;
+                    if (c < 16) {
+                        pos = 8 * (c & 7);
+                        src = reinterpret_cast<const char*>(c < 8 ? a.cv.idxK : a.cv.idxV) + (t.unit0 + pos) * 2;
+                        want = c < 8 ? !full_k : !full_v;
+                    } else {
+                        const int side = c - 16 >= 4 * DUB, off = 16 * (c - 16 - (side ? 4 * DUB : 0));
+                        pos = off / (DUB > 0 ? DUB : 1);
+                        src = reinterpret_cast<const char*>(side ? a.cv.userV : a.cv.userK) + t.unit0 * DUB + off;
+                        want = (side ? !full_v : !full_k) && c < 16 + 8 * DUB;
                     }
-                    if (!ok && !*abort_flag) note_site(abort_flag, SITE_QTURN);
-                    if (ok && st.useq >= NQ)
-                        ok = mbar_wait(bar(BAR_QEMPTY + st.useq % NQ), ((st.useq / NQ) - 1) & 1, abort_flag, SITE_QBUF);
-                    if (ok) abort_flag[4] = st.useq + 1;
+                    if (want && pos < room) cp_async16_once(dst + 16 * c, src, 16u);
                 }
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok) break;
-                const uint32_t qdst = sbase + kOffQ + (st.useq % NQ) * kTileK + kv_lane;
-                const int rows_in = st.u.wk.M - st.u.row0;
-                const uint16_t* qsrc = Q + ((int64_t)(st.u.wk.q0 + st.u.row0 + q) * G + st.u.grp) * D + chunk * 8;
-#pragma unroll 2
-                for (int rr = 0; rr < 16; ++rr) {  // rows 8 rr + q
-                    const bool in = 8 * rr + q < rows_in;
-                    cp_async16_once(qdst + 512 * rr, in ? qsrc + (int64_t)8 * rr * G * D : Q, in ? 16u : 0u);
+                if (++j == u.n_tiles) {
+                    j = 0;
+                    un.next();
                 }
             }
-            const int64_t tile_unit0 = st.u.wk.base + (int64_t)st.u.grp * st.u.wk.Lpad + st.u.wk.begin + st.j * TK;
-            const char* pk = full_k ? rowsK0 + tile_unit0 * (D * 2) : poolK0 + st.u.grp * pool_stride;
-            const char* pv = full_v ? rowsV0 + tile_unit0 * (D * 2) : poolV0 + st.u.grp * pool_stride;
-            const uint32_t kdst = sbase + kOffK + s * kTileK + kv_lane, vdst = sbase + kOffV + s * kTileV + kv_lane;
-            const int valid = st.j == st.u.n_tiles - 1 ? st.u.last_valid : TK;
-            // The indices of positions 32 rb + 4 q .. + 3 are with lane 8 rb + q (it fetched them as one 8-byte
-            // word per side); all sixteen of a side come over by shuffles before the first copy is issued, so that
-            // the copies are not strung out between dependent loads.
-            uint32_t ik[8], iv[8];
-#pragma unroll
-            for (int rb = 0; rb < 4; ++rb) {
-                ik[2 * rb] = __shfl_sync(0xffffffffu, xk_cur.x, 8 * rb + q);
-                ik[2 * rb + 1] = __shfl_sync(0xffffffffu, xk_cur.y, 8 * rb + q);
-                iv[2 * rb] = __shfl_sync(0xffffffffu, xv_cur.x, 8 * rb + q);
-                iv[2 * rb + 1] = __shfl_sync(0xffffffffu, xv_cur.y, 8 * rb + q);
-            }
-#pragma unroll
-            for (int it = 0; it < 16; ++it) {  // rb = it / 4, i = it % 4: position 32 rb + 4 q + i -> tile row 32 rb + 8 i + q
-                const int pos = 32 * (it >> 2) + 4 * q + (it & 3);
-                const uint32_t nb = pos < valid ? 16u : 0u;  // rows of positions beyond the history are zero
-                const int jk = (int)((ik[it >> 1] >> (16 * (it & 1))) & 0xffffu), jv = (int)((iv[it >> 1] >> (16 * (it & 1))) & 0xffffu);
-                // (range-checked build: pool indices below n_entries, destinations inside the stage)
-                (void)CKV_CLAMP((int)(512 * it + kv_lane), kTileK - 15, err_flag);
-                (void)CKV_CLAMP((int)(kVGroup * it + kv_lane), kTileV - 15, err_flag);
-                cp_async16(kdst + 512 * it, pk + (size_t)CKV_CLAMP(jk, full_k ? TK : a.cv.n_entries, err_flag) * (D * 2), nb);
-                cp_async16(vdst + kVGroup * it, pv + (size_t)CKV_CLAMP(jv, full_v ? TK : a.cv.n_entries, err_flag) * (D * 2), nb);
-            }
-            cp_async_commit();
-            // what this warp's next tile needs travels while the copies land
-            st.advance_by(kProducerWarps);
-            fetch();
-            cp_async_wait<0>();
-            __syncwarp();  // a row's chunks were copied by four lanes of this warp
+            mslot = (mslot + 1) & (L::META_SLOTS - 1);
+            return t;
+        };
+        Tile t0 = request(), t1 = request();
+        cp_async_commit();
+        cp_async_wait<0>();
+        __syncwarp();
+        int p_valid = 0, p_s = 0, p_m = 0;  // the tile whose copies are in flight: positions, stage, request slot
+        auto publish = [&]() {  // its copies have landed: patch, and hand it to the issuing thread
+            __syncwarp();       // a row's chunks were copied by four lanes of this warp
             if constexpr (DUB > 0) {
 #pragma unroll
-                for (int rb = 0; rb < 4; ++rb) {
-                    if (32 * rb + patch_pos < valid) {  // zero rows beyond the history stay zero
-                        if (!full_k) uk[rb].store(smem + kOffK + s * kTileK + k_off(32 * rb + lane, 0));
-                        if (!full_v) uv[rb].store(smem + kOffV + s * kTileV + v_off(32 * rb + lane, 0));
+                for (int rb = 0; rb < 2; ++rb) {
+                    if (32 * rb + patch_pos < p_valid) {  // zero rows beyond the history stay zero
+                        const unsigned char* up = metap + p_m * L::META + 256 + (32 * rb + patch_pos) * DUB;
+                        UserPart<DUB> x;
+                        if (!full_k) {
+                            x.take(up);
+                            x.store(smem + b * L::WORKER + L::K + p_s * kTileK + k_off(32 * rb + lane, 0));
+                        }
+                        if (!full_v) {
+                            x.take(up + TH * DUB);
+                            x.store(smem + b * L::WORKER + L::V + p_s * kTileV + v_off(32 * rb + lane, 0));
+                        }
                     }
                 }
             }
             fence_proxy_async();  // by the writing threads themselves: a fence on the reading side alone is not enough
             __syncwarp();
-            if (lane == 0) {
-                if (q_slot >= 0) mbar_arrive(bar(BAR_QFULL + q_slot));
-                mbar_arrive(bar(BAR_FULL + s));
+            if (lane == 0) mbar_arrive(bar(BAR_FULL + p_s));
+            p_valid = 0;
+        };
+        int s = 0, useq = 0, m = 0;
+        uint32_t par = 1;  // parity of the release of stage s that the next copy into it waits for (the first round passes)
+        while (t0.valid > 0) {
+            // a free stage, and for a unit's first tile the Q block of the unit before the last
+            bool free = mbar_test(bar(BAR_EMPTY + s), par) && (t0.q_rows < 0 || mbar_test(bar(BAR_QEMPTY + (useq & 1)), ((useq >> 1) & 1) ^ 1));
+            if (!__all_sync(0xffffffffu, free)) {
+                if (p_valid > 0) {
+                    cp_async_wait<0>();
+                    publish();
+                }
+                ok = mbar_wait(bar(BAR_EMPTY + s), par, abort_flag, SITE_STAGE) &&
+                     (t0.q_rows < 0 || mbar_wait(bar(BAR_QEMPTY + (useq & 1)), ((useq >> 1) & 1) ^ 1, abort_flag, SITE_QBUF));
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
             }
+            if (t0.q_rows >= 0) {  // stage the unit's Q block (rows beyond M are zero)
+                const uint32_t qdst = wbase + L::Q + (useq & 1) * kTileQ + kv_lane;
+                const uint16_t* qsrc = Q + ((t0.q_row + q) * G + t0.grp) * D + chunk * 8;
+#pragma unroll 2
+                for (int rr = 0; rr < 16; ++rr) {  // rows 8 rr + q
+                    const bool in = 8 * rr + q < t0.q_rows;
+                    cp_async16_once(qdst + 512 * rr, in ? qsrc + (int64_t)8 * rr * G * D : Q, in ? 16u : 0u);
+                }
+                ++useq;
+            }
+            const char* pk = full_k ? rowsK0 + t0.unit0 * (D * 2) : poolK0 + t0.grp * pool_stride;
+            const char* pv = full_v ? rowsV0 + t0.unit0 * (D * 2) : poolV0 + t0.grp * pool_stride;
+            const uint32_t kdst = wbase + L::K + s * kTileK + kv_lane, vdst = wbase + L::V + s * kTileV + kv_lane;
+#pragma unroll
+            for (int rb = 0; rb < 2; ++rb) {
+                const int p4 = 32 * rb + 4 * q;  // this lane's four positions of the block
+                uint2 xk = make_uint2(p4 | ((p4 + 1) << 16), (p4 + 2) | ((p4 + 3) << 16)), xv = xk;
+                if (!full_k) xk = *reinterpret_cast<const uint2*>(metap + m * L::META + 2 * p4);
+                if (!full_v) xv = *reinterpret_cast<const uint2*>(metap + m * L::META + 128 + 2 * p4);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {  // position 32 rb + 4 q + i -> tile row 32 rb + 8 i + q
+                    const uint32_t nb = p4 + i < t0.valid ? 16u : 0u;  // rows of positions beyond the history are zero
+                    uint32_t jk = ((i < 2 ? xk.x : xk.y) >> (16 * (i & 1))) & 0xffffu, jv = ((i < 2 ? xv.x : xv.y) >> (16 * (i & 1))) & 0xffffu;
+                    if (p4 + i >= t0.valid) jk = jv = 0;  // (behind the history the slot may hold anything)
+                    // (range-checked build: pool indices below n_entries, destinations inside the stage)
+                    const int it = 4 * rb + i;
+                    (void)CKV_CLAMP((int)(512 * it + kv_lane), kTileK - 15, err_flag);
+                    (void)CKV_CLAMP((int)(kVGroup * it + kv_lane), kTileV - 15, err_flag);
+                    cp_async16(kdst + 512 * it, pk + (size_t)CKV_CLAMP((int)jk, full_k ? TH : a.cv.n_entries, err_flag) * (D * 2), nb);
+                    cp_async16(vdst + kVGroup * it, pv + (size_t)CKV_CLAMP((int)jv, full_v ? TH : a.cv.n_entries, err_flag) * (D * 2), nb);
+                }
+            }
+            Tile t2 = request();
+            cp_async_commit();
+            if (p_valid > 0) {
+                cp_async_wait<1>();  // the copies of the tile before, and the requests of the tile behind this one
+                publish();
+            } else {
+                cp_async_wait<1>();
+                __syncwarp();
+            }
+            p_valid = t0.valid;
+            p_s = s;
+            p_m = m;
+            m = (m + 1) & (L::META_SLOTS - 1);
+            if (++s == NS) {
+                s = 0;
+                par ^= 1;
+            }
+            t0 = t1;
+            t1 = t2;
         }
         cp_async_wait<0>();
+        if (ok && p_valid > 0) publish();
         if (!ok) {
             *abort_flag = 1;
             if (lane == 0) atomicOr(err_flag, ERR_PRODUCER);
@@ -1226,16 +1070,18 @@ cudaError_t launch_attend_umma(int max_M, const AttendArgs& a, int n_sms, int* e
     if (a.n_items == 0) return cudaSuccess;
     const int n_mb = (max_M + 127) / 128;
     const int64_t n_work = (int64_t)a.n_items * n_mb * a.cv.n_groups;
-    if (n_work + n_sms >= (int64_t)1 << 32) return cudaErrorInvalidValue;  // the kernel counts units in 32 bits
+    if (n_work + NW * (int64_t)n_sms >= (int64_t)1 << 32) return cudaErrorInvalidValue;  // the kernel counts units in 32 bits
     const unsigned grid = (unsigned)(n_work < n_sms ? n_work : n_sms);
-    auto go = [&](auto kernel) {
-        return launch_kernel(l, kernel, grid, kThreads, kSmemBytes, 1, a, n_mb, n_work, err_flag);
+    auto go = [&](auto kernel, int smem_bytes) {
+        return launch_kernel(l, kernel, grid, kThreads, smem_bytes, 1, a, n_mb, n_work, err_flag);
     };
     const bool sm = a.mode == CKV_SOFTMAX, vis = a.vis != nullptr;
     if (vis && a.vmax == nullptr) return cudaErrorInvalidValue;
 #define CKV_UMMA_GO(DUB)                                                                                          \
-    (vis ? (sm ? go(attend_umma_kernel<CKV_SOFTMAX, DUB, true>) : go(attend_umma_kernel<CKV_SILU_OVER_L, DUB, true>)) \
-         : (sm ? go(attend_umma_kernel<CKV_SOFTMAX, DUB, false>) : go(attend_umma_kernel<CKV_SILU_OVER_L, DUB, false>)))
+    (vis ? (sm ? go(attend_umma_kernel<CKV_SOFTMAX, DUB, true>, Map<DUB>::BYTES)                                  \
+               : go(attend_umma_kernel<CKV_SILU_OVER_L, DUB, true>, Map<DUB>::BYTES))                             \
+         : (sm ? go(attend_umma_kernel<CKV_SOFTMAX, DUB, false>, Map<DUB>::BYTES)                                 \
+               : go(attend_umma_kernel<CKV_SILU_OVER_L, DUB, false>, Map<DUB>::BYTES)))
     switch (a.cv.full_k && a.cv.full_v ? 0 : a.cv.d_user) {  // the user-specific width of the shared side(s)
         case 0: return CKV_UMMA_GO(0);
         case 1: return CKV_UMMA_GO(2);
