@@ -137,9 +137,10 @@ struct Plan {
     int64_t opt_split = 0, opt_kernel = 0;
     bool with_vis = false;   // planned for a call with visible lengths (other kernel choice)
     // The request list cut into n_ranges runs of consecutive users (host-buffer calls are pipelined range by
-    // range): items and the split list are grouped by range, r_item / r_split give each range's slice.
+    // range): items, the split list and the works are grouped by range, r_item / r_split / r_work give each range's slice.
     int32_t n_ranges = 1;
-    int32_t r_user[kMaxRanges + 1] = {}, r_item[kMaxRanges + 1] = {}, r_split[kMaxRanges + 1] = {};
+    int32_t r_user[kMaxRanges + 1] = {}, r_item[kMaxRanges + 1] = {}, r_split[kMaxRanges + 1] = {},
+            r_work[kMaxRanges + 1] = {};
     DevBuf dev;              // reqs | items | split list | works
     void* host = nullptr;    // pinned mirror the tables are built in
     size_t host_cap = 0;
@@ -148,7 +149,7 @@ struct Plan {
     Item* d_items = nullptr;
     int32_t* d_split = nullptr;
     Work* d_works = nullptr;
-    int32_t n_items = 0, n_split = 0, split_items = 0, max_M = 0, max_L = 0, n_req = 0, family = 1, n_vblocks = 0;
+    int32_t n_items = 0, n_split = 0, split_items = 0, max_M = 0, max_L = 0, n_req = 0, family = 1, n_works = 0;
     int32_t parts = 1;       // family 2: warps that share a unit
     int64_t part_rows = 0;
     uint64_t last_use = 0;
@@ -626,7 +627,9 @@ ckv_status build_plan(ckv_ctx* ctx, Plan& pl, int32_t n, const int64_t* users, c
     pl.part_rows = part_rows;
 
     // the tables are laid out in the slot's pinned block and go to the device in one copy
-    const size_t n_works = pl.family == 3 ? items.size() : 0;
+    size_t n_works = 0;
+    if (pl.family == 3)
+        for (const Item& it : items) n_works += (size_t)(reqs[it.req].M + 127) / 128;
     const size_t b_req = sizeof(Req) * reqs.size(), b_item = sizeof(Item) * items.size(),
                  b_split = sizeof(int32_t) * split.size(), b_work = sizeof(Work) * n_works;
     const size_t o_item = (b_req + 255) / 256 * 256, o_split = o_item + (b_item + 255) / 256 * 256,
@@ -648,18 +651,25 @@ ckv_status build_plan(ckv_ctx* ctx, Plan& pl, int32_t n, const int64_t* users, c
     for (size_t i = 0; i < items.size(); ++i) h_items[i] = items[order[i]];
     if (b_split) std::memcpy(h + o_split, split.data(), b_split);
     Work* h_works = (Work*)(h + o_work);
-    // where each request's blocks of 128 queries start in the table of largest visible lengths
-    std::vector<int32_t> vb_off(n_works ? reqs.size() : 0);
-    pl.n_vblocks = 0;
-    for (size_t k = 0; k < vb_off.size(); ++k) {
-        vb_off[k] = pl.n_vblocks;
-        pl.n_vblocks += (reqs[k].M + 127) / 128;
+    // The tcgen05 kernel's records, in order of falling cost inside every range: an item's query blocks one behind the
+    // other, all of the same cost, items longest first; or, with visible lengths, where a late block usually sees more
+    // than an early one, the late blocks of all items first.
+    size_t w = 0;
+    for (int rg = 0; rg < n_ranges && n_works > 0; ++rg) {
+        pl.r_work[rg] = (int32_t)w;
+        int32_t levels = 1;
+        if (with_vis)
+            for (int32_t i = pl.r_item[rg]; i < pl.r_item[rg + 1]; ++i) levels = std::max(levels, (reqs[h_items[i].req].M + 127) / 128);
+        for (int32_t lv = levels - 1; lv >= 0; --lv)
+            for (int32_t i = pl.r_item[rg]; i < pl.r_item[rg + 1]; ++i) {
+                const Item& it = h_items[i];
+                const Req& r = reqs[it.req];
+                const int32_t b0 = with_vis ? lv : 0, b1 = with_vis ? lv + 1 : (r.M + 127) / 128;
+                for (int32_t b = b0; b < b1 && b * 128 < r.M; ++b)
+                    h_works[w++] = Work{r.base, r.L, r.Lpad, r.q0, r.M, it.begin, it.len, it.part_row, b * 128, {0, 0}};
+            }
     }
-    for (size_t i = 0; i < n_works; ++i) {
-        const Item& it = h_items[i];
-        const Req& r = reqs[it.req];
-        h_works[i] = Work{r.base, r.L, r.Lpad, r.q0, r.M, it.begin, it.len, it.part_row, {vb_off[it.req], 0, 0}};
-    }
+    pl.r_work[n_ranges] = pl.n_works = (int32_t)w;
     pl.d_reqs = (Req*)pl.dev.p;
     pl.d_items = (Item*)((char*)pl.dev.p + o_item);
     pl.d_split = (int32_t*)((char*)pl.dev.p + o_split);
@@ -1370,13 +1380,15 @@ ckv_status timed(ckv_ctx* ctx, bool time_it, cudaStream_t s, F&& attend)
     return CKV_OK;
 }
 
-// The kernels of one slice of a plan (items [i0, i1), split requests [s0, s1)) on stream s.
-ckv_status launch_slice(ckv_ctx* ctx, const Plan* pl, AttendArgs a, int i0, int i1, int s0, int s1, bool time_it,
-                        cudaStream_t s)
+// The kernels of one slice of a plan (items [i0, i1), split requests [s0, s1), works [w0, w1)) on stream s.
+ckv_status launch_slice(ckv_ctx* ctx, const Plan* pl, AttendArgs a, int i0, int i1, int s0, int s1, int w0, int w1,
+                        bool time_it, cudaStream_t s)
 {
     const int D = ctx->cfg.head_dim, G = ctx->cfg.n_groups;
     a.items = pl->d_items + i0;
-    a.works = pl->d_works ? pl->d_works + i0 : nullptr;
+    a.works = pl->d_works ? pl->d_works + w0 : nullptr;
+    a.n_works = w1 - w0;
+    if (a.vmax) a.vmax += w0;
     a.n_items = i1 - i0;
     a.inl = 0;
     const Launch l = launch_on(ctx, s);
@@ -1388,7 +1400,7 @@ ckv_status launch_slice(ckv_ctx* ctx, const Plan* pl, AttendArgs a, int i0, int 
                                   tw + (size_t)pl->n_req * G * fact_row_floats(ctx->n_entries), l));
             ctx->st_launches += 2;
         } else if (pl->family == 3)
-            CK(launch_attend_umma(pl->max_M, a, ctx->n_sms, ctx->d_err, l));
+            CK(launch_attend_umma(a, ctx->n_sms, ctx->d_err, l));
         else if (pl->family == 2) {
             ckv_status st2 = run_mma(ctx, D, pl->max_M, pl->parts, a, nullptr, l);
             if (st2 != CKV_OK) return st2;
@@ -1487,7 +1499,7 @@ ckv_status attend_impl(ckv_ctx* ctx, int32_t n, const int64_t* users, const int3
         a.reqs = nullptr;
         a.items = nullptr;
         a.works = nullptr;
-        a.n_items = a.inl = 0;
+        a.n_items = a.n_works = a.inl = 0;
         a.queries = d_q;
         a.vis = d_vis;
         a.vmax = nullptr;
@@ -1558,11 +1570,12 @@ ckv_status attend_impl(ckv_ctx* ctx, int32_t n, const int64_t* users, const int3
     a.n_items = pl->n_items;
     a.partials = (float*)ctx->partials.p;
     a.works = pl->d_works;
+    a.n_works = pl->n_works;
     a.part_rows = pl->family == 4 ? 0 : pl->part_rows;
     ctx->ev_valid = false;
     if (d_vis && pl->family == 3 && pl->n_items > 0) {
         // the tcgen05 kernel's roles skip what lies behind every row's limit: the largest limit per block of queries
-        CK(grow(ctx->vmax, (size_t)std::max(pl->n_vblocks, 1) * sizeof(int32_t), &ctx->st_allocs));
+        CK(grow(ctx->vmax, (size_t)std::max(pl->n_works, 1) * sizeof(int32_t), &ctx->st_allocs));
         cudaStream_t vs = n_ranges > 1 ? ctx->pipe_stream[0] : s;
         if (n_ranges > 1) CK(cudaStreamWaitEvent(vs, ctx->pipe_plan, 0));
         CK(launch_vis_block_max(a, (int32_t*)ctx->vmax.p, vs));
@@ -1577,7 +1590,7 @@ ckv_status attend_impl(ckv_ctx* ctx, int32_t n, const int64_t* users, const int3
         if (time_it)
             for (auto& e : ctx->ev)
                 if (!e) CK(cudaEventCreate(&e));
-        st = launch_slice(ctx, pl, a, 0, pl->n_items, 0, pl->n_split, time_it, s);
+        st = launch_slice(ctx, pl, a, 0, pl->n_items, 0, pl->n_split, 0, pl->n_works, time_it, s);
         if (st != CKV_OK) return st;
         ctx->ev_valid = time_it;
         if (o_host) CK(cudaMemcpyAsync(out, d_out, o_bytes, cudaMemcpyDeviceToHost, s));
@@ -1592,7 +1605,7 @@ ckv_status attend_impl(ckv_ctx* ctx, int32_t n, const int64_t* users, const int3
         cudaStream_t ps = ctx->pipe_stream[0];
         CK(cudaStreamWaitEvent(ps, ctx->pipe_plan, 0));
         for (int r = 1; r < n_ranges; ++r) CK(cudaStreamWaitEvent(ps, ctx->pipe_h2d[r], 0));
-        result = launch_slice(ctx, pl, a, 0, pl->n_items, 0, pl->n_split, false, ps);
+        result = launch_slice(ctx, pl, a, 0, pl->n_items, 0, pl->n_split, 0, pl->n_works, false, ps);
         if (result == CKV_OK) {
             cudaError_t e = cudaMemcpyAsync(out, d_out, o_bytes, cudaMemcpyDeviceToHost, ps);
             if (e != cudaSuccess) result = ctx->fail(e);
@@ -1601,7 +1614,8 @@ ckv_status attend_impl(ckv_ctx* ctx, int32_t n, const int64_t* users, const int3
         for (int r = 0; r < n_ranges && result == CKV_OK; ++r) {
             cudaStream_t ps = ctx->pipe_stream[r];
             CK(cudaStreamWaitEvent(ps, ctx->pipe_plan, 0));
-            result = launch_slice(ctx, pl, a, pl->r_item[r], pl->r_item[r + 1], pl->r_split[r], pl->r_split[r + 1], false, ps);
+            result = launch_slice(ctx, pl, a, pl->r_item[r], pl->r_item[r + 1], pl->r_split[r], pl->r_split[r + 1],
+                                  pl->r_work[r], pl->r_work[r + 1], false, ps);
             const size_t r0 = (size_t)q_off[r_user[r]], r1 = (size_t)q_off[r_user[r + 1]];
             if (result == CKV_OK && r1 > r0) {
                 cudaError_t e = cudaMemcpyAsync((char*)out + r0 * o_row, (const char*)d_out + r0 * o_row, (r1 - r0) * o_row,
@@ -1990,6 +2004,7 @@ extern "C" ckv_status ckv_attend_static(ckv_ctx* ctx, int32_t n, const int64_t* 
     a.reqs = (const Req*)base;
     a.items = (const Item*)(base + kOffItems);
     a.works = nullptr;
+    a.n_works = 0;
     a.n_items = n_items;
     a.inl = 0;
     a.queries = queries;

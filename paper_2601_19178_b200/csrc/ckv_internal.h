@@ -41,14 +41,15 @@ struct InlineTable {
     InlineReq r[kInlineReqs];
 };
 
-// An Item merged with its request row, for kernels that read their work list once per unit
+// A block of up to 128 query rows of an Item, merged with its request row, for kernels that read their work list once per unit
 // with plain 16-byte loads (48 bytes, 16-byte aligned).
 struct Work {
     int64_t base;      // Req::base
     int32_t L, Lpad;   // Req::L, Req::Lpad
     int32_t q0, M;     // Req::q0, Req::M
     int32_t begin, len, part_row;  // Item::begin, Item::len, Item::part_row
-    int32_t pad[3];    // [0]: with visible lengths, where the request's query blocks start in AttendArgs::vmax
+    int32_t row0;      // first query row of the block
+    int32_t pad[2];
 };
 
 // Everything a kernel needs to find the compressed cache and the pool.
@@ -73,12 +74,13 @@ struct AttendArgs {
     CacheView cv;
     const Req* reqs;
     const Item* items;
-    const Work* works;     // one per item, same order (tcgen05 family only, else null)
+    const Work* works;     // tcgen05 family only: one per (item, block of 128 queries)
+    int32_t n_works;
     int32_t n_items;
     int32_t inl;           // the requests are kernel arguments (InlineTable), one unsplit item each; reqs and items are null
     const void* queries;   // [Q][G][D]
     const int32_t* vis;    // null, or per query row the number of leading history positions it attends [Q]
-    const int32_t* vmax;   // tcgen05 family with visible lengths: largest limit per (request, block of 128 queries)
+    const int32_t* vmax;   // tcgen05 family with visible lengths: largest limit per work record
     void* out;             // [Q][G][D]
     float* partials;       // [part rows][G][D + 2]  (m, l, acc[D])
     int32_t out_dtype;     // ckv_dtype
@@ -241,8 +243,8 @@ cudaError_t launch_project(int d_in, int d_out, int G, const void* x, const void
 bool umma_supported(int dtype, int head_dim, int d_user, int idx_bytes);
 // err_flag: device int, OR-ed with a non-zero code if a bounded wait inside the kernel ran out.
 // Persistent: one CTA per SM (n_sms of them at most).
-cudaError_t launch_attend_umma(int max_M, const AttendArgs& a, int n_sms, int* err_flag, const Launch& l);
-// Fills vmax (one int per request and block of 128 queries, at Work::pad[0] + block) from a.vis; a.works as for the attend.
+cudaError_t launch_attend_umma(const AttendArgs& a, int n_sms, int* err_flag, const Launch& l);
+// Fills vmax (one int per work record) from a.vis; a.works as for the attend.
 cudaError_t launch_vis_block_max(const AttendArgs& a, int32_t* vmax, cudaStream_t s);
 
 }  // namespace ckv

@@ -44,6 +44,8 @@
 #include <cuda_bf16.h>
 #include <math_constants.h>
 
+#include <type_traits>
+
 #include "ckv_internal.h"
 #include "ptx_helpers.cuh"
 
@@ -495,7 +497,7 @@ struct Unit {
     Work wk;
     int grp;
     int row0;        // first query row of the block
-    int n_tiles;     // > 0: tiles to process; 0: empty history (zero output rows); < 0: nothing at all
+    int n_tiles;     // > 0: tiles to process; 0: empty history (zero output rows)
     int last_valid;  // real positions in the last tile
 };
 
@@ -513,93 +515,72 @@ __device__ __forceinline__ Work load_work(const Work* p)
     return u.w;
 }
 
-// A worker's units: worker b of block x takes units x + gridDim.x b, then every (NW gridDim.x)-th.  Every role walks an
-// identical copy, so stage and buffer indices need no communication.  The record of the following unit is always in
-// flight while the current one is processed.  Unit w stands for (item, group, query block) = (w / n_mb / G,
-// w / n_mb % G, w % n_mb); the coordinates are stepped with carries instead of divided out each time.
+// A worker's units.  Worker k = x + gridDim.x b (worker b of block x) takes one unit of every run of NW gridDim.x
+// consecutive ones, number k of the even runs and number k from the end of the odd ones, so that units in order of falling
+// cost come out even.  Every role walks an identical copy, so stage and buffer indices need no communication.  The record
+// of the following unit is always in flight while the current one is processed.
+// Unit w stands for (work record, group) = (w / G, w % G), a record for every (item, query block) that exists.
 // KEEP_EMPTY: also stop at units with an empty history (the role that writes their zero rows).
 template <bool KEEP_EMPTY, bool VIS>
 struct Units {
     const Work* works;
-    const int32_t* vmax;         // VIS: per (request, query block) the largest visible length of its rows
-    uint32_t n_mb, n_groups;
-    uint32_t w, n_work, stride;  // the host keeps n_work + stride below 2^32
-    uint32_t item, grp, mb;      // coordinates of unit w
-    uint32_t d_item, d_grp, d_mb;  // the stride in the same mixed radix
+    const int32_t* vmax;       // VIS: per record the largest visible length of its rows
+    uint32_t n_groups, n_work, run, k;  // the host keeps n_work + 2 run below 2^32
+    uint32_t base;             // first unit of the run behind the current one
+    bool odd;                  // that run is an odd one
+    uint32_t w_nxt, grp_nxt;   // the unit taken from it
+    int vmax_nxt;
     Unit u;
-    Work nxt;    // record of unit w + stride (valid if that is < n_work)
+    Work nxt;                  // its record (valid if w_nxt < n_work)
     bool valid;
-    __device__ __forceinline__ void step(uint32_t& it, uint32_t& gr, uint32_t& m) const
+    __device__ __forceinline__ void request()
     {
-        m += d_mb;
-        gr += d_grp;
-        it += d_item;
-        if (m >= n_mb) {
-            m -= n_mb;
-            ++gr;
-        }
-        if (gr >= n_groups) {
-            gr -= n_groups;
-            ++it;
-        }
-    }
-    __device__ __forceinline__ void take()
-    {
-        valid = false;
-        while (w < n_work) {
-            u.wk = nxt;
-            u.grp = (int)grp;
-            u.row0 = (int)mb * 128;
-            const uint32_t wn = w + stride;
-            uint32_t ni = item, ng = grp, nm = mb;
-            step(ni, ng, nm);
-            if (wn < n_work) nxt = load_work(works + ni);
-            // with visible lengths nothing behind the block's largest limit is touched (every role decodes the same)
-            int len = u.wk.len;
-            if constexpr (VIS) {
-                if (u.row0 < u.wk.M) len = min(len, max(__ldg(vmax + u.wk.pad[0] + mb) - u.wk.begin, 0));
-            }
-            u.n_tiles = u.row0 < u.wk.M ? (len + TH - 1) / TH : -1;
-            u.last_valid = len - (u.n_tiles - 1) * TH;
-            if (u.n_tiles > 0 || (KEEP_EMPTY && u.n_tiles == 0)) {
-                valid = true;
-                return;
-            }
-            w = wn;
-            item = ni;
-            grp = ng;
-            mb = nm;
-        }
+        w_nxt = base + (odd ? run - 1 - k : k);
+        base += run;
+        odd = !odd;
+        if (w_nxt >= n_work) return;  // (a later run lies behind the end altogether)
+        const uint32_t i = w_nxt / n_groups;
+        grp_nxt = w_nxt - i * n_groups;
+        nxt = load_work(works + i);
+        if constexpr (VIS) vmax_nxt = __ldg(vmax + i);
     }
     __device__ __forceinline__ void next()
     {
-        w += stride;
-        step(item, grp, mb);
-        take();
+        valid = false;
+        while (w_nxt < n_work) {
+            u.wk = nxt;
+            u.grp = (int)grp_nxt;
+            u.row0 = u.wk.row0;
+            // with visible lengths nothing behind the block's largest limit is touched (every role decodes the same)
+            int len = u.wk.len;
+            if constexpr (VIS) len = min(len, max(vmax_nxt - u.wk.begin, 0));
+            request();
+            u.n_tiles = (len + TH - 1) / TH;
+            u.last_valid = len - (u.n_tiles - 1) * TH;
+            if (u.n_tiles > 0 || KEEP_EMPTY) {
+                valid = true;
+                return;
+            }
+        }
     }
-    __device__ __forceinline__ void init(const AttendArgs& a, int n_mb_, int64_t n_work_, int worker)
+    __device__ __forceinline__ void init(const AttendArgs& a, int64_t n_work_, int worker)
     {
         works = a.works;
         if constexpr (VIS) vmax = a.vmax;
-        n_mb = (uint32_t)n_mb_;
         n_groups = (uint32_t)a.cv.n_groups;
         n_work = (uint32_t)n_work_;
-        stride = NW * gridDim.x;
-        w = blockIdx.x + gridDim.x * (uint32_t)worker;
-        mb = w % n_mb;
-        grp = (w / n_mb) % n_groups;
-        item = (w / n_mb) / n_groups;
-        d_mb = stride % n_mb;
-        d_grp = (stride / n_mb) % n_groups;
-        d_item = (stride / n_mb) / n_groups;
-        if (w < n_work) nxt = load_work(works + item);
-        take();
+        run = NW * gridDim.x;
+        k = blockIdx.x + gridDim.x * (uint32_t)worker;
+        base = 0;
+        odd = false;
+        request();
+        next();
     }
 };
 
 // VIS: visible lengths (a.vis, a.vmax); the plain instantiations carry none of that code.
 template <int MODE, int DUB, bool VIS>
-__global__ void __launch_bounds__(kThreads, 1) attend_umma_kernel(const AttendArgs a, int n_mb, int64_t n_work, int* err_flag)
+__global__ void __launch_bounds__(kThreads, 1) attend_umma_kernel(const AttendArgs a, int64_t n_work, int* err_flag)
 {
     using L = Map<DUB>;
     constexpr int NS = L::STAGES;
@@ -648,7 +629,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma_kernel(const AttendAr
         bool ok = true;
         uint32_t sa[32];  // one 32-column chunk of a tile's scores
         Units<true, VIS> un;
-        un.init(a, n_mb, n_work, b);
+        un.init(a, n_work, b);
         for (; un.valid && ok; un.next()) {
             const Unit& u = un.u;
             const int r = u.row0 + row;
@@ -784,7 +765,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma_kernel(const AttendAr
                            dv0 = smem_desc(wbase + L::V, kVGroup, 128);
             auto at = [](uint64_t d, uint32_t byte_off) { return d + (uint64_t)(byte_off >> 4); };  // no carry out of the address field
             Units<false, VIS> un;
-            un.init(a, n_mb, n_work, b);
+            un.init(a, n_work, b);
             int cnt = 0, done = 0;    // steps whose scores / weighted sum have been issued; at most two apart
             int s = 0, par = 0;       // stage of step cnt and the phase parity of its tile
             int pv_s = 0;             // stage of step `done`
@@ -862,7 +843,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma_kernel(const AttendAr
         const char* rowsK0 = reinterpret_cast<const char*>(a.cv.userK) + chunk * 16;
         const char* rowsV0 = reinterpret_cast<const char*>(a.cv.userV) + chunk * 16;
         Units<false, VIS> un;
-        un.init(a, n_mb, n_work, b);
+        un.init(a, n_work, b);
         bool ok = true;
         struct Tile {
             int valid;               // real positions; 0: no tile
@@ -921,21 +902,24 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma_kernel(const AttendAr
         __syncwarp();
         int p_valid = 0, p_s = 0, p_m = 0;  // the tile whose copies are in flight: positions, stage, request slot
         auto publish = [&]() {  // its copies have landed: patch, and hand it to the issuing thread
-            __syncwarp();       // a row's chunks were copied by four lanes of this warp
+            UserPart<DUB> xk[2], xv[2];
             if constexpr (DUB > 0) {
 #pragma unroll
                 for (int rb = 0; rb < 2; ++rb) {
+                    const unsigned char* up = metap + p_m * L::META + 256 + (32 * rb + patch_pos) * DUB;
+                    xk[rb].take(up);
+                    xv[rb].take(up + TH * DUB);
+                }
+            }
+            __syncwarp();       // a row's chunks were copied by four lanes of this warp
+            if constexpr (DUB > 0) {
+                unsigned char *kt = smem + b * L::WORKER + L::K + p_s * kTileK + k_off(lane, 0),
+                              *vt = smem + b * L::WORKER + L::V + p_s * kTileV + v_off(lane, 0);
+#pragma unroll
+                for (int rb = 0; rb < 2; ++rb) {
                     if (32 * rb + patch_pos < p_valid) {  // zero rows beyond the history stay zero
-                        const unsigned char* up = metap + p_m * L::META + 256 + (32 * rb + patch_pos) * DUB;
-                        UserPart<DUB> x;
-                        if (!full_k) {
-                            x.take(up);
-                            x.store(smem + b * L::WORKER + L::K + p_s * kTileK + k_off(32 * rb + lane, 0));
-                        }
-                        if (!full_v) {
-                            x.take(up + TH * DUB);
-                            x.store(smem + b * L::WORKER + L::V + p_s * kTileV + v_off(32 * rb + lane, 0));
-                        }
+                        if (!full_k) xk[rb].store(kt + rb * 4 * 512);
+                        if (!full_v) xv[rb].store(vt + rb * 4 * kVGroup);
                     }
                 }
             }
@@ -946,9 +930,10 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma_kernel(const AttendAr
         };
         int s = 0, useq = 0, m = 0;
         uint32_t par = 1;  // parity of the release of stage s that the next copy into it waits for (the first round passes)
+        bool stage_free = true;  // of stage s, as seen an iteration ago
         while (t0.valid > 0) {
             // a free stage, and for a unit's first tile the Q block of the unit before the last
-            bool free = mbar_test(bar(BAR_EMPTY + s), par) && (t0.q_rows < 0 || mbar_test(bar(BAR_QEMPTY + (useq & 1)), ((useq >> 1) & 1) ^ 1));
+            bool free = stage_free && (t0.q_rows < 0 || mbar_test(bar(BAR_QEMPTY + (useq & 1)), ((useq >> 1) & 1) ^ 1));
             if (!__all_sync(0xffffffffu, free)) {
                 if (p_valid > 0) {
                     cp_async_wait<0>();
@@ -972,27 +957,39 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma_kernel(const AttendAr
             const char* pk = full_k ? rowsK0 + t0.unit0 * (D * 2) : poolK0 + t0.grp * pool_stride;
             const char* pv = full_v ? rowsV0 + t0.unit0 * (D * 2) : poolV0 + t0.grp * pool_stride;
             const uint32_t kdst = wbase + L::K + s * kTileK + kv_lane, vdst = wbase + L::V + s * kTileV + kv_lane;
+            uint2 xk[2], xv[2];  // pool rows of this lane's positions 32 rb + 4 q .. + 3
 #pragma unroll
             for (int rb = 0; rb < 2; ++rb) {
-                const int p4 = 32 * rb + 4 * q;  // this lane's four positions of the block
-                uint2 xk = make_uint2(p4 | ((p4 + 1) << 16), (p4 + 2) | ((p4 + 3) << 16)), xv = xk;
-                if (!full_k) xk = *reinterpret_cast<const uint2*>(metap + m * L::META + 2 * p4);
-                if (!full_v) xv = *reinterpret_cast<const uint2*>(metap + m * L::META + 128 + 2 * p4);
+                const int p4 = 32 * rb + 4 * q;
+                xk[rb] = xv[rb] = make_uint2(p4 | ((p4 + 1) << 16), (p4 + 2) | ((p4 + 3) << 16));
+                if (!full_k) xk[rb] = *reinterpret_cast<const uint2*>(metap + m * L::META + 2 * p4);
+                if (!full_v) xv[rb] = *reinterpret_cast<const uint2*>(metap + m * L::META + 128 + 2 * p4);
+            }
+            auto copies = [&](auto tail) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {  // position 32 rb + 4 q + i -> tile row 32 rb + 8 i + q
-                    const uint32_t nb = p4 + i < t0.valid ? 16u : 0u;  // rows of positions beyond the history are zero
-                    uint32_t jk = ((i < 2 ? xk.x : xk.y) >> (16 * (i & 1))) & 0xffffu, jv = ((i < 2 ? xv.x : xv.y) >> (16 * (i & 1))) & 0xffffu;
-                    if (p4 + i >= t0.valid) jk = jv = 0;  // (behind the history the slot may hold anything)
+                for (int it = 0; it < 8; ++it) {  // position 32 rb + 4 q + i -> tile row 32 rb + 8 i + q   (rb = it / 4, i = it % 4)
+                    const int i = it & 3, pos = 32 * (it >> 2) + 4 * q + i;
+                    uint32_t jk = __byte_perm(i < 2 ? xk[it >> 2].x : xk[it >> 2].y, 0, i & 1 ? 0x4432 : 0x4410),
+                             jv = __byte_perm(i < 2 ? xv[it >> 2].x : xv[it >> 2].y, 0, i & 1 ? 0x4432 : 0x4410);
+                    uint32_t nb = 16u;
+                    if (decltype(tail)::value && pos >= t0.valid) jk = jv = nb = 0;  // rows behind the history are zero
                     // (range-checked build: pool indices below n_entries, destinations inside the stage)
-                    const int it = 4 * rb + i;
                     (void)CKV_CLAMP((int)(512 * it + kv_lane), kTileK - 15, err_flag);
                     (void)CKV_CLAMP((int)(kVGroup * it + kv_lane), kTileV - 15, err_flag);
-                    cp_async16(kdst + 512 * it, pk + (size_t)CKV_CLAMP((int)jk, full_k ? TH : a.cv.n_entries, err_flag) * (D * 2), nb);
-                    cp_async16(vdst + kVGroup * it, pv + (size_t)CKV_CLAMP((int)jv, full_v ? TH : a.cv.n_entries, err_flag) * (D * 2), nb);
+                    cp_async16(kdst + 512 * it, pk + (size_t)CKV_CLAMP(jk, (uint32_t)(full_k ? TH : a.cv.n_entries), err_flag) * (D * 2), nb);
+                    cp_async16(vdst + kVGroup * it, pv + (size_t)CKV_CLAMP(jv, (uint32_t)(full_v ? TH : a.cv.n_entries), err_flag) * (D * 2), nb);
                 }
-            }
+            };
+            if (t0.valid == TH) copies(std::false_type{});
+            else copies(std::true_type{});
             Tile t2 = request();
             cp_async_commit();
+            const int s_cur = s;
+            if (++s == NS) {
+                s = 0;
+                par ^= 1;
+            }
+            stage_free = mbar_test(bar(BAR_EMPTY + s), par);
             if (p_valid > 0) {
                 cp_async_wait<1>();  // the copies of the tile before, and the requests of the tile behind this one
                 publish();
@@ -1001,13 +998,9 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma_kernel(const AttendAr
                 __syncwarp();
             }
             p_valid = t0.valid;
-            p_s = s;
+            p_s = s_cur;
             p_m = m;
             m = (m + 1) & (L::META_SLOTS - 1);
-            if (++s == NS) {
-                s = 0;
-                par ^= 1;
-            }
             t0 = t1;
             t1 = t2;
         }
@@ -1038,42 +1031,38 @@ bool umma_supported(int dtype, int head_dim, int d_user, int idx_bytes)
 
 namespace {
 
-// vmax[off(req) + mb] = largest visible length (clamped to the history) among the rows of query block mb of a
-// request; off(req) is pad[0] of the request's work records.  One block per work item (its request's blocks are
-// written once per item: the same values).
-__global__ void vis_block_max_kernel(const Work* __restrict__ works, int n_items, const int32_t* __restrict__ vis,
+// vmax[i] = largest visible length (clamped to the history) among the rows of work record i.  One warp per record.
+__global__ void vis_block_max_kernel(const Work* __restrict__ works, int n_works, const int32_t* __restrict__ vis,
                                      int32_t* __restrict__ vmax)
 {
-    const Work w = works[blockIdx.x];
-    const int n_mb = (w.M + 127) / 128;
-    for (int mb = threadIdx.x >> 5; mb < n_mb; mb += blockDim.x >> 5) {
-        int m = 0;
-        for (int r = 128 * mb + (threadIdx.x & 31); r < min(w.M, 128 * mb + 128); r += 32)
-            m = max(m, min(max(__ldg(vis + w.q0 + r), 0), w.L));
+    const int i = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
+    if (i >= n_works) return;
+    const Work w = works[i];
+    int m = 0;
+    for (int r = w.row0 + (threadIdx.x & 31); r < min(w.M, w.row0 + 128); r += 32)
+        m = max(m, min(max(__ldg(vis + w.q0 + r), 0), w.L));
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if ((threadIdx.x & 31) == 0) vmax[w.pad[0] + mb] = m;
-    }
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) vmax[i] = m;
 }
 
 }  // namespace
 
 cudaError_t launch_vis_block_max(const AttendArgs& a, int32_t* vmax, cudaStream_t s)
 {
-    if (a.n_items == 0) return cudaSuccess;
-    vis_block_max_kernel<<<a.n_items, 128, 0, s>>>(a.works, a.n_items, a.vis, vmax);
+    if (a.n_works == 0) return cudaSuccess;
+    vis_block_max_kernel<<<(a.n_works + 3) / 4, 128, 0, s>>>(a.works, a.n_works, a.vis, vmax);
     return cudaGetLastError();
 }
 
-cudaError_t launch_attend_umma(int max_M, const AttendArgs& a, int n_sms, int* err_flag, const Launch& l)
+cudaError_t launch_attend_umma(const AttendArgs& a, int n_sms, int* err_flag, const Launch& l)
 {
-    if (a.n_items == 0) return cudaSuccess;
-    const int n_mb = (max_M + 127) / 128;
-    const int64_t n_work = (int64_t)a.n_items * n_mb * a.cv.n_groups;
-    if (n_work + NW * (int64_t)n_sms >= (int64_t)1 << 32) return cudaErrorInvalidValue;  // the kernel counts units in 32 bits
+    if (a.n_works == 0) return cudaSuccess;
+    const int64_t n_work = (int64_t)a.n_works * a.cv.n_groups;
+    if (n_work + 2 * NW * (int64_t)n_sms >= (int64_t)1 << 32) return cudaErrorInvalidValue;  // the kernel counts units in 32 bits
     const unsigned grid = (unsigned)(n_work < n_sms ? n_work : n_sms);
     auto go = [&](auto kernel, int smem_bytes) {
-        return launch_kernel(l, kernel, grid, kThreads, smem_bytes, 1, a, n_mb, n_work, err_flag);
+        return launch_kernel(l, kernel, grid, kThreads, smem_bytes, 1, a, n_work, err_flag);
     };
     const bool sm = a.mode == CKV_SOFTMAX, vis = a.vis != nullptr;
     if (vis && a.vmax == nullptr) return cudaErrorInvalidValue;
