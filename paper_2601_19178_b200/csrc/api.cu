@@ -448,12 +448,9 @@ int choose_family(const ckv_ctx* ctx, bool with_vis, int32_t n, int64_t n_active
     const bool can_umma = ctx->has_umma;
     // tcgen05 from three 16-query blocks on, else the warp-level tensor-core kernel (faster than the CUDA-core
     // kernel from a single query on); the CUDA-core kernel serves what neither supports
-    // One query per user: the pool-side factorisation trades the row gathers for two tables per (user, group) in
-    // HBM (n_entries floats per request and group: not beyond 2 GiB of workspace).
+    // One query per user: the pool-side factorisation trades the row gathers for two tables per (user, group).
     const bool can_fact = plain && all_single && n_active > 0 &&
-                          fact_max_history(ctx->cfg.dtype, ctx->cfg.head_dim, ctx->d_user, ctx->n_entries) >= max_L &&
-                          (int64_t)n * ctx->cfg.n_groups * (fact_row_floats(ctx->n_entries) + fact_aux_floats()) *
-                                  (int64_t)sizeof(float) <= ((int64_t)2 << 30);
+                          fact_supported(ctx->cfg.dtype, ctx->cfg.head_dim, ctx->d_user, ctx->n_entries);
     // It pays when histories are long against the pool and there are enough (user, group) pairs to fill the SMs
     // (one CTA holds a whole pair; the gathering kernel splits long histories over CTAs).  Cost lines fitted to
     // B200 measurements, in microseconds of one SM: a pair costs a + b n_entries + c L on the factorised path,
@@ -1395,10 +1392,9 @@ ckv_status launch_slice(ckv_ctx* ctx, const Plan* pl, AttendArgs a, int i0, int 
     if (time_it) CK(cudaEventRecord(ctx->ev[0], s));
     if (a.n_items > 0) {
         if (pl->family == 4) {
-            float* tw = (float*)ctx->partials.p;
-            CK(launch_attend_fact(D, a, pl->n_req, pl->max_L, ctx->n_sms, tw,
-                                  tw + (size_t)pl->n_req * G * fact_row_floats(ctx->n_entries), l));
-            ctx->st_launches += 2;
+            int launched = -1;  // (one is counted below)
+            CK(launch_attend_fact(D, a, ctx->n_sms, (float*)ctx->partials.p, l, &launched));
+            ctx->st_launches += launched;
         } else if (pl->family == 3)
             CK(launch_attend_umma(a, ctx->n_sms, ctx->d_err, l));
         else if (pl->family == 2) {
@@ -1558,7 +1554,7 @@ ckv_status attend_impl(ckv_ctx* ctx, int32_t n, const int64_t* users, const int3
 
     // split-reduction partials, or the factorisation's tables (per request and group: n_entries + a few floats)
     const size_t ws = pl->family == 4
-                          ? (size_t)pl->n_req * G * ((size_t)fact_row_floats(ctx->n_entries) + fact_aux_floats()) * sizeof(float)
+                          ? (size_t)fact_workspace_floats(pl->n_items, G, ctx->n_entries) * sizeof(float)
                           : (size_t)pl->part_rows * G * (D + 2) * sizeof(float);
     if (ws) CK(grow(ctx->partials, ws, &ctx->st_allocs));
     ctx->st_ws = (int64_t)ws;

@@ -212,15 +212,11 @@ int mma_warps_per_sm(int head_dim, int max_M);
 bool make_pool_tensor_maps(int head_dim, int64_t rows, const void* poolK, const void* poolV, void* maps_out);
 
 // ---- kernels_fact.cu : pool-side factorisation for one query per user (bf16, head_dim 32 or 64, d_user <= 8)
-// Largest history the family can take for this shape (its tables and scores share one CTA's shared memory),
-// or -1 if the shape is not supported.
-int fact_max_history(int dtype, int head_dim, int d_user, int n_entries);
-int fact_aux_floats();
-int fact_row_floats(int n_entries);
-// a.items: one unsplit item per request with a query.  tw: [n_req][G][fact_row_floats(n_entries)] floats,
-// aux: [n_req][G][fact_aux_floats()].
-cudaError_t launch_attend_fact(int head_dim, const AttendArgs& a, int n_req, int max_L, int n_sms, float* tw,
-                               float* aux, const Launch& l);
+bool fact_supported(int dtype, int head_dim, int d_user, int n_entries);
+// Floats of workspace for a list of n_items requests.
+int64_t fact_workspace_floats(int n_items, int n_groups, int n_entries);
+// a.items: one unsplit item per request with a query.  Adds the kernels launched to *launches.
+cudaError_t launch_attend_fact(int head_dim, const AttendArgs& a, int n_sms, float* ws, const Launch& l, int* launches);
 
 // ---- kernels_route.cu : prefill router, fused scores + row arg-max (bf16, d_in 32 / 64 / 128)
 bool route_supported(int d_in);

@@ -18,6 +18,7 @@
 #include <math_constants.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "ckv_internal.h"
 #include "ptx_helpers.cuh"
@@ -27,9 +28,26 @@ namespace {
 
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr int kMainThreads = 1024;
+constexpr int64_t kSlabBytes = (int64_t)1 << 30;
+constexpr size_t kMainSmem = 226 * 1024, kMainExtra = 32 * 9 * 4 + 64;  // shared memory for tables; sums and barriers
 constexpr int kOutWarps = 16;
 
 __device__ __forceinline__ float bf16_bits_to_float(uint32_t b) { return __uint_as_float(b << 16); }
+
+enum { ERR_FACT_TABLE = 128 };  // a bounded wait for a table row ran out
+__device__ __forceinline__ bool table_wait(uint32_t bar, uint32_t parity)
+{
+    for (int i = 0; i < (1 << 22); ++i) {
+        uint32_t ok;
+        asm volatile(
+            "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity)
+            : "memory");
+        if (ok) return true;
+    }
+    return false;
+}
 // ------------------------------------------------------------------------------------------------ T = P_k q
 // T / w rows in HBM are this many floats apart: 32-byte aligned rows, room for zero-filled bf16 pairs up to a
 // multiple of 8 entries
@@ -37,13 +55,31 @@ __host__ __device__ __forceinline__ int row_floats(int n_entries) { return (n_en
 
 constexpr int kTableMT = 4;  // 16-request tiles per warp: every pool row fetched serves 64 requests
 
+// What the main kernel needs to know of a pair, written by the table kernel (in place of a chain of three loads per pair).
+struct __align__(16) PairRec {
+    int64_t unit0;    // arena unit of position 0
+    int32_t L, pad;
+    uint4 q_head;     // the query's first eight elements (the user part meets them), bf16
+};
+
+// Rows of the tables follow the items: row = item * G + group.
 template <int D>
-__global__ void __launch_bounds__(128) fact_table_kernel(const AttendArgs a, int n_req, float* __restrict__ tw)
+__global__ void __launch_bounds__(128)
+    fact_table_kernel(const __grid_constant__ AttendArgs a, float* __restrict__ tw, PairRec* __restrict__ recs)
 {
     constexpr int KS = D / 16, MT = kTableMT;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gl = lane >> 2, t = lane & 3;
     const int m = a.cv.n_entries, G = a.cv.n_groups, grp = blockIdx.z;
     const int j0 = blockIdx.x * 256 + warp * 64, r0 = blockIdx.y * (16 * MT);
+    if (blockIdx.x == 0 && threadIdx.x < 16 * MT && r0 + (int)threadIdx.x < a.n_items) {
+        const Req rq = a.reqs[a.items[r0 + threadIdx.x].req];
+        PairRec rec;
+        rec.unit0 = rq.base + (int64_t)grp * rq.Lpad;
+        rec.L = rq.L;
+        rec.pad = 0;
+        rec.q_head = __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const uint16_t*>(a.queries) + ((int64_t)rq.q0 * G + grp) * D));
+        recs[(int64_t)(r0 + threadIdx.x) * G + grp] = rec;
+    }
     if (j0 >= m) return;
     // Which feature sits in which k-slot of the MMA is free as long as Q and the pool rows agree: a lane reads
     // D / 4 contiguous bytes of "its" rows, and k-step ks, slots (2t, 2t+1, 2t+8, 2t+9) hold features
@@ -55,16 +91,17 @@ __global__ void __launch_bounds__(128) fact_table_kernel(const AttendArgs a, int
 #pragma unroll
     for (int mt = 0; mt < MT; ++mt) {
         const int r_lo = r0 + 16 * mt + gl, r_hi = r_lo + 8;
-        v_lo[mt] = r_lo < n_req && a.reqs[r_lo].M > 0;
-        v_hi[mt] = r_hi < n_req && a.reqs[r_hi].M > 0;
+        v_lo[mt] = r_lo < a.n_items;
+        v_hi[mt] = r_hi < a.n_items;
+        const int64_t q0_lo = v_lo[mt] ? a.reqs[a.items[r_lo].req].q0 : 0, q0_hi = v_hi[mt] ? a.reqs[a.items[r_hi].req].q0 : 0;
         uint32_t q_lo[W], q_hi[W];
 #pragma unroll
         for (int h = 0; h < W / 4; ++h) {
             uint4 x = make_uint4(0, 0, 0, 0), y = x;
             if (v_lo[mt])
-                x = __ldg(reinterpret_cast<const uint4*>(Q + ((int64_t)a.reqs[r_lo].q0 * G + grp) * D + 2 * W * t) + h);
+                x = __ldg(reinterpret_cast<const uint4*>(Q + (q0_lo * G + grp) * D + 2 * W * t) + h);
             if (v_hi[mt])
-                y = __ldg(reinterpret_cast<const uint4*>(Q + ((int64_t)a.reqs[r_hi].q0 * G + grp) * D + 2 * W * t) + h);
+                y = __ldg(reinterpret_cast<const uint4*>(Q + (q0_hi * G + grp) * D + 2 * W * t) + h);
             q_lo[4 * h] = x.x; q_lo[4 * h + 1] = x.y; q_lo[4 * h + 2] = x.z; q_lo[4 * h + 3] = x.w;
             q_hi[4 * h] = y.x; q_hi[4 * h + 1] = y.y; q_hi[4 * h + 2] = y.z; q_hi[4 * h + 3] = y.w;
         }
@@ -78,261 +115,313 @@ __global__ void __launch_bounds__(128) fact_table_kernel(const AttendArgs a, int
     }
     const uint16_t* P = reinterpret_cast<const uint16_t*>(a.cv.poolK) + (int64_t)grp * m * D;
     const int ms = row_floats(m);
-#pragma unroll 2
-    for (int nt = 0; nt < 8; ++nt) {
-        const int jb = j0 + 8 * nt + gl;  // pool entry whose row is this lane's B column
-        const uint4* row = reinterpret_cast<const uint4*>(P + (int64_t)(jb < m ? jb : m - 1) * D + 2 * W * t);
-        uint32_t pw[W];
+    // Four n-tiles at a time, their columns dealt out so that a lane's accumulators are eight consecutive entries of a row
+    // (column n of tile i is entry 8 (n / 2) + 2 i + n % 2): a row gets 128 contiguous bytes per store instruction pair.
+    // 512 requests x 4 groups x 16384 entries (134 MB of T): FIGURES us, with one 8-byte store per tile 39.7.
+#pragma unroll 1
+    for (int jb = j0; jb < min(j0 + 64, m); jb += 32) {
+        uint32_t pw[4][W];
 #pragma unroll
-        for (int h = 0; h < W / 4; ++h) {
-            const uint4 x = __ldg(row + h);
-            pw[4 * h] = x.x; pw[4 * h + 1] = x.y; pw[4 * h + 2] = x.z; pw[4 * h + 3] = x.w;
+        for (int i = 0; i < 4; ++i) {
+            const int j = jb + 8 * (gl >> 1) + 2 * i + (gl & 1);  // pool entry whose row is this lane's B column
+            const uint4* row = reinterpret_cast<const uint4*>(P + (int64_t)min(j, m - 1) * D + 2 * W * t);
+#pragma unroll
+            for (int h = 0; h < W / 4; ++h) {
+                const uint4 x = __ldg(row + h);
+                pw[i][4 * h] = x.x; pw[i][4 * h + 1] = x.y; pw[i][4 * h + 2] = x.z; pw[i][4 * h + 3] = x.w;
+            }
         }
-        const int jc = j0 + 8 * nt + 2 * t;  // columns of the accumulator fragment
+        const int jc = jb + 8 * t;  // this lane's eight entries (rows of T are padded to a multiple of eight)
 #pragma unroll
         for (int mt = 0; mt < MT; ++mt) {
-            float c[4] = {0.f, 0.f, 0.f, 0.f};
+            float c[4][4];
 #pragma unroll
-            for (int ks = 0; ks < KS; ++ks) mma_bf16(c, qa[mt][ks], pw[2 * ks], pw[2 * ks + 1]);
-            float* t_lo = tw + ((int64_t)(r0 + 16 * mt + gl) * G + grp) * ms;
-            float* t_hi = t_lo + (int64_t)8 * G * ms;
-            // the two columns of a lane are one aligned 8-byte store (a column past the last entry lands in the row's padding)
-            if (v_lo[mt] && jc < m) *reinterpret_cast<float2*>(t_lo + jc) = make_float2(c[0], c[1]);
-            if (v_hi[mt] && jc < m) *reinterpret_cast<float2*>(t_hi + jc) = make_float2(c[2], c[3]);
+            for (int i = 0; i < 4; ++i) {
+                c[i][0] = c[i][1] = c[i][2] = c[i][3] = 0.f;
+#pragma unroll
+                for (int ks = 0; ks < KS; ++ks) mma_bf16(c[i], qa[mt][ks], pw[i][2 * ks], pw[i][2 * ks + 1]);
+            }
+            if (jc >= ms) continue;
+            float4* t_lo = reinterpret_cast<float4*>(tw + ((int64_t)(r0 + 16 * mt + gl) * G + grp) * ms + jc);
+            float4* t_hi = t_lo + (int64_t)2 * G * ms;
+            if (v_lo[mt]) {
+                t_lo[0] = make_float4(c[0][0], c[0][1], c[1][0], c[1][1]);
+                t_lo[1] = make_float4(c[2][0], c[2][1], c[3][0], c[3][1]);
+            }
+            if (v_hi[mt]) {
+                t_hi[0] = make_float4(c[0][2], c[0][3], c[1][2], c[1][3]);
+                t_hi[1] = make_float4(c[2][2], c[2][3], c[3][2], c[3][3]);
+            }
         }
     }
 }
 
 // ------------------------------------------------------------------------------------------------ main
-template <bool IDX16>
-__device__ __forceinline__ int load_index(const void* base, int64_t unit)
-{
-    if constexpr (IDX16) return __ldg(reinterpret_cast<const uint16_t*>(base) + unit);
-    else return __ldg(reinterpret_cast<const int32_t*>(base) + unit);
-}
-
-// user part of one position (d_user <= 8 bf16 elements) as raw bits, two elements per word
-__device__ __forceinline__ uint4 load_user(const uint16_t* u, int64_t unit, int d_user)
-{
-    uint4 r = make_uint4(0, 0, 0, 0);
-    switch (d_user) {
-        case 0: break;
-        case 1: r.x = __ldg(u + unit); break;
-        case 2: r.x = __ldg(reinterpret_cast<const uint32_t*>(u + unit * 2)); break;
-        case 4: {
-            const uint2 w = __ldg(reinterpret_cast<const uint2*>(u + unit * 4));
-            r.x = w.x;
-            r.y = w.y;
-            break;
-        }
-        case 8: r = __ldg(reinterpret_cast<const uint4*>(u + unit * 8)); break;
-        default: {
-            uint32_t w[4] = {0, 0, 0, 0};
-#pragma unroll
-            for (int e = 0; e < 8; ++e)
-                if (e < d_user) w[e >> 1] |= (uint32_t)__ldg(u + unit * d_user + e) << (16 * (e & 1));
-            r = make_uint4(w[0], w[1], w[2], w[3]);
-        }
-    }
-    return r;
-}
-// acc + sum_e c[e] * x[e]
-__device__ __forceinline__ float dot_user(const float (&c)[8], const uint4& x, float acc)
-{
-    acc = fmaf(c[0], bf16_bits_to_float(x.x & 0xffffu), acc); acc = fmaf(c[1], __uint_as_float(x.x & 0xffff0000u), acc);
-    acc = fmaf(c[2], bf16_bits_to_float(x.y & 0xffffu), acc); acc = fmaf(c[3], __uint_as_float(x.y & 0xffff0000u), acc);
-    acc = fmaf(c[4], bf16_bits_to_float(x.z & 0xffffu), acc); acc = fmaf(c[5], __uint_as_float(x.z & 0xffff0000u), acc);
-    acc = fmaf(c[6], bf16_bits_to_float(x.w & 0xffffu), acc); acc = fmaf(c[7], __uint_as_float(x.w & 0xffff0000u), acc);
-    return acc;
-}
-// acc[e] += p * x[e]
-__device__ __forceinline__ void axpy_user(float (&acc)[8], float p, const uint4& x)
-{
-    acc[0] = fmaf(p, bf16_bits_to_float(x.x & 0xffffu), acc[0]); acc[1] = fmaf(p, __uint_as_float(x.x & 0xffff0000u), acc[1]);
-    acc[2] = fmaf(p, bf16_bits_to_float(x.y & 0xffffu), acc[2]); acc[3] = fmaf(p, __uint_as_float(x.y & 0xffff0000u), acc[3]);
-    acc[4] = fmaf(p, bf16_bits_to_float(x.z & 0xffffu), acc[4]); acc[5] = fmaf(p, __uint_as_float(x.z & 0xffff0000u), acc[5]);
-    acc[6] = fmaf(p, bf16_bits_to_float(x.w & 0xffffu), acc[6]); acc[7] = fmaf(p, __uint_as_float(x.w & 0xffff0000u), acc[7]);
-}
-
-__device__ __forceinline__ float block_reduce(float v, bool is_max, float* red)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float x = __shfl_xor_sync(0xffffffffu, v, o);
-        v = is_max ? fmaxf(v, x) : v + x;
-    }
-    __syncthreads();  // red may still be read from the previous reduction
-    if (lane == 0) red[warp] = v;
-    __syncthreads();
-    float r = red[0];
-    for (int w = 1; w < kMainThreads / 32; ++w) r = is_max ? fmaxf(r, red[w]) : r + red[w];  // fixed order
-    return r;
-}
-
+constexpr int kCrowd = 3;  // lanes of a warp's first positions that share a pool entry from which on additions are combined
 constexpr int kAux = 16;  // floats per (request, group): [0] row sum l, [1..8] user-part output (not normalised)
 
-// Persistent: CTA c takes (item, group) pairs c, c + gridDim.x, ... of the list ordered longest history first
-// (pair = item * G + group, so neighbours in the list weigh about the same).  While a pair is processed, the T row
-// of the CTA's next pair is already on its way into the other table buffer.
-template <int D, int MODE, bool IDX16>
-__global__ void __launch_bounds__(kMainThreads, 1)
-    fact_main_kernel(const AttendArgs a, float* __restrict__ tw, float* __restrict__ aux, int s_cap)
+// User parts of two neighbouring positions, DU bf16 elements each (DU < 0: `d_user` of them, any number up to 8), as the
+// words they are stored in.
+template <int DU>
+struct UserPair {
+    static constexpr int W = DU < 0 ? 8 : DU == 0 ? 1 : DU;  // 32-bit words
+    uint32_t w[W];
+    __device__ __forceinline__ void load(const uint16_t* u, int64_t unit, int d_user)
+    {
+        if constexpr (DU == 1) w[0] = __ldcs(reinterpret_cast<const uint32_t*>(u + unit));
+        if constexpr (DU == 2) {
+            const uint2 x = __ldcs(reinterpret_cast<const uint2*>(u + unit * 2));
+            w[0] = x.x; w[1] = x.y;
+        }
+        if constexpr (DU == 4 || DU == 8) {
+#pragma unroll
+            for (int h = 0; h < DU / 4; ++h) {
+                const uint4 x = __ldcs(reinterpret_cast<const uint4*>(u + unit * DU) + h);
+                w[4 * h] = x.x; w[4 * h + 1] = x.y; w[4 * h + 2] = x.z; w[4 * h + 3] = x.w;
+            }
+        }
+        if constexpr (DU < 0) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {  // element e of position 0 in word e / 2, of position 1 in word 4 + e / 2
+                const uint32_t x = e < d_user ? __ldg(u + unit * d_user + e) : 0u, y = e < d_user ? __ldg(u + (unit + 1) * d_user + e) : 0u;
+                w[e >> 1] = e & 1 ? w[e >> 1] | x << 16 : x;
+                w[4 + (e >> 1)] = e & 1 ? w[4 + (e >> 1)] | y << 16 : y;
+            }
+        }
+    }
+    __device__ __forceinline__ float at(int pos, int e) const  // element e of position pos
+    {
+        const int i = (DU < 0 ? 8 : DU) * pos + e;
+        return i & 1 ? __uint_as_float(w[i >> 1] & 0xffff0000u) : bf16_bits_to_float(w[i >> 1] & 0xffffu);
+    }
+};
+
+__device__ __forceinline__ int order_bits(float f)  // monotone in f
 {
-    extern __shared__ __align__(16) float fsm[];
-    const int m = a.cv.n_entries, G = a.cv.n_groups, d_user = a.cv.d_user, tid = threadIdx.x;
-    const int n_pairs = a.n_items * G;
-    // fsm[0 .. 2m): two table buffers; a pair's T row, dead after the scores, then its weight histogram
-    float* Sb = fsm + 2 * (size_t)m;     // [s_cap] scores (softmax), half scores (SiLU); at the end the warps' sums
-    float* red = Sb + s_cap;             // [32]
+    const int i = __float_as_int(f);
+    return i ^ ((i >> 31) & 0x7fffffff);
+}
+
+// Persistent: CTA c takes (item, group) pairs c, c + gridDim.x, ... of the list ordered longest history first
+// (pair = item * G + group, so neighbours in the list weigh about the same).  One pass over the history: index, user
+// part, T entry, weight, histogram.  The weights are taken relative to 2^0 and not to the largest score, which would
+// need a pass of its own (fp32 and bf16 have the exponent range for weights of 2^-60 .. 2^60); a pair whose largest score
+// turns out beyond that is worked out again relative to it.  While a pair is processed, the T row of the CTA's next pair
+// is on its way into the other table buffer (one bulk copy), and every thread has two pairs of positions in flight.
+// Bound by HBM: 20 bytes per position at d_u = 4 are 4 us per pair and SM at an even share of the bandwidth.  512 users,
+// 4 groups, 16384 entries, 1000..16384 positions: FIGURES
+template <int D, int MODE, int DU>
+__global__ void __launch_bounds__(kMainThreads, 1)
+    fact_main_kernel(const __grid_constant__ AttendArgs a, float* __restrict__ tw, float* __restrict__ aux,
+                     const PairRec* __restrict__ recs, int n_tab)
+{
+    extern __shared__ __align__(128) float fsm[];
+    constexpr int NU = DU < 0 ? 8 : DU;
+    const int m = a.cv.n_entries, G = a.cv.n_groups, d_user = a.cv.d_user, ms = row_floats(m), tid = threadIdx.x, nt = blockDim.x;
+    const int lane = tid & 31, warp = tid >> 5, n_pairs = a.n_items * G;
+    float* const Ws = fsm + n_tab * (size_t)ms;      // the pair's weight histogram, all zero between pairs
+    float* const red = Ws + ms;                      // [32][9] the warps' sums
+    int* const smax = reinterpret_cast<int*>(red + 32 * 9);  // largest score of the pair, order_bits
+    const uint32_t bar = smem_u32(smax + 4);         // [2] the table buffers' arrivals
     const uint16_t* uK = reinterpret_cast<const uint16_t*>(a.cv.userK);
     const uint16_t* uV = reinterpret_cast<const uint16_t*>(a.cv.userV);
+    const uint16_t* iK = reinterpret_cast<const uint16_t*>(a.cv.idxK);
+    const uint16_t* iV = reinterpret_cast<const uint16_t*>(a.cv.idxV);
     const float sc = a.scale * (MODE == CKV_SOFTMAX ? kLog2e : 0.5f);
-    constexpr int B = 4;  // positions per thread whose loads are in flight together
-    int ix[B];
-    uint4 x[B];
 
-    struct Pair {
-        int req, grp, L, q0;
-        int64_t unit0;
+    auto fetch_table = [&](int row, int k) {  // one thread
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar + 8 * k), "r"(4 * ms) : "memory");
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                         smem_u32(fsm + k * (size_t)ms)),
+                     "l"(tw + (int64_t)row * ms), "r"(4 * ms), "r"(bar + 8 * k)
+                     : "memory");
     };
-    auto get_pair = [&](int p) {
-        Pair r;
-        const Item it = a.items[p / G];
-        const Req rq = a.reqs[it.req];
-        r.req = it.req;
-        r.grp = p - (p / G) * G;
-        r.L = rq.L;
-        r.q0 = rq.q0;
-        r.unit0 = rq.base + (int64_t)r.grp * rq.Lpad;
-        return r;
+    struct Step {
+        uint32_t ik, iv;
+        UserPair<DU> k, v;
     };
-    auto table_row = [&](const Pair& pr) { return tw + ((int64_t)pr.req * G + pr.grp) * row_floats(m); };
-    auto fetch_table = [&](const Pair& pr, float* dstp) {  // all of the row in flight at once
-        const float* row = table_row(pr);
-        if ((m & 3) == 0) {
-            const uint32_t dst = smem_u32(dstp);
-            for (int j = 4 * tid; j < m; j += 4 * kMainThreads)
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 4 * j), "l"(row + j) : "memory");
-        } else {
-            for (int j = tid; j < m; j += kMainThreads) dstp[j] = row[j];
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    };
-    auto load_batch = [&](const void* idx, const uint16_t* u, const Pair& pr, int i0) {
-#pragma unroll
-        for (int b = 0; b < B; ++b) {
-            const int i = i0 + b * kMainThreads;
-            ix[b] = 0;
-            x[b] = make_uint4(0, 0, 0, 0);
-            if (i < pr.L) {
-                ix[b] = load_index<IDX16>(idx, CKV_CLAMP(pr.unit0 + i, a.arena_units, a.err));
-                x[b] = load_user(u, pr.unit0 + i, d_user);
-            }
-        }
+    auto load_step = [&](Step& s, const PairRec& pr, int i) {  // positions i, i + 1 (the arena is padded: i + 1 may be read)
+        if (i >= pr.L) return;
+        const int64_t u = CKV_CLAMP(pr.unit0 + i, a.arena_units, a.err);
+        s.ik = __ldcs(reinterpret_cast<const uint32_t*>(iK + u));
+        s.iv = __ldcs(reinterpret_cast<const uint32_t*>(iV + u));
+        s.k.load(uK, u, d_user);
+        s.v.load(uV, u, d_user);
     };
 
+    if (tid == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar + 8) : "memory");
+        *smax = INT32_MIN;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    for (int j = tid; j < ms; j += nt) Ws[j] = 0.f;
+    __syncthreads();
     int p = blockIdx.x, k = 0;
+    uint32_t phase[2] = {0, 0};
     if (p >= n_pairs) return;
-    Pair cur = get_pair(p);
-    fetch_table(cur, fsm);
-    load_batch(a.cv.idxK, uK, cur, tid);
+    PairRec cur = recs[p], nxt = recs[min(p + (int)gridDim.x, n_pairs - 1)];
+    Step A, B;
+    load_step(A, cur, 2 * tid);
+    load_step(B, cur, 2 * (tid + nt));
+    if (tid == 0) fetch_table(p, 0);
+    bool ok = true;
     for (;;) {
-        float* Ts = fsm + (size_t)k * m;
-        float* Ws = Ts;
-        const int L = cur.L;
-        float qu[8], ou[8];
-        {
-            const uint16_t* q = reinterpret_cast<const uint16_t*>(a.queries) + ((int64_t)cur.q0 * G + cur.grp) * D;
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                qu[e] = e < d_user ? bf16_bits_to_float(__ldg(q + e)) : 0.f;
-                ou[e] = 0.f;
-            }
-        }
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        __syncthreads();  // T of this pair is in place; the other buffer's histogram has been written out
+        const float* Ts = fsm + k * (size_t)ms;
         const int p_next = p + gridDim.x;
         const bool more = p_next < n_pairs;
-        Pair nxt = cur;
-        if (more) {
-            nxt = get_pair(p_next);
-            fetch_table(nxt, fsm + (size_t)(k ^ 1) * m);
-        }
-
-        // scores: Sb[i] = scale * (q_u . K_u[i] + T[I_k[i]])   (softmax: in log2 units; SiLU: half the score)
-        float mx = -CUDART_INF_F, lsum = 0.f;
-        for (int i0 = tid; i0 < L;) {
+        const PairRec behind = recs[min(p_next + (int)gridDim.x, n_pairs - 1)];  // used a pair later
+        float qu[NU > 0 ? NU : 1], ou[NU > 0 ? NU : 1];
+        {
+            const uint32_t w[4] = {cur.q_head.x, cur.q_head.y, cur.q_head.z, cur.q_head.w};
 #pragma unroll
-            for (int b = 0; b < B; ++b) {
-                const int i = i0 + b * kMainThreads;
-                if (i < L) {
-                    const float sv = dot_user(qu, x[b], Ts[CKV_CLAMP(ix[b], m, a.err)]) * sc;
-                    Sb[i] = sv;
-                    mx = fmaxf(mx, sv);
-                }
-            }
-            i0 += B * kMainThreads;
-            if (i0 < L) load_batch(a.cv.idxK, uK, cur, i0);
+            for (int e = 0; e < NU; ++e)
+                qu[e] = (DU >= 0 || e < d_user) ? (e & 1 ? __uint_as_float(w[e >> 1] & 0xffff0000u) : bf16_bits_to_float(w[e >> 1] & 0xffffu)) : 0.f;
         }
-        load_batch(a.cv.idxV, uV, cur, tid);  // the first V-side batch travels during the reduction
-        if constexpr (MODE == CKV_SOFTMAX) mx = block_reduce(mx, true, red);
-        else __syncthreads();
-        // T is dead: the same memory becomes the histogram
-        for (int j = tid; j < m; j += kMainThreads) Ws[j] = 0.f;
-        __syncthreads();
-        // weights: p_i into w[I_v[i]], p_i V_u[i] into the user-part output (every thread reads back its own scores)
-        for (int i0 = tid; i0 < L;) {
+        ok = ok && table_wait(bar + 8 * k, phase[k]);
+        phase[k] ^= 1;
+        if (more && n_tab == 2 && tid == 0) {  // (its buffer was last read before the barrier behind the previous pair's pass)
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            fetch_table(p_next, k ^ 1);
+        }
+        float m_ref = 0.f, mx, lsum;
+        for (bool again = false;; again = true) {
+            mx = -CUDART_INF_F;
+            lsum = 0.f;
 #pragma unroll
-            for (int b = 0; b < B; ++b) {
-                const int i = i0 + b * kMainThreads;
-                if (i < L) {
-                    float pw;
-                    if constexpr (MODE == CKV_SOFTMAX) {
-                        pw = ex2(Sb[i] - mx);
-                        lsum += pw;
-                    } else {
-                        const float h = Sb[i];  // silu(x) = x sigmoid(x) = h (1 + tanh(h)), h = x / 2
-                        pw = fmaf(h, tanh_fast(h), h);
+            for (int e = 0; e < NU; ++e) ou[e] = 0.f;
+            // CROWD: lanes of a warp often hit the same entry (skewed indices), and colliding additions to one address take
+            // turns: they are summed by shuffles first, and one lane adds
+            auto step = [&](const Step& s, int i, auto crowd) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const bool in = i + h < cur.L;
+                    if (!decltype(crowd)::value && !in) break;
+                    float pw = 0.f;
+                    uint32_t j = 0x10000u + lane;
+                    if (in) {
+                        float d = Ts[CKV_CLAMP(h ? s.ik >> 16 : s.ik & 0xffffu, (uint32_t)m, a.err)];
+#pragma unroll
+                        for (int e = 0; e < NU; ++e) d = fmaf(qu[e], s.k.at(h, e), d);
+                        d *= sc;
+                        if constexpr (MODE == CKV_SOFTMAX) {
+                            mx = fmaxf(mx, d);
+                            pw = ex2(d - m_ref);
+                            lsum += pw;
+                        } else {  // silu(x) = x sigmoid(x) = h (1 + tanh(h)), h = x / 2
+                            pw = fmaf(d, tanh_fast(d), d);
+                        }
+                        j = CKV_CLAMP(h ? s.iv >> 16 : s.iv & 0xffffu, (uint32_t)m, a.err);
+#pragma unroll
+                        for (int e = 0; e < NU; ++e) ou[e] = fmaf(pw, s.v.at(h, e), ou[e]);
                     }
-                    atomicAdd(&Ws[CKV_CLAMP(ix[b], m, a.err)], pw);
-                    axpy_user(ou, pw, x[b]);
+                    if constexpr (decltype(crowd)::value) {
+                        uint32_t peers = __match_any_sync(0xffffffffu, j);
+                        uint32_t rank = __popc(peers & ((1u << lane) - 1u));
+                        const bool leads = rank == 0;
+                        peers &= 0xfffffffeu << lane;  // the peers above this lane
+                        while (__any_sync(0xffffffffu, peers != 0)) {  // pairs, pairs of pairs, ...
+                            const int nx = __ffs(peers);
+                            const float t = __shfl_sync(0xffffffffu, pw, (nx - 1) & 31);
+                            if (nx) pw += t;
+                            peers &= __ballot_sync(0xffffffffu, !(rank & 1));
+                            rank >>= 1;
+                        }
+                        if (in && leads) atomicAdd(&Ws[j], pw);
+                    } else {
+                        atomicAdd(&Ws[j], pw);
+                    }
+                }
+            };
+            if (again) {
+                load_step(A, cur, 2 * tid);
+                load_step(B, cur, 2 * (tid + nt));
+            }
+            auto pass = [&](auto crowd) {
+                for (int i0 = 64 * warp; i0 < cur.L; i0 += 4 * nt) {
+                    const int i = i0 + 2 * lane;
+                    step(A, i, crowd);
+                    load_step(A, cur, i + 4 * nt);
+                    step(B, i + 2 * nt, crowd);
+                    load_step(B, cur, i + 6 * nt);
+                }
+            };
+            const uint32_t alike = __match_any_sync(0xffffffffu, 2 * tid < cur.L ? A.iv & 0xffffu : 0x10000u + lane);
+            if (__reduce_max_sync(0xffffffffu, __popc(alike)) >= kCrowd) pass(std::true_type{});
+            else pass(std::false_type{});
+            if (MODE != CKV_SOFTMAX || again) break;
+            const int wmax = __reduce_max_sync(0xffffffffu, order_bits(mx));
+            if (lane == 0) atomicMax(smax, wmax);
+            __syncthreads();
+            const int bits = *smax;
+            const float top = __int_as_float(bits ^ ((bits >> 31) & 0x7fffffff));
+            if (cur.L == 0 || (top <= 60.f && top >= -60.f)) break;
+            m_ref = top;  // far from 2^0: once more, relative to the largest score
+            for (int j = tid; j < ms; j += nt) Ws[j] = 0.f;
+            __syncthreads();
+        }
+        if (more) {  // the next pair's first positions travel during the write-out
+            load_step(A, nxt, 2 * tid);
+            load_step(B, nxt, 2 * (tid + nt));
+        }
+        // row sum and user-part output: warp sums, then one thread per value adds the warps' sums in fixed order.  At every
+        // step of the butterfly a lane gives away half of its values and keeps the other half's sums (9 shuffles for five
+        // values instead of 25).
+        constexpr int NV = NU == 0 ? 1 : NU == 1 ? 2 : NU <= 3 ? 4 : NU <= 7 ? 8 : 16;  // 1 + NU values, padded
+        {
+            float vals[NV];
+#pragma unroll
+            for (int v = 0; v < NV; ++v) vals[v] = v == 0 ? lsum : v <= NU ? ou[v <= NU && NU > 0 ? v - 1 : 0] : 0.f;
+            int id = 0;  // which value this lane ends up with
+#pragma unroll
+            for (int o = 16, n = NV; o > 0; o >>= 1) {
+                if (n > 1) {
+                    n >>= 1;
+                    const bool up = lane & o;
+#pragma unroll
+                    for (int v = 0; v < NV / 2; ++v)
+                        if (v < n) {
+                            const float give = up ? vals[v] : vals[v + n], keep = up ? vals[v + n] : vals[v];
+                            vals[v] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+                        }
+                    id = 2 * id + (up ? 1 : 0);
+                } else {
+                    vals[0] += __shfl_xor_sync(0xffffffffu, vals[0], o);
                 }
             }
-            i0 += B * kMainThreads;
-            if (i0 < L) load_batch(a.cv.idxV, uV, cur, i0);
+            constexpr int spare = 32 / NV - 1;  // the lanes of a value differ in these low bits
+            if ((lane & spare) == 0 && id <= NU) red[warp * 9 + id] = vals[0];
         }
-        if (more) load_batch(a.cv.idxK, uK, nxt, tid);  // the next pair's first K-side batch travels during the write-out
-        // row sum and user-part output: warp sums, then one thread per value adds the warps' sums in fixed order
-        float vals[9] = {lsum, ou[0], ou[1], ou[2], ou[3], ou[4], ou[5], ou[6], ou[7]};
-#pragma unroll
-        for (int q9 = 0; q9 < 9; ++q9)
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) vals[q9] += __shfl_xor_sync(0xffffffffu, vals[q9], o);
-        __syncthreads();  // the histogram is complete; Sb is free
-        if ((tid & 31) == 0) {
-#pragma unroll
-            for (int q9 = 0; q9 < 9; ++q9) Sb[(tid >> 5) * 9 + q9] = vals[q9];
+        __syncthreads();  // the histogram and the warps' sums are complete; T is dead
+        if (more && n_tab == 1 && tid == 0) {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            fetch_table(p_next, 0);
         }
         // w goes back to HBM rounded to bf16 (the precision the output product takes it in), two entries per word,
-        // over the head of the T row, zero-filled up to a multiple of 8 entries
+        // over the head of the T row, zero up to a multiple of 8 entries; what has been read is cleared for the next pair
         {
-            uint32_t* wrow = reinterpret_cast<uint32_t*>(table_row(cur));
-            for (int j2 = tid; 2 * j2 < row_floats(m); j2 += kMainThreads)
-                wrow[j2] = pack_bf16(2 * j2 < m ? Ws[2 * j2] : 0.f, 2 * j2 + 1 < m ? Ws[2 * j2 + 1] : 0.f);
+            uint2* wrow = reinterpret_cast<uint2*>(tw + (int64_t)p * ms);
+            for (int j4 = tid; 4 * j4 < ms; j4 += nt) {
+                float4* w4 = reinterpret_cast<float4*>(Ws) + j4;
+                const float4 x = *w4;
+                wrow[j4] = make_uint2(pack_bf16(x.x, x.y), pack_bf16(x.z, x.w));
+                *w4 = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
         }
-        __syncthreads();
-        if (tid < 9) {
+        if (tid <= NU) {
             float v = 0.f;
-            for (int w = 0; w < kMainThreads / 32; ++w) v += Sb[w * 9 + tid];
-            aux[((int64_t)cur.req * G + cur.grp) * kAux + tid] = v;
+            for (int w = 0; w < nt / 32; ++w) v += red[w * 9 + tid];
+            aux[(int64_t)p * kAux + tid] = v;
         }
+        if (tid == 0) *smax = INT32_MIN;
         if (!more) break;
-        __syncthreads();  // Sb (the warps' sums) is read before the next pair's scores overwrite it
+        __syncthreads();  // the histogram is clear, the warps' sums have been read
         cur = nxt;
+        nxt = behind;
         p = p_next;
-        k ^= 1;
+        if (n_tab == 2) k ^= 1;
     }
+    if (!ok && tid == 0) atomicOr(a.err, ERR_FACT_TABLE);
 }
 
 // ------------------------------------------------------------------------------------------------ out = w P_v
@@ -348,7 +437,7 @@ __device__ __forceinline__ int swz(int r)
 
 template <int D>
 __global__ void __launch_bounds__(kOutWarps * 32, 1)
-    fact_out_kernel(const AttendArgs a, int n_req, const float* __restrict__ tw, const float* __restrict__ aux)
+    fact_out_kernel(const __grid_constant__ AttendArgs a, const float* __restrict__ tw, const float* __restrict__ aux)
 {
     constexpr int NTD = D / 8, ROWB = D * 2, CPR = ROWB / 16, RPI = 32 / CPR, TILE_B = 32 * ROWB;
     extern __shared__ __align__(128) unsigned char osm[];
@@ -357,7 +446,7 @@ __global__ void __launch_bounds__(kOutWarps * 32, 1)
     const int span = ((m + kOutWarps - 1) / kOutWarps + 31) / 32 * 32;
     const int jbeg = warp * span, jend = min(m, jbeg + span);
     const int r_lo = r0 + gl, r_hi = r_lo + 8;
-    const bool v_lo = r_lo < n_req && a.reqs[r_lo].M > 0, v_hi = r_hi < n_req && a.reqs[r_hi].M > 0;
+    const bool v_lo = r_lo < a.n_items, v_hi = r_hi < a.n_items;
     const float* w_lo = tw + ((int64_t)(v_lo ? r_lo : 0) * G + grp) * row_floats(m);
     const float* w_hi = tw + ((int64_t)(v_hi ? r_hi : 0) * G + grp) * row_floats(m);
     const char* pV = reinterpret_cast<const char*>(a.cv.poolV) + (int64_t)grp * m * ROWB;
@@ -450,66 +539,87 @@ __global__ void __launch_bounds__(kOutWarps * 32, 1)
     __syncthreads();
     for (int x = threadIdx.x; x < 16 * D; x += kOutWarps * 32) {
         const int rr = x / D, f = x - rr * D, r = r0 + rr;
-        if (r >= n_req || a.reqs[r].M <= 0) continue;
+        if (r >= a.n_items) continue;
+        const Req rq = a.reqs[a.items[r].req];
         float v = 0.f;
         for (int w = 0; w < kOutWarps; ++w) v += red[((size_t)w * 16 + rr) * D + f];
         const float* ax = aux + ((int64_t)r * G + grp) * kAux;
         if (f < a.cv.d_user) v += ax[1 + f];
         float inv;
         if (a.mode == CKV_SOFTMAX) inv = ax[0] > 0.f ? 1.0f / ax[0] : 0.f;
-        else inv = a.reqs[r].L > 0 ? 1.0f / (float)a.reqs[r].L : 0.f;
+        else inv = rq.L > 0 ? 1.0f / (float)rq.L : 0.f;
         v *= inv;
-        const int64_t oi = ((int64_t)a.reqs[r].q0 * G + grp) * D + f;
+        const int64_t oi = ((int64_t)rq.q0 * G + grp) * D + f;
         if (a.out_dtype == CKV_BF16) reinterpret_cast<__nv_bfloat16*>(a.out)[oi] = __float2bfloat16_rn(v);
         else reinterpret_cast<float*>(a.out)[oi] = v;
     }
 }
 
 template <int D>
-cudaError_t launch_fact(const AttendArgs& a, int n_req, int max_L, int n_sms, float* tw, float* aux, const Launch& l)
+cudaError_t launch_slab(const AttendArgs& a, int n_sms, float* tw, float* aux, const Launch& l)
 {
-    const int m = a.cv.n_entries, G = a.cv.n_groups;
-    const bool i16 = a.cv.idx_bytes == 2, soft = a.mode == CKV_SOFTMAX;
+    const int m = a.cv.n_entries, G = a.cv.n_groups, n_pairs = a.n_items * G;
+    PairRec* recs = reinterpret_cast<PairRec*>(aux + (size_t)n_pairs * kAux);
     cudaError_t e = launch_kernel(l, fact_table_kernel<D>,
-                                  dim3((m + 255) / 256, (n_req + 16 * kTableMT - 1) / (16 * kTableMT), G), 128, 0, 1, a, n_req, tw);
+                                  dim3((m + 255) / 256, (a.n_items + 16 * kTableMT - 1) / (16 * kTableMT), G), 128, 0, 1, a, tw, recs);
     if (e != cudaSuccess) return e;
-    const int s_cap = std::max((max_L + 31) / 32 * 32, 9 * (kMainThreads / 32));  // scores; later the warps' sums
-    const size_t smem_main = (2 * (size_t)m + s_cap + 32) * sizeof(float);
-    const int n_pairs = a.n_items * G;
-    const dim3 grid(n_pairs < n_sms ? n_pairs : n_sms);
-#define CKV_FACT_MAIN(MODE, I16) \
-    launch_kernel(l, fact_main_kernel<D, MODE, I16>, grid, kMainThreads, smem_main, 1, a, tw, aux, s_cap)
-    if (soft) e = i16 ? CKV_FACT_MAIN(CKV_SOFTMAX, true) : CKV_FACT_MAIN(CKV_SOFTMAX, false);
-    else e = i16 ? CKV_FACT_MAIN(CKV_SILU_OVER_L, true) : CKV_FACT_MAIN(CKV_SILU_OVER_L, false);
+    // two table buffers if they fit next to the histogram; two CTAs of half the threads per SM if that leaves room for both
+    const size_t table = (size_t)row_floats(m) * sizeof(float);
+    const int n_tab = 3 * table + kMainExtra <= kMainSmem ? 2 : 1;
+    const size_t smem_main = (n_tab + 1) * table + kMainExtra;
+    const int per_sm = smem_main <= kMainSmem / 2 ? 2 : 1;
+    const dim3 grid((unsigned)std::min(n_pairs, per_sm * n_sms));
+#define CKV_FACT_MAIN(MODE, DU) \
+    launch_kernel(l, fact_main_kernel<D, MODE, DU>, grid, kMainThreads / per_sm, smem_main, 1, a, tw, aux, (const PairRec*)recs, n_tab)
+#define CKV_FACT_DU(MODE)                                                                                   \
+    (a.cv.d_user == 0   ? CKV_FACT_MAIN(MODE, 0) : a.cv.d_user == 1 ? CKV_FACT_MAIN(MODE, 1)                \
+     : a.cv.d_user == 2 ? CKV_FACT_MAIN(MODE, 2) : a.cv.d_user == 4 ? CKV_FACT_MAIN(MODE, 4)                \
+     : a.cv.d_user == 8 ? CKV_FACT_MAIN(MODE, 8) : CKV_FACT_MAIN(MODE, -1))
+    e = a.mode == CKV_SOFTMAX ? CKV_FACT_DU(CKV_SOFTMAX) : CKV_FACT_DU(CKV_SILU_OVER_L);
+#undef CKV_FACT_DU
 #undef CKV_FACT_MAIN
     if (e != cudaSuccess) return e;
     const size_t smem_out = std::max((size_t)kOutWarps * 2 * 32 * D * 2, (size_t)kOutWarps * 16 * D * sizeof(float));
-    return launch_kernel(l, fact_out_kernel<D>, dim3((n_req + 15) / 16, G), kOutWarps * 32, smem_out, 1, a, n_req,
+    return launch_kernel(l, fact_out_kernel<D>, dim3((a.n_items + 15) / 16, G), kOutWarps * 32, smem_out, 1, a,
                          (const float*)tw, (const float*)aux);
 }
 
 }  // namespace
 
-// Largest history (positions) the main kernel can hold next to its two tables, or -1 if the shape is not supported.
-int fact_max_history(int dtype, int head_dim, int d_user, int n_entries)
+// Whether the family takes the shape: one table and one histogram in a CTA's shared memory (so stored indices have 16 bits).
+bool fact_supported(int dtype, int head_dim, int d_user, int n_entries)
 {
-    if (dtype != CKV_BF16 || (head_dim != 32 && head_dim != 64) || d_user > 8) return -1;
-    const int64_t floats = 220 * 1024 / 4 - 32 - 2 * (int64_t)n_entries;  // two table buffers + one score per position
-    if (floats < 9 * (kMainThreads / 32)) return -1;
-    return (int)(floats / 32 * 32);
+    return dtype == CKV_BF16 && (head_dim == 32 || head_dim == 64) && d_user <= 8 &&
+           2 * (size_t)row_floats(std::min(n_entries, 65536)) * sizeof(float) + kMainExtra <= kMainSmem;
 }
 
-int fact_aux_floats() { return kAux; }
-int fact_row_floats(int n_entries) { return row_floats(n_entries); }
-
-// Three launches; a.items holds one unsplit item per request with a query; tw: [n_req][G][fact_row_floats()] floats,
-// aux: [n_req][G][fact_aux_floats()] floats.
-cudaError_t launch_attend_fact(int D, const AttendArgs& a, int n_req, int max_L, int n_sms, float* tw, float* aux,
-                               const Launch& l)
+// Items per slab: the tables take at most kSlabBytes of workspace.  (Slabs whose tables stay in L2 were no faster: the main
+// kernel gained 7 %, the other two lost more to grids too small for the SMs.)
+int fact_slab_items(int n_items, int n_groups, int n_entries)
 {
-    if (a.n_items == 0) return cudaSuccess;
-    return D == 64 ? launch_fact<64>(a, n_req, max_L, n_sms, tw, aux, l)
-                   : launch_fact<32>(a, n_req, max_L, n_sms, tw, aux, l);
+    const int64_t row = (int64_t)row_floats(n_entries) * sizeof(float) * n_groups;
+    const int64_t slabs = std::max<int64_t>(1, (n_items * row + kSlabBytes - 1) / kSlabBytes);
+    return (int)std::min<int64_t>(n_items, ((n_items + slabs - 1) / slabs + 63) / 64 * 64);
+}
+int64_t fact_workspace_floats(int n_items, int n_groups, int n_entries)
+{
+    return (int64_t)fact_slab_items(n_items, n_groups, n_entries) * n_groups *
+           (row_floats(n_entries) + kAux + (int)(sizeof(PairRec) / sizeof(float)));
+}
+
+cudaError_t launch_attend_fact(int D, const AttendArgs& a, int n_sms, float* ws, const Launch& l, int* launches)
+{
+    const int slab = fact_slab_items(a.n_items, a.cv.n_groups, a.cv.n_entries);
+    float* aux = ws + (size_t)slab * a.cv.n_groups * row_floats(a.cv.n_entries);
+    for (int i0 = 0; i0 < a.n_items; i0 += slab) {
+        AttendArgs s = a;
+        s.items = a.items + i0;
+        s.n_items = std::min(slab, a.n_items - i0);
+        const cudaError_t e = D == 64 ? launch_slab<64>(s, n_sms, ws, aux, l) : launch_slab<32>(s, n_sms, ws, aux, l);
+        if (e != cudaSuccess) return e;
+        *launches += 3;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace ckv
