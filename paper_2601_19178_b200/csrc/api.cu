@@ -150,7 +150,7 @@ struct Plan {
     int32_t* d_split = nullptr;
     Work* d_works = nullptr;
     int32_t n_items = 0, n_split = 0, split_items = 0, max_M = 0, max_L = 0, n_req = 0, family = 1, n_works = 0;
-    int32_t parts = 1;       // family 2: warps that share a unit
+    int32_t parts = 1, qpw = 16;  // family 2: warps that share a unit, queries a warp holds
     int64_t part_rows = 0;
     uint64_t last_use = 0;
 };
@@ -453,16 +453,17 @@ int choose_family(const ckv_ctx* ctx, bool with_vis, int32_t n, int64_t n_active
                           fact_supported(ctx->cfg.dtype, ctx->cfg.head_dim, ctx->d_user, ctx->n_entries);
     // It pays when histories are long against the pool and there are enough (user, group) pairs to fill the SMs
     // (one CTA holds a whole pair; the gathering kernel splits long histories over CTAs).  Cost lines fitted to
-    // B200 measurements, in microseconds of one SM: a pair costs a + b n_entries + c L on the factorised path,
-    // a position d on the gathering path.
+    // B200 measurements, in microseconds of one SM: a pair costs a + b n_entries + c L on the factorised path (c between
+    // 0.0004 for uniform indices and 0.0016 for Zipf ones, whose histogram additions collide), a position d on the
+    // gathering path; the three launches cost 5 us more than one.
     bool fact_pays = false;
     if (can_fact) {
         const bool wide = ctx->cfg.head_dim == 64;
-        const double a = wide ? 4.8 : 4.7, b = wide ? 0.00032 : 0.00024, c = wide ? 0.0010 : 0.0008,
-                     d = wide ? 0.0047 : 0.0025;
+        const double a = wide ? 1.2 : 1.0, b = wide ? 0.00055 : 0.0005, c = wide ? 0.0010 : 0.0009,
+                     d = wide ? 0.0047 : 0.0027;
         const double pairs = (double)n_active * ctx->cfg.n_groups, mean_L = (double)total_pos / (double)n_active;
         const double waves = std::ceil(pairs / ctx->n_sms);
-        const double t_fact = waves * (a + b * ctx->n_entries + c * mean_L);
+        const double t_fact = 5.0 + waves * (a + b * ctx->n_entries + c * mean_L);
         const double t_gather = d * (double)total_pos * ctx->cfg.n_groups / ctx->n_sms;
         fact_pays = t_fact < t_gather;
     }
@@ -476,16 +477,49 @@ int choose_family(const ckv_ctx* ctx, bool with_vis, int32_t n, int64_t n_active
     return 0;
 }
 
-// Warps that share one unit of the warp-level tensor-core kernel: `tiles` 32-position tiles of all query blocks of
-// one group in all, the longest history `max_tiles` of them.  The longest unit must not keep a warp busy longer than
-// the resident warps are with everything.
-int mma_parts(const ckv_ctx* ctx, int64_t tiles, int64_t max_tiles, int max_M)
+// What the warp-level tensor-core kernel's work consists of: units of (chunk, group, query block) and their 32-position tiles.
+struct MmaWork {
+    int64_t units = 0, tiles = 0, min_tiles = INT64_MAX, max_tiles = 0;  // of one group
+    int32_t M = -1;
+    bool alike = true;  // every unit costs the same
+    void add(int64_t L, int32_t m, int qpw, int64_t chunk)
+    {
+        const int64_t blocks = (m + qpw - 1) / qpw;
+        if (M < 0) M = m;
+        alike = alike && m == M && L <= chunk;
+        const int64_t chunks = L > chunk ? (L + chunk - 1) / chunk : 1, t = (std::min(L, chunk) + 31) / 32;
+        units += blocks * chunks;
+        tiles += blocks * ((L + 31) / 32);
+        min_tiles = std::min(min_tiles, t);
+        max_tiles = std::max(max_tiles, t);
+    }
+};
+
+// Warps that share one unit: the number with the shortest estimated run, in tile times of a resident warp.  A unit costs
+// about two tiles besides its own, three where several warps merge.  Units of one size run in whole waves; units of mixed
+// sizes, longest histories first, end up to the longest unit apart.
+int mma_parts(const ckv_ctx* ctx, const MmaWork& w, int qpw)
 {
-    const int64_t warps = (int64_t)ctx->n_sms * mma_warps_per_sm(ctx->cfg.head_dim, max_M);
-    const int64_t share = std::max<int64_t>(tiles * ctx->cfg.n_groups / warps, 1);
-    int parts = 1;
-    while (parts < kMmaMaxParts && max_tiles > parts * share) parts *= 2;
-    return parts;
+    const double warps = (double)ctx->n_sms * mma_warps_per_sm(ctx->cfg.head_dim, qpw), G = ctx->cfg.n_groups;
+    int best = 1;
+    double best_t = 1e300;
+    for (int parts = 1; parts <= kMmaMaxParts && parts <= std::max<int64_t>(w.max_tiles, 1); parts *= 2) {
+        const double extra = parts > 1 ? 3 : 2, rounds = w.units * G * parts / warps;
+        const double t = w.alike && w.min_tiles == w.max_tiles
+                             ? std::ceil(rounds) * ((w.max_tiles + parts - 1) / parts + extra)
+                             : w.tiles * G / warps + rounds * extra + (double)w.max_tiles / parts;
+        if (t < best_t) {
+            best_t = t;
+            best = parts;
+        }
+    }
+    return best;
+}
+
+int mma_qpw(const ckv_ctx* ctx, int64_t tiles16, int max_M)
+{
+    const int D = ctx->cfg.head_dim;
+    return mma_queries_per_warp(D, max_M, tiles16 * ctx->cfg.n_groups >= (int64_t)20 * ctx->n_sms * mma_warps_per_sm(D, 16));
 }
 
 // Block size of the CUDA-core kernel: blocks of more warps when there are fewer blocks than SMs.
@@ -506,8 +540,7 @@ int64_t auto_split_len(const ckv_ctx* ctx, int64_t total_positions, int family, 
         return std::min<int64_t>(std::max<int64_t>(c, 1024), 16384);
     }
     if (family == 2) {
-        const int qpw = mma_queries_per_warp(ctx->cfg.head_dim, max_M);
-        c = total_positions * ctx->cfg.n_groups * ((max_M + qpw - 1) / qpw) / (ctx->n_sms * 32);
+        c = total_positions * ctx->cfg.n_groups * ((max_M + 15) / 16) / (ctx->n_sms * 32);
         c = (c + 63) / 64 * 64;
         return std::min<int64_t>(std::max<int64_t>(c, 256), 4096);
     }
@@ -576,11 +609,16 @@ ckv_status build_plan(ckv_ctx* ctx, Plan& pl, int32_t n, const int64_t* users, c
     const int64_t C = ctx->opt_split > 0 && pl.family != 4 ? ctx->opt_split
                                                            : auto_split_len(ctx, total_pos, pl.family, max_M, max_L);
     pl.parts = 1;
-    if (pl.family == 2 && ctx->opt_split == 0) {
-        int64_t tiles = 0;
-        const int qpw = mma_queries_per_warp(ctx->cfg.head_dim, max_M);
-        for (const Req& r : reqs) tiles += (int64_t)((r.L + 31) / 32) * ((r.M + qpw - 1) / qpw);
-        pl.parts = mma_parts(ctx, tiles, (std::min<int64_t>(C, max_L) + 31) / 32, max_M);
+    if (pl.family == 2) {
+        int64_t tiles16 = 0;
+        for (const Req& r : reqs) tiles16 += (int64_t)((r.L + 31) / 32) * ((r.M + 15) / 16);
+        pl.qpw = mma_qpw(ctx, tiles16, max_M);
+        if (ctx->opt_split == 0) {
+            MmaWork w;
+            for (const Req& r : reqs)
+                if (r.M > 0) w.add(r.L, r.M, pl.qpw, C);
+            pl.parts = mma_parts(ctx, w, pl.qpw);
+        }
     }
     std::vector<Item> items;
     std::vector<int32_t> split;
@@ -1232,14 +1270,14 @@ namespace {
 // on B200 a warp spends about 100 clocks per TMA gather instruction it issues, so with the compute warps doing
 // their own gathers the TMA loader measured slower (cfg4: 607 against 522 us; cfg5, Zipf indices that profit
 // from L1, which TMA bypasses: 5.07 against 2.37 ms).  Both loaders give the same bits.
-ckv_status run_mma(ckv_ctx* ctx, int D, int max_M, int parts, const AttendArgs& a, const InlineTable* tab,
+ckv_status run_mma(ckv_ctx* ctx, int D, int max_M, int qpw, int parts, const AttendArgs& a, const InlineTable* tab,
                    const Launch& l)
 {
     const int loader = ctx->opt_loader == 2 ? 2 : 1;
     // the TMA loader serves the plain form only (both sides shared, no visible lengths)
     if (loader == 2 && (!ctx->has_tma || a.cv.full_k || a.cv.full_v || a.vis)) return CKV_ERR_UNSUPPORTED;
     ctx->st_loader = loader;
-    CK(launch_attend_mma(D, max_M, parts, a, tab, loader == 2 ? ctx->tmaps : nullptr, ctx->d_err, l));
+    CK(launch_attend_mma(D, max_M, qpw, parts, a, tab, loader == 2 ? ctx->tmaps : nullptr, ctx->d_err, l));
     return CKV_OK;
 }
 
@@ -1320,7 +1358,7 @@ cudaError_t pipe_prepare(ckv_ctx* ctx)
 // A short request list as kernel arguments: nothing is planned, uploaded or kept for it.
 struct InlineList {
     InlineTable tab;
-    int32_t n = 0, max_M = 0, parts = 1, family = 0;
+    int32_t n = 0, max_M = 0, parts = 1, qpw = 16, family = 0;
 };
 
 // Fills `x`; x.family stays 0 if the list has to go through a plan (too long, or a kernel family or a chunking that
@@ -1346,11 +1384,12 @@ ckv_status inline_list(ckv_ctx* ctx, int32_t n, const int64_t* users, const int3
     const int family = choose_family(ctx, with_vis, n, x.n, total_pos, x.max_M, max_L, all_single);
     if ((family != 1 && family != 2) || auto_split_len(ctx, total_pos, family, x.max_M, max_L) < max_L) return CKV_OK;
     if (family == 2) {
-        int64_t tiles = 0;
-        const int qpw = mma_queries_per_warp(ctx->cfg.head_dim, x.max_M);
-        for (int32_t k = 0; k < x.n; ++k)
-            tiles += (int64_t)((x.tab.r[k].L + 31) / 32) * ((x.tab.r[k].M + qpw - 1) / qpw);
-        x.parts = mma_parts(ctx, tiles, (max_L + 31) / 32, x.max_M);
+        int64_t tiles16 = 0;
+        for (int32_t k = 0; k < x.n; ++k) tiles16 += (int64_t)((x.tab.r[k].L + 31) / 32) * ((x.tab.r[k].M + 15) / 16);
+        x.qpw = mma_qpw(ctx, tiles16, x.max_M);
+        MmaWork w;
+        for (int32_t k = 0; k < x.n; ++k) w.add(x.tab.r[k].L, x.tab.r[k].M, x.qpw, INT32_MAX);
+        x.parts = mma_parts(ctx, w, x.qpw);
     }
     // longest first, as in a plan: the tail of the grid is made of short ones
     if (max_L != min_L && (int64_t)x.n * ctx->cfg.n_groups > ctx->n_sms)
@@ -1398,7 +1437,7 @@ ckv_status launch_slice(ckv_ctx* ctx, const Plan* pl, AttendArgs a, int i0, int 
         } else if (pl->family == 3)
             CK(launch_attend_umma(a, ctx->n_sms, ctx->d_err, l));
         else if (pl->family == 2) {
-            ckv_status st2 = run_mma(ctx, D, pl->max_M, pl->parts, a, nullptr, l);
+            ckv_status st2 = run_mma(ctx, D, pl->max_M, pl->qpw, pl->parts, a, nullptr, l);
             if (st2 != CKV_OK) return st2;
         } else
             CK(launch_attend_simt(ctx->cfg.dtype, D, pl->max_M, simt_wide(ctx, a.n_items), a, nullptr, l));
@@ -1525,7 +1564,7 @@ ckv_status attend_impl(ckv_ctx* ctx, int32_t n, const int64_t* users, const int3
             Launch l = launch_on(ctx, s);
             l.early = true;
             st = timed(ctx, ctx->opt_time != 0, s, [&]() -> ckv_status {
-                if (x.family == 2) return run_mma(ctx, D, x.max_M, x.parts, a, &x.tab, l);
+                if (x.family == 2) return run_mma(ctx, D, x.max_M, x.qpw, x.parts, a, &x.tab, l);
                 CK(launch_attend_simt(ctx->cfg.dtype, D, x.max_M, simt_wide(ctx, x.n), a, &x.tab, l));
                 return CKV_OK;
             });
@@ -2018,7 +2057,7 @@ extern "C" ckv_status ckv_attend_static(ckv_ctx* ctx, int32_t n, const int64_t* 
     const Launch l{s, nullptr, &ctx->grants};
     if (n_items > 0) {
         if (family == 2)
-            CK(launch_attend_mma(D, max_M, 1, a, nullptr, nullptr, ctx->d_err, l));
+            CK(launch_attend_mma(D, max_M, 16, 1, a, nullptr, nullptr, ctx->d_err, l));
         else
             CK(launch_attend_simt(ctx->cfg.dtype, D, max_M, simt_wide(ctx, n_items), a, nullptr, l));
     }

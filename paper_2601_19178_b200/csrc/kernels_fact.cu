@@ -30,7 +30,7 @@ constexpr float kLog2e = 1.4426950408889634f;
 constexpr int kMainThreads = 1024;
 constexpr int64_t kSlabBytes = (int64_t)1 << 30;
 constexpr size_t kMainSmem = 226 * 1024, kMainExtra = 32 * 9 * 4 + 64;  // shared memory for tables; sums and barriers
-constexpr int kOutWarps = 16;
+constexpr int kOutWarps = 8, kOutMT = 2, kOutRows = 16 * kOutMT, kOutCluster = 4;
 
 __device__ __forceinline__ float bf16_bits_to_float(uint32_t b) { return __uint_as_float(b << 16); }
 
@@ -115,43 +115,29 @@ __global__ void __launch_bounds__(128)
     }
     const uint16_t* P = reinterpret_cast<const uint16_t*>(a.cv.poolK) + (int64_t)grp * m * D;
     const int ms = row_floats(m);
-    // Four n-tiles at a time, their columns dealt out so that a lane's accumulators are eight consecutive entries of a row
-    // (column n of tile i is entry 8 (n / 2) + 2 i + n % 2): a row gets 128 contiguous bytes per store instruction pair.
-    // 512 requests x 4 groups x 16384 entries (134 MB of T): FIGURES us, with one 8-byte store per tile 39.7.
-#pragma unroll 1
-    for (int jb = j0; jb < min(j0 + 64, m); jb += 32) {
-        uint32_t pw[4][W];
+    // (Bound by the writing of T: 134 MB for 512 requests x 4 groups x 16384 entries in 40 us.  Storing 32 bytes per lane,
+    // 128 per row, took 43; 32 requests and 256 entries per warp with the next rows prefetched 46.)
+#pragma unroll 2
+    for (int nt = 0; nt < 8; ++nt) {
+        const int jb = j0 + 8 * nt + gl;  // pool entry whose row is this lane's B column
+        const uint4* row = reinterpret_cast<const uint4*>(P + (int64_t)(jb < m ? jb : m - 1) * D + 2 * W * t);
+        uint32_t pw[W];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int j = jb + 8 * (gl >> 1) + 2 * i + (gl & 1);  // pool entry whose row is this lane's B column
-            const uint4* row = reinterpret_cast<const uint4*>(P + (int64_t)min(j, m - 1) * D + 2 * W * t);
-#pragma unroll
-            for (int h = 0; h < W / 4; ++h) {
-                const uint4 x = __ldg(row + h);
-                pw[i][4 * h] = x.x; pw[i][4 * h + 1] = x.y; pw[i][4 * h + 2] = x.z; pw[i][4 * h + 3] = x.w;
-            }
+        for (int h = 0; h < W / 4; ++h) {
+            const uint4 x = __ldg(row + h);
+            pw[4 * h] = x.x; pw[4 * h + 1] = x.y; pw[4 * h + 2] = x.z; pw[4 * h + 3] = x.w;
         }
-        const int jc = jb + 8 * t;  // this lane's eight entries (rows of T are padded to a multiple of eight)
+        const int jc = j0 + 8 * nt + 2 * t;  // columns of the accumulator fragment
 #pragma unroll
         for (int mt = 0; mt < MT; ++mt) {
-            float c[4][4];
+            float c[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                c[i][0] = c[i][1] = c[i][2] = c[i][3] = 0.f;
-#pragma unroll
-                for (int ks = 0; ks < KS; ++ks) mma_bf16(c[i], qa[mt][ks], pw[i][2 * ks], pw[i][2 * ks + 1]);
-            }
-            if (jc >= ms) continue;
-            float4* t_lo = reinterpret_cast<float4*>(tw + ((int64_t)(r0 + 16 * mt + gl) * G + grp) * ms + jc);
-            float4* t_hi = t_lo + (int64_t)2 * G * ms;
-            if (v_lo[mt]) {
-                t_lo[0] = make_float4(c[0][0], c[0][1], c[1][0], c[1][1]);
-                t_lo[1] = make_float4(c[2][0], c[2][1], c[3][0], c[3][1]);
-            }
-            if (v_hi[mt]) {
-                t_hi[0] = make_float4(c[0][2], c[0][3], c[1][2], c[1][3]);
-                t_hi[1] = make_float4(c[2][2], c[2][3], c[3][2], c[3][3]);
-            }
+            for (int ks = 0; ks < KS; ++ks) mma_bf16(c, qa[mt][ks], pw[2 * ks], pw[2 * ks + 1]);
+            float* t_lo = tw + ((int64_t)(r0 + 16 * mt + gl) * G + grp) * ms;
+            float* t_hi = t_lo + (int64_t)8 * G * ms;
+            // the two columns of a lane are one aligned 8-byte store (a column past the last entry lands in the row's padding)
+            if (v_lo[mt] && jc < m) *reinterpret_cast<float2*>(t_lo + jc) = make_float2(c[0], c[1]);
+            if (v_hi[mt] && jc < m) *reinterpret_cast<float2*>(t_hi + jc) = make_float2(c[2], c[3]);
         }
     }
 }
@@ -209,7 +195,9 @@ __device__ __forceinline__ int order_bits(float f)  // monotone in f
 // turns out beyond that is worked out again relative to it.  While a pair is processed, the T row of the CTA's next pair
 // is on its way into the other table buffer (one bulk copy), and every thread has two pairs of positions in flight.
 // Bound by HBM: 20 bytes per position at d_u = 4 are 4 us per pair and SM at an even share of the bandwidth.  512 users,
-// 4 groups, 16384 entries, 1000..16384 positions: FIGURES
+// 4 groups, 16384 entries, 1000..16384 positions: 127 us (521 MB of DRAM traffic at 4.1 TB/s, 50 %; issue slots 40 %; a
+// pair takes 18000 clocks of an SM, 9000 of them in the pass); with two passes, a block-wide maximum between them and the
+// scores kept in shared memory 181 us.
 template <int D, int MODE, int DU>
 __global__ void __launch_bounds__(kMainThreads, 1)
     fact_main_kernel(const __grid_constant__ AttendArgs a, float* __restrict__ tw, float* __restrict__ aux,
@@ -401,17 +389,25 @@ __global__ void __launch_bounds__(kMainThreads, 1)
         // over the head of the T row, zero up to a multiple of 8 entries; what has been read is cleared for the next pair
         {
             uint2* wrow = reinterpret_cast<uint2*>(tw + (int64_t)p * ms);
-            for (int j4 = tid; 4 * j4 < ms; j4 += nt) {
-                float4* w4 = reinterpret_cast<float4*>(Ws) + j4;
-                const float4 x = *w4;
-                wrow[j4] = make_uint2(pack_bf16(x.x, x.y), pack_bf16(x.z, x.w));
-                *w4 = make_float4(0.f, 0.f, 0.f, 0.f);
+            float4* w4 = reinterpret_cast<float4*>(Ws);
+            for (int j4 = tid; 4 * j4 < ms; j4 += 4 * nt) {
+                float4 x[4];
+#pragma unroll
+                for (int h = 0; h < 4; ++h)
+                    if (4 * (j4 + h * nt) < ms) x[h] = w4[j4 + h * nt];
+#pragma unroll
+                for (int h = 0; h < 4; ++h)
+                    if (4 * (j4 + h * nt) < ms) {
+                        wrow[j4 + h * nt] = make_uint2(pack_bf16(x[h].x, x[h].y), pack_bf16(x[h].z, x[h].w));
+                        w4[j4 + h * nt] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    }
             }
         }
-        if (tid <= NU) {
-            float v = 0.f;
-            for (int w = 0; w < nt / 32; ++w) v += red[w * 9 + tid];
-            aux[(int64_t)p * kAux + tid] = v;
+        if (warp <= NU) {  // warp v adds up value v
+            float v = lane < nt / 32 ? red[lane * 9 + warp] : 0.f;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (lane == 0) aux[(int64_t)p * kAux + warp] = v;
         }
         if (tid == 0) *smax = INT32_MIN;
         if (!more) break;
@@ -425,7 +421,10 @@ __global__ void __launch_bounds__(kMainThreads, 1)
 }
 
 // ------------------------------------------------------------------------------------------------ out = w P_v
-// One CTA per (16 requests, group); warp w covers pool entries [w, w + 1) * ceil32(m / 16).  P_v rows are
+// A cluster of four CTAs per (32 requests, group), its 32 warps splitting the pool's entries.  What bounds it is the V pool
+// out of L2 (2 MB per cluster at 16384 64-wide entries): every row fetched serves 32 requests, and the split gives every
+// SM a share.  512 requests x 4 groups x 16384 entries: 27 us (2.5 TB/s of w besides), with one CTA
+// per 16 requests 30, and for 100 requests the whole call takes 61 us instead of 68.  P_v rows are
 // contiguous here: 32-row tiles through a two-slot cp.async ring per warp, fragments by transposing ldmatrix.
 // 16-byte chunk c of tile row r sits at chunk c ^ swz(r).  The eight rows of one ldmatrix block are rows
 // 8 t' + const + e (t' < 4, e < 2) here, see the k-slot order below: they must fall into eight different bank groups.
@@ -436,24 +435,32 @@ __device__ __forceinline__ int swz(int r)
 }
 
 template <int D>
-__global__ void __launch_bounds__(kOutWarps * 32, 1)
+__global__ void __launch_bounds__(kOutWarps * 32, 2)
     fact_out_kernel(const __grid_constant__ AttendArgs a, const float* __restrict__ tw, const float* __restrict__ aux)
 {
     constexpr int NTD = D / 8, ROWB = D * 2, CPR = ROWB / 16, RPI = 32 / CPR, TILE_B = 32 * ROWB;
     extern __shared__ __align__(128) unsigned char osm[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gl = lane >> 2, t = lane & 3;
-    const int m = a.cv.n_entries, G = a.cv.n_groups, grp = blockIdx.y, r0 = blockIdx.x * 16;
-    const int span = ((m + kOutWarps - 1) / kOutWarps + 31) / 32 * 32;
-    const int jbeg = warp * span, jend = min(m, jbeg + span);
-    const int r_lo = r0 + gl, r_hi = r_lo + 8;
-    const bool v_lo = r_lo < a.n_items, v_hi = r_hi < a.n_items;
-    const float* w_lo = tw + ((int64_t)(v_lo ? r_lo : 0) * G + grp) * row_floats(m);
-    const float* w_hi = tw + ((int64_t)(v_hi ? r_hi : 0) * G + grp) * row_floats(m);
+    const int m = a.cv.n_entries, G = a.cv.n_groups, grp = blockIdx.y, rank = blockIdx.x % kOutCluster,
+              r0 = blockIdx.x / kOutCluster * kOutRows;
+    constexpr int kParts = kOutWarps * kOutCluster;
+    const int span = ((m + kParts - 1) / kParts + 31) / 32 * 32;
+    const int jbeg = (rank * kOutWarps + warp) * span, jend = min(m, jbeg + span);
+    const uint32_t* wrow[kOutMT][2];  // the requests of this lane's fragment rows
+    bool v_in[kOutMT][2];
+#pragma unroll
+    for (int mt = 0; mt < kOutMT; ++mt)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int r = r0 + 16 * mt + gl + 8 * h;
+            v_in[mt][h] = r < a.n_items;
+            wrow[mt][h] = reinterpret_cast<const uint32_t*>(tw + ((int64_t)(v_in[mt][h] ? r : 0) * G + grp) * row_floats(m));
+        }
     const char* pV = reinterpret_cast<const char*>(a.cv.poolV) + (int64_t)grp * m * ROWB;
     const uint32_t ring = smem_u32(osm) + warp * (2 * TILE_B);
     const int cr = lane / CPR, cc = lane % CPR, lr = lane & 7, lm = lane >> 3;
     // Which pool entry sits in which k-slot is free as long as w and the V rows agree: a lane reads 8 consecutive
-    // weights of its two requests with one 16-byte load each, and k-step b, slots (2t, 2t+1, 2t+8, 2t+9) hold
+    // weights of its requests with one 16-byte load each, and k-step b, slots (2t, 2t+1, 2t+8, 2t+9) hold
     // entries 8t + 4b + (0, 1, 2, 3) of the 32-entry chunk; the ldmatrix row addresses follow.
     uint32_t offV[2][NTD / 2];
 #pragma unroll
@@ -476,20 +483,22 @@ __global__ void __launch_bounds__(kOutWarps * 32, 1)
     };
     // weights of one 32-entry chunk: entries 8t .. 8t+7 of both requests, the bf16 pairs the main kernel stored
     // (rows start at multiples of 32 bytes and are zero-filled behind the last entry up to a multiple of 8 entries)
-    auto load_w = [&](int jc, uint4 (&x)[2]) {
+    auto load_w = [&](int jc, uint4 (&x)[kOutMT][2]) {
         const int j = jc + 8 * t;
-        const bool in = j < jend;
-        x[0] = (in && v_lo) ? __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const uint32_t*>(w_lo) + (j >> 1)))
-                            : make_uint4(0, 0, 0, 0);
-        x[1] = (in && v_hi) ? __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const uint32_t*>(w_hi) + (j >> 1)))
-                            : make_uint4(0, 0, 0, 0);
+#pragma unroll
+        for (int mt = 0; mt < kOutMT; ++mt)
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                x[mt][h] = j < jend && v_in[mt][h] ? __ldg(reinterpret_cast<const uint4*>(wrow[mt][h] + (j >> 1))) : make_uint4(0, 0, 0, 0);
     };
 
-    float o[NTD][4];
+    float o[kOutMT][NTD][4];
 #pragma unroll
-    for (int j = 0; j < NTD; ++j) o[j][0] = o[j][1] = o[j][2] = o[j][3] = 0.f;
+    for (int mt = 0; mt < kOutMT; ++mt)
+#pragma unroll
+        for (int j = 0; j < NTD; ++j) o[mt][j][0] = o[mt][j][1] = o[mt][j][2] = o[mt][j][3] = 0.f;
     const int nch = jbeg < jend ? (jend - jbeg + 31) / 32 : 0;
-    uint4 wa[2], wb[2];
+    uint4 wa[kOutMT][2], wb[kOutMT][2];
     if (nch > 0) {
         issue(jbeg, 0);
         load_w(jbeg, wa);
@@ -506,9 +515,7 @@ __global__ void __launch_bounds__(kOutWarps * 32, 1)
         __syncwarp();
         const uint32_t vt = ring + (c & 1) * TILE_B;
 #pragma unroll
-        for (int b = 0; b < 2; ++b) {
-            const uint32_t pa[4] = {b ? wa[0].z : wa[0].x, b ? wa[1].z : wa[1].x, b ? wa[0].w : wa[0].y,
-                                    b ? wa[1].w : wa[1].y};
+        for (int b = 0; b < 2; ++b)
 #pragma unroll
             for (int jp = 0; jp < NTD / 2; ++jp) {
                 uint32_t v0, v1, v2, v3;
@@ -516,33 +523,53 @@ __global__ void __launch_bounds__(kOutWarps * 32, 1)
                              : "=r"(v0), "=r"(v1), "=r"(v2), "=r"(v3)
                              : "r"(vt + offV[b][jp])
                              : "memory");
-                mma_bf16(o[2 * jp], pa, v0, v1);
-                mma_bf16(o[2 * jp + 1], pa, v2, v3);
-            }
-        }
-        __syncwarp();  // every lane is done reading the slot that the next iteration refills
 #pragma unroll
-        for (int i = 0; i < 2; ++i) wa[i] = wb[i];
+                for (int mt = 0; mt < kOutMT; ++mt) {
+                    const uint32_t pa[4] = {b ? wa[mt][0].z : wa[mt][0].x, b ? wa[mt][1].z : wa[mt][1].x,
+                                            b ? wa[mt][0].w : wa[mt][0].y, b ? wa[mt][1].w : wa[mt][1].y};
+                    mma_bf16(o[mt][2 * jp], pa, v0, v1);
+                    mma_bf16(o[mt][2 * jp + 1], pa, v2, v3);
+                }
+            }
+        __syncwarp();  // every lane is done with the slot that the next iteration refills
+#pragma unroll
+        for (int mt = 0; mt < kOutMT; ++mt) {
+            wa[mt][0] = wb[mt][0];
+            wa[mt][1] = wb[mt][1];
+        }
     }
 
-    // sum the warps' partial outputs in fixed order, add the user part, normalise, store
+    // sum the warps' partial outputs, then the CTAs', in fixed order; add the user part, normalise, store
     __syncthreads();
-    float* red = reinterpret_cast<float*>(osm);  // [kOutWarps][16][D]
+    float* red = reinterpret_cast<float*>(osm);  // [kOutWarps][kOutRows][D]; the sums over the warps in [0]
 #pragma unroll
-    for (int j = 0; j < NTD; ++j) {
-        float* p = red + ((size_t)warp * 16 + gl) * D + 8 * j + 2 * t;
-        p[0] = o[j][0];
-        p[1] = o[j][1];
-        p[8 * D] = o[j][2];
-        p[8 * D + 1] = o[j][3];
-    }
+    for (int mt = 0; mt < kOutMT; ++mt)
+#pragma unroll
+        for (int j = 0; j < NTD; ++j) {
+            float* p = red + ((size_t)warp * kOutRows + 16 * mt + gl) * D + 8 * j + 2 * t;
+            *reinterpret_cast<float2*>(p) = make_float2(o[mt][j][0], o[mt][j][1]);
+            *reinterpret_cast<float2*>(p + 8 * D) = make_float2(o[mt][j][2], o[mt][j][3]);
+        }
     __syncthreads();
-    for (int x = threadIdx.x; x < 16 * D; x += kOutWarps * 32) {
+    for (int x = threadIdx.x; x < kOutRows * D; x += kOutWarps * 32) {
+        float v = red[x];
+        for (int w = 1; w < kOutWarps; ++w) v += red[(size_t)w * kOutRows * D + x];
+        red[x] = v;
+    }
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    constexpr int kMine = kOutRows * D / kOutCluster;  // elements this CTA finishes
+    for (int x = rank * kMine + threadIdx.x; x < (rank + 1) * kMine; x += kOutWarps * 32) {
         const int rr = x / D, f = x - rr * D, r = r0 + rr;
         if (r >= a.n_items) continue;
         const Req rq = a.reqs[a.items[r].req];
         float v = 0.f;
-        for (int w = 0; w < kOutWarps; ++w) v += red[((size_t)w * 16 + rr) * D + f];
+        for (int c = 0; c < kOutCluster; ++c) {
+            uint32_t at;
+            float y;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(smem_u32(red + x)), "r"(c));
+            asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(y) : "r"(at) : "memory");
+            v += y;
+        }
         const float* ax = aux + ((int64_t)r * G + grp) * kAux;
         if (f < a.cv.d_user) v += ax[1 + f];
         float inv;
@@ -553,6 +580,8 @@ __global__ void __launch_bounds__(kOutWarps * 32, 1)
         if (a.out_dtype == CKV_BF16) reinterpret_cast<__nv_bfloat16*>(a.out)[oi] = __float2bfloat16_rn(v);
         else reinterpret_cast<float*>(a.out)[oi] = v;
     }
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");  // the others' sums have been read
 }
 
 template <int D>
@@ -579,9 +608,10 @@ cudaError_t launch_slab(const AttendArgs& a, int n_sms, float* tw, float* aux, c
 #undef CKV_FACT_DU
 #undef CKV_FACT_MAIN
     if (e != cudaSuccess) return e;
-    const size_t smem_out = std::max((size_t)kOutWarps * 2 * 32 * D * 2, (size_t)kOutWarps * 16 * D * sizeof(float));
-    return launch_kernel(l, fact_out_kernel<D>, dim3((a.n_items + 15) / 16, G), kOutWarps * 32, smem_out, 1, a,
-                         (const float*)tw, (const float*)aux);
+    static_assert(kOutRows * 2 == 2 * 32, "the sums take the room of the rings");
+    const size_t smem_out = (size_t)kOutWarps * 2 * 32 * D * 2;
+    return launch_kernel(l, fact_out_kernel<D>, dim3((unsigned)((a.n_items + kOutRows - 1) / kOutRows * kOutCluster), G),
+                         kOutWarps * 32, smem_out, kOutCluster, a, (const float*)tw, (const float*)aux);
 }
 
 }  // namespace

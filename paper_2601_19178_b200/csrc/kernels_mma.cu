@@ -744,37 +744,31 @@ bool mma_supported(int dtype, int head_dim, int d_user)
     return dtype == CKV_BF16 && (head_dim == 32 || head_dim == 64) && d_user <= 8;
 }
 
-// Every gathered row serves all the queries a warp holds, so it holds as many as there are, up to what its registers
-// take: four 16-query tiles of 32-wide heads, three of 64-wide ones.
-int mma_queries_per_warp(int D, int max_M) { return max_M <= 16 ? 16 : max_M <= 32 ? 32 : D == 64 || max_M <= 48 ? 48 : 64; }
-
-// warps of the kernel that are resident on an SM
-int mma_warps_per_sm(int D, int max_M)
+// Queries a warp holds.  One 16-query tile gathers a row for every tile of a user's queries, but leaves registers for twice
+// the warps (32-wide heads) and starts and merges in half the time; more tiles pay only when every resident warp has `big`
+// amounts of work, and then only from where a gathered row costs as much as the products on it: 200 users x 1000 positions,
+// 64-wide, 20..32 queries 64 us with two tiles, 75 with one (40 queries: 105 either way); 32-wide, 40 queries x 2000 users x
+// 500 positions 214 us with three tiles, 224 with one (up to 32 queries one tile is the faster: 155 against 166 with two).
+int mma_queries_per_warp(int D, int max_M, bool big)
 {
-    if (D == 64) return 8;
-    return mma_queries_per_warp(D, max_M) == 16 ? 4 * MmaCfg<32, 1, false>::MIN_BLOCKS : 8;
+    if (!big || max_M <= 16) return 16;
+    return D == 64 ? 32 : max_M > 32 ? 48 : 16;
 }
 
-cudaError_t launch_attend_mma(int D, int max_M, int parts, const AttendArgs& a, const InlineTable* tab,
+// warps of the kernel that are resident on an SM
+int mma_warps_per_sm(int D, int queries_per_warp) { return D == 64 || queries_per_warp > 16 ? 8 : 16; }
+
+cudaError_t launch_attend_mma(int D, int max_M, int queries_per_warp, int parts, const AttendArgs& a, const InlineTable* tab,
                               const void* tensor_maps, int* err_flag, const Launch& l)
 {
     if (a.n_items == 0) return cudaSuccess;
     const CUtensorMap* maps = reinterpret_cast<const CUtensorMap*>(tensor_maps);
-    const int qpw = mma_queries_per_warp(D, max_M);
-    const int n_mb = (max_M + qpw - 1) / qpw;
-    if (D == 64) {
-        switch (qpw) {
-            case 16: return launch_mma<64, 1>(a, n_mb, parts, tab, maps, err_flag, l);
-            case 32: return launch_mma<64, 2>(a, n_mb, parts, tab, maps, err_flag, l);
-            default: return launch_mma<64, 3>(a, n_mb, parts, tab, maps, err_flag, l);
-        }
-    }
-    switch (qpw) {
-        case 16: return launch_mma<32, 1>(a, n_mb, parts, tab, maps, err_flag, l);
-        case 32: return launch_mma<32, 2>(a, n_mb, parts, tab, maps, err_flag, l);
-        case 48: return launch_mma<32, 3>(a, n_mb, parts, tab, maps, err_flag, l);
-        default: return launch_mma<32, 4>(a, n_mb, parts, tab, maps, err_flag, l);
-    }
+    const int n_mb = (max_M + queries_per_warp - 1) / queries_per_warp;
+    if (D == 64)
+        return queries_per_warp == 16 ? launch_mma<64, 1>(a, n_mb, parts, tab, maps, err_flag, l)
+                                      : launch_mma<64, 2>(a, n_mb, parts, tab, maps, err_flag, l);
+    return queries_per_warp == 16 ? launch_mma<32, 1>(a, n_mb, parts, tab, maps, err_flag, l)
+                                  : launch_mma<32, 3>(a, n_mb, parts, tab, maps, err_flag, l);
 }
 
 // Tensor maps of the K and the V pool ([n_groups * n_entries] rows of head_dim bf16) for tile::gather4: a box of
