@@ -149,7 +149,7 @@ struct Plan {
     Item* d_items = nullptr;
     int32_t* d_split = nullptr;
     Work* d_works = nullptr;
-    int32_t n_items = 0, n_split = 0, split_items = 0, max_M = 0, max_L = 0, n_req = 0, family = 1, n_works = 0;
+    int32_t n_items = 0, n_split = 0, split_items = 0, max_M = 0, n_req = 0, family = 1, n_works = 0;
     int32_t parts = 1, qpw = 16;  // family 2: warps that share a unit, queries a warp holds
     int64_t part_rows = 0;
     uint64_t last_use = 0;
@@ -435,48 +435,6 @@ void arena_give(ckv_ctx* ctx, int64_t base, int64_t units)
     }
 }
 
-int64_t units_of_len(const ckv_ctx* ctx, int64_t L) { return (int64_t)ctx->cfg.n_groups * ((L + 31) / 32 * 32); }
-
-// The kernel family of a request list (0: the forced one cannot take it).
-int choose_family(const ckv_ctx* ctx, bool with_vis, int32_t n, int64_t n_active, int64_t total_pos, int32_t max_M,
-                  int32_t max_L, bool all_single)
-{
-    const bool can_mma = ctx->has_mma;
-    // visible lengths and sides that are not shared are served by every gathering kernel, not by the pool-side
-    // factorisation
-    const bool plain = !with_vis && !ctx->full_k && !ctx->full_v;
-    const bool can_umma = ctx->has_umma;
-    // tcgen05 from three 16-query blocks on, else the warp-level tensor-core kernel (faster than the CUDA-core
-    // kernel from a single query on); the CUDA-core kernel serves what neither supports
-    // One query per user: the pool-side factorisation trades the row gathers for two tables per (user, group).
-    const bool can_fact = plain && all_single && n_active > 0 &&
-                          fact_supported(ctx->cfg.dtype, ctx->cfg.head_dim, ctx->d_user, ctx->n_entries);
-    // It pays when histories are long against the pool and there are enough (user, group) pairs to fill the SMs
-    // (one CTA holds a whole pair; the gathering kernel splits long histories over CTAs).  Cost lines fitted to
-    // B200 measurements, in microseconds of one SM: a pair costs a + b n_entries + c L on the factorised path (c between
-    // 0.0004 for uniform indices and 0.0016 for Zipf ones, whose histogram additions collide), a position d on the
-    // gathering path; the three launches cost 5 us more than one.
-    bool fact_pays = false;
-    if (can_fact) {
-        const bool wide = ctx->cfg.head_dim == 64;
-        const double a = wide ? 1.2 : 1.0, b = wide ? 0.00055 : 0.0005, c = wide ? 0.0010 : 0.0009,
-                     d = wide ? 0.0047 : 0.0027;
-        const double pairs = (double)n_active * ctx->cfg.n_groups, mean_L = (double)total_pos / (double)n_active;
-        const double waves = std::ceil(pairs / ctx->n_sms);
-        const double t_fact = 5.0 + waves * (a + b * ctx->n_entries + c * mean_L);
-        const double t_gather = d * (double)total_pos * ctx->cfg.n_groups / ctx->n_sms;
-        fact_pays = t_fact < t_gather;
-    }
-    switch (ctx->opt_kernel) {
-        case 0: return can_umma && max_M >= 48 ? 3 : fact_pays ? 4 : can_mma ? 2 : 1;
-        case 1: return 1;
-        case 2: return can_mma ? 2 : 0;
-        case 3: return can_umma ? 3 : 0;
-        case 4: return can_fact ? 4 : 0;
-    }
-    return 0;
-}
-
 // What the warp-level tensor-core kernel's work consists of: units of (chunk, group, query block) and their 32-position tiles.
 struct MmaWork {
     int64_t units = 0, tiles = 0, min_tiles = INT64_MAX, max_tiles = 0;  // of one group
@@ -495,24 +453,30 @@ struct MmaWork {
     }
 };
 
-// Warps that share one unit: the number with the shortest estimated run, in tile times of a resident warp.  A unit costs
-// about two tiles besides its own, three where several warps merge.  Units of one size run in whole waves; units of mixed
-// sizes, longest histories first, end up to the longest unit apart.
-int mma_parts(const ckv_ctx* ctx, const MmaWork& w, int qpw)
+// Warps that share one unit: the number with the shortest estimated run, in tile times of a resident warp.  A unit costs two
+// tiles besides its own.  Every further warp per unit shortens the units but adds blocks, and a round of blocks costs
+// about five tiles, six across a cluster (head_dim 64 with clusters of eight: nine).  Units of one size run in whole rounds;
+// mixed ones, longest histories first, leave SMs idle for about half of the longest.  (Fitted to sweeps of 1..32 warps over
+// 1..300 users of 200..16384 positions; within 15 % of most, and the number it picks within 6 % of the best.)
+int mma_parts(const ckv_ctx* ctx, const MmaWork& w, int qpw, double* tile_times)
 {
-    const double warps = (double)ctx->n_sms * mma_warps_per_sm(ctx->cfg.head_dim, qpw), G = ctx->cfg.n_groups;
+    const int D = ctx->cfg.head_dim;
+    const double warps = (double)ctx->n_sms * mma_warps_per_sm(D, qpw), G = ctx->cfg.n_groups;
     int best = 1;
     double best_t = 1e300;
     for (int parts = 1; parts <= kMmaMaxParts && parts <= std::max<int64_t>(w.max_tiles, 1); parts *= 2) {
-        const double extra = parts > 1 ? 3 : 2, rounds = w.units * G * parts / warps;
+        const double rounds = w.units * G * parts / warps;
+        const double extra = parts == 1 ? 2 : D != 64 || parts <= 4 ? 5 : parts <= 16 ? 6 : 9;
         const double t = w.alike && w.min_tiles == w.max_tiles
-                             ? std::ceil(rounds) * ((w.max_tiles + parts - 1) / parts + extra)
-                             : w.tiles * G / warps + rounds * extra + (double)w.max_tiles / parts;
+                             ? std::ceil(rounds) * ((w.max_tiles + parts - 1) / parts + 2) + rounds * (extra - 2) +
+                                   (parts > 16 ? 2 : parts > 1 ? 1 : 0)
+                             : w.tiles * G / warps + rounds * extra + 0.5 * (double)w.max_tiles / parts;
         if (t < best_t) {
             best_t = t;
             best = parts;
         }
     }
+    *tile_times = best_t;
     return best;
 }
 
@@ -522,29 +486,151 @@ int mma_qpw(const ckv_ctx* ctx, int64_t tiles16, int max_M)
     return mma_queries_per_warp(D, max_M, tiles16 * ctx->cfg.n_groups >= (int64_t)20 * ctx->n_sms * mma_warps_per_sm(D, 16));
 }
 
+// Queries per warp and warps per unit; `each(add)` calls add(L, M) for every request with a query.  Holding more queries
+// per warp saves gathers and lengthens a tile (measured 1.45 times for 32 queries at head_dim 64, 1.3 for 48 at 32), but
+// leaves fewer units to spread: lists of few long histories are better off with 16.
+template <typename F>
+void mma_shape(const ckv_ctx* ctx, int64_t tiles16, int max_M, int64_t chunk, F&& each, int& qpw, int& parts)
+{
+    auto estimate = [&](int q, int& p) {
+        MmaWork w;
+        each([&](int32_t L, int32_t M) { w.add(L, M, q, chunk); });
+        double t;
+        p = mma_parts(ctx, w, q, &t);
+        return t;
+    };
+    qpw = mma_qpw(ctx, tiles16, max_M);
+    const double t = estimate(qpw, parts);
+    int p16;
+    if (qpw > 16 && estimate(16, p16) < (qpw == 32 ? 1.45 : 1.3) * t) {
+        qpw = 16;
+        parts = p16;
+    }
+}
+
+// A request list as the dispatch sees it.
+struct ListShape {
+    int32_t n = 0, max_M = 0, max_L = 0;
+    int64_t active = 0, positions = 0;  // requests with a query, their history lengths in all
+    int64_t blocks128 = 0, tiles64 = 0; // blocks of 128 queries, and (block, 64 positions) tiles
+    bool single = true;                 // one query each
+    MmaWork mma;                        // for 16 queries per warp
+    void add(int32_t L, int32_t M)
+    {
+        ++n;
+        max_M = std::max(max_M, M);
+        if (M <= 0) return;
+        ++active;
+        positions += L;
+        max_L = std::max(max_L, L);
+        single = single && M == 1;
+        const int64_t b = (M + 127) / 128;
+        blocks128 += b;
+        tiles64 += b * ((L + 63) / 64);
+        mma.add(L, M, 16, INT32_MAX);
+    }
+};
+
+// Chunk length of the tcgen05 kernel: the one with the shortest estimated run, in microseconds.  Three persistent workers
+// per SM walk a (chunk, group, 128 queries) unit alone; measured, a worker takes 1 us per 64 positions when it has the SM
+// to itself and 1.4 next to two others, 1.5 per unit, the launch 6, and merging chunks 6 and more.  Units of one size
+// run in whole rounds; mixed ones are dealt out longest first, and only the longest of them bounds the run from below.
+int64_t umma_chunk(const ckv_ctx* ctx, const ListShape& s, double* time = nullptr)
+{
+    const double workers = 3.0 * ctx->n_sms, G = ctx->cfg.n_groups;
+    const bool alike = s.mma.alike && s.mma.min_tiles == s.mma.max_tiles;
+    int64_t best = 16384;
+    double best_t = 1e300;
+    for (int64_t n = (s.max_L + 16383) / 16384, last = 0; n <= 512 && last != 256; n += (n + 15) / 16) {
+        const int64_t c = std::max<int64_t>((s.max_L / std::max<int64_t>(n, 1) + 63) / 64 * 64, 256);
+        if (c == last) continue;
+        last = c;
+        const bool split = c < s.max_L;
+        const double cut = alike ? (double)((s.max_L + c - 1) / c) * s.blocks128 : s.tiles64 * 64.0 / c + (split ? 0.5 : 0) * s.blocks128;
+        const double units = G * std::max<double>(cut, s.blocks128), tiles = c / 64;
+        const double tile_us = 0.8 + 0.2 * std::min(3.0, std::max(1.0, units / ctx->n_sms));
+        const double longest = std::min<double>(tiles, (s.max_L + 63) / 64) * tile_us + 1.5;
+        const double t = 6 + (split ? 6 + 0.003 * units : 0) +
+                         (alike ? std::ceil(units / workers) * longest
+                                : std::max(longest, (s.tiles64 * G * tile_us + 1.5 * units) / workers));
+        if (t < best_t) {
+            best_t = t;
+            best = c;
+        }
+    }
+    if (time) *time = best_t;
+    return std::min<int64_t>(best, 16384);
+}
+
+// The kernel family of a request list (0: the forced one cannot take it).
+int choose_family(const ckv_ctx* ctx, bool with_vis, const ListShape& s)
+{
+    const int64_t n_active = s.active, total_pos = s.positions;
+    const int32_t max_M = s.max_M;
+    const bool can_mma = ctx->has_mma;
+    // visible lengths and sides that are not shared are served by every gathering kernel, not by the pool-side
+    // factorisation
+    const bool plain = !with_vis && !ctx->full_k && !ctx->full_v;
+    const bool can_umma = ctx->has_umma;
+    // tcgen05 from three 16-query blocks on, else the warp-level tensor-core kernel (faster than the CUDA-core
+    // kernel from a single query on); the CUDA-core kernel serves what neither supports.  Up to six blocks the
+    // warp-level kernel also takes lists too small to fill the tcgen05 kernel's workers (measured: 1.2 us per tile time of
+    // its resident warps and 4 us besides).
+    bool few = false;
+    if (can_umma && can_mma && !with_vis && max_M >= 48 && max_M <= 96 && n_active > 0) {
+        double tile_times, t_umma;
+        mma_parts(ctx, s.mma, 16, &tile_times);
+        umma_chunk(ctx, s, &t_umma);
+        few = 4 + 1.2 * tile_times < t_umma;
+    }
+    // One query per user: the pool-side factorisation trades the row gathers for two tables per (user, group).
+    const bool can_fact = plain && s.single && n_active > 0 &&
+                          fact_supported(ctx->cfg.dtype, ctx->cfg.head_dim, ctx->d_user, ctx->n_entries);
+    // It pays when histories are long against the pool and there are enough (user, group) pairs to fill the SMs
+    // (one CTA holds a whole pair; the gathering kernel splits long histories over CTAs).  Cost lines fitted to
+    // B200 measurements, in microseconds of one SM: a pair costs a + b n_entries + c L on the factorised path (c between
+    // 0.0004 for uniform indices and 0.0016 for Zipf ones, whose histogram additions collide), a position d on the
+    // gathering path; the three launches cost 5 us more than one.
+    bool fact_pays = false;
+    if (can_fact) {
+        const bool wide = ctx->cfg.head_dim == 64;
+        const double a = wide ? 1.2 : 1.0, b = wide ? 0.00055 : 0.0005, c = wide ? 0.0010 : 0.0009,
+                     d = wide ? 0.0047 : 0.0027;
+        const double pairs = (double)n_active * ctx->cfg.n_groups, mean_L = (double)total_pos / (double)n_active;
+        const double waves = std::ceil(pairs / ctx->n_sms);
+        const double t_fact = 5.0 + waves * (a + b * ctx->n_entries + c * mean_L);
+        const double t_gather = d * (double)total_pos * ctx->cfg.n_groups / ctx->n_sms;
+        fact_pays = t_fact < t_gather;
+    }
+    switch (ctx->opt_kernel) {
+        case 0: return can_umma && max_M >= 48 && !few ? 3 : fact_pays ? 4 : can_mma ? 2 : 1;
+        case 1: return 1;
+        case 2: return can_mma ? 2 : 0;
+        case 3: return can_umma ? 3 : 0;
+        case 4: return can_fact ? 4 : 0;
+    }
+    return 0;
+}
+
 // Block size of the CUDA-core kernel: blocks of more warps when there are fewer blocks than SMs.
 bool simt_wide(const ckv_ctx* ctx, int64_t n_items) { return n_items * ctx->cfg.n_groups <= ctx->n_sms; }
 
-int64_t auto_split_len(const ckv_ctx* ctx, int64_t total_positions, int family, int max_M, int max_L)
+int64_t auto_split_len(const ckv_ctx* ctx, const ListShape& s, int family)
 {
     if (family == 4) return INT32_MAX;  // one CTA holds a whole history
+    if (family == 3) return umma_chunk(ctx, s);
     // up to 64 Ki positions the warps that share a unit of the warp-level tensor-core kernel are enough (64 tiles
     // for each of them), up to 4096 the 16 warps of a CUDA-core block are
-    if ((family == 2 && max_L <= 65536) || (family == 1 && max_L <= 4096)) return INT32_MAX;
+    if ((family == 2 && s.max_L <= 65536) || (family == 1 && s.max_L <= 4096)) return INT32_MAX;
     // Enough (chunk, group) blocks to fill the SMs several times over, but chunks long
     // enough that the merge of partial results stays a small fraction of the work.
     int64_t c;
-    if (family == 3) {  // persistent CTAs share (chunk, group, 128 queries) units round-robin: a few units per SM
-        c = total_positions * ctx->cfg.n_groups * ((max_M + 127) / 128) / (ctx->n_sms * 4);
-        c = (c + 127) / 128 * 128;
-        return std::min<int64_t>(std::max<int64_t>(c, 1024), 16384);
-    }
     if (family == 2) {
-        c = total_positions * ctx->cfg.n_groups * ((max_M + 15) / 16) / (ctx->n_sms * 32);
+        c = s.positions * ctx->cfg.n_groups * ((s.max_M + 15) / 16) / (ctx->n_sms * 32);
         c = (c + 63) / 64 * 64;
         return std::min<int64_t>(std::max<int64_t>(c, 256), 4096);
     }
-    c = total_positions * ctx->cfg.n_groups / (ctx->n_sms * 16);
+    c = s.positions * ctx->cfg.n_groups / (ctx->n_sms * 16);
     c = (c + 63) / 64 * 64;
     return std::min<int64_t>(std::max<int64_t>(c, 256), 2048);
 }
@@ -578,9 +664,7 @@ ckv_status build_plan(ckv_ctx* ctx, Plan& pl, int32_t n, const int64_t* users, c
                       int n_ranges, const int32_t* r_user, cudaStream_t s)
 {
     std::vector<Req> reqs((size_t)n);
-    int64_t total_pos = 0, n_active = 0;
-    int32_t max_M = 0, max_L = 0;
-    bool all_single = true;
+    ListShape shape;
     for (int32_t k = 0; k < n; ++k) {
         if (k + 12 < n) ctx->users.prefetch(users[k + 12]);
         const UserEntry* f = ctx->users.find(users[k]);
@@ -593,32 +677,21 @@ ckv_status build_plan(ckv_ctx* ctx, Plan& pl, int32_t n, const int64_t* users, c
         r.M = q_off[k + 1] - q_off[k];
         r.part0 = -1;
         r.n_chunks = 1;
-        if (r.M > 0) {
-            total_pos += r.L;
-            max_L = std::max(max_L, r.L);
-            n_active++;
-            all_single = all_single && r.M == 1;
-        }
-        max_M = std::max(max_M, r.M);
+        shape.add(r.L, r.M);
     }
-    pl.max_M = max_M;
-    pl.max_L = max_L;
+    const int32_t max_M = pl.max_M = shape.max_M;
     pl.n_req = n;
-    pl.family = choose_family(ctx, with_vis, n, n_active, total_pos, max_M, max_L, all_single);
+    pl.family = choose_family(ctx, with_vis, shape);
     if (pl.family == 0) return CKV_ERR_UNSUPPORTED;
-    const int64_t C = ctx->opt_split > 0 && pl.family != 4 ? ctx->opt_split
-                                                           : auto_split_len(ctx, total_pos, pl.family, max_M, max_L);
+    const int64_t C = ctx->opt_split > 0 && pl.family != 4 ? ctx->opt_split : auto_split_len(ctx, shape, pl.family);
     pl.parts = 1;
     if (pl.family == 2) {
-        int64_t tiles16 = 0;
-        for (const Req& r : reqs) tiles16 += (int64_t)((r.L + 31) / 32) * ((r.M + 15) / 16);
-        pl.qpw = mma_qpw(ctx, tiles16, max_M);
-        if (ctx->opt_split == 0) {
-            MmaWork w;
-            for (const Req& r : reqs)
-                if (r.M > 0) w.add(r.L, r.M, pl.qpw, C);
-            pl.parts = mma_parts(ctx, w, pl.qpw);
-        }
+        if (ctx->opt_split > 0) pl.qpw = mma_qpw(ctx, shape.mma.tiles, max_M);
+        else
+            mma_shape(ctx, shape.mma.tiles, max_M, C, [&](auto&& add) {
+                for (const Req& r : reqs)
+                    if (r.M > 0) add(r.L, r.M);
+            }, pl.qpw, pl.parts);
     }
     std::vector<Item> items;
     std::vector<int32_t> split;
@@ -1366,33 +1439,26 @@ struct InlineList {
 ckv_status inline_list(ckv_ctx* ctx, int32_t n, const int64_t* users, const int32_t* q_off, bool with_vis, InlineList& x)
 {
     if (n > kInlineReqs || ctx->opt_split > 0 || ctx->opt_kernel > 2 || ctx->opt_loader == 2) return CKV_OK;
-    int64_t total_pos = 0;
-    int32_t max_L = 0, min_L = INT32_MAX;
-    bool all_single = true;
+    ListShape shape;
+    int32_t min_L = INT32_MAX;
     for (int32_t k = 0; k < n; ++k) {
         const UserEntry* f = ctx->users.find(users[k]);
         if (!f) return CKV_ERR_UNKNOWN_USER;
         const int32_t M = q_off[k + 1] - q_off[k];
+        shape.add(f->L, M);
         if (M <= 0) continue;
         x.tab.r[x.n++] = InlineReq{(uint32_t)(f->base >> 5), f->L, q_off[k], M};
-        total_pos += f->L;
-        max_L = std::max(max_L, f->L);
         min_L = std::min(min_L, f->L);
-        x.max_M = std::max(x.max_M, M);
-        all_single = all_single && M == 1;
     }
-    const int family = choose_family(ctx, with_vis, n, x.n, total_pos, x.max_M, max_L, all_single);
-    if ((family != 1 && family != 2) || auto_split_len(ctx, total_pos, family, x.max_M, max_L) < max_L) return CKV_OK;
-    if (family == 2) {
-        int64_t tiles16 = 0;
-        for (int32_t k = 0; k < x.n; ++k) tiles16 += (int64_t)((x.tab.r[k].L + 31) / 32) * ((x.tab.r[k].M + 15) / 16);
-        x.qpw = mma_qpw(ctx, tiles16, x.max_M);
-        MmaWork w;
-        for (int32_t k = 0; k < x.n; ++k) w.add(x.tab.r[k].L, x.tab.r[k].M, x.qpw, INT32_MAX);
-        x.parts = mma_parts(ctx, w, x.qpw);
-    }
+    x.max_M = shape.max_M;
+    const int family = choose_family(ctx, with_vis, shape);
+    if ((family != 1 && family != 2) || auto_split_len(ctx, shape, family) < shape.max_L) return CKV_OK;
+    if (family == 2)
+        mma_shape(ctx, shape.mma.tiles, x.max_M, INT32_MAX, [&](auto&& add) {
+            for (int32_t k = 0; k < x.n; ++k) add(x.tab.r[k].L, x.tab.r[k].M);
+        }, x.qpw, x.parts);
     // longest first, as in a plan: the tail of the grid is made of short ones
-    if (max_L != min_L && (int64_t)x.n * ctx->cfg.n_groups > ctx->n_sms)
+    if (shape.max_L != min_L && (int64_t)x.n * ctx->cfg.n_groups > ctx->n_sms)
         std::sort(x.tab.r, x.tab.r + x.n, [](const InlineReq& a, const InlineReq& b) { return a.L > b.L; });
     x.family = family;
     return CKV_OK;
@@ -1445,7 +1511,7 @@ ckv_status launch_slice(ckv_ctx* ctx, const Plan* pl, AttendArgs a, int i0, int 
     }
     if (time_it) CK(cudaEventRecord(ctx->ev[1], s));
     if (s1 > s0) {
-        CK(launch_combine(D, a, pl->d_split + s0, s1 - s0, l));
+        CK(launch_combine(D, pl->max_M, a, pl->d_split + s0, s1 - s0, l));
         ctx->st_launches++;
     }
     if (time_it) CK(cudaEventRecord(ctx->ev[2], s));
@@ -1980,8 +2046,7 @@ extern "C" ckv_status ckv_attend_static(ckv_ctx* ctx, int32_t n, const int64_t* 
     // the plan, in fixed-size host arrays; nothing is enqueued before the request is known to fit
     StaticRow rows[kStaticMaxReqs];
     const int D = ctx->cfg.head_dim, G = ctx->cfg.n_groups;
-    int64_t total_pos = 0;
-    int32_t max_M = 0;
+    ListShape shape;
     for (int32_t k = 0; k < n; ++k) {
         const UserEntry* f = ctx->users.find(users[k]);
         if (!f) return CKV_ERR_UNKNOWN_USER;
@@ -1993,15 +2058,16 @@ extern "C" ckv_status ckv_attend_static(ckv_ctx* ctx, int32_t n, const int64_t* 
         r.M = q_off[k + 1] - q_off[k];
         r.part0 = -1;
         r.n_chunks = 1;
-        if (r.M > 0) total_pos += r.L;
-        max_M = std::max(max_M, r.M);
+        shape.add(r.L, r.M);
     }
+    const int32_t max_M = shape.max_M;
+    shape.max_L = INT32_MAX;  // (chunks here, not warps sharing a unit: the chunks' limits are part of this call's contract)
     int family;
     if (ctx->opt_kernel == 0) family = ctx->has_mma ? 2 : 1;
     else if (ctx->opt_kernel == 1) family = 1;
     else if (ctx->opt_kernel == 2 && ctx->has_mma) family = 2;
     else return CKV_ERR_UNSUPPORTED;
-    const int64_t C = ctx->opt_split > 0 ? ctx->opt_split : auto_split_len(ctx, total_pos, family, max_M, INT32_MAX);
+    const int64_t C = ctx->opt_split > 0 ? ctx->opt_split : auto_split_len(ctx, shape, family);
     const int64_t row_floats = (int64_t)G * (D + 2);
     const int64_t cap_rows = (int64_t)((kStaticBytes - kOffPartials) / sizeof(float)) / row_floats;
     int32_t n_items = 0, n_split = 0;
@@ -2061,6 +2127,6 @@ extern "C" ckv_status ckv_attend_static(ckv_ctx* ctx, int32_t n, const int64_t* 
         else
             CK(launch_attend_simt(ctx->cfg.dtype, D, max_M, simt_wide(ctx, n_items), a, nullptr, l));
     }
-    if (n_split > 0) CK(launch_combine(D, a, (const int32_t*)(base + kOffSplit), n_split, l));
+    if (n_split > 0) CK(launch_combine(D, max_M, a, (const int32_t*)(base + kOffSplit), n_split, l));
     return CKV_OK;
 }

@@ -82,7 +82,7 @@ struct AttendArgs {
     const int32_t* vis;    // null, or per query row the number of leading history positions it attends [Q]
     const int32_t* vmax;   // tcgen05 family with visible lengths: largest limit per work record
     void* out;             // [Q][G][D]
-    float* partials;       // [part rows][G][D + 2]  (m, l, acc[D])
+    float* partials;       // [part rows][G][D] accumulators, behind them [part rows][G] (m, l)
     int32_t out_dtype;     // ckv_dtype
     int32_t mode;          // ckv_mode
     float scale;
@@ -92,6 +92,18 @@ struct AttendArgs {
     int64_t part_rows;     // rows of `partials`
     int* err;              // device error word (the context's)
 };
+
+#ifdef __CUDACC__
+// Where the partial result of (part row, group) stands: rows on 16-byte boundaries, so that they move four floats at a time.
+__device__ __forceinline__ float* part_acc(const AttendArgs& a, int D, int64_t row, int g)
+{
+    return a.partials + (row * a.cv.n_groups + g) * D;
+}
+__device__ __forceinline__ float2* part_ml(const AttendArgs& a, int D, int64_t row, int g)
+{
+    return reinterpret_cast<float2*>(a.partials + a.part_rows * a.cv.n_groups * D) + row * a.cv.n_groups + g;
+}
+#endif
 
 // How a launcher launches: stream, the access-policy window over the pool (null: none) as a launch attribute, and the
 // context's record of which kernels have been allowed how much dynamic shared memory (the permission belongs to the
@@ -196,7 +208,7 @@ cudaError_t launch_check_indices(int idx_bytes, int n_entries, const void* idxK,
 cudaError_t launch_attend_simt(int dtype, int D, int max_M, bool wide, const AttendArgs& a, const InlineTable* tab,
                                const Launch& l);
 // Merges the partial results of split requests into `out`.
-cudaError_t launch_combine(int D, const AttendArgs& a, const int32_t* split_reqs, int n_split, const Launch& l);
+cudaError_t launch_combine(int D, int max_M, const AttendArgs& a, const int32_t* split_reqs, int n_split, const Launch& l);
 
 // ---- kernels_mma.cu : warp-level tensor-core family (bf16, head_dim 32 or 64, d_user <= 8)
 bool mma_supported(int dtype, int head_dim, int d_user);  // d_user of the shared side(s)

@@ -684,14 +684,12 @@ __global__ void __launch_bounds__(128, MmaCfg<D, MT, TMA>::MIN_BLOCKS)
                             make_float2(x, y);
                 }
             } else {
-                float* pr = a.partials + (CKV_CLAMP((int64_t)(it.part_row + r), a.part_rows, err_flag) * G + grp) * (D + 2);
-                if (t == 0) {
-                    pr[0] = m_run[mt][h];
-                    pr[1] = l;
-                }
+                const int64_t row = CKV_CLAMP((int64_t)(it.part_row + r), a.part_rows, err_flag);
+                if (t == 0) *part_ml(a, D, row, grp) = make_float2(m_run[mt][h], l);
+                float* pr = part_acc(a, D, row, grp);
 #pragma unroll
                 for (int j = 0; j < NTD; ++j)
-                    *reinterpret_cast<float2*>(pr + 2 + 8 * j + 2 * t) =
+                    *reinterpret_cast<float2*>(pr + 8 * j + 2 * t) =
                         make_float2(o[mt][j][2 * h], o[mt][j][2 * h + 1]);
             }
         }

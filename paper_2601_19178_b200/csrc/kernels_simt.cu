@@ -16,6 +16,8 @@
 #include <cuda_bf16.h>
 #include <math_constants.h>
 
+#include <algorithm>
+
 #include "ckv_internal.h"
 #include "ptx_helpers.cuh"
 
@@ -351,49 +353,70 @@ __global__ void __launch_bounds__(kWarps * 32, QB == 1 && kWarps == 4 ? 5 : 1)
                 else res = rq.L > 0 ? o / (float)rq.L : 0.f;
                 store_out(a.out, (CKV_CLAMP((int64_t)(rq.q0 + qb + r), a.q_rows, a.err) * G + g) * D + c, res, a.out_dtype);
             } else {
-                float* pr = a.partials + (CKV_CLAMP((int64_t)(it.part_row + qb + r), a.part_rows, a.err) * G + g) * (D + 2);
-                if (c == 0) {
-                    pr[0] = mt;
-                    pr[1] = lt;
-                }
-                pr[2 + c] = o;
+                const int64_t row = CKV_CLAMP((int64_t)(it.part_row + qb + r), a.part_rows, a.err);
+                if (c == 0) *part_ml(a, D, row, g) = make_float2(mt, lt);
+                part_acc(a, D, row, g)[c] = o;
             }
         }
         __syncthreads();
     }
 }
 
-// One block per (split request, group): out = merge over the request's chunks.
+// out = merge over a split request's chunks.  D / 4 lanes share a (query row, group), four columns each, so that a warp
+// has several rows in work, and eight chunks are requested before the first is used: the kernel is a chain of loads
+// (split list, request, partial results) and little else.  FIGURES
 template <int MODE>
-__global__ void __launch_bounds__(128) combine_kernel(const AttendArgs a, const int32_t* split_reqs,
-                                                      int D)
+__global__ void __launch_bounds__(256) combine_kernel(const AttendArgs a, const int32_t* split_reqs, int D)
 {
     const Req rq = a.reqs[split_reqs[blockIdx.x]];
-    const int g = blockIdx.y, G = a.cv.n_groups;
-    const int W = D + 2;
-    for (int t = threadIdx.x; t < rq.M * D; t += blockDim.x) {
-        const int r = t / D, c = t - r * D;
-        float res;
-        if constexpr (MODE == CKV_SOFTMAX) {
-            float mt = -CUDART_INF_F;
-            for (int k = 0; k < rq.n_chunks; ++k)
-                mt = fmaxf(mt, a.partials[(CKV_CLAMP((int64_t)(rq.part0 + k * rq.M + r), a.part_rows, a.err) * G + g) * W]);
-            const float ms = mt == -CUDART_INF_F ? 0.f : mt;
-            float lt = 0.f, o = 0.f;
-            for (int k = 0; k < rq.n_chunks; ++k) {
-                const float* pr = a.partials + ((int64_t)(rq.part0 + k * rq.M + r) * G + g) * W;
-                const float ck = exp2f(pr[0] - ms);
-                lt += pr[1] * ck;
-                o += pr[2 + c] * ck;
+    const int G = a.cv.n_groups, lanes = D / 4, col = threadIdx.x % lanes * 4, per_block = 256 / lanes;
+    const int64_t n = (int64_t)rq.M * G;
+    for (int64_t x = (int64_t)blockIdx.y * per_block + threadIdx.x / lanes; x < n; x += (int64_t)gridDim.y * per_block) {
+        const int r = (int)(x / G), g = (int)(x % G);
+        const int64_t row0 = CKV_CLAMP((int64_t)(rq.part0 + r), a.part_rows, a.err);
+        const float* acc = part_acc(a, D, row0, g) + col;
+        const float2* ml = part_ml(a, D, row0, g);
+        float m = -CUDART_INF_F, l = 0.f;
+        float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int k0 = 0; k0 < rq.n_chunks; k0 += 8) {
+            float2 p[8];
+            float4 v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                p[i] = make_float2(-CUDART_INF_F, 0.f);
+                v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (k0 + i < rq.n_chunks) {
+                    if constexpr (MODE == CKV_SOFTMAX) p[i] = ml[(k0 + i) * n];
+                    v[i] = *reinterpret_cast<const float4*>(acc + (k0 + i) * n * D);
+                }
             }
-            res = lt > 0.f ? o / lt : 0.f;
-        } else {
-            float o = 0.f;
-            for (int k = 0; k < rq.n_chunks; ++k)
-                o += a.partials[((int64_t)(rq.part0 + k * rq.M + r) * G + g) * W + 2 + c];
-            res = rq.L > 0 ? o / (float)rq.L : 0.f;
+            if constexpr (MODE == CKV_SOFTMAX) {
+                float mn = m;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) mn = fmaxf(mn, p[i].x);
+                const float ref = mn == -CUDART_INF_F ? 0.f : mn, c = exp2f(m - ref);
+                m = mn;
+                l *= c;
+                o = make_float4(o.x * c, o.y * c, o.z * c, o.w * c);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const float w = exp2f(p[i].x - ref);
+                    l = fmaf(p[i].y, w, l);
+                    o = make_float4(fmaf(v[i].x, w, o.x), fmaf(v[i].y, w, o.y), fmaf(v[i].z, w, o.z), fmaf(v[i].w, w, o.w));
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) o = make_float4(o.x + v[i].x, o.y + v[i].y, o.z + v[i].z, o.w + v[i].w);
+            }
         }
-        store_out(a.out, (CKV_CLAMP((int64_t)(rq.q0 + r), a.q_rows, a.err) * G + g) * D + c, res, a.out_dtype);
+        float inv;
+        if constexpr (MODE == CKV_SOFTMAX) inv = l > 0.f ? 1.0f / l : 0.f;
+        else inv = rq.L > 0 ? 1.0f / (float)rq.L : 0.f;
+        const int64_t out = (CKV_CLAMP((int64_t)(rq.q0 + r), a.q_rows, a.err) * G + g) * D + col;
+        store_out(a.out, out, o.x * inv, a.out_dtype);
+        store_out(a.out, out + 1, o.y * inv, a.out_dtype);
+        store_out(a.out, out + 2, o.z * inv, a.out_dtype);
+        store_out(a.out, out + 3, o.w * inv, a.out_dtype);
     }
 }
 
@@ -429,12 +452,13 @@ cudaError_t launch_attend_simt(int dtype, int D, int max_M, bool wide, const Att
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_combine(int D, const AttendArgs& a, const int32_t* split_reqs, int n_split, const Launch& l)
+cudaError_t launch_combine(int D, int max_M, const AttendArgs& a, const int32_t* split_reqs, int n_split, const Launch& l)
 {
     if (n_split == 0) return cudaSuccess;
-    const dim3 grid(n_split, a.cv.n_groups);
-    return a.mode == CKV_SOFTMAX ? launch_kernel(l, combine_kernel<CKV_SOFTMAX>, grid, 128, 0, 1, a, split_reqs, D)
-                                 : launch_kernel(l, combine_kernel<CKV_SILU_OVER_L>, grid, 128, 0, 1, a, split_reqs, D);
+    const int64_t rows = 256 / (D / 4), blocks = ((int64_t)max_M * a.cv.n_groups + rows - 1) / rows;
+    const dim3 grid(n_split, (unsigned)std::min<int64_t>(blocks, 4096));
+    return a.mode == CKV_SOFTMAX ? launch_kernel(l, combine_kernel<CKV_SOFTMAX>, grid, 256, 0, 1, a, split_reqs, D)
+                                 : launch_kernel(l, combine_kernel<CKV_SILU_OVER_L>, grid, 256, 0, 1, a, split_reqs, D);
 }
 
 }  // namespace ckv

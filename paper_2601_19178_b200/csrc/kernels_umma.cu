@@ -638,9 +638,10 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma_kernel(const AttendAr
             if (u.n_tiles == 0) {  // empty history, or a chunk behind every row's visible length: zero rows
                 if (r < u.wk.M) {
                     if (u.wk.part_row >= 0) {  // (only with visible lengths) an empty partial result
-                        float* pr = a.partials + (CKV_CLAMP((int64_t)(u.wk.part_row + r), a.part_rows, err_flag) * G + u.grp) * (D + 2);
-                        pr[0] = -CUDART_INF_F;
-                        for (int e = 1; e < D + 2; ++e) pr[e] = 0.f;
+                        const int64_t pr = CKV_CLAMP((int64_t)(u.wk.part_row + r), a.part_rows, err_flag);
+                        *part_ml(a, D, pr, u.grp) = make_float2(-CUDART_INF_F, 0.f);
+                        float4* dst = reinterpret_cast<float4*>(part_acc(a, D, pr, u.grp));
+                        for (int q4 = 0; q4 < 8; ++q4) dst[q4] = make_float4(0.f, 0.f, 0.f, 0.f);
                     } else if (a.out_dtype == CKV_BF16) {
                         uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(a.out) + out_base);
                         for (int q4 = 0; q4 < 4; ++q4) dst[q4] = make_uint4(0, 0, 0, 0);
@@ -742,11 +743,12 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma_kernel(const AttendAr
                             dst[q4] = make_float4(o(4 * q4) * inv, o(4 * q4 + 1) * inv, o(4 * q4 + 2) * inv, o(4 * q4 + 3) * inv);
                     }
                 } else {
-                    float* pr = a.partials + (CKV_CLAMP((int64_t)(u.wk.part_row + r), a.part_rows, err_flag) * G + u.grp) * (D + 2);
-                    pr[0] = m_ref;
-                    pr[1] = l;
+                    const int64_t pr = CKV_CLAMP((int64_t)(u.wk.part_row + r), a.part_rows, err_flag);
+                    *part_ml(a, D, pr, u.grp) = make_float2(m_ref, l);
+                    float4* dst = reinterpret_cast<float4*>(part_acc(a, D, pr, u.grp));
 #pragma unroll
-                    for (int e = 0; e < 32; ++e) pr[2 + e] = o(e);
+                    for (int q4 = 0; q4 < 8; ++q4)
+                        dst[q4] = make_float4(o(4 * q4), o(4 * q4 + 1), o(4 * q4 + 2), o(4 * q4 + 3));
                 }
             }
         }
