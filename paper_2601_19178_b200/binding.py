@@ -90,8 +90,9 @@ try:
     from . import _pycall
 except ImportError as e:
     raise ImportError(f"{e}: build it with `python paper_2601_19178_b200/build.py`") from e
-_ATTEND, _ATTEND_VISIBLE, _ATTEND_STATIC = (
-    ctypes.cast(f, ctypes.c_void_p).value for f in (lib.ckv_attend, lib.ckv_attend_visible, lib.ckv_attend_static))
+_ATTEND, _ATTEND_VISIBLE, _ATTEND_STATIC, _APPEND = (
+    ctypes.cast(f, ctypes.c_void_p).value
+    for f in (lib.ckv_attend, lib.ckv_attend_visible, lib.ckv_attend_static, lib.ckv_cache_append))
 
 
 def _ptr(x) -> Optional[int]:
@@ -187,6 +188,10 @@ def ckv_cache_put_batch(ctx, users, hist_off, idx_K, idx_V, user_K, user_V, d_us
 
 
 def ckv_cache_append(ctx, user: int, L_new: int, idx_K, idx_V, user_K, user_V, d_user: int, stream=None) -> None:
+    stream = _stream(stream)
+    st = _pycall.append(_APPEND, ctx or 0, int(user), int(L_new), idx_K, idx_V, user_K, user_V, d_user, stream or 0)
+    if st is not None:
+        return _check(ctx, st, "ckv_cache_append")
     _check(ctx, lib.ckv_cache_append(ctx, int(user), int(L_new), _ptr(idx_K), _ptr(idx_V), _ptr(user_K),
                                      _ptr(user_V), d_user, _stream(stream)), "ckv_cache_append")
 

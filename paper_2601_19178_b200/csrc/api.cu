@@ -1,6 +1,8 @@
 // Host side of the library: context, pool and compressed-cache management, attend
 // planning (history chunking for the split-along-history reduction) and kernel dispatch.
 #include <algorithm>
+#include <atomic>
+#include <chrono>
 #include <cmath>
 #include <cstring>
 #include <map>
@@ -200,7 +202,7 @@ struct ckv_ctx {
     uint64_t generation = 1;
     // scratch
     DevBuf stage_q, stage_out, stage_vis, vmax, partials;
-    int* h_flag = nullptr;     // pinned, mapped: a kernel that checks indices raises it, the host reads it behind a synchronise
+    int* h_flag = nullptr;     // pinned, mapped: {bad, done} of a kernel that checks indices (d_err + 1: its counter)
     void* put_host = nullptr;  // pinned table of a put of many users
     size_t put_host_cap = 0;
     DevBuf put_dev, put_in[4];  // its device copy; staged host inputs up to kKeepStaged bytes each
@@ -272,6 +274,31 @@ cudaError_t grow(DevBuf& b, size_t bytes, int64_t* allocs = nullptr)
     }
     b.cap = want;
     return cudaSuccess;
+}
+
+// Waits until the kernel just launched on `s` has written the host-mapped word `done`, which it writes last.  Short kernels
+// are over within microseconds of the launch, before a stream synchronise returns, so the word is watched first; after
+// that, and for every error, the stream is waited for.
+cudaError_t wait_done(volatile int* done, cudaStream_t s)
+{
+    const auto t0 = std::chrono::steady_clock::now();
+    while (!*done && std::chrono::steady_clock::now() - t0 < std::chrono::microseconds(40)) {
+    }
+    const cudaError_t e = *done ? cudaSuccess : cudaStreamSynchronize(s);
+    std::atomic_thread_fence(std::memory_order_acquire);
+    return e;
+}
+
+// Runs `launch(report)` and waits for its kernel: *bad tells whether it met a bad index.
+template <typename F>
+cudaError_t run_checked(ckv_ctx* ctx, cudaStream_t s, bool* bad, F&& launch)
+{
+    volatile int* const flag = ctx->h_flag;
+    flag[0] = flag[1] = 0;
+    cudaError_t e = launch(Report{ctx->h_flag, ctx->h_flag + 1, reinterpret_cast<unsigned*>(ctx->d_err + 1)});
+    if (e == cudaSuccess) e = wait_done(flag + 1, s);
+    *bad = flag[0] != 0;
+    return e;
 }
 
 constexpr size_t kKeepStaged = size_t(16) << 20;
@@ -931,15 +958,15 @@ ckv_status ckv_create(const ckv_config* cfg, ckv_ctx** out)
     ctx->scale = cfg->scale > 0.f ? cfg->scale
                                   : (cfg->mode == CKV_SOFTMAX ? 1.0f / std::sqrt((float)cfg->head_dim) : 1.0f);
     DeviceGuard dg(cfg->device);
-    if (!dg.ok || cudaMalloc((void**)&ctx->d_err, sizeof(int)) != cudaSuccess ||
-        cudaMemset(ctx->d_err, 0, sizeof(int)) != cudaSuccess ||
-        cudaHostAlloc((void**)&ctx->h_flag, sizeof(int), cudaHostAllocMapped) != cudaSuccess) {
+    if (!dg.ok || cudaMalloc((void**)&ctx->d_err, 2 * sizeof(int)) != cudaSuccess ||
+        cudaMemset(ctx->d_err, 0, 2 * sizeof(int)) != cudaSuccess ||
+        cudaHostAlloc((void**)&ctx->h_flag, 2 * sizeof(int), cudaHostAllocMapped) != cudaSuccess) {
         cudaGetLastError();
         if (ctx->d_err) cudaFree(ctx->d_err);
         delete ctx;
         return CKV_ERR_CUDA;
     }
-    *ctx->h_flag = 0;
+    ctx->h_flag[0] = ctx->h_flag[1] = 0;
     if (cudaDeviceGetAttribute(&ctx->n_sms, cudaDevAttrMultiProcessorCount, cfg->device) != cudaSuccess || ctx->n_sms < 1) {
         cudaGetLastError();
         ctx->n_sms = 148;
@@ -1104,14 +1131,13 @@ ckv_status ckv_cache_put_batch(ckv_ctx* ctx, int32_t n, const int64_t* users, co
             CK(cudaMemcpyAsync(ctx->put_dev.p, tab, sizeof(PutUser) * (size_t)n, cudaMemcpyHostToDevice, s));
         ckv_status st = arena_take(ctx, total_units, s, &base);
         if (st != CKV_OK) return st;
-        volatile int* const flag = ctx->h_flag;
-        *flag = 0;
-        cudaError_t e = launch_pack(ctx->cfg.dtype, G, ctx->n_entries, ctx->idx_bytes, n,
-                                    n > kInlinePuts ? (const PutUser*)ctx->put_dev.p : nullptr, &inl,
-                                    total_units / (32 * (int64_t)G), base, (const int32_t*)sik.dev, (const int32_t*)siv.dev,
-                                    suk.dev, suv.dev, view_of(ctx), ctx->cfg.head_dim, ctx->h_flag, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        const bool bad = *flag != 0;
+        bool bad;
+        const cudaError_t e = run_checked(ctx, s, &bad, [&](const Report& report) {
+            return launch_pack(ctx->cfg.dtype, G, ctx->n_entries, ctx->idx_bytes, n,
+                               n > kInlinePuts ? (const PutUser*)ctx->put_dev.p : nullptr, &inl,
+                               total_units / (32 * (int64_t)G), base, (const int32_t*)sik.dev, (const int32_t*)siv.dev,
+                               suk.dev, suv.dev, view_of(ctx), ctx->cfg.head_dim, report, s);
+        });
         if (e != cudaSuccess || bad) {  // nothing was stored: the units go back
             arena_give(ctx, base, total_units);
             return e != cudaSuccess ? ctx->fail(e) : CKV_ERR_INDEX_RANGE;
@@ -1172,18 +1198,16 @@ ckv_status ckv_cache_append(ckv_ctx* ctx, int64_t user, int32_t L_new, const int
         ckv_status st = arena_take(ctx, units, s, &base);
         if (st != CKV_OK) return st;
     }
-    volatile int* const flag = ctx->h_flag;
-    *flag = 0;
-    auto append = [&](int32_t n_new) {
+    auto append = [&](int32_t n_new, const Report& report) {
         return launch_append(ctx->cfg.dtype, G, ctx->n_entries, ctx->idx_bytes, old.base, old.L, old.Lpad, base, n_new,
                              Lpad_tot, (const int32_t*)sik.dev, (const int32_t*)siv.dev, suk.dev, suv.dev, view_of(ctx),
-                             ctx->cfg.head_dim, ctx->h_flag, s);
+                             ctx->cfg.head_dim, report, s);
     };
-    cudaError_t e = append(L_new);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess || *flag) {  // the user keeps the old history
+    bool bad;
+    cudaError_t e = run_checked(ctx, s, &bad, [&](const Report& report) { return append(L_new, report); });
+    if (e != cudaSuccess || bad) {  // the user keeps the old history
         if (!in_place) arena_give(ctx, base, units);
-        else if (e == cudaSuccess) e = append(0);  // padding again
+        else if (e == cudaSuccess) e = append(0, Report{ctx->h_flag});  // padding again
         return e != cudaSuccess ? ctx->fail(e) : CKV_ERR_INDEX_RANGE;
     }
     if (!in_place) arena_give(ctx, old.base, (int64_t)G * old.Lpad);
@@ -1360,10 +1384,10 @@ ckv_status run_mma(ckv_ctx* ctx, int D, int max_M, int qpw, int parts, const Att
 
 namespace {
 
-// An error word in pinned host memory for one call of the context-free router: 64 of them for the process, handed out
-// and given back under a lock (a call beyond that many at the same time gets one of its own).
+// Two words {error, done} in pinned host memory for one call of the context-free router: 64 pairs for the process, handed
+// out and given back under a lock (a call beyond that many at the same time gets one of its own, without the second word).
 class HostFlag {
-    static constexpr int kSlots = 64, kStride = 16;  // a cache line each
+    static constexpr int kSlots = kRouteSlots, kStride = 16;  // a cache line each
     static std::mutex mu_;
     static int* pool_;
     static uint64_t used_;
@@ -1371,6 +1395,7 @@ class HostFlag {
 
 public:
     int* p = nullptr;
+    int slot() const { return slot_; }
     HostFlag()
     {
         {
@@ -1388,11 +1413,11 @@ public:
                 p = pool_ + slot_ * kStride;
             }
         }
-        if (!p && cudaHostAlloc((void**)&p, sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
+        if (!p && cudaHostAlloc((void**)&p, 2 * sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
             cudaGetLastError();
             p = nullptr;
         }
-        if (p) *p = 0;
+        if (p) p[0] = p[1] = 0;
     }
     ~HostFlag()
     {
@@ -1824,8 +1849,8 @@ ckv_status ckv_route(int32_t device, int32_t n, int32_t n_groups, int32_t d_in, 
     } else {
         HostFlag flag;
         if (!flag.p) return CKV_ERR_OOM;
-        e = launch_route_umma(d_in, x, W, bias, n, n_entries, n_groups, idx_out, flag.p, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        e = launch_route_umma(d_in, x, W, bias, n, n_entries, n_groups, idx_out, flag.p, flag.slot(), s);
+        if (e == cudaSuccess) e = wait_done(flag.p + 1, s);
         // a bounded wait inside the kernel ran out: the output is not valid
         if (e == cudaSuccess && *(volatile int*)flag.p) return CKV_ERR_CUDA;
     }

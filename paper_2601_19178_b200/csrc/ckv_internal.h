@@ -182,19 +182,41 @@ struct PutTable {
     PutUser u[kInlinePuts];
 };
 // Packs n users' [P][G] indices and [P][G][d_user] user parts into arena units and validates the index range;
-// *bad_flag (host-mapped int) becomes 1 on a bad index.  The users come from `table` (device memory) or, if that is
+// How a kernel that checks indices reports to the host, in host-mapped memory: *bad becomes 1 on a bad index, and *done
+// (if not null) behind the last block's last access, which the host sees some microseconds before a stream synchronise
+// returns.  `count` is a device counter, zero between launches, used by one launch at a time.
+struct Report {
+    int* bad = nullptr;
+    int* done = nullptr;
+    unsigned* count = nullptr;
+};
+#ifdef __CUDACC__
+// The end of a kernel that reports, reached by all threads of its n_blocks blocks: every thread's accesses lie before *done.
+__device__ __forceinline__ void report_done(const Report& r, unsigned n_blocks)
+{
+    if (!r.done) return;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    __threadfence_system();
+    if (atomicAdd(r.count, 1u) != n_blocks - 1) return;
+    *r.count = 0;
+    __threadfence_system();
+    *reinterpret_cast<volatile int*>(r.done) = 1;
+}
+#endif
+// The users come from `table` (device memory) or, if that is
 // null, from *inl.  The arena arrays and the sides' widths come from `cv` (head_dim D).
 cudaError_t launch_pack(int dtype, int G, int n_entries, int idx_bytes, int n_users, const PutUser* table,
                         const PutTable* inl, int64_t total_tiles, int64_t arena_base, const int32_t* idxK,
                         const int32_t* idxV, const void* userK, const void* userV, const CacheView& cv, int D,
-                        int* bad_flag, cudaStream_t s);
+                        const Report& report, cudaStream_t s);
 // Writes a user's units for L_old + L_new positions at arena unit dst_base: the first L_old positions copied from
 // the units at old_base (same arena), the rest packed from the new [L_new][G] indices and [L_new][G][d_user] parts.  dst_base = old_base (and
 // Lpad_tot = Lpad_old): the new positions are written behind the old ones, in place.
 cudaError_t launch_append(int dtype, int G, int n_entries, int idx_bytes, int64_t old_base, int L_old,
                           int Lpad_old, int64_t dst_base, int L_new, int Lpad_tot, const int32_t* idxK,
                           const int32_t* idxV, const void* userK, const void* userV, const CacheView& cv, int D,
-                          int* bad_flag, cudaStream_t s);
+                          const Report& report, cudaStream_t s);
 cudaError_t launch_materialize(int dtype, int D, const CacheView& cv, int64_t base, int L, int Lpad,
                                void* K_out, void* V_out, cudaStream_t s);
 
@@ -239,9 +261,11 @@ cudaError_t launch_route(int d_in, const void* x, const void* W, const float* bi
                          int32_t* out, cudaStream_t s);
 
 // ---- kernels_route_umma.cu : the same router on tcgen05 (TMEM accumulators, warp-specialised)
-// err_flag: host-mapped int, set to a non-zero code if a bounded wait inside the kernel ran out (nothing is written then).
+// flags: two host-mapped ints.  flags[0] becomes a non-zero code if a bounded wait inside the kernel ran out (nothing is
+// written then); flags[1] becomes 1 at its end if slot is in [0, kRouteSlots) and no other launch uses it at the time.
+constexpr int kRouteSlots = 64;
 cudaError_t launch_route_umma(int d_in, const void* x, const void* W, const float* bias, int n, int n_entries, int G,
-                              int32_t* out, int* err_flag, cudaStream_t s);
+                              int32_t* out, int* flags, int slot, cudaStream_t s);
 
 // out[i][g][c] = x_i . W[g][c] + bias[g][c] (bf16 in and out, fp32 sums); W [G][d_out][d_in], bias [G][d_out] or null.
 bool project_supported(int d_in, int d_out, int n_groups);

@@ -30,7 +30,8 @@ struct SideDst {
     void* idx;     // arena indices, null for a side that is not shared
     void* user;    // arena user parts / full rows
     int width;     // elements per unit in `user`
-    int vec;       // bytes per unit if they can be moved as one word, else 0
+    int vec;       // bytes per unit if they can be moved from the caller's array as one word, else 0
+    int vec_arena; // the same between units of the arena
 };
 // A unit's user part is one word if its size is a power of two of 4 to 16 bytes and the caller's array is aligned to it
 // (the arena is: units start at multiples of the size).
@@ -41,7 +42,8 @@ inline int vec_bytes(int bytes, const void* src)
 inline SideDst side_dst(bool full, const void* idx, const void* user, int d_user, int D, int elem, const void* src)
 {
     const int width = full ? D : d_user;
-    return SideDst{full ? nullptr : const_cast<void*>(idx), const_cast<void*>(user), width, vec_bytes(width * elem, src)};
+    return SideDst{full ? nullptr : const_cast<void*>(idx), const_cast<void*>(user), width, vec_bytes(width * elem, src),
+                   vec_bytes(width * elem, nullptr)};
 }
 
 // `bytes` bytes of one unit: one access where they are a word of 4 to 16 bytes (aligned on both sides, see vec_bytes),
@@ -86,14 +88,13 @@ template <typename E, typename I>
 __global__ void __launch_bounds__(256) pack_kernel(int G, int n_entries, int n_users, const PutUser* __restrict__ table,
                                                    int64_t total_tiles, int64_t arena_base, const int32_t* __restrict__ idxK,
                                                    const int32_t* __restrict__ idxV, const E* __restrict__ userK,
-                                                   const E* __restrict__ userV, SideDst dK, SideDst dV, int* bad_flag,
+                                                   const E* __restrict__ userV, SideDst dK, SideDst dV, Report report,
                                                    const __grid_constant__ PutTable inl)
 {
     const PutUser* tab = table ? table : inl.u;
     const int lane = threadIdx.x & 31;
     const int64_t n_warps = (int64_t)gridDim.x * (blockDim.x / 32), w = blockIdx.x * (int64_t)(blockDim.x / 32) + (threadIdx.x >> 5);
     const int64_t t0 = total_tiles * w / n_warps, t1 = total_tiles * (w + 1) / n_warps;
-    if (t0 >= t1) return;
     int u = 0, hi = n_users;  // last user whose first tile is <= t0
     while (hi - u > 1) {
         const int mid = (u + hi) >> 1;
@@ -107,17 +108,18 @@ __global__ void __launch_bounds__(256) pack_kernel(int G, int n_entries, int n_u
         const bool real = i < e.L;
 #pragma unroll 4
         for (int g = 0; g < G; ++g) {
-            store_unit<E, I>(dK, dst + (int64_t)g * Lpad, idxK, userK, src + g, real, n_entries, bad_flag);
-            store_unit<E, I>(dV, dst + (int64_t)g * Lpad, idxV, userV, src + g, real, n_entries, bad_flag);
+            store_unit<E, I>(dK, dst + (int64_t)g * Lpad, idxK, userK, src + g, real, n_entries, report.bad);
+            store_unit<E, I>(dV, dst + (int64_t)g * Lpad, idxV, userV, src + g, real, n_entries, report.bad);
         }
     }
+    report_done(report, gridDim.x);
 }
 
 template <typename E, typename I>
 __device__ __forceinline__ void copy_unit(const SideDst& d, int64_t dst, int64_t src)
 {
     E* du = reinterpret_cast<E*>(d.user);
-    for (int c = 0; c < d.width; ++c) du[dst * d.width + c] = du[src * d.width + c];
+    copy_user<E>(du + dst * d.width, du + src * d.width, d.width, d.vec_arena, true);
     if (d.idx) reinterpret_cast<I*>(d.idx)[dst] = reinterpret_cast<I*>(d.idx)[src];
 }
 
@@ -128,7 +130,7 @@ template <typename E, typename I>
 __global__ void append_kernel(int G, int n_entries, int64_t old_base, int L_old, int Lpad_old,
                               int64_t dst_base, int L_new, int Lpad_tot, const int32_t* __restrict__ idxK,
                               const int32_t* __restrict__ idxV, const E* __restrict__ userK,
-                              const E* __restrict__ userV, SideDst dK, SideDst dV, int* bad_flag)
+                              const E* __restrict__ userV, SideDst dK, SideDst dV, Report report)
 {
     const int first = dst_base == old_base ? L_old : 0, n = Lpad_tot - first;
     const int64_t total = (int64_t)G * n;
@@ -143,10 +145,11 @@ __global__ void append_kernel(int G, int n_entries, int64_t old_base, int L_old,
         } else {
             const int64_t src = (int64_t)(i - L_old) * G + g;
             const bool real = i < L_old + L_new;
-            store_unit<E, I>(dK, dst, idxK, userK, src, real, n_entries, bad_flag);
-            store_unit<E, I>(dV, dst, idxV, userV, src, real, n_entries, bad_flag);
+            store_unit<E, I>(dK, dst, idxK, userK, src, real, n_entries, report.bad);
+            store_unit<E, I>(dV, dst, idxV, userV, src, real, n_entries, report.bad);
         }
     }
+    report_done(report, gridDim.x);
 }
 
 template <typename E, typename I>
@@ -208,15 +211,20 @@ cudaError_t launch_pool_layout(int dtype, int G, int m, int d_shared, int D, con
     return cudaGetLastError();
 }
 
+// Beyond this many blocks a kernel takes so long that a synchronise costs nothing in comparison.
+constexpr int kMaxReporting = 1024;
+
 cudaError_t launch_pack(int dtype, int G, int n_entries, int idx_bytes, int n_users, const PutUser* table,
                         const PutTable* inl, int64_t total_tiles, int64_t arena_base, const int32_t* idxK,
                         const int32_t* idxV, const void* userK, const void* userV, const CacheView& cv, int D,
-                        int* bad_flag, cudaStream_t s)
+                        const Report& to, cudaStream_t s)
 {
     if (total_tiles == 0) return cudaSuccess;
     // two warps per block while that leaves SMs without a block, then eight; at most 16 blocks of eight per SM
     const int block = total_tiles <= 148 * 8 ? 64 : 256, wpb = block / 32;
     const int grid = (int)std::min<int64_t>((total_tiles + wpb - 1) / wpb, 148 * 16);
+    Report report = to;
+    if (grid > kMaxReporting) report.done = nullptr;
     static const PutTable none{};
     const PutTable& pt = inl ? *inl : none;
     const int es = dtype == CKV_BF16 ? 2 : 4;
@@ -224,7 +232,7 @@ cudaError_t launch_pack(int dtype, int G, int n_entries, int idx_bytes, int n_us
     const SideDst dV = side_dst(cv.full_v, cv.idxV, cv.userV, cv.d_user, D, es, userV);
 #define CKV_PACK(E, I)                                                                                         \
     pack_kernel<E, I><<<grid, block, 0, s>>>(G, n_entries, n_users, table, total_tiles, arena_base, idxK, idxV, \
-                                             (const E*)userK, (const E*)userV, dK, dV, bad_flag, pt)
+                                             (const E*)userK, (const E*)userV, dK, dV, report, pt)
     if (dtype == CKV_BF16) {
         if (idx_bytes == 2) CKV_PACK(uint16_t, uint16_t); else CKV_PACK(uint16_t, int32_t);
     } else {
@@ -237,18 +245,20 @@ cudaError_t launch_pack(int dtype, int G, int n_entries, int idx_bytes, int n_us
 cudaError_t launch_append(int dtype, int G, int n_entries, int idx_bytes, int64_t old_base, int L_old,
                           int Lpad_old, int64_t dst_base, int L_new, int Lpad_tot, const int32_t* idxK,
                           const int32_t* idxV, const void* userK, const void* userV, const CacheView& cv, int D,
-                          int* bad_flag, cudaStream_t s)
+                          const Report& to, cudaStream_t s)
 {
     const int64_t total = (int64_t)G * (Lpad_tot - (dst_base == old_base ? L_old : 0));
     if (total == 0) return cudaSuccess;
     const int grid = grid_for(total, 256);
+    Report report = to;
+    if (grid > kMaxReporting) report.done = nullptr;
     const int es = dtype == CKV_BF16 ? 2 : 4;
     const SideDst dK = side_dst(cv.full_k, cv.idxK, cv.userK, cv.d_user, D, es, userK);
     const SideDst dV = side_dst(cv.full_v, cv.idxV, cv.userV, cv.d_user, D, es, userV);
 #define CKV_APPEND(E, I)                                                                                       \
     append_kernel<E, I><<<grid, 256, 0, s>>>(G, n_entries, old_base, L_old, Lpad_old, dst_base, L_new,        \
                                              Lpad_tot, idxK, idxV, (const E*)userK, (const E*)userV, dK, dV,  \
-                                             bad_flag)
+                                             report)
     if (dtype == CKV_BF16) {
         if (idx_bytes == 2) CKV_APPEND(uint16_t, uint16_t); else CKV_APPEND(uint16_t, int32_t);
     } else {

@@ -163,10 +163,12 @@ __device__ __forceinline__ uint64_t swz_desc(uint32_t addr)
 // K-major core matrices of 16 bf16 per row, no swizzle: row r, 16-byte chunk c
 __device__ __forceinline__ uint32_t step_off(int r, int c) { return (uint32_t)((r >> 3) * 256 + c * 128 + (r & 7) * 16); }
 
+__device__ unsigned route_count[kRouteSlots];  // finished CTAs of the launch that holds the slot, zero between launches
+
 template <int DIN>
 __global__ void __launch_bounds__(kThreadsRU, 1)
     route_umma_kernel(const uint16_t* __restrict__ x, const __grid_constant__ CUtensorMap tmW, const float* __restrict__ bias,
-                      int n, int m, int G, int32_t* __restrict__ out, int* err_flag, int n_split)
+                      int n, int m, int G, int32_t* __restrict__ out, int* flags, int slot, int n_split)
 {
     using L = RU<DIN>;
     extern __shared__ __align__(1024) unsigned char usm[];
@@ -420,7 +422,8 @@ __global__ void __launch_bounds__(kThreadsRU, 1)
         asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     }
     if (warp < kEpiWarps && split == 0 && !*abort_flag && row0 + row < n) out[(row0 + row) * G + grp] = arg;
-    if (tid == 0 && *abort_flag) *reinterpret_cast<volatile int*>(err_flag) = ERR_ROUTE;
+    if (tid == 0 && *abort_flag) *reinterpret_cast<volatile int*>(flags) = ERR_ROUTE;
+    if (slot >= 0) report_done(Report{flags, flags + 1, &route_count[slot]}, gridDim.x * gridDim.y);
 }
 
 // The weights as rows of `d_in` inputs, boxes of 128 rows and at most 64 inputs.
@@ -445,8 +448,8 @@ bool make_weight_map(int d_in, int64_t rows, const void* W, CUtensorMap* map)
 }
 
 template <int DIN>
-cudaError_t launch_t(const void* x, const void* W, const float* bias, int n, int m, int G, int32_t* out, int* err_flag,
-                     cudaStream_t s)
+cudaError_t launch_t(const void* x, const void* W, const float* bias, int n, int m, int G, int32_t* out, int* flags,
+                     int slot, cudaStream_t s)
 {
     CUtensorMap map;
     if (!make_weight_map(DIN, (int64_t)G * m, W, &map)) return cudaErrorInvalidValue;
@@ -466,21 +469,21 @@ cudaError_t launch_t(const void* x, const void* W, const float* bias, int n, int
         }
     }
     const dim3 grid((unsigned)((n + kRows - 1) / kRows * split), (unsigned)G);
+    if (ctas * split > sms) slot = -1;  // several rounds: the report at the end of each CTA would delay the next
     return launch_kernel(Launch{s, nullptr, nullptr}, route_umma_kernel<DIN>, grid, kThreadsRU, RU<DIN>::SMEM, split,
-                         (const uint16_t*)x, map, bias, n, m, G, out, err_flag, split);
+                         (const uint16_t*)x, map, bias, n, m, G, out, flags, slot, split);
 }
 
 }  // namespace
 
-// err_flag: host-mapped int, set to a non-zero code if a bounded wait inside the kernel ran out (nothing is written then).
 cudaError_t launch_route_umma(int d_in, const void* x, const void* W, const float* bias, int n, int n_entries, int G,
-                              int32_t* out, int* err_flag, cudaStream_t s)
+                              int32_t* out, int* flags, int slot, cudaStream_t s)
 {
     if (n == 0) return cudaSuccess;
     switch (d_in) {
-        case 32: return launch_t<32>(x, W, bias, n, n_entries, G, out, err_flag, s);
-        case 64: return launch_t<64>(x, W, bias, n, n_entries, G, out, err_flag, s);
-        default: return launch_t<128>(x, W, bias, n, n_entries, G, out, err_flag, s);
+        case 32: return launch_t<32>(x, W, bias, n, n_entries, G, out, flags, slot, s);
+        case 64: return launch_t<64>(x, W, bias, n, n_entries, G, out, flags, slot, s);
+        default: return launch_t<128>(x, W, bias, n, n_entries, G, out, flags, slot, s);
     }
 }
 

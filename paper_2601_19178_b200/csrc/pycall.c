@@ -1,5 +1,5 @@
 /*
- * CPython helper of binding.py: marshals the arguments of the decode calls.  A decode call of a few users takes the
+ * CPython helper of binding.py: marshals the arguments of the decode and append calls.  A decode call of a few users takes the
  * GPU about 6 us; taking two array addresses, two tensor addresses and going through ctypes took Python another 4.
  * Marshalling only: the call itself is the C-ABI function whose address is passed in.
  */
@@ -81,7 +81,39 @@ static PyObject* attend(PyObject* self, PyObject* const* args, Py_ssize_t n_args
     return PyLong_FromLong(status);
 }
 
+typedef int32_t (*append_fn)(void*, int64_t, int32_t, const void*, const void*, const void*, const void*, int32_t, void*);
+
+/* append(function address, context, user, L_new, idx_K, idx_V, user_K, user_V, d_user, stream): as attend, every array a
+ * contiguous tensor. */
+static PyObject* append(PyObject* self, PyObject* const* args, Py_ssize_t n_args)
+{
+    (void)self;
+    if (n_args != 10) {
+        PyErr_SetString(PyExc_TypeError, "append takes 10 arguments");
+        return NULL;
+    }
+    void* fn = PyLong_AsVoidPtr(args[0]);
+    void* ctx = PyLong_AsVoidPtr(args[1]);
+    const long long user = PyLong_AsLongLong(args[2]);
+    const long L_new = PyLong_AsLong(args[3]), d_user = PyLong_AsLong(args[8]);
+    void* stream = PyLong_AsVoidPtr(args[9]);
+    if (PyErr_Occurred()) return NULL;
+    void* p[4];
+    for (int i = 0; i < 4; ++i)
+        if (!tensor_address(args[4 + i], &p[i])) {
+            if (PyErr_Occurred()) return NULL;
+            Py_RETURN_NONE;
+        }
+    if (L_new != (int32_t)L_new || d_user != (int32_t)d_user) Py_RETURN_NONE;
+    int32_t status;
+    Py_BEGIN_ALLOW_THREADS;
+    status = ((append_fn)fn)(ctx, user, (int32_t)L_new, p[0], p[1], p[2], p[3], (int32_t)d_user, stream);
+    Py_END_ALLOW_THREADS;
+    return PyLong_FromLong(status);
+}
+
 static PyMethodDef methods[] = {{"attend", (PyCFunction)(void (*)(void))attend, METH_FASTCALL, "one decode call"},
+                                {"append", (PyCFunction)(void (*)(void))append, METH_FASTCALL, "one append"},
                                 {NULL, NULL, 0, NULL}};
 static struct PyModuleDef module = {PyModuleDef_HEAD_INIT, "_pycall", NULL, -1, methods, NULL, NULL, NULL, NULL};
 
