@@ -366,42 +366,43 @@ __global__ void __launch_bounds__(128, MmaCfg<D, MT, TMA>::MIN_BLOCKS)
         }
     };
 
-    // prologue: tiles 0 .. NST-2 in flight, indices two tiles further, user parts two tiles ahead
-    int ikA, ivA, ikB, ivB, ikC, ivC;
+    // prologue: tiles 0 .. NST-2 in flight, indices of the next two and user parts of the first two requested.  All
+    // requests before the first use: a block's life begins with this chain of latencies.
+    struct Ahead {
+        int ik, iv;     // indices of tile step + NST - 1
+        uint4 uk, uv;   // user parts of tile step
+    } even, odd;
+    int ik0[NST - 1], iv0[NST - 1];
+#pragma unroll
+    for (int s0 = 0; s0 < NST - 1; ++s0) fetch_idx(s0, ik0[s0], iv0[s0]);
+    fetch_idx(NST - 1, even.ik, even.iv);
+    fetch_idx(NST, odd.ik, odd.iv);
+    even.uk = even.uv = odd.uk = odd.uv = make_uint4(0, 0, 0, 0);
+    fetch_user(0, even.uk, even.uv);
+    fetch_user(1, odd.uk, odd.uv);
 #pragma unroll
     for (int s0 = 0; s0 < NST - 1; ++s0) {
-        fetch_idx(s0, ikA, ivA);
-        if (s0 < nsteps) issue(s0, ikA, ivA);
+        if (s0 < nsteps) issue(s0, ik0[s0], iv0[s0]);
         if constexpr (!TMA) cp_async_commit();
     }
-    fetch_idx(NST - 1, ikA, ivA);
-    fetch_idx(NST, ikB, ivB);
-    fetch_idx(NST + 1, ikC, ivC);
-    uint4 ukA, uvA, ukB, uvB;
-    ukA = uvA = ukB = uvB = make_uint4(0, 0, 0, 0);
-    fetch_user(0, ukA, uvA);
-    fetch_user(1, ukB, uvB);
 
-    bool ok = true;
-    for (int step = 0; step < nsteps; ++step) {
+    // one tile; its registers of `w` are requested again for the tile two steps further
+    auto body = [&](int step, Ahead& w) {
         const int p0 = it.begin + 32 * part + stride * step;
-        if (step + NST - 1 < nsteps) issue(step + NST - 1, ikA, ivA);
+        if (step + NST - 1 < nsteps) issue(step + NST - 1, w.ik, w.iv);
         if constexpr (!TMA) cp_async_commit();
-        ikA = ikB; ivA = ivB; ikB = ikC; ivB = ivC;
-        fetch_idx(step + NST + 2, ikC, ivC);
+        fetch_idx(step + NST + 1, w.ik, w.iv);
         if constexpr (TMA) {
             const uint32_t bar = bars + 8 * (step % NST), parity = (step / NST) & 1;
+            bool here = true;
             int spins = 0;
             while (!mbar_try_wait(bar, parity)) {
                 if (++spins > kTmaSpinLimit) {
-                    ok = false;
+                    here = false;
                     break;
                 }
             }
-            if (!__all_sync(0xffffffffu, ok)) {  // give up: nothing more is issued, nothing is stored
-                ok = false;
-                break;
-            }
+            if (!__all_sync(0xffffffffu, here)) return false;  // give up: nothing more is issued, nothing is stored
         } else {
             cp_async_wait<NST - 1>();
         }
@@ -409,10 +410,9 @@ __global__ void __launch_bounds__(128, MmaCfg<D, MT, TMA>::MIN_BLOCKS)
         const uint32_t kt = ring + (step % NST) * (2 * C::TILE_B), vt = kt + C::TILE_B;
         // Eq. K: dims [0, d_user) of every row come from the user-specific part
         if (wide_user) {
-            if (!full_k) store_user_part(kt + offU, ukA, d_user);
-            if (!full_v) store_user_part(vt + offU, uvA, d_user);
-            ukA = ukB; uvA = uvB;
-            fetch_user(step + 2, ukB, uvB);
+            if (!full_k) store_user_part(kt + offU, w.uk, d_user);
+            if (!full_v) store_user_part(vt + offU, w.uv, d_user);
+            fetch_user(step + 2, w.uk, w.uv);
         } else if (d_user > 0 && !(full_k && full_v)) {
             for (int e = 0; e < d_user; ++e) {
                 if (!full_k) {
@@ -575,6 +575,12 @@ __global__ void __launch_bounds__(128, MmaCfg<D, MT, TMA>::MIN_BLOCKS)
         // and loads are ordered before the asynchronous-proxy writes of the refill)
         if constexpr (TMA) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
+        return true;
+    };
+    bool ok = true;
+    for (int step = 0; ok && step < nsteps; step += 2) {
+        ok = body(step, even);
+        if (ok && step + 1 < nsteps) ok = body(step + 1, odd);
     }
     if constexpr (TMA) {
         // (a warp that gave up still takes part in the merge: the error word says that the outputs are not valid)
