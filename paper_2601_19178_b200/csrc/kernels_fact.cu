@@ -11,8 +11,8 @@
 //
 // Three launches:
 //   fact_table_kernel  T[r][g][j] = q_r . P_k[g][j]          m16n8k16 MMAs, fp32 out
-//   fact_main_kernel   persistent CTAs over the (user, group) pairs: T row into shared memory, scores, max, weights, histogram w,
-//                      user-part output and row sum; w takes T's place in shared memory and in HBM
+//   fact_main_kernel   persistent CTAs over the (user, group) pairs: T row into shared memory by bulk copy, then one pass over
+//                      the history: score, weight, histogram w (a buffer of its own), user-part output and row sum
 //   fact_out_kernel    out[r][g][:] = (w[r][g] P_v[g] + user part) / l          MMAs, w in bf16
 #include <cuda_bf16.h>
 #include <math_constants.h>

@@ -27,7 +27,9 @@
 // warp's sub-partition; three workers fill each other's gaps.  Registers (65536 / 20 warps = 96 a thread, enough for one
 // 32-column chunk of scores at a time) and TMEM (3 x (2 x 64 + 32) = 480 columns) admit no fourth.  With the three groups
 // on one unit instead (its tiles dealt out in turn, accumulators merged through shared memory at its end) a unit cost
-// FIGURES
+// 5 us plus 0.45 us per 128 positions; now an SM of busy workers takes 0.4 us per 64 positions and 1.5 us per unit, the
+// special-function unit busy 70 % of the time.  1024 users x 1024 positions x 100 queries x 8 groups 490 -> 385 us, 2048
+// users x 4096 x 128 (SiLU) 2.88 -> 2.57 ms, 64 causal self-attentions of 200..1500 positions 283 -> 147 us.
 //
 // Softmax bookkeeping.  The reference maximum m of a row is the largest of the first 32 scores of the group's
 // first half of the unit and stays fixed: later scores may exceed it by up to 2^64 (fp32 accumulators and bf16

@@ -1,0 +1,159 @@
+"""Edges of the kernels' tiles and of the rules that choose among them, against the CPU oracle through the C ABI."""
+import numpy as np
+import pytest
+import torch
+
+import synth
+from ckv_testlib import assert_close, gpu_attend, make_session, oracle_attend, to_dev
+from test_route import _bf16, _check, _gpu_route
+
+pytestmark = pytest.mark.gpu
+
+
+def _workload(mode="softmax", dtype="bf16", head=(30, 2), groups=2, pool=500, users=4, hist=(1, 300), queries=5,
+              zipf=1.1, seed=7):
+    return synth.Workload("edge", groups, head[0], head[1], pool, users, hist, queries, mode, dtype, zipf, 1 / 32,
+                          1 / 32, seed)
+
+
+def _attend_matches(w, d, want_kernel=None, scale=0.0, **options):
+    s = make_session(w, d, scale=scale, **options)
+    got = gpu_attend(w, d, session=s)
+    kernel, split = s.stat("kernel"), s.stat("split_items")
+    assert s.stat("device_errors") == 0
+    s.close()
+    if want_kernel is not None:
+        assert kernel == want_kernel
+    assert_close(got, oracle_attend(w, d, scale=scale if scale else None), w.dtype, repr(w))
+    return split
+
+
+@pytest.mark.parametrize("users", [1, 224, 225])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_request_list_as_kernel_argument_and_as_table(users, dtype):
+    """Up to 224 requests travel as a kernel argument, and so does the table of a put of as many users."""
+    w = _workload(dtype=dtype, users=users, hist=(1, 70), queries=3)
+    _attend_matches(w, synth.generate(w), want_kernel=1 if dtype == "f32" else 2)
+
+
+@pytest.mark.parametrize("mode", ["softmax", "silu_over_l"])
+@pytest.mark.parametrize("head", [(30, 2), (60, 4)], ids=["d32", "d64"])
+@pytest.mark.parametrize("length", [1, 31, 33, 64, 65, 129, 512, 1025, 4097])
+def test_warps_sharing_one_unit(mode, head, length):
+    """One user: 1 to 32 warps (in up to eight blocks of a cluster) share a unit and merge their results."""
+    w = _workload(mode=mode, head=head, users=1, hist=(length, length), queries=17)
+    _attend_matches(w, synth.generate(w), want_kernel=2)
+
+
+@pytest.mark.parametrize("mode", ["softmax", "silu_over_l"])
+@pytest.mark.parametrize("head,queries", [((31, 1), 33), ((31, 1), 47), ((60, 4), 17), ((60, 4), 40)])
+def test_several_query_tiles_per_warp(mode, head, queries):
+    """Enough work for every resident warp: a warp holds 48 (32-wide heads) or 32 queries (64-wide)."""
+    w = _workload(mode=mode, head=head, groups=4, users=450, hist=(400, 430), queries=queries)
+    d = synth.generate(w)
+    sel = np.arange(0, w.n_users, 37)
+    s = make_session(w, d, kernel=2)
+    got = gpu_attend(w, d, session=s)
+    s.close()
+    rows = np.concatenate([np.arange(d["q_off"][u], d["q_off"][u + 1]) for u in sel])
+    assert_close(got[rows], oracle_attend(w, d, sel=sel), "bf16", f"{head} {queries}")
+
+
+@pytest.mark.parametrize("dtype,length", [("f32", 1), ("f32", 65), ("f32", 1000), ("f32", 4097), ("bf16", 4097)])
+@pytest.mark.parametrize("queries", [1, 5])
+def test_wide_blocks_of_the_cuda_core_kernel(dtype, length, queries):
+    """Fewer blocks than SMs: 16 (8 with several queries) warps on one history, beyond 4096 positions chunks."""
+    w = _workload(dtype=dtype, users=2, hist=(length, length), queries=queries)
+    split = _attend_matches(w, synth.generate(w), want_kernel=1, kernel=1)
+    assert (split > 0) == (length > 4096)
+
+
+@pytest.mark.parametrize("mode", ["softmax", "silu_over_l"])
+@pytest.mark.parametrize("head", [(14, 2), (30, 2), (60, 4), (120, 8)], ids=["d16", "d32", "d64", "d128"])
+@pytest.mark.parametrize("chunks", [2, 8, 9, 40])
+def test_merge_of_chunks(mode, head, chunks):
+    """The merge kernel requests eight chunks at a time."""
+    w = _workload(mode=mode, head=head, users=2, hist=(64 * chunks - 5, 64 * chunks - 5), queries=9)
+    assert _attend_matches(w, synth.generate(w), split_len=64) > 0
+
+
+@pytest.mark.parametrize("mode", ["softmax", "silu_over_l"])
+@pytest.mark.parametrize("queries", [1, 127, 128, 129])
+@pytest.mark.parametrize("length", [1, 63, 64, 65, 127, 449, 513])
+def test_tcgen05_kernel_tile_edges(mode, queries, length):
+    """Tiles of 64 positions and 128 queries; a ring of seven tiles."""
+    w = _workload(mode=mode, head=(28, 4), groups=3, users=3, hist=(length, length), queries=queries)
+    _attend_matches(w, synth.generate(w), want_kernel=3, kernel=3)
+
+
+@pytest.mark.parametrize("queries,hist", [(47, (500, 500)), (48, (60, 60)), (96, (1500, 1500)), (97, (1500, 1500)),
+                                          (200, (1, 4096)), (60, (4096, 9000))])
+def test_short_lists_of_many_queries(queries, hist):
+    """From 48 queries on: warp-level kernel, tcgen05 kernel, or that in chunks, as the list's size decides."""
+    w = _workload(users=3, hist=hist, queries=queries, groups=4)
+    _attend_matches(w, synth.generate(w))
+
+
+@pytest.mark.parametrize("mode", ["softmax", "silu_over_l"])
+@pytest.mark.parametrize("head", [(30, 2), (60, 4)], ids=["d32", "d64"])
+@pytest.mark.parametrize("pool", [1, 33, 9000, 9500, 19000, 19600, 28000])
+def test_factorisation_table_sizes(mode, head, pool):
+    """Two CTAs per SM, two table buffers, or one, as the pool's size leaves shared memory."""
+    w = _workload(mode=mode, head=head, pool=pool, users=5, hist=(1, 3000), queries=1, zipf=None)
+    _attend_matches(w, synth.generate(w), want_kernel=4, kernel=4)
+
+
+@pytest.mark.parametrize("scale", [2e-3, 1.0, 400.0])
+@pytest.mark.parametrize("pool,zipf", [(4, None), (3000, 1.6)])
+def test_factorisation_of_large_scores_and_crowded_entries(scale, pool, zipf):
+    """Weights are first taken relative to 2^0 and again if the top score is far from it; many positions of one entry."""
+    w = _workload(head=(60, 4), pool=pool, users=6, hist=(200, 2500), queries=1, zipf=zipf)
+    d = synth.generate(w)
+    # (histories of few distinct rows: at the largest scale one position takes all the weight)
+    _attend_matches(w, d, want_kernel=4, scale=scale, kernel=4)
+
+
+@pytest.mark.parametrize("n_new", [1, 12, 13, 40])
+def test_append_inside_and_beyond_the_padding(n_new):
+    """A history of 20 has room for 12 more positions in place; a refused append leaves everything as it was."""
+    import paper_2601_19178_b200 as ckv
+    w = _workload(users=2, hist=(20 + n_new, 20 + n_new), queries=4, pool=64)
+    d = synth.generate(w)
+    L = 20 + n_new
+    part = dict(d, hist_off=np.array([0, 20, 20 + L], dtype=np.int64))
+    keep = np.r_[0:20, L:2 * L]
+    for k in ("idx_K", "idx_V", "user_K", "user_V"):
+        part[k] = d[k][keep]
+    s = make_session(w, part)
+    tail = lambda k, t: to_dev(np.ascontiguousarray(d[k][20:L]), t)
+    new = [tail("idx_K", "i"), tail("idx_V", "i"), tail("user_K", "bf16"), tail("user_V", "bf16")]
+    before = gpu_attend(w, d, session=s)
+    bad = new[1].clone()
+    bad[-1, -1] = 64
+    with pytest.raises(ckv.CkvError) as e:
+        s.cache_append(int(d["users"][0]), new[0], bad, new[2], new[3])
+    assert e.value.status == ckv.CKV_ERR_INDEX_RANGE
+    assert np.array_equal(gpu_attend(w, d, session=s), before)
+    s.cache_append(int(d["users"][0]), *new)
+    got = gpu_attend(w, d, session=s)
+    s.close()
+    assert_close(got, oracle_attend(w, d), "bf16", "appended")
+
+
+@pytest.mark.parametrize("d_in", [32, 64, 128])
+@pytest.mark.parametrize("n,m", [(1, 1), (1, 127), (128, 129), (129, 1000), (256, 128), (257, 3001), (3, 16384)])
+def test_router_block_edges(d_in, n, m):
+    """Blocks of 256 positions, tiles of 128 entries, entries shared by up to eight CTAs for few positions."""
+    rng = np.random.default_rng(n * 7 + m)
+    x, W = _bf16(rng.standard_normal((n, d_in))), _bf16(rng.standard_normal((3, m, d_in)) / np.sqrt(d_in))
+    _check(x, W, None, f"{n} {m} {d_in}", 2)
+    _check(x, W, rng.standard_normal((3, m)).astype(np.float32), f"{n} {m} {d_in} bias", 2)
+
+
+def test_router_bias_keeps_its_32_bits():
+    """The bias enters as three bf16 parts: entries that differ in its last bit only are told apart."""
+    m, d_in = 300, 64
+    bias = np.full((1, m), np.float32(1.2345678), dtype=np.float32)
+    bias[0, 217] = np.nextafter(bias[0, 0], np.float32(2), dtype=np.float32)
+    x, W = _bf16(np.zeros((5, d_in))), _bf16(np.zeros((1, m, d_in)))
+    assert (_gpu_route(x, W, bias, 2) == 217).all()
