@@ -21,8 +21,8 @@
  *     host data through its own device buffers on `stream`.  With host *output* memory the
  *     call returns after the copy has been enqueued; synchronise the stream before reading.
  *   - `stream` is a cudaStream_t passed as void* (NULL = the legacy default stream).
- *     Calls enqueue work on it and return; ckv_cache_put* additionally wait for their own
- *     index validation (one 4-byte read-back).
+ *     Calls enqueue work on it and return; ckv_cache_put*, ckv_cache_append, ckv_cache_import and
+ *     ckv_route additionally wait for their own kernel, whose error word they read.
  *   - The library copies what it is given: inputs may be released once the stream has
  *     passed the call.  Outputs are caller-owned.
  *   - Errors are return codes.  Nothing aborts, traps or throws across the boundary.  After
@@ -261,8 +261,8 @@ CKV_API ckv_status ckv_materialize(ckv_ctx* ctx, int64_t user, void* K_out, void
  *   idx_out  device, int32 [n][n_groups]        what ckv_cache_put takes as idx_K / idx_V
  *   variant  0 = default (tcgen05 kernel), 1 = warp-level tensor-core kernel, 2 = tcgen05 kernel
  * Products are exact, sums fp32; entries whose scores are equal in that arithmetic resolve to the
- * lowest index.  The tcgen05 kernel's waits are bounded; the call reads its error word back and
- * therefore synchronises `stream` (variant 1 is only stream-ordered).
+ * lowest index.  The tcgen05 kernel's waits are bounded; the call reads its error word and
+ * therefore waits for the kernel (variant 1 is only stream-ordered).
  * Errors: INVALID_ARG (sizes, null or host pointers), UNSUPPORTED (d_in), OOM, CUDA (also: a wait
  * inside the kernel ran out; idx_out is not valid then).
  */
@@ -286,9 +286,10 @@ CKV_API ckv_status ckv_project(int32_t device, int32_t n, int32_t n_groups, int3
 
 /*
  * Appends L_new positions (new interactions) behind a cached user's history; arguments as for
- * ckv_cache_put, describing only the new positions.  The user's compressed cache moves to other
- * storage holding the old and the new positions; the old storage is reused by later calls.
- * Synchronises `stream`.
+ * ckv_cache_put, describing only the new positions.  Histories are stored in multiples of 32
+ * positions: new positions that fit behind the old ones are written there, otherwise the user's
+ * compressed cache moves to other storage holding the old and the new positions and the old storage
+ * is reused by later calls.  Waits for its kernel (and so for what `stream` held before it).
  * Errors: INVALID_ARG, STATE (no pool), SHAPE (d_user), UNKNOWN_USER, INDEX_RANGE (an index
  * outside [0, n_entries); the user keeps the old history), OOM, CUDA.
  */
@@ -349,9 +350,9 @@ CKV_API ckv_status ckv_cache_bytes(ckv_ctx* ctx, int64_t* compressed, int64_t* f
  *                  0 or 1 = 16-byte asynchronous copies through L1 (default), 2 = TMA row gathers
  *                  (UNSUPPORTED from ckv_attend if the driver cannot encode the tensor maps);
  *                  the results are the same bits either way
- *   "l2_persist"   1 (default) = every ckv_attend puts an access-policy window over the pool
- *                  (persisting hits) on the caller's stream while it enqueues its kernels and restores
- *                  the stream's previous window before it returns; 0 = leave the stream alone
+ *   "l2_persist"   1 (default) = ckv_attend launches its kernels with an access-policy window over the
+ *                  pool (persisting hits), an attribute of the launch: the caller's stream keeps its own;
+ *                  0 = without
  *   "time_kernels" 1 = record CUDA events around the kernels of each ckv_attend (see ckv_last_stat)
  */
 CKV_API ckv_status ckv_set_option(ckv_ctx* ctx, const char* name, int64_t value);

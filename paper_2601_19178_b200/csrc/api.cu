@@ -482,8 +482,8 @@ struct MmaWork {
 
 // Warps that share one unit: the number with the shortest estimated run, in tile times of a resident warp.  A unit costs two
 // tiles besides its own.  Every further warp per unit shortens the units but adds blocks, and a round of blocks costs
-// about five tiles, six across a cluster (head_dim 64 with clusters of eight: nine).  Units of one size run in whole rounds;
-// mixed ones, longest histories first, leave SMs idle for about half of the longest.  (Fitted to sweeps of 1..32 warps over
+// about four tiles, across a cluster five (head_dim 64: six, with clusters of eight nine).  Units of one size run in whole
+// rounds; mixed ones, longest histories first, leave SMs idle for about three quarters of the longest.  (Fitted to sweeps of 1..32 warps over
 // 1..300 users of 200..16384 positions; within 15 % of most, and the number it picks within 6 % of the best.)
 int mma_parts(const ckv_ctx* ctx, const MmaWork& w, int qpw, double* tile_times)
 {
@@ -493,11 +493,11 @@ int mma_parts(const ckv_ctx* ctx, const MmaWork& w, int qpw, double* tile_times)
     double best_t = 1e300;
     for (int parts = 1; parts <= kMmaMaxParts && parts <= std::max<int64_t>(w.max_tiles, 1); parts *= 2) {
         const double rounds = w.units * G * parts / warps;
-        const double extra = parts == 1 ? 2 : D != 64 || parts <= 4 ? 5 : parts <= 16 ? 6 : 9;
+        const double extra = parts == 1 ? 2 : parts <= 4 ? 4 : D != 64 ? 5 : parts <= 16 ? 6 : 9;
         const double t = w.alike && w.min_tiles == w.max_tiles
                              ? std::ceil(rounds) * ((w.max_tiles + parts - 1) / parts + 2) + rounds * (extra - 2) +
                                    (parts > 16 ? 2 : parts > 1 ? 1 : 0)
-                             : w.tiles * G / warps + rounds * extra + 0.5 * (double)w.max_tiles / parts;
+                             : w.tiles * G / warps + rounds * extra + 0.75 * (double)w.max_tiles / parts;
         if (t < best_t) {
             best_t = t;
             best = parts;
