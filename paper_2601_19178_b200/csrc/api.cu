@@ -560,7 +560,7 @@ struct ListShape {
 
 // Chunk length of the tcgen05 kernel: the one with the shortest estimated run, in microseconds.  Three persistent workers
 // per SM walk a (chunk, group, 128 queries) unit alone; measured, a worker takes 1 us per 64 positions when it has the SM
-// to itself and 1.4 next to two others, 1.5 per unit, the launch 6, and merging chunks 6 and more.  Units of one size
+// to itself and 1.4 next to two others, 1.5 per unit, the launch 6, and merging chunks 6 and 0.007 per chunk.  Units of one size
 // run in whole rounds; mixed ones are dealt out longest first, and only the longest of them bounds the run from below.
 int64_t umma_chunk(const ckv_ctx* ctx, const ListShape& s, double* time = nullptr)
 {
@@ -575,11 +575,16 @@ int64_t umma_chunk(const ckv_ctx* ctx, const ListShape& s, double* time = nullpt
         const bool split = c < s.max_L;
         const double cut = alike ? (double)((s.max_L + c - 1) / c) * s.blocks128 : s.tiles64 * 64.0 / c + (split ? 0.5 : 0) * s.blocks128;
         const double units = G * std::max<double>(cut, s.blocks128), tiles = c / 64;
-        const double tile_us = 0.8 + 0.2 * std::min(3.0, std::max(1.0, units / ctx->n_sms));
-        const double longest = std::min<double>(tiles, (s.max_L + 63) / 64) * tile_us + 1.5;
-        const double t = 6 + (split ? 6 + 0.003 * units : 0) +
-                         (alike ? std::ceil(units / workers) * longest
-                                : std::max(longest, (s.tiles64 * G * tile_us + 1.5 * units) / workers));
+        auto unit_us = [&](double n_tiles, double n) {  // of n units that run at a time
+            return n_tiles * (0.8 + 0.2 * std::min(3.0, std::max(1.0, n / ctx->n_sms))) + 1.5;
+        };
+        const double longest = std::min<double>(tiles, (s.max_L + 63) / 64);
+        double t = 6 + (split ? 6 + 0.007 * units : 0);
+        if (alike) {
+            const double full = std::floor(units / workers), rest = units - full * workers;
+            t += full * unit_us(longest, workers) + (rest > 0 ? unit_us(longest, rest) : 0);
+        } else
+            t += std::max(unit_us(longest, units), (unit_us(s.tiles64 * G, units) + 1.5 * (units - 1)) / workers);
         if (t < best_t) {
             best_t = t;
             best = c;
