@@ -90,9 +90,10 @@ try:
     from . import _pycall
 except ImportError as e:
     raise ImportError(f"{e}: build it with `python paper_2601_19178_b200/build.py`") from e
-_ATTEND, _ATTEND_VISIBLE, _ATTEND_STATIC, _APPEND = (
+_ATTEND, _ATTEND_VISIBLE, _ATTEND_STATIC, _APPEND, _PUT, _ROUTE, _PROJECT = (
     ctypes.cast(f, ctypes.c_void_p).value
-    for f in (lib.ckv_attend, lib.ckv_attend_visible, lib.ckv_attend_static, lib.ckv_cache_append))
+    for f in (lib.ckv_attend, lib.ckv_attend_visible, lib.ckv_attend_static, lib.ckv_cache_append, lib.ckv_cache_put_batch,
+              lib.ckv_route, lib.ckv_project))
 
 
 def _ptr(x) -> Optional[int]:
@@ -179,6 +180,10 @@ def ckv_cache_put(ctx, user: int, L: int, idx_K, idx_V, user_K, user_V, d_user: 
 
 
 def ckv_cache_put_batch(ctx, users, hist_off, idx_K, idx_V, user_K, user_V, d_user: int, stream=None) -> None:
+    stream = _stream(stream)
+    st = _pycall.put(_PUT, ctx or 0, users, hist_off, idx_K, idx_V, user_K, user_V, d_user, stream or 0)
+    if st is not None:
+        return _check(ctx, st, "ckv_cache_put_batch")
     users, hist_off = _host_i64(users), _host_i64(hist_off)
     if hist_off.shape[0] != users.shape[0] + 1:
         raise ValueError("hist_off must have len(users) + 1 entries")
@@ -321,6 +326,10 @@ def ckv_route(device: int, n: int, n_groups: int, d_in: int, n_entries: int, x, 
               stream=None) -> None:
     """Router indices of n positions: x [n][d_in], W [G][n_entries][d_in] (bf16, device), bias [G][n_entries] fp32
     or None, idx_out [n][G] int32 (device); variant 0 / 2 = tcgen05 kernel, 1 = warp-level tensor-core kernel."""
+    stream = _stream(stream)
+    st = _pycall.prefill(_ROUTE, device, n, n_groups, d_in, n_entries, x, W, bias, idx_out, int(variant), stream or 0)
+    if st is not None:
+        return _check(None, st, "ckv_route")
     _check(None, lib.ckv_route(device, n, n_groups, d_in, n_entries, _ptr(x), _ptr(W), _ptr(bias), _ptr(idx_out),
                                int(variant), _stream(stream)), "ckv_route")
 
@@ -328,5 +337,9 @@ def ckv_route(device: int, n: int, n_groups: int, d_in: int, n_entries: int, x, 
 def ckv_project(device: int, n: int, n_groups: int, d_in: int, d_out: int, x, W, bias, out, stream=None) -> None:
     """User-specific low-dimensional projection: x [n][d_in], W [G][d_out][d_in] (bf16, device), bias [G][d_out]
     fp32 or None, out [n][G][d_out] bf16 (device)."""
+    stream = _stream(stream)
+    st = _pycall.prefill(_PROJECT, device, n, n_groups, d_in, d_out, x, W, bias, out, None, stream or 0)
+    if st is not None:
+        return _check(None, st, "ckv_project")
     _check(None, lib.ckv_project(device, n, n_groups, d_in, d_out, _ptr(x), _ptr(W), _ptr(bias), _ptr(out),
                                  _stream(stream)), "ckv_project")
