@@ -465,13 +465,11 @@ void arena_give(ckv_ctx* ctx, int64_t base, int64_t units)
 // What the warp-level tensor-core kernel's work consists of: units of (chunk, group, query block) and their 32-position tiles.
 struct MmaWork {
     int64_t units = 0, tiles = 0, min_tiles = INT64_MAX, max_tiles = 0;  // of one group
-    int32_t M = -1;
-    bool alike = true;  // every unit costs the same
-    void add(int64_t L, int32_t m, int qpw, int64_t chunk)
+    bool alike = true;  // every unit costs the same, if min_tiles = max_tiles
+    // a request of `blocks` query blocks (as many as every other if `same`), chunks of `chunk` positions
+    void add(int64_t L, int64_t blocks, bool same, int64_t chunk)
     {
-        const int64_t blocks = (m + qpw - 1) / qpw;
-        if (M < 0) M = m;
-        alike = alike && m == M && L <= chunk;
+        alike = alike && same && L <= chunk;
         const int64_t chunks = L > chunk ? (L + chunk - 1) / chunk : 1, t = (std::min(L, chunk) + 31) / 32;
         units += blocks * chunks;
         tiles += blocks * ((L + 31) / 32);
@@ -507,26 +505,74 @@ int mma_parts(const ckv_ctx* ctx, const MmaWork& w, int qpw, double* tile_times)
     return best;
 }
 
-int mma_qpw(const ckv_ctx* ctx, int64_t tiles16, int max_M)
+// Query blocks of a request for a warp that holds qpw = 16, 32 or 48 of them (constants, so that planning a long list does
+// not divide).
+inline int64_t mma_blocks(uint32_t M, int qpw) { return qpw == 16 ? (M + 15) / 16 : qpw == 32 ? (M + 31) / 32 : (M + 47) / 48; }
+
+// A request list as the dispatch sees it.  One loop of its own over the requests, which gathers what every estimate below
+// needs: next to the look-ups the sums cost 17 ns a request instead of 3 (a look-up is a cache miss, and fewer of them are
+// in flight with more work between them), and a walk per estimate another 3 each.
+struct ListShape {
+    const int qpw_wide;                 // queries of a warp that holds several tiles of them
+    int32_t max_M = 0, min_M = INT32_MAX, max_L = 0, min_L = INT32_MAX;  // of requests with a query
+    int64_t active = 0, positions = 0;  // how many have one, their history lengths in all
+    int64_t blocks128 = 0, tiles64 = 0; // blocks of 128 queries, and (block, 64 positions) tiles
+    int64_t units16 = 0, tiles16 = 0, units_wide = 0, tiles_wide = 0;  // MmaWork of unchunked histories
+    explicit ListShape(int head_dim) : qpw_wide(mma_wide_queries(head_dim)) {}
+    void add(int32_t length, int32_t queries)
+    {
+        if (queries <= 0) return;
+        const uint32_t L = (uint32_t)length, M = (uint32_t)queries;
+        ++active;
+        max_M = std::max(max_M, queries);
+        min_M = std::min(min_M, queries);
+        max_L = std::max(max_L, length);
+        min_L = std::min(min_L, length);
+        positions += L;
+        const int64_t b = (M + 127) / 128, b16 = mma_blocks(M, 16), bw = mma_blocks(M, qpw_wide), t = (L + 31) / 32;
+        blocks128 += b;
+        tiles64 += b * ((L + 63) / 64);
+        units16 += b16;
+        tiles16 += b16 * t;
+        units_wide += bw;
+        tiles_wide += bw * t;
+    }
+    bool same_M() const { return min_M == max_M || active == 0; }
+    bool single() const { return active > 0 && max_M == 1; }  // one query each
+    MmaWork mma(int qpw) const  // unchunked, qpw = 16 or qpw_wide
+    {
+        MmaWork w;
+        if (active == 0) return w;
+        w.units = qpw == 16 ? units16 : units_wide;
+        w.tiles = qpw == 16 ? tiles16 : tiles_wide;
+        w.min_tiles = (min_L + 31) / 32;
+        w.max_tiles = (max_L + 31) / 32;
+        w.alike = same_M();
+        return w;
+    }
+};
+
+int mma_qpw(const ckv_ctx* ctx, const ListShape& s)
 {
     const int D = ctx->cfg.head_dim;
-    return mma_queries_per_warp(D, max_M, tiles16 * ctx->cfg.n_groups >= (int64_t)20 * ctx->n_sms * mma_warps_per_sm(D, 16));
+    return mma_queries_per_warp(D, s.max_M, s.tiles16 * ctx->cfg.n_groups >= (int64_t)20 * ctx->n_sms * mma_warps_per_sm(D, 16));
 }
 
-// Queries per warp and warps per unit; `each(add)` calls add(L, M) for every request with a query.  Holding more queries
-// per warp saves gathers and lengthens a tile (measured 1.45 times for 32 queries at head_dim 64, 1.3 for 48 at 32), but
-// leaves fewer units to spread: lists of few long histories are better off with 16.
+// Queries per warp and warps per unit of histories cut into chunks of `chunk`; `each(add)` calls add(L, M) for every request
+// with a query.  Holding more queries per warp saves gathers and lengthens a tile (measured 1.45 times for 32 queries at
+// head_dim 64, 1.3 for 48 at 32), but leaves fewer units to spread: lists of few long histories are better off with 16.
 template <typename F>
-void mma_shape(const ckv_ctx* ctx, int64_t tiles16, int max_M, int64_t chunk, F&& each, int& qpw, int& parts)
+void mma_shape(const ckv_ctx* ctx, const ListShape& s, int64_t chunk, F&& each, int& qpw, int& parts)
 {
     auto estimate = [&](int q, int& p) {
         MmaWork w;
-        each([&](int32_t L, int32_t M) { w.add(L, M, q, chunk); });
+        if (chunk >= s.max_L) w = s.mma(q);
+        else each([&](int32_t L, int32_t M) { w.add(L, mma_blocks(M, q), s.same_M(), chunk); });
         double t;
         p = mma_parts(ctx, w, q, &t);
         return t;
     };
-    qpw = mma_qpw(ctx, tiles16, max_M);
+    qpw = mma_qpw(ctx, s);
     const double t = estimate(qpw, parts);
     int p16;
     if (qpw > 16 && estimate(16, p16) < (qpw == 32 ? 1.45 : 1.3) * t) {
@@ -535,29 +581,6 @@ void mma_shape(const ckv_ctx* ctx, int64_t tiles16, int max_M, int64_t chunk, F&
     }
 }
 
-// A request list as the dispatch sees it.
-struct ListShape {
-    int32_t n = 0, max_M = 0, max_L = 0;
-    int64_t active = 0, positions = 0;  // requests with a query, their history lengths in all
-    int64_t blocks128 = 0, tiles64 = 0; // blocks of 128 queries, and (block, 64 positions) tiles
-    bool single = true;                 // one query each
-    MmaWork mma;                        // for 16 queries per warp
-    void add(int32_t L, int32_t M)
-    {
-        ++n;
-        max_M = std::max(max_M, M);
-        if (M <= 0) return;
-        ++active;
-        positions += L;
-        max_L = std::max(max_L, L);
-        single = single && M == 1;
-        const int64_t b = (M + 127) / 128;
-        blocks128 += b;
-        tiles64 += b * ((L + 63) / 64);
-        mma.add(L, M, 16, INT32_MAX);
-    }
-};
-
 // Chunk length of the tcgen05 kernel: the one with the shortest estimated run, in microseconds.  Three persistent workers
 // per SM walk a (chunk, group, 128 queries) unit alone; measured, a worker takes 1 us per 64 positions when it has the SM
 // to itself and 1.4 next to two others, 1.5 per unit, the launch 6, and merging chunks 6 and 0.007 per chunk.  Units of one size
@@ -565,7 +588,8 @@ struct ListShape {
 int64_t umma_chunk(const ckv_ctx* ctx, const ListShape& s, double* time = nullptr)
 {
     const double workers = 3.0 * ctx->n_sms, G = ctx->cfg.n_groups;
-    const bool alike = s.mma.alike && s.mma.min_tiles == s.mma.max_tiles;
+    const MmaWork w16 = s.mma(16);
+    const bool alike = w16.alike && w16.min_tiles == w16.max_tiles;
     int64_t best = 16384;
     double best_t = 1e300;
     for (int64_t n = (s.max_L + 16383) / 16384, last = 0; n <= 512 && last != 256; n += (n + 15) / 16) {
@@ -611,12 +635,12 @@ int choose_family(const ckv_ctx* ctx, bool with_vis, const ListShape& s)
     bool few = false;
     if (can_umma && can_mma && !with_vis && max_M >= 48 && max_M <= 96 && n_active > 0) {
         double tile_times, t_umma;
-        mma_parts(ctx, s.mma, 16, &tile_times);
+        mma_parts(ctx, s.mma(16), 16, &tile_times);
         umma_chunk(ctx, s, &t_umma);
         few = 4 + 1.2 * tile_times < t_umma;
     }
     // One query per user: the pool-side factorisation trades the row gathers for two tables per (user, group).
-    const bool can_fact = plain && s.single && n_active > 0 &&
+    const bool can_fact = plain && s.single() &&
                           fact_supported(ctx->cfg.dtype, ctx->cfg.head_dim, ctx->d_user, ctx->n_entries);
     // It pays when histories are long against the pool and there are enough (user, group) pairs to fill the SMs
     // (one CTA holds a whole pair; the gathering kernel splits long histories over CTAs).  Cost lines fitted to
@@ -696,7 +720,6 @@ ckv_status build_plan(ckv_ctx* ctx, Plan& pl, int32_t n, const int64_t* users, c
                       int n_ranges, const int32_t* r_user, cudaStream_t s)
 {
     std::vector<Req> reqs((size_t)n);
-    ListShape shape;
     for (int32_t k = 0; k < n; ++k) {
         if (k + 12 < n) ctx->users.prefetch(users[k + 12]);
         const UserEntry* f = ctx->users.find(users[k]);
@@ -709,18 +732,19 @@ ckv_status build_plan(ckv_ctx* ctx, Plan& pl, int32_t n, const int64_t* users, c
         r.M = q_off[k + 1] - q_off[k];
         r.part0 = -1;
         r.n_chunks = 1;
-        shape.add(r.L, r.M);
     }
-    const int32_t max_M = pl.max_M = shape.max_M;
+    ListShape shape(ctx->cfg.head_dim);
+    for (const Req& r : reqs) shape.add(r.L, r.M);
+    pl.max_M = shape.max_M;
     pl.n_req = n;
     pl.family = choose_family(ctx, with_vis, shape);
     if (pl.family == 0) return CKV_ERR_UNSUPPORTED;
     const int64_t C = ctx->opt_split > 0 && pl.family != 4 ? ctx->opt_split : auto_split_len(ctx, shape, pl.family);
     pl.parts = 1;
     if (pl.family == 2) {
-        if (ctx->opt_split > 0) pl.qpw = mma_qpw(ctx, shape.mma.tiles, max_M);
+        if (ctx->opt_split > 0) pl.qpw = mma_qpw(ctx, shape);
         else
-            mma_shape(ctx, shape.mma.tiles, max_M, C, [&](auto&& add) {
+            mma_shape(ctx, shape, C, [&](auto&& add) {
                 for (const Req& r : reqs)
                     if (r.M > 0) add(r.L, r.M);
             }, pl.qpw, pl.parts);
@@ -729,6 +753,7 @@ ckv_status build_plan(ckv_ctx* ctx, Plan& pl, int32_t n, const int64_t* users, c
     std::vector<int32_t> split;
     items.reserve((size_t)n);
     int64_t part_rows = 0;
+    pl.split_items = 0;
     if (pl.family == 4) n_ranges = 1;  // its three launches work on all requests at once
     pl.n_ranges = n_ranges;
     for (int32_t k = 0, rg = 0; k <= n; ++k) {
@@ -741,7 +766,7 @@ ckv_status build_plan(ckv_ctx* ctx, Plan& pl, int32_t n, const int64_t* users, c
         if (k == n) break;
         Req& r = reqs[k];
         if (r.M <= 0) continue;
-        const int64_t nc = r.L == 0 ? 1 : (r.L + C - 1) / C;
+        const int64_t nc = r.L <= C ? 1 : (r.L + C - 1) / C;  // (most lists are not cut: no division for them)
         r.n_chunks = (int32_t)nc;
         if (nc == 1) {
             items.push_back(Item{k, 0, r.L, -1});
@@ -755,6 +780,7 @@ ckv_status build_plan(ckv_ctx* ctx, Plan& pl, int32_t n, const int64_t* users, c
             items.push_back(Item{k, b, (int32_t)std::min<int64_t>(C, r.L - b), (int32_t)(part_rows + c * r.M)});
         }
         part_rows += nc * r.M;
+        pl.split_items += (int32_t)nc;
     }
     // longest chunks first (inside every range): the tail of a grid is made of short ones
     std::vector<uint32_t> order(items.size()), tmp, count;
@@ -762,8 +788,6 @@ ckv_status build_plan(ckv_ctx* ctx, Plan& pl, int32_t n, const int64_t* users, c
         order_longest_first(items, (size_t)pl.r_item[rg], (size_t)pl.r_item[rg + 1], order, tmp, count);
     pl.n_items = (int32_t)items.size();
     pl.n_split = (int32_t)split.size();
-    pl.split_items = 0;
-    for (const Item& it : items) pl.split_items += it.part_row >= 0;
     pl.part_rows = part_rows;
 
     // the tables are laid out in the slot's pinned block and go to the device in one copy
@@ -1469,8 +1493,7 @@ struct InlineList {
 ckv_status inline_list(ckv_ctx* ctx, int32_t n, const int64_t* users, const int32_t* q_off, bool with_vis, InlineList& x)
 {
     if (n > kInlineReqs || ctx->opt_split > 0 || ctx->opt_kernel > 2 || ctx->opt_loader == 2) return CKV_OK;
-    ListShape shape;
-    int32_t min_L = INT32_MAX;
+    ListShape shape(ctx->cfg.head_dim);
     for (int32_t k = 0; k < n; ++k) {
         const UserEntry* f = ctx->users.find(users[k]);
         if (!f) return CKV_ERR_UNKNOWN_USER;
@@ -1478,17 +1501,14 @@ ckv_status inline_list(ckv_ctx* ctx, int32_t n, const int64_t* users, const int3
         shape.add(f->L, M);
         if (M <= 0) continue;
         x.tab.r[x.n++] = InlineReq{(uint32_t)(f->base >> 5), f->L, q_off[k], M};
-        min_L = std::min(min_L, f->L);
     }
     x.max_M = shape.max_M;
     const int family = choose_family(ctx, with_vis, shape);
     if ((family != 1 && family != 2) || auto_split_len(ctx, shape, family) < shape.max_L) return CKV_OK;
     if (family == 2)
-        mma_shape(ctx, shape.mma.tiles, x.max_M, INT32_MAX, [&](auto&& add) {
-            for (int32_t k = 0; k < x.n; ++k) add(x.tab.r[k].L, x.tab.r[k].M);
-        }, x.qpw, x.parts);
+        mma_shape(ctx, shape, INT32_MAX, [](auto&&) {}, x.qpw, x.parts);
     // longest first, as in a plan: the tail of the grid is made of short ones
-    if (shape.max_L != min_L && (int64_t)x.n * ctx->cfg.n_groups > ctx->n_sms)
+    if (shape.max_L != shape.min_L && (int64_t)x.n * ctx->cfg.n_groups > ctx->n_sms)
         std::sort(x.tab.r, x.tab.r + x.n, [](const InlineReq& a, const InlineReq& b) { return a.L > b.L; });
     x.family = family;
     return CKV_OK;
@@ -2076,7 +2096,7 @@ extern "C" ckv_status ckv_attend_static(ckv_ctx* ctx, int32_t n, const int64_t* 
     // the plan, in fixed-size host arrays; nothing is enqueued before the request is known to fit
     StaticRow rows[kStaticMaxReqs];
     const int D = ctx->cfg.head_dim, G = ctx->cfg.n_groups;
-    ListShape shape;
+    ListShape shape(ctx->cfg.head_dim);
     for (int32_t k = 0; k < n; ++k) {
         const UserEntry* f = ctx->users.find(users[k]);
         if (!f) return CKV_ERR_UNKNOWN_USER;

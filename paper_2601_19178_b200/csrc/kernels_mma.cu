@@ -756,7 +756,7 @@ bool mma_supported(int dtype, int head_dim, int d_user)
 int mma_queries_per_warp(int D, int max_M, bool big)
 {
     if (!big || max_M <= 16) return 16;
-    return D == 64 ? 32 : max_M > 32 ? 48 : 16;
+    return D == 64 || max_M > 32 ? mma_wide_queries(D) : 16;
 }
 
 // warps of the kernel that are resident on an SM

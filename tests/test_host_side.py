@@ -1,0 +1,84 @@
+"""The library's host side on the CPU: its object files linked with tests/fake_cudart.cpp instead of the CUDA runtime.
+Kernels do not run there; what is tested is what a call does before and between them."""
+import ctypes as C
+import glob
+import importlib.util
+import os
+import subprocess
+import time
+
+import numpy as np
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+class Config(C.Structure):
+    _fields_ = [(n, C.c_int32) for n in ("n_groups", "head_dim", "dtype", "out_dtype", "mode")] + \
+        [("scale", C.c_float), ("device", C.c_int32)]
+
+
+def ptr(a):
+    return a.ctypes.data_as(C.c_void_p)
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    spec = importlib.util.spec_from_file_location("ckv_build", os.path.join(ROOT, "paper_2601_19178_b200", "build.py"))
+    mod = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(mod)
+    mod.build()
+    so = str(tmp_path_factory.mktemp("host") / "libckv_host.so")
+    subprocess.run(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-Wl,-Bsymbolic", "-I/usr/local/cuda/include", "-o", so,
+                    *sorted(glob.glob(os.path.join(mod.OBJ, "*.o"))), os.path.join(ROOT, "tests", "fake_cudart.cpp")],
+                   check=True)
+    lib = C.CDLL(so)
+    lib.fake_count.restype = C.c_long
+    return lib
+
+
+def device_block(lib, size):
+    p = C.c_void_p()
+    assert lib.cudaMalloc(C.byref(p), C.c_size_t(size)) == 0
+    return p
+
+
+def context(lib, G=4, D=32, d_user=1, m=2048):
+    """A bf16 softmax context with a pool, and a block that stands for any device input."""
+    ctx = C.c_void_p()
+    assert lib.ckv_create(C.byref(Config(G, D, 1, 1, 0, 0.0, 0)), C.byref(ctx)) == 0
+    block = device_block(lib, G * m * D * 2)
+    assert lib.ckv_pool_load(ctx, block, block, m, D - d_user, None) == 0
+    return ctx, block
+
+
+def put(lib, ctx, block, users, lens, d_user=1):
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    return lib.ckv_cache_put_batch(ctx, len(users), ptr(users), ptr(off), block, block, block, block, d_user, None)
+
+
+def test_planning_a_list_costs_little_more_than_its_tables(lib):
+    """A request list that the context has not seen: at most half as much again as looking its users up and writing and
+    copying its tables (1.3 times; sums for the dispatch next to the look-ups, further walks over the list for its estimates
+    and a division per request made it 1.6)."""
+    n = 65536
+    ctx, block = context(lib)
+    users = np.arange(n, dtype=np.int64) * 7919 + 3
+    assert put(lib, ctx, block, users, np.full(n, 512)) == 0
+    q_off = np.arange(n + 1, dtype=np.int32) * 16
+    rng = np.random.default_rng(0)
+    lists = [rng.permutation(users) for _ in range(9)]  # more than the context keeps plans
+    ratio = 1e9
+    for _ in range(4):
+        plan, floor = [], []
+        for u in lists:
+            t0 = time.perf_counter()
+            assert lib.ckv_attend(ctx, n, ptr(u), ptr(q_off), block, block, None) == 0
+            t1 = time.perf_counter()
+            assert lib.fake_plan_floor(lib.ckv_user_length, ctx, n, ptr(u), ptr(q_off)) == 0
+            t2 = time.perf_counter()
+            plan.append(t1 - t0)
+            floor.append(t2 - t1)
+        ratio = min(ratio, min(plan) / min(floor))
+    lib.ckv_destroy(ctx)
+    assert ratio < 1.5
