@@ -6,6 +6,7 @@
 #include <cmath>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <string>
@@ -157,6 +158,75 @@ struct Plan {
     uint64_t last_use = 0;
 };
 
+// Two words {error, done} in mapped host memory, through which a kernel reports to the host: for one call of the
+// context-free router, or for the life of a context.  They are handed out of one block that the process keeps, and given back,
+// under a lock (a block of its own for every context made ckv_create take 1.8 to 3.4 ms instead of 0.4); who finds none left
+// gets an allocation of its own.
+class HostFlag {
+    static constexpr int kSlots = 512, kStride = 16;  // a cache line each
+    struct Pool {
+        int* p = nullptr;
+        uint64_t generation = 0, used[kSlots / 64] = {};
+    };
+    static std::mutex mu_;
+    static Pool pool_;
+    int slot_ = -1;
+    uint64_t generation_ = 0;
+
+    static bool alloc(int** p, int words)
+    {
+        if (cudaHostAlloc((void**)p, words * sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable) == cudaSuccess) return true;
+        cudaGetLastError();
+        *p = nullptr;
+        return false;
+    }
+    // the block, anew if it went with a device that the process has reset since
+    static bool have_block()
+    {
+        cudaPointerAttributes at;
+        if (pool_.p && cudaPointerGetAttributes(&at, pool_.p) == cudaSuccess && at.type == cudaMemoryTypeHost) return true;
+        cudaGetLastError();
+        const uint64_t generation = pool_.generation + 1;
+        pool_ = Pool();
+        pool_.generation = generation;
+        return alloc(&pool_.p, kSlots * kStride);
+    }
+
+public:
+    enum Use { kRoute, kContext };  // the router's are the first kRouteSlots: the kernel counts its blocks per slot
+    int* p = nullptr;
+    int slot() const { return slot_; }
+    explicit HostFlag(Use use)
+    {
+        {
+            std::lock_guard<std::mutex> lock(mu_);
+            if (!have_block()) return;
+            const int end = use == kRoute ? kRouteSlots : kSlots;
+            for (int i = use == kRoute ? 0 : kRouteSlots; i < end && slot_ < 0; ++i)
+                if (!(pool_.used[i / 64] >> (i % 64) & 1)) slot_ = i;
+            if (slot_ >= 0) {
+                pool_.used[slot_ / 64] |= 1ull << (slot_ % 64);
+                generation_ = pool_.generation;
+                p = pool_.p + slot_ * kStride;
+            }
+        }
+        if (p || alloc(&p, 2)) p[0] = p[1] = 0;
+    }
+    ~HostFlag()
+    {
+        if (slot_ < 0) {
+            if (p) cudaFreeHost(p);
+            return;
+        }
+        std::lock_guard<std::mutex> lock(mu_);
+        if (generation_ == pool_.generation) pool_.used[slot_ / 64] &= ~(1ull << (slot_ % 64));
+    }
+    HostFlag(const HostFlag&) = delete;
+    HostFlag& operator=(const HostFlag&) = delete;
+};
+std::mutex HostFlag::mu_;
+HostFlag::Pool HostFlag::pool_;
+
 constexpr int kMaxPlans = 4;
 
 struct DeviceGuard {
@@ -202,7 +272,8 @@ struct ckv_ctx {
     uint64_t generation = 1;
     // scratch
     DevBuf stage_q, stage_out, stage_vis, vmax, partials;
-    int* h_flag = nullptr;     // pinned, mapped: {bad, done} of a kernel that checks indices (d_err + 1: its counter)
+    std::unique_ptr<HostFlag> words;
+    int* h_flag = nullptr;     // its words: {bad, done} of a kernel that checks indices (d_err + 1: its counter)
     void* put_host = nullptr;  // pinned table of a put of many users
     size_t put_host_cap = 0;
     DevBuf put_dev, put_in[4];  // its device copy; staged host inputs up to kKeepStaged bytes each
@@ -988,14 +1059,19 @@ ckv_status ckv_create(const ckv_config* cfg, ckv_ctx** out)
                                   : (cfg->mode == CKV_SOFTMAX ? 1.0f / std::sqrt((float)cfg->head_dim) : 1.0f);
     DeviceGuard dg(cfg->device);
     if (!dg.ok || cudaMalloc((void**)&ctx->d_err, 2 * sizeof(int)) != cudaSuccess ||
-        cudaMemset(ctx->d_err, 0, 2 * sizeof(int)) != cudaSuccess ||
-        cudaHostAlloc((void**)&ctx->h_flag, 2 * sizeof(int), cudaHostAllocMapped) != cudaSuccess) {
+        cudaMemset(ctx->d_err, 0, 2 * sizeof(int)) != cudaSuccess) {
         cudaGetLastError();
         if (ctx->d_err) cudaFree(ctx->d_err);
         delete ctx;
         return CKV_ERR_CUDA;
     }
-    ctx->h_flag[0] = ctx->h_flag[1] = 0;
+    ctx->words.reset(new (std::nothrow) HostFlag(HostFlag::kContext));
+    if (!ctx->words || !ctx->words->p) {
+        cudaFree(ctx->d_err);
+        delete ctx;
+        return CKV_ERR_CUDA;
+    }
+    ctx->h_flag = ctx->words->p;
     if (cudaDeviceGetAttribute(&ctx->n_sms, cudaDevAttrMultiProcessorCount, cfg->device) != cudaSuccess || ctx->n_sms < 1) {
         cudaGetLastError();
         ctx->n_sms = 148;
@@ -1014,7 +1090,7 @@ ckv_status ckv_destroy(ckv_ctx* ctx)
                     ctx->put_dev.p, ctx->put_in[0].p, ctx->put_in[1].p, ctx->put_in[2].p, ctx->put_in[3].p};
     for (void* b : bufs)
         if (b) cudaFree(b);
-    if (ctx->h_flag) cudaFreeHost(ctx->h_flag);
+    ctx->words.reset();  // (behind cudaFree, which waits: no kernel of the context can write them any more)
     if (ctx->put_host) cudaFreeHost(ctx->put_host);
     for (auto& e : ctx->ev)
         if (e) cudaEventDestroy(e);
@@ -1412,57 +1488,6 @@ ckv_status run_mma(ckv_ctx* ctx, int D, int max_M, int qpw, int parts, const Att
 }  // extern "C"
 
 namespace {
-
-// Two words {error, done} in pinned host memory for one call of the context-free router: 64 pairs for the process, handed
-// out and given back under a lock (a call beyond that many at the same time gets one of its own, without the second word).
-class HostFlag {
-    static constexpr int kSlots = kRouteSlots, kStride = 16;  // a cache line each
-    static std::mutex mu_;
-    static int* pool_;
-    static uint64_t used_;
-    int slot_ = -1;
-
-public:
-    int* p = nullptr;
-    int slot() const { return slot_; }
-    HostFlag()
-    {
-        {
-            std::lock_guard<std::mutex> lock(mu_);
-            if (!pool_ && cudaHostAlloc((void**)&pool_, kSlots * kStride * sizeof(int),
-                                        cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
-                cudaGetLastError();
-                pool_ = nullptr;
-                return;
-            }
-            for (int i = 0; i < kSlots && slot_ < 0; ++i)
-                if (!(used_ >> i & 1)) slot_ = i;
-            if (slot_ >= 0) {
-                used_ |= 1ull << slot_;
-                p = pool_ + slot_ * kStride;
-            }
-        }
-        if (!p && cudaHostAlloc((void**)&p, 2 * sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
-            cudaGetLastError();
-            p = nullptr;
-        }
-        if (p) p[0] = p[1] = 0;
-    }
-    ~HostFlag()
-    {
-        if (slot_ < 0) {
-            if (p) cudaFreeHost(p);
-            return;
-        }
-        std::lock_guard<std::mutex> lock(mu_);
-        used_ &= ~(1ull << slot_);
-    }
-    HostFlag(const HostFlag&) = delete;
-    HostFlag& operator=(const HostFlag&) = delete;
-};
-std::mutex HostFlag::mu_;
-int* HostFlag::pool_ = nullptr;
-uint64_t HostFlag::used_ = 0;
 
 constexpr size_t kPipeMinBytes = size_t(4) << 20;  // host query buffers below this are not worth pipelining
 constexpr size_t kPipeManyBytes = size_t(96) << 20;  // from here on: eight ranges instead of four
@@ -1872,7 +1897,7 @@ ckv_status ckv_route(int32_t device, int32_t n, int32_t n_groups, int32_t d_in, 
     if (variant == 1) {
         e = launch_route(d_in, x, W, bias, n, n_entries, n_groups, idx_out, s);
     } else {
-        HostFlag flag;
+        HostFlag flag(HostFlag::kRoute);
         if (!flag.p) return CKV_ERR_OOM;
         e = launch_route_umma(d_in, x, W, bias, n, n_entries, n_groups, idx_out, flag.p, flag.slot(), s);
         if (e == cudaSuccess) e = wait_done(flag.p + 1, s);

@@ -16,7 +16,7 @@
 namespace {
 std::mutex mu;
 std::map<std::string, long> counts, fail_at;        // calls so far; the call that fails (counted from the reset)
-std::map<const char*, size_t> device_blocks;
+std::map<const char*, size_t> device_blocks, host_blocks;
 long launched[6];                                    // of the last cudaLaunchKernelExC: grid, threads, shared memory, cluster
 
 cudaError_t called(const char* name)
@@ -31,11 +31,21 @@ cudaError_t called(const char* name)
 cudaError_t take(void** p, size_t bytes, bool device)
 {
     *p = std::aligned_alloc(512, (bytes + 511) / 512 * 512 + 512);
-    if (device) {
-        std::lock_guard<std::mutex> lock(mu);
-        device_blocks[(const char*)*p] = bytes;
-    }
+    std::lock_guard<std::mutex> lock(mu);
+    (device ? device_blocks : host_blocks)[(const char*)*p] = bytes;
     return cudaSuccess;
+}
+cudaError_t give(void* p, std::map<const char*, size_t>& blocks)
+{
+    std::lock_guard<std::mutex> lock(mu);
+    blocks.erase((const char*)p);
+    std::free(p);
+    return cudaSuccess;
+}
+bool holds(const std::map<const char*, size_t>& blocks, const char* p)
+{
+    auto it = blocks.upper_bound(p);
+    return it != blocks.begin() && p < std::prev(it)->first + std::prev(it)->second;
 }
 int encode(...) { return 0; }  // cuTensorMapEncodeTiled
 }  // namespace
@@ -56,21 +66,20 @@ API void fake_fail(const char* name, long nth)
     std::lock_guard<std::mutex> lock(mu);
     fail_at[name] = counts[name] + nth;
 }
+API void fake_device_reset()  // what the runtime has allocated is gone
+{
+    std::lock_guard<std::mutex> lock(mu);
+    device_blocks.clear();
+    host_blocks.clear();
+}
 API const long* fake_launched() { return launched; }
 
 // ---- the runtime calls the library makes
 API cudaError_t cudaMalloc(void** p, size_t n) { CALLED(); return take(p, n, true); }
-API cudaError_t cudaFree(void* p)
-{
-    CALLED();
-    std::lock_guard<std::mutex> lock(mu);
-    device_blocks.erase((const char*)p);
-    std::free(p);
-    return cudaSuccess;
-}
+API cudaError_t cudaFree(void* p) { CALLED(); return give(p, device_blocks); }
 API cudaError_t cudaMallocHost(void** p, size_t n) { CALLED(); return take(p, n, false); }
 API cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { CALLED(); return take(p, n, false); }
-API cudaError_t cudaFreeHost(void* p) { CALLED(); std::free(p); return cudaSuccess; }
+API cudaError_t cudaFreeHost(void* p) { CALLED(); return give(p, host_blocks); }
 API cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) { CALLED(); std::memcpy(d, s, n); return cudaSuccess; }
 API cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) { CALLED(); std::memcpy(d, s, n); return cudaSuccess; }
 API cudaError_t cudaMemset(void* d, int v, size_t n) { CALLED(); std::memset(d, v, n); return cudaSuccess; }
@@ -79,9 +88,8 @@ API cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void* p
     CALLED();
     std::memset(a, 0, sizeof *a);
     std::lock_guard<std::mutex> lock(mu);
-    auto it = device_blocks.upper_bound((const char*)p);
-    a->type = cudaMemoryTypeUnregistered;
-    if (it != device_blocks.begin() && (const char*)p < std::prev(it)->first + std::prev(it)->second) a->type = cudaMemoryTypeDevice;
+    a->type = holds(device_blocks, (const char*)p) ? cudaMemoryTypeDevice
+              : holds(host_blocks, (const char*)p) ? cudaMemoryTypeHost : cudaMemoryTypeUnregistered;
     return cudaSuccess;
 }
 API cudaError_t cudaGetDeviceCount(int* n) { *n = 1; return cudaSuccess; }

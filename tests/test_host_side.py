@@ -82,3 +82,35 @@ def test_planning_a_list_costs_little_more_than_its_tables(lib):
         ratio = min(ratio, min(plan) / min(floor))
     lib.ckv_destroy(ctx)
     assert ratio < 1.5
+
+
+def test_contexts_share_one_block_of_mapped_words(lib):
+    """Pinned memory is what creating a context spent its time on.  A reset of the device takes the block along."""
+    def create(n):
+        ctxs = [C.c_void_p() for _ in range(n)]
+        for c in ctxs:
+            assert lib.ckv_create(C.byref(Config(4, 32, 1, 1, 0, 0.0, 0)), C.byref(c)) == 0
+        return ctxs
+
+    def destroy(ctxs):
+        for c in ctxs:
+            assert lib.ckv_destroy(c) == 0
+
+    destroy(create(2))
+    lib.fake_reset()
+    for _ in range(3):
+        destroy(create(20))
+    assert lib.fake_count(b"cudaHostAlloc") + lib.fake_count(b"cudaMallocHost") == 0
+    live = create(500)  # no words for two at once: 448 in the block, an allocation for each of the others
+    assert lib.fake_count(b"cudaHostAlloc") == 500 - 448
+    destroy(live)
+    assert lib.fake_count(b"cudaFreeHost") == 500 - 448
+    before = create(2)
+    lib.fake_device_reset()
+    lib.fake_reset()
+    after = create(447)
+    assert lib.fake_count(b"cudaHostAlloc") == 1
+    destroy(before)  # words of the old block: nothing of the new one comes free
+    after += create(2)
+    assert lib.fake_count(b"cudaHostAlloc") == 2
+    destroy(after)
