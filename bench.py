@@ -53,7 +53,7 @@ XU_PER_SM_CLK = 16
 L1_PIPE_BYTES_PER_SM_CLK = 128
 TRAFFIC_JSON = os.path.join(ROOT, "profiles", "traffic.json")
 CSRC = os.path.join(ROOT, "paper_2601_19178_b200", "csrc")
-KERNEL_SOURCES = {1: ["kernels_simt.cu"], 2: ["kernels_mma.cu"], 3: ["kernels_umma.cu"], 4: ["kernels_fact.cu"]}
+KERNEL_SOURCES = {1: ["kernels_simt.cu"], 2: ["attend_mma.cuh", "kernels_mma.cu"], 3: ["kernels_umma.cu"], 4: ["kernels_fact.cu"]}
 
 
 def _peaks():

@@ -232,7 +232,7 @@ cudaError_t launch_attend_simt(int dtype, int D, int max_M, bool wide, const Att
 // Merges the partial results of split requests into `out`.
 cudaError_t launch_combine(int D, int max_M, const AttendArgs& a, const int32_t* split_reqs, int n_split, const Launch& l);
 
-// ---- kernels_mma.cu : warp-level tensor-core family (bf16, head_dim 32 or 64, d_user <= 8)
+// ---- kernels_mma.cu, attend_mma.cuh, kernels_mma_*.cu : warp-level tensor-core family (bf16, head_dim 32 or 64, d_user <= 8)
 bool mma_supported(int dtype, int head_dim, int d_user);  // d_user of the shared side(s)
 // big: every resident warp has some twenty tiles of 32 positions x 16 queries to do
 int mma_queries_per_warp(int head_dim, int max_M, bool big);

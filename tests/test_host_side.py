@@ -23,14 +23,20 @@ def ptr(a):
 
 
 @pytest.fixture(scope="module")
-def lib(tmp_path_factory):
+def objects():
+    """The library's object files, one per source file."""
     spec = importlib.util.spec_from_file_location("ckv_build", os.path.join(ROOT, "paper_2601_19178_b200", "build.py"))
     mod = importlib.util.module_from_spec(spec)
     spec.loader.exec_module(mod)
     mod.build()
+    return [os.path.join(mod.OBJ, os.path.basename(f)[:-3] + ".o") for f in sorted(glob.glob(os.path.join(mod.CSRC, "*.cu")))]
+
+
+@pytest.fixture(scope="module")
+def lib(objects, tmp_path_factory):
     so = str(tmp_path_factory.mktemp("host") / "libckv_host.so")
     subprocess.run(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-Wl,-Bsymbolic", "-I/usr/local/cuda/include", "-o", so,
-                    *sorted(glob.glob(os.path.join(mod.OBJ, "*.o"))), os.path.join(ROOT, "tests", "fake_cudart.cpp")],
+                    *objects, os.path.join(ROOT, "tests", "fake_cudart.cpp")],
                    check=True)
     lib = C.CDLL(so)
     lib.fake_count.restype = C.c_long
@@ -55,6 +61,13 @@ def context(lib, G=4, D=32, d_user=1, m=2048):
 def put(lib, ctx, block, users, lens, d_user=1):
     off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
     return lib.ckv_cache_put_batch(ctx, len(users), ptr(users), ptr(off), block, block, block, block, d_user, None)
+
+
+def test_no_object_file_holds_many_forms_of_the_warp_level_kernel(objects):
+    """Its 96 forms in one file took three times as long to compile as all others side by side."""
+    per_file = [subprocess.run(["nm", "-C", o], capture_output=True, text=True, check=True).stdout.count("::attend_mma_kernel<")
+                for o in objects]
+    assert 0 < max(per_file) <= 32
 
 
 def test_planning_a_list_costs_little_more_than_its_tables(lib):
