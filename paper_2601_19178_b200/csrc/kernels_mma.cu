@@ -1,7 +1,6 @@
 // Dispatch of the warp-level tensor-core attention kernel (attend_mma.cuh) and the tensor maps of its TMA loader.
-#include <cuda.h>
-
 #include "ckv_internal.h"
+#include "tensor_map.h"
 
 namespace ckv {
 
@@ -46,30 +45,13 @@ cudaError_t launch_attend_mma(int D, int max_M, int queries_per_warp, int parts,
 // chunk ^ ((row >> 1) & 3)).  maps_out: 2 x 128 bytes, 64-byte aligned.  false if the driver cannot encode them.
 bool make_pool_tensor_maps(int D, int64_t rows, const void* poolK, const void* poolV, void* maps_out)
 {
-    typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                 const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                 CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
     if ((D != 32 && D != 64) || rows < 1 || rows > INT32_MAX) return false;
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q) != cudaSuccess || !fn ||
-        q != cudaDriverEntryPointSuccess) {
-        cudaGetLastError();
-        return false;
-    }
     CUtensorMap* maps = reinterpret_cast<CUtensorMap*>(maps_out);
     const void* src[2] = {poolK, poolV};
-    for (int i = 0; i < 2; ++i) {
-        const cuuint64_t dims[2] = {(cuuint64_t)D, (cuuint64_t)rows};
-        const cuuint64_t strides[1] = {(cuuint64_t)D * 2};
-        const cuuint32_t box[2] = {(cuuint32_t)D, 1};
-        const cuuint32_t estr[2] = {1, 1};
-        const CUresult r = reinterpret_cast<EncodeFn>(fn)(
-            &maps[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(src[i]), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, D == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
-            CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r != CUDA_SUCCESS) return false;
-    }
+    for (int i = 0; i < 2; ++i)
+        if (!encode_rows(&maps[i], src[i], D, rows, D, 1, D == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+                         CU_TENSOR_MAP_L2_PROMOTION_NONE))
+            return false;
     return true;
 }
 

@@ -17,11 +17,11 @@
 // read-out group: 1.41.
 // Every wait is bounded: a time-out raises the CTA's abort flag, the CTA drains, frees its TMEM, reports through
 // the error word and writes nothing.
-#include <cuda.h>
 #include <cuda_bf16.h>
 #include <math_constants.h>
 
 #include "ckv_internal.h"
+#include "tensor_map.h"
 
 namespace ckv {
 namespace {
@@ -429,22 +429,8 @@ __global__ void __launch_bounds__(kThreadsRU, 1)
 // The weights as rows of `d_in` inputs, boxes of 128 rows and at most 64 inputs.
 bool make_weight_map(int d_in, int64_t rows, const void* W, CUtensorMap* map)
 {
-    typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                 const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                 CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-    static const EncodeFn encode = [] {
-        void* fn = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        const bool ok = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q) == cudaSuccess &&
-                        q == cudaDriverEntryPointSuccess;
-        return ok ? reinterpret_cast<EncodeFn>(fn) : nullptr;
-    }();
-    if (!encode) return false;
-    const cuuint64_t dims[2] = {(cuuint64_t)d_in, (cuuint64_t)rows}, strides[1] = {(cuuint64_t)d_in * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)(d_in < 64 ? d_in : 64), (cuuint32_t)kTileN}, estr[2] = {1, 1};
-    return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(W), dims, strides, box, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, d_in < 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
-                  CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    return encode_rows(map, W, d_in, rows, d_in < 64 ? d_in : 64, kTileN, d_in < 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                       CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
 }
 
 template <int DIN>

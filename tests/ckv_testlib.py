@@ -58,3 +58,20 @@ def assert_close(got, want, dtype, what=""):
         if rows.any():
             rel = (err.max(axis=-1)[rows] / denom[..., 0][rows]).max()
             assert rel <= ROW_TOL[dtype], f"{what}: row-normalised error {rel:.3e} > {ROW_TOL[dtype]}"
+
+
+def random_session(dtype, users, length, seed=0, groups=2, head_dim=32, d_user=2, pool=300, scale=0.5):
+    """A context whose outputs are of the size of its queries (so that they can be the next call's): values ~N(0, 1)."""
+    import paper_2601_19178_b200 as ckv
+    g = torch.Generator(device="cuda").manual_seed(seed)
+
+    def rnd(*shape):
+        return torch.randn(shape, generator=g, device="cuda").to(dtype)
+
+    s = ckv.CollectiveKV(groups, head_dim, dtype, "softmax", scale)
+    s.pool_load(rnd(groups, pool, head_dim - d_user), rnd(groups, pool, head_dim - d_user))
+    ids = np.arange(users, dtype=np.int64) * 13 + 5
+    off = np.arange(users + 1, dtype=np.int64) * length
+    idx = [torch.randint(0, pool, (users * length, groups), generator=g, device="cuda", dtype=torch.int32) for _ in range(2)]
+    s.cache_put_batch(ids, off, *idx, rnd(users * length, groups, d_user), rnd(users * length, groups, d_user))
+    return s, ids, rnd

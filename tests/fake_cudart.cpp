@@ -17,10 +17,14 @@ namespace {
 std::mutex mu;
 std::map<std::string, long> counts, fail_at;        // calls so far; the call that fails (counted from the reset)
 std::map<const char*, size_t> device_blocks, host_blocks;
+thread_local bool has_context = false;                // as made by the calls that need one, and by cudaSetDevice
 long launched[6];                                    // of the last cudaLaunchKernelExC: grid, threads, shared memory, cluster
 
 cudaError_t called(const char* name)
 {
+    if (!std::strcmp(name, "cudaSetDevice") || !std::strcmp(name, "cudaMalloc") || !std::strncmp(name, "cudaLaunch", 10) ||
+        !std::strncmp(name, "cudaMem", 7) || !std::strncmp(name, "cudaStream", 10))
+        has_context = true;
     std::lock_guard<std::mutex> lock(mu);
     const long n = ++counts[name];
     auto f = fail_at.find(name);
@@ -47,7 +51,7 @@ bool holds(const std::map<const char*, size_t>& blocks, const char* p)
     auto it = blocks.upper_bound(p);
     return it != blocks.begin() && p < std::prev(it)->first + std::prev(it)->second;
 }
-int encode(...) { return 0; }  // cuTensorMapEncodeTiled
+int encode(...) { return has_context ? 0 : 201; }      // cuTensorMapEncodeTiled: CUDA_ERROR_INVALID_CONTEXT
 }  // namespace
 
 API long fake_count(const char* name)

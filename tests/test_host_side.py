@@ -5,6 +5,7 @@ import glob
 import importlib.util
 import os
 import subprocess
+import threading
 import time
 
 import numpy as np
@@ -127,3 +128,31 @@ def test_contexts_share_one_block_of_mapped_words(lib):
     after += create(2)
     assert lib.fake_count(b"cudaHostAlloc") == 2
     destroy(after)
+
+
+def test_a_threads_first_call_may_need_a_tensor_map(lib):
+    """Encoding one is a driver call, which makes no context current by itself as a launch does: the router's calls, and a
+    pool loaded again into storage that is there, on a thread that has not used the GPU."""
+    G, d, m, n = 2, 64, 1024, 200
+    block = device_block(lib, G * m * d * 2)
+    status = {}
+
+    def route():
+        status["route"] = lib.ckv_route(0, n, G, d, m, block, block, None, block, 0, None)
+
+    ctx, pool = context(lib, G=2, D=64, d_user=4, m=m)
+
+    def load():
+        status["load"] = lib.ckv_pool_load(ctx, pool, pool, m, 60, None)
+
+    for f in (route, load):
+        t = threading.Thread(target=f)
+        t.start()
+        t.join()
+    assert status == {"route": 0, "load": 0}
+    # with its maps the pool can be gathered by TMA
+    users = np.arange(300, dtype=np.int64)
+    assert put(lib, ctx, block, users, np.full(300, 40), d_user=4) == 0
+    assert lib.ckv_set_option(ctx, b"mma_loader", C.c_int64(2)) == 0
+    assert lib.ckv_attend(ctx, 300, ptr(users), ptr(np.arange(301, dtype=np.int32)), block, block, None) == 0
+    lib.ckv_destroy(ctx)
