@@ -4,7 +4,8 @@
 // a cluster share the positions when there are too few of them to fill the SMs).  The positions' inputs sit in TMEM
 // (A operand, lane = position); the group's weight rows stream through a ring of shared-memory stages in tiles of 128
 // entries (B operand, one swizzled TMA box per tile), and every tile is multiplied with both blocks.  The bias is one
-// more K = 16 step of the product, ones times the bias cut into three bf16 parts whose sum is the fp32 bias exactly, so
+// more K = 16 step of the product, ones times the bias cut into three bf16 parts whose sum is the fp32 bias exactly (below
+// 2^-100 the parts are those of 2^100 times the bias and meet 2^-100: bf16 has no room for the last of them there), so
 // the read-out touches no shared memory.  One thread per block issues the products into three 128-column TMEM
 // accumulators in turn; two groups of four warps, one per block (thread = position = TMEM lane), fetch their accumulator
 // into registers, release it at once, and keep a running (best score, entry); the score matrix never leaves the SM.
@@ -31,6 +32,7 @@ constexpr int kEpiWarps = 8, kIssueWarp = kEpiWarps, kIssuers = 2, kLoadWarp = k
 constexpr int kThreadsRU = (kBiasWarp + 1) * 32;  // twelve warps: 168 registers for a read-out thread's 128 columns
 constexpr int kMaxClusterRU = 8;
 constexpr uint32_t kSpin = 1u << 18, kSuspend = 4000;
+constexpr float kTinyBias = 0x1p-100f;  // 0x0d80 in bf16
 enum { ERR_ROUTE = 64 };
 
 // A step k is (tile, block); it uses accumulator k mod 3.  With two blocks an accumulator goes from one block to the
@@ -206,9 +208,10 @@ __global__ void __launch_bounds__(kThreadsRU, 1)
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (warp == kBiasWarp) {
-        // A operand of the bias step: three ones per position; and the second chunk of every bias slot stays zero
+        // A operand of the bias step: three ones and three times kTinyBias per position; and the second chunk of every
+        // bias slot stays zero
         for (int r = lane; r < 128; r += 32) {
-            *reinterpret_cast<uint4*>(usm + L::OFF_ONES + step_off(r, 0)) = make_uint4(0x3f803f80u, 0x3f80u, 0, 0);
+            *reinterpret_cast<uint4*>(usm + L::OFF_ONES + step_off(r, 0)) = make_uint4(0x3f803f80u, 0x0d803f80u, 0x0d800d80u, 0);
             *reinterpret_cast<uint4*>(usm + L::OFF_ONES + step_off(r, 1)) = make_uint4(0, 0, 0, 0);
         }
         for (int r = lane; r < kTileN * L::STAGES; r += 32)  // (slots are whole groups of eight rows, one behind the other)
@@ -375,12 +378,14 @@ __global__ void __launch_bounds__(kThreadsRU, 1)
 #pragma unroll
                 for (int i = 0; i < 2 * kPer; ++i) {
                     if (i >= kPer && n_t < 2) break;
-                    const float b = cur[i];
-                    const uint32_t hi = __float_as_uint(b) & 0xffff0000u;
+                    const bool tiny = fabsf(cur[i]) < kTinyBias;
+                    const float b = tiny ? cur[i] / kTinyBias : cur[i];
+                    // (a NaN whose upper half alone would be an infinity stays one)
+                    const uint32_t hi = (__float_as_uint(b) & 0xffff0000u) | (b != b ? 0x400000u : 0u);
                     const float r1 = isfinite(b) ? b - __uint_as_float(hi) : 0.f;
                     const uint32_t mid = __float_as_uint(r1) & 0xffff0000u, lo = __float_as_uint(r1 - __uint_as_float(mid));
-                    *reinterpret_cast<uint4*>(usm + L::OFF_BIAS + (t + i / kPer) % L::STAGES * L::BIAS +
-                                              step_off(32 * (i % kPer) + lane, 0)) = make_uint4((hi >> 16) | mid, lo >> 16, 0, 0);
+                    *reinterpret_cast<uint4*>(usm + L::OFF_BIAS + (t + i / kPer) % L::STAGES * L::BIAS + step_off(32 * (i % kPer) + lane, 0)) =
+                        tiny ? make_uint4(0, hi, (mid >> 16) | lo, 0) : make_uint4((hi >> 16) | mid, lo >> 16, 0, 0);
                 }
                 fence_async();
             }

@@ -216,3 +216,37 @@ def test_prefill_outputs_feed_the_decode_path():
     want = O.attend("bf16", "softmax", 1.0 / np.sqrt(dg + du), pool["K"], pool["V"], hist_off, o_idx["K"], o_idx["V"],
                     o_usr["K"], o_usr["V"], q_off, q)
     assert_close(got, want, "bf16", "prefill -> decode")
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("variant", [0, 1])
+@pytest.mark.parametrize("n,G,d,m", [(200, 2, 64, 1024), (5, 1, 32, 1000), (40000, 2, 128, 1111)])
+def test_gpu_route_biases_out_of_the_ordinary(n, G, d, m, variant):
+    """A bias is an fp32 summand, whatever its size: one that is not a number never wins (also where its upper sixteen bits
+    alone are an infinity), denormal ones count to their last bit."""
+    rng = np.random.default_rng(5)
+    x = _bf16(rng.standard_normal((n, d)) / np.sqrt(d))
+    W = _bf16(rng.standard_normal((G, m, d)))
+    bias = (0.1 * rng.standard_normal((G, m))).astype(np.float32)
+    nan = bias.copy()
+    nan.view(np.uint32)[:, 3] = 0x7f800001
+    nan.view(np.uint32)[:, 700] = 0xff80ffff
+    without = np.where(np.isnan(nan), np.float32(-np.inf), nan)
+    if variant == 0:
+        assert np.array_equal(_gpu_route(x, W, nan, variant), _gpu_route(x, W, without, variant))
+    got = _gpu_route(x, W, np.where(np.arange(m) == 700, np.float32(np.inf), bias).astype(np.float32), variant)
+    assert (got == 700).all()
+    # no weights: the largest bias wins by its own bits, at every size
+    zero = np.zeros_like(W)
+    for low in (-149, -140, -126, -110, -101, -100, -99, -60, 0):
+        top = np.ldexp(np.float32(1), max(low, -126)).astype(np.float32) if low > -126 else np.float32(0)
+        b = np.full((G, m), top, np.float32)
+        winner = rng.integers(0, m, G)
+        for g in range(G):  # one unit in the last place more than all others
+            b[g, winner[g]] = np.ldexp(1.0, low) if low <= -126 else np.nextafter(top, np.float32(np.inf))
+        assert (_gpu_route(x, zero, b, variant) == winner[None]).all(), low
+        b = -b  # and one less
+        want = np.zeros(G, int)
+        for g in range(G):
+            want[g] = 1 if winner[g] == 0 else 0
+        assert (_gpu_route(x, zero, b, variant) == want[None]).all(), -low
