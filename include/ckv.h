@@ -260,8 +260,10 @@ CKV_API ckv_status ckv_materialize(ckv_ctx* ctx, int64_t user, void* K_out, void
  *   bias     device, fp32 [n_groups][n_entries], or NULL for none
  *   idx_out  device, int32 [n][n_groups]        what ckv_cache_put takes as idx_K / idx_V
  *   variant  0 = default (tcgen05 kernel), 1 = warp-level tensor-core kernel, 2 = tcgen05 kernel
- * Products are exact, sums fp32; entries whose scores are equal in that arithmetic resolve to the
- * lowest index.  The tcgen05 kernel's waits are bounded; the call reads its error word and
+ * Products are exact, sums fp32; scores equal in that arithmetic resolve to the lowest index.  The bias
+ * is one of the summands, unrounded: the tensor cores add it with the products (variant 1: it is added
+ * behind them), so scores no further apart than the rounding of such a sum may resolve differently in
+ * the two variants.  The tcgen05 kernel's waits are bounded; the call reads its error word and
  * therefore waits for the kernel (variant 1 is only stream-ordered).
  * Errors: INVALID_ARG (sizes, null or host pointers), UNSUPPORTED (d_in), OOM, CUDA (also: a wait
  * inside the kernel ran out; idx_out is not valid then).

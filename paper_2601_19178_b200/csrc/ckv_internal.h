@@ -181,7 +181,6 @@ constexpr int kInlinePuts = 224;  // users whose table travels as a kernel argum
 struct PutTable {
     PutUser u[kInlinePuts];
 };
-// Packs n users' [P][G] indices and [P][G][d_user] user parts into arena units and validates the index range;
 // How a kernel that checks indices reports to the host, in host-mapped memory: *bad becomes 1 on a bad index, and *done
 // (if not null) behind the last block's last access, which the host sees some microseconds before a stream synchronise
 // returns.  `count` is a device counter, zero between launches, used by one launch at a time.
@@ -204,8 +203,9 @@ __device__ __forceinline__ void report_done(const Report& r, unsigned n_blocks)
     *reinterpret_cast<volatile int*>(r.done) = 1;
 }
 #endif
-// The users come from `table` (device memory) or, if that is
-// null, from *inl.  The arena arrays and the sides' widths come from `cv` (head_dim D).
+// Packs n users' [P][G] indices and [P][G][d_user] user parts into arena units and validates the index range.  The users
+// come from `table` (device memory) or, if that is null, from *inl; the arena arrays and the sides' widths from `cv`
+// (head_dim D).
 cudaError_t launch_pack(int dtype, int G, int n_entries, int idx_bytes, int n_users, const PutUser* table,
                         const PutTable* inl, int64_t total_tiles, int64_t arena_base, const int32_t* idxK,
                         const int32_t* idxV, const void* userK, const void* userV, const CacheView& cv, int D,
@@ -262,8 +262,8 @@ cudaError_t launch_route(int d_in, const void* x, const void* W, const float* bi
                          int32_t* out, cudaStream_t s);
 
 // ---- kernels_route_umma.cu : the same router on tcgen05 (TMEM accumulators, warp-specialised)
-// flags: two host-mapped ints.  flags[0] becomes a non-zero code if a bounded wait inside the kernel ran out (nothing is
-// written then); flags[1] becomes 1 at its end if slot is in [0, kRouteSlots) and no other launch uses it at the time.
+// flags: two host-mapped ints.  flags[0] becomes a non-zero code if a bounded wait inside the kernel ran out (`out` is not
+// valid then, whether written or not); flags[1] becomes 1 at its end if slot is in [0, kRouteSlots) and no other launch uses it at the time.
 constexpr int kRouteSlots = 64;
 cudaError_t launch_route_umma(int d_in, const void* x, const void* W, const float* bias, int n, int n_entries, int G,
                               int32_t* out, int* flags, int slot, cudaStream_t s);

@@ -16,8 +16,9 @@
 // shared memory, whose fetch competed with the B operand for its 128 bytes per clock, 2.04.  Four issuing threads leave
 // the read-out 128 registers (spills: 1.34 ms); four accumulators of 96 columns, each with its own issuing thread and
 // read-out group: 1.41.
-// Every wait is bounded: a time-out raises the CTA's abort flag, the CTA drains, frees its TMEM, reports through
-// the error word and writes nothing.
+// Every wait is bounded: a time-out raises the CTA's abort flag, the CTA drains, frees its TMEM and reports through
+// the error word.  The call then returns an error and its whole output is not valid: the CTA itself writes none, but others
+// have, among them the first of its cluster, which takes the best entries of all of them as they stand.
 #include <cuda_bf16.h>
 #include <math_constants.h>
 

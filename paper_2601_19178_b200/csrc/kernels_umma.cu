@@ -19,7 +19,7 @@
 //   O   += P_i V_tile                 UMMA 128 x 32 x 64, A = P from TMEM, B = V tile (MN-major)
 // The issuing thread issues the weighted sum of step t, then the scores of step t + 2 (into the buffer the weighted sum
 // has just read): the tensor core runs one thread's instructions in order, so the buffer needs no completion hand-off in
-// between, and the scores of step t + 1 are there while the group normalises step t.
+// between, and the scores of step t + 1 are there while step t is normalised.
 //
 // What bounds it: the special-function unit (one ex2 or tanh per score, 16 per clock per SM).  The normalisation of a
 // tile is a chain of dependent work for its warp (wait for the scores, TMEM load, arithmetic, TMEM store, publish; at a
@@ -31,11 +31,11 @@
 // special-function unit busy 70 % of the time.  1024 users x 1024 positions x 100 queries x 8 groups 490 -> 385 us, 2048
 // users x 4096 x 128 (SiLU) 2.88 -> 2.57 ms, 64 causal self-attentions of 200..1500 positions 283 -> 147 us.
 //
-// Softmax bookkeeping.  The reference maximum m of a row is the largest of the first 32 scores of the group's
-// first half of the unit and stays fixed: later scores may exceed it by up to 2^64 (fp32 accumulators and bf16
+// Softmax bookkeeping.  The reference maximum m of a row is the largest of the first 32 scores of the unit's
+// first tile and stays fixed: later scores may exceed it by up to 2^64 (fp32 accumulators and bf16
 // P have the exponent range for that).  The row sum l is added up by the row's thread in fp32, chunk by chunk, and
 // a chunk's share of it also tells when a row has left that bound (32 weights within it sum to at most 2^69); only
-// then is the reference moved, O_b and the row sum rescaled (TMEM read-modify-write) and the chunk worked out again.
+// then is the reference moved, O and the row sum rescaled (TMEM read-modify-write) and the chunk worked out again.
 //
 // Shared-memory tiles use the no-swizzle UMMA canonical layout: groups of 8 rows (512 bytes), inside a
 // group one 128-byte core matrix per 16-byte row chunk, inside a core matrix row r%8 at 16 r.
@@ -314,7 +314,7 @@ __device__ __forceinline__ uint32_t v_off(int r, int c) { return (uint32_t)((r >
 // position a score column belongs to.
 __device__ __forceinline__ int pos_of_col(int c, int e) { return 32 * c + 4 * (e & 7) + (e >> 3); }
 
-// ---- normalisation of one 128 x 64 score tile by its group (thread = query row = TMEM lane) ----
+// ---- normalisation of one 128 x 64 score tile by the worker's four warps (thread = query row = TMEM lane) ----
 
 // Multiplies this thread's row of O (32 columns) by f.
 __device__ __noinline__ void rescale_row(uint32_t tO, float f)
@@ -374,17 +374,17 @@ __device__ __noinline__ float chunk_max(const uint32_t* cur, float sc, float nm,
 // Softmax weights of one 32-column chunk (c = 0, 1) of a 128 x 64 score tile: p = exp2(s c - m) as bf16
 // pairs written over the head of the scores (columns 0..31 of the buffer; chunk 1 of the scores, columns 32..63,
 // is still to be read when chunk 0's weights land on columns 0..15, and chunk 1's weights
-// land on columns 16..31, whose scores have been consumed).  The chunk's weights are added to the row sum l.  With `first` (chunk 0 of the group's first half
-// tile of a unit) the row's reference m is set from these 32 scores (column 0 is the half's position 0, always a
-// real one).  A chunk whose largest exponent argument leaves the headroom moves the reference up by a whole
-// number of octaves and is written again from the scores still in the registers; what O_b holds so far
+// land on columns 16..31, whose scores have been consumed).  The chunk's weights are added to the row sum l.  With `first`
+// (the unit's first tile) chunk 0 sets the row's reference m from its 32 scores (column 0 is the tile's position 0, always a
+// real one).  A chunk whose sum gives away that a score has left the headroom moves the reference up by a whole
+// number of octaves and is written again from its scores, read once more; what O holds so far
 // (`have_o`; wait_prev() waits for the previous step's MMAs) and, for chunk 1, the weights of chunk 0 are
 // multiplied by the same power of two.  Returns false if that wait ran out.
-// `valid` counts the real positions of the half (1..64); column (c, e) of the half holds position
-// pos_of_col(c, e) of the half.  TAIL = true (end of a history, at most once per unit and group) masks the
+// `valid` counts the real positions of the tile (1..64); column e of chunk c holds position
+// pos_of_col(c, e) of the tile.  TAIL = true (the last tile of a history, at most once per unit) masks the
 // columns beyond.
 // VIS (visible lengths): `valid` differs from thread to thread and may be zero or negative (the row sees nothing
-// of this half tile); a row's reference is then set by the first chunk in which it sees a position.
+// of this tile); a row's reference is then set by the first chunk in which it sees a position.
 template <bool TAIL, bool VIS, typename WaitPrev>
 __device__ __forceinline__ bool softmax_chunk(const uint32_t (&cur)[32], int c, uint32_t tS, uint32_t tO, float sc,
                                               int valid, bool first, bool have_o, float& m_ref, float& l, WaitPrev&& wait_prev)
@@ -720,7 +720,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma_kernel(const AttendAr
             tc_fence_after();
             tmem_ld32(tO, sa);
             tmem_wait_ld32(sa);
-            tc_fence_before();  // (the next unit overwrites O behind this group's next hand-over)
+            tc_fence_before();  // (the next unit overwrites O behind these warps' next hand-over)
             if (r < u.wk.M) {
                 auto o = [&](int e) { return __uint_as_float(sa[e]); };
                 if (u.wk.part_row < 0) {
@@ -776,7 +776,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma_kernel(const AttendAr
             uint32_t acc0 = 0, acc1 = 0;  // of the steps in flight, oldest first: O already holds earlier tiles of the unit
             int useq = 0;             // units begun
             bool ok = true;
-            // O += P_i V for step `done`, once the group has written P_i
+            // O += P_i V for step `done`, once the normalisation warps have written P_i
             auto issue_pv = [&]() {
                 const int i = done & 1;
                 if (!mbar_wait_fast(bar(BAR_PREADY + i), (done >> 1) & 1, abort_flag, SITE_PREADY)) return false;
@@ -795,7 +795,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma_kernel(const AttendAr
                 const uint64_t dq = at(dq0, (uint32_t)(useq & 1) * kTileQ);
                 for (int j = 0; j < un.u.n_tiles; ++j) {
                     // buffer i still holds the weights of step cnt - 2: its weighted sum goes first (and before the wait
-                    // for the tile: at a unit's end the group is waiting for exactly this weighted sum).  The tensor
+                    // for the tile: at a unit's end the normalisation warps wait for exactly this weighted sum).  The tensor
                     // core runs this thread's instructions in order, so the scores below need not wait for it to finish.
                     if (cnt - done == 2) ok = issue_pv();
                     if (ok) ok = mbar_wait_fast(bar(BAR_FULL + s), par, abort_flag, SITE_TILE);
