@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(128, MmaCfg<D, MT, TMA>::MIN_BLOCKS)
     const char* pK = reinterpret_cast<const char*>(a.cv.poolK) + (int64_t)grp * a.cv.n_entries * ROWB + cc * 16;
     const char* pV = reinterpret_cast<const char*>(a.cv.poolV) + (int64_t)grp * a.cv.n_entries * ROWB + cc * 16;
     const int64_t chunk0 = rq.base + (int64_t)grp * rq.Lpad + it.begin;  // the chunk's first unit
-    (void)CKV_CLAMP(chunk0 + ((it.len + 31) & ~31) - 1, a.arena_units, err_flag);  // the chunk's last (padded) unit
+    if (it.len > 0) (void)CKV_CLAMP(chunk0 + ((it.len + 31) & ~31) - 1, a.arena_units, err_flag);  // the chunk's last (padded) unit
     const int64_t unit0 = chunk0 + 32 * part + lane;  // this lane's position of step 0
     const int stride = 32 * parts;                    // positions between two of this warp's steps
     const uint16_t* uK = reinterpret_cast<const uint16_t*>(a.cv.userK);

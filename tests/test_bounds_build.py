@@ -47,8 +47,40 @@ for name, kw, kernel in cases:
 print("BOUNDS_OK", len(cases))
 """
 
+# The forms that split_len keeps from running: requests as kernel arguments, warps sharing a unit across a block or a
+# cluster, several query tiles per warp, the chunks the library chooses; lists with empty histories among them.
+CHILD_DEFAULT = r"""
+import numpy as np, torch, synth
+from ckv_testlib import assert_close, gpu_attend, make_session, oracle_attend
+import paper_2601_19178_b200 as ckv
+assert ckv.LIB_PATH.endswith("libckv_bounds.so")
+W = synth.WORKLOADS
+cases = [("cfg1", dict(n_users=5, hist_len=(0, 300))), ("cfg1", dict(n_users=230, hist_len=(0, 40))),
+         ("cfg2", dict(n_users=5, hist_len=(0, 3000))), ("cfg5", dict(n_users=1, hist_len=(0, 0))),
+         ("cfg5", dict(n_users=1, hist_len=(5000, 5000))), ("cfg5", dict(n_users=230, hist_len=(0, 90))),
+         ("cfg5", dict(n_users=600, hist_len=(300, 400), n_queries=40)), ("cfg4", dict(n_users=2, hist_len=(0, 9000))),
+         ("cfg4", dict(n_users=400, hist_len=(300, 400), n_queries=20))]
+for name, kw in cases:
+    w = synth.scaled(W[name], **kw)
+    d = synth.generate(w)
+    s = make_session(w, d)
+    got = gpu_attend(w, d, session=s)
+    assert s.stat("device_errors") == 0, (name, kw, s.stat("device_errors"))
+    s.close()
+    assert_close(got, oracle_attend(w, d), w.dtype, f"{name} {kw}")
+print("BOUNDS_OK", len(cases))
+"""
+
 
 def test_sample_of_parity_cases_on_the_range_checked_build():
+    _run(CHILD)
+
+
+def test_default_dispatch_on_the_range_checked_build():
+    _run(CHILD_DEFAULT)
+
+
+def _run(child):
     if not os.path.exists(LIB):
         sys.path.insert(0, os.path.join(ROOT, "paper_2601_19178_b200"))
         import importlib.util
@@ -57,5 +89,5 @@ def test_sample_of_parity_cases_on_the_range_checked_build():
         spec.loader.exec_module(mod)
         mod.build(bounds=True)
     env = dict(os.environ, CKV_LIBRARY=LIB, PYTHONPATH=os.pathsep.join([ROOT, os.path.join(ROOT, "tests")]))
-    r = subprocess.run([sys.executable, "-c", CHILD], capture_output=True, text=True, env=env, cwd=ROOT, timeout=900)
+    r = subprocess.run([sys.executable, "-c", child], capture_output=True, text=True, env=env, cwd=ROOT, timeout=900)
     assert r.returncode == 0 and "BOUNDS_OK" in r.stdout, (r.stdout[-2000:], r.stderr[-3000:])
