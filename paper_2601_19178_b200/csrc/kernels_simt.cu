@@ -83,8 +83,17 @@ __device__ __forceinline__ void store_out(void* out, int64_t i, float v, int out
         reinterpret_cast<float*>(out)[i] = v;
 }
 
+// Blocks an SM is to hold: with one query per pass 20 warps, 24 of fp32 heads of 64 or more; with four, fp32, 16 of those and
+// 12 of narrower ones.  The kernels fit the 80, 128 and 168 registers that this leaves, but the compiler exceeds them by a
+// few unasked (64-wide, 146 users x 101 positions x 1..16 queries x 4 groups: 49.4 us with 135 registers, 46.9 with 116).
+constexpr int simt_min_blocks(bool bf16, int D, int QB, int warps)
+{
+    const bool light = !bf16 && D >= 64;
+    return QB == 1 ? (warps == 4 ? (light ? 6 : 5) : 1) : bf16 ? 1 : (light ? 16 : 12) / warps;
+}
+
 template <bool BF16, int D, int QB, int MODE, int kWarps>
-__global__ void __launch_bounds__(kWarps * 32, QB == 1 && kWarps == 4 ? 5 : 1)
+__global__ void __launch_bounds__(kWarps * 32, simt_min_blocks(BF16, D, QB, kWarps))
     attend_simt_kernel(const __grid_constant__ AttendArgs a, const __grid_constant__ InlineTable tab)
 {
     constexpr int ES = BF16 ? 2 : 4;
