@@ -154,6 +154,7 @@ struct Plan {
     Work* d_works = nullptr;
     int32_t n_items = 0, n_split = 0, split_items = 0, max_M = 0, n_req = 0, family = 1, n_works = 0;
     int32_t parts = 1, qpw = 16;  // family 2: warps that share a unit, queries a warp holds
+    bool wide = false;            // family 1: blocks of more warps
     int64_t part_rows = 0;
     uint64_t last_use = 0;
 };
@@ -589,6 +590,7 @@ struct ListShape {
     int64_t active = 0, positions = 0;  // how many have one, their history lengths in all
     int64_t blocks128 = 0, tiles64 = 0; // blocks of 128 queries, and (block, 64 positions) tiles
     int64_t units16 = 0, tiles16 = 0, units_wide = 0, tiles_wide = 0;  // MmaWork of unchunked histories
+    int64_t passes = 0, pass_positions = 0;  // of the CUDA-core kernel, four queries at a time; their history lengths in all
     explicit ListShape(int head_dim) : qpw_wide(mma_wide_queries(head_dim)) {}
     void add(int32_t length, int32_t queries)
     {
@@ -600,7 +602,9 @@ struct ListShape {
         max_L = std::max(max_L, length);
         min_L = std::min(min_L, length);
         positions += L;
-        const int64_t b = (M + 127) / 128, b16 = mma_blocks(M, 16), bw = mma_blocks(M, qpw_wide), t = (L + 31) / 32;
+        const int64_t b = (M + 127) / 128, b16 = mma_blocks(M, 16), bw = mma_blocks(M, qpw_wide), t = (L + 31) / 32, p = (M + 3) / 4;
+        passes += p;
+        pass_positions += p * L;
         blocks128 += b;
         tiles64 += b * ((L + 63) / 64);
         units16 += b16;
@@ -739,18 +743,82 @@ int choose_family(const ckv_ctx* ctx, bool with_vis, const ListShape& s)
     return 0;
 }
 
-// Block size of the CUDA-core kernel: blocks of more warps when there are fewer blocks than SMs.
+// Block size of the CUDA-core kernel where the chunks' length is given: blocks of more warps when there are fewer than SMs.
 bool simt_wide(const ckv_ctx* ctx, int64_t n_items) { return n_items * ctx->cfg.n_groups <= ctx->n_sms; }
+
+// The CUDA-core kernel's chunk length (INT32_MAX: none) and block size with the shortest estimated run, in microseconds.  A
+// block is a chain of passes (one or four queries) of steps (what its warps load at a time), and a step takes tau, a memory
+// latency and its arithmetic, or longer once enough warps share the SM; blocks that do not fit the SMs at once follow one
+// another, in whole rounds where they are alike.  Wide blocks shorten the chain, chunks add blocks, which a second launch
+// merges.  Fitted to 80 fp32 lists of 4 to 4000 users,
+// 50..16000 positions, 1..16 queries, run in six ways each; the choice is within 5 % of the best in most, 15 % in all.
+// With wide blocks up to one per SM and no chunks otherwise, lists of a few hundred blocks took up to 2.8 times as long
+// (75 users of 50..1000 positions, 1..16 queries, 2 groups of 32-wide SiLU 131 us, now 42).
+int64_t simt_shape(const ckv_ctx* ctx, const ListShape& s, bool* wide)
+{
+    const int D = ctx->cfg.head_dim, lanes = D * ctx->elem / 16, unroll = lanes >= 16 ? 2 : 4;
+    const bool one = s.max_M <= 1;
+    const double G = ctx->cfg.n_groups, n = (double)s.active, step = 32 / lanes * unroll;  // positions a warp loads at a time
+    const double slow = (unroll == 2 ? 0.5 : 1) * (!one && ctx->cfg.mode == CKV_SILU_OVER_L ? 1.2 : 1);
+    *wide = false;
+    if (s.active == 0) return INT32_MAX;
+    // a list that is cut is planned and uploaded: behind a call of few blocks, some 20 us of the host that show in its latency
+    const double plan = n * G <= ctx->n_sms ? 19.5 : n <= kInlineReqs ? 2 : 0;
+    double best_t = 1e300;
+    int64_t best = INT32_MAX;
+    auto consider = [&](int64_t c, bool w) {
+        const bool split = c < s.max_L;
+        const double len = (double)std::min<int64_t>(c, s.max_L), warps = w ? (one ? 16 : 8) : 4;
+        // warps an SM holds, by the kernels' registers
+        const bool light = ctx->elem == 4 && D >= 64;
+        const double room = one ? (w ? 16 : light ? 24 : 20) : light ? 16 : w || ctx->elem == 2 ? 8 : 12;
+        const double chunks = !split ? n : s.min_L == s.max_L ? n * std::ceil(s.max_L / len)
+                                                              : std::max(n, (double)s.positions / len + 0.5 * n);
+        const double passes = s.passes * chunks / n;
+        const double blocks = chunks * G, slots = ctx->n_sms * room / warps, pass = one ? 0.8 : 0.45;
+        auto tau = [&](double n_blocks) {  // a step, with that many blocks at a time
+            const double load = std::min(n_blocks * warps / ctx->n_sms, room);
+            return slow * (one ? std::max(1.2, 0.07 * load) : std::max(1.5, 0.16 * load));
+        };
+        auto longest = [&](double n_blocks) {
+            return 0.25 + (s.max_M + 3) / 4 * (pass + std::ceil(len / (warps * step)) * tau(n_blocks));
+        };
+        double t = 6.5;
+        if (blocks <= slots) {
+            t += longest(blocks);
+        } else if (!split && s.min_L == s.max_L && s.same_M()) {
+            const double rounds = std::floor(blocks / slots), rest = blocks - rounds * slots;
+            t += rounds * longest(slots) + (rest > 0 ? longest(rest) : 0);
+        } else {
+            const double all = G * (0.25 * chunks + pass * passes + (s.pass_positions / (warps * step) + 0.5 * passes) * tau(slots));
+            t += std::max(longest(slots), all / slots + 0.4 * longest(slots));
+        }
+        // the second launch, and the partial results there and back
+        if (split) t += 2 + plan + passes * (one ? 1 : 4) * G * (D + 2) * 8 / 4e6;
+        if (t < best_t) {
+            best_t = t;
+            best = c;
+            *wide = w;
+        }
+    };
+    if (n * G > ctx->n_sms || s.max_L <= 4096) {
+        consider(INT32_MAX, false);
+        consider(INT32_MAX, true);
+    }
+    for (int64_t c = 64; c <= 4096 && c < s.max_L; c *= 2) consider(c, false);
+    return best;
+}
 
 int64_t auto_split_len(const ckv_ctx* ctx, const ListShape& s, int family)
 {
     if (family == 4) return INT32_MAX;  // one CTA holds a whole history
     if (family == 3) return umma_chunk(ctx, s);
     // up to 64 Ki positions the warps that share a unit of the warp-level tensor-core kernel are enough (64 tiles
-    // for each of them), up to 4096 the 16 warps of a CUDA-core block are
-    if ((family == 2 && s.max_L <= 65536) || (family == 1 && s.max_L <= 4096)) return INT32_MAX;
+    // for each of them)
+    if (family == 2 && s.max_L <= 65536) return INT32_MAX;
     // Enough (chunk, group) blocks to fill the SMs several times over, but chunks long
-    // enough that the merge of partial results stays a small fraction of the work.
+    // enough that the merge of partial results stays a small fraction of the work.  (Family 1 comes here from
+    // ckv_attend_static alone, see simt_shape.)
     int64_t c;
     if (family == 2) {
         c = s.positions * ctx->cfg.n_groups * ((s.max_M + 15) / 16) / (ctx->n_sms * 32);
@@ -762,8 +830,8 @@ int64_t auto_split_len(const ckv_ctx* ctx, const ListShape& s, int family)
     return std::min<int64_t>(std::max<int64_t>(c, 256), 2048);
 }
 
-// Orders the item indices [begin, end) by descending chunk length, equal lengths in their original order (two
-// 16-bit counting passes over the complemented length: linear in the number of items).
+// Orders the item indices [begin, end) by descending chunk length, equal lengths in their original order: a sort up to
+// 2048 items, else two 16-bit counting passes over the complemented length, which cost 66 us whatever the number.
 void order_longest_first(const std::vector<Item>& items, size_t begin, size_t end, std::vector<uint32_t>& order,
                          std::vector<uint32_t>& tmp, std::vector<uint32_t>& count)
 {
@@ -774,6 +842,13 @@ void order_longest_first(const std::vector<Item>& items, size_t begin, size_t en
         same = same && items[i].len == items[begin].len;
     }
     if (same || n < 2) return;
+    if (n <= 2048) {
+        uint64_t key[2048];
+        for (size_t i = 0; i < n; ++i) key[i] = (uint64_t)(~(uint32_t)items[begin + i].len) << 32 | (begin + i);
+        std::sort(key, key + n);
+        for (size_t i = 0; i < n; ++i) order[begin + i] = (uint32_t)key[i];
+        return;
+    }
     tmp.resize(items.size());
     count.resize(65536 + 1);
     for (int pass = 0; pass < 2; ++pass) {
@@ -810,7 +885,10 @@ ckv_status build_plan(ckv_ctx* ctx, Plan& pl, int32_t n, const int64_t* users, c
     pl.n_req = n;
     pl.family = choose_family(ctx, with_vis, shape);
     if (pl.family == 0) return CKV_ERR_UNSUPPORTED;
-    const int64_t C = ctx->opt_split > 0 && pl.family != 4 ? ctx->opt_split : auto_split_len(ctx, shape, pl.family);
+    pl.wide = false;
+    const int64_t C = ctx->opt_split > 0 && pl.family != 4 ? ctx->opt_split
+                      : pl.family == 1                     ? simt_shape(ctx, shape, &pl.wide)
+                                                           : auto_split_len(ctx, shape, pl.family);
     pl.parts = 1;
     if (pl.family == 2) {
         if (ctx->opt_split > 0) pl.qpw = mma_qpw(ctx, shape);
@@ -1511,6 +1589,7 @@ cudaError_t pipe_prepare(ckv_ctx* ctx)
 struct InlineList {
     InlineTable tab;
     int32_t n = 0, max_M = 0, parts = 1, qpw = 16, family = 0;
+    bool wide = false;
 };
 
 // Fills `x`; x.family stays 0 if the list has to go through a plan (too long, or a kernel family or a chunking that
@@ -1529,7 +1608,9 @@ ckv_status inline_list(ckv_ctx* ctx, int32_t n, const int64_t* users, const int3
     }
     x.max_M = shape.max_M;
     const int family = choose_family(ctx, with_vis, shape);
-    if ((family != 1 && family != 2) || auto_split_len(ctx, shape, family) < shape.max_L) return CKV_OK;
+    if ((family != 1 && family != 2) ||
+        (family == 1 ? simt_shape(ctx, shape, &x.wide) : auto_split_len(ctx, shape, family)) < shape.max_L)
+        return CKV_OK;
     if (family == 2)
         mma_shape(ctx, shape, INT32_MAX, [](auto&&) {}, x.qpw, x.parts);
     // longest first, as in a plan: the tail of the grid is made of short ones
@@ -1581,7 +1662,8 @@ ckv_status launch_slice(ckv_ctx* ctx, const Plan* pl, AttendArgs a, int i0, int 
             ckv_status st2 = run_mma(ctx, D, pl->max_M, pl->qpw, pl->parts, a, nullptr, l);
             if (st2 != CKV_OK) return st2;
         } else
-            CK(launch_attend_simt(ctx->cfg.dtype, D, pl->max_M, simt_wide(ctx, a.n_items), a, nullptr, l));
+            CK(launch_attend_simt(ctx->cfg.dtype, D, pl->max_M,
+                                  pl->wide || ((pl->n_split == 0 || pl->opt_split > 0) && simt_wide(ctx, a.n_items)), a, nullptr, l));
         ctx->st_launches++;
     }
     if (time_it) CK(cudaEventRecord(ctx->ev[1], s));
@@ -1706,7 +1788,7 @@ ckv_status attend_impl(ckv_ctx* ctx, int32_t n, const int64_t* users, const int3
             l.early = true;
             st = timed(ctx, ctx->opt_time != 0, s, [&]() -> ckv_status {
                 if (x.family == 2) return run_mma(ctx, D, x.max_M, x.qpw, x.parts, a, &x.tab, l);
-                CK(launch_attend_simt(ctx->cfg.dtype, D, x.max_M, simt_wide(ctx, x.n), a, &x.tab, l));
+                CK(launch_attend_simt(ctx->cfg.dtype, D, x.max_M, x.wide, a, &x.tab, l));
                 return CKV_OK;
             });
             if (st != CKV_OK) return st;

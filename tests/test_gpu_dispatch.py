@@ -70,6 +70,15 @@ def test_wide_blocks_of_the_cuda_core_kernel(dtype, length, queries):
 
 @pytest.mark.parametrize("mode", ["softmax", "silu_over_l"])
 @pytest.mark.parametrize("head", [(14, 2), (30, 2), (60, 4), (120, 8)], ids=["d16", "d32", "d64", "d128"])
+@pytest.mark.parametrize("users,hist,queries", [(149, (17, 130), 1), (80, (17, 700), 9), (230, (63, 65), 4), (20, (17, 2500), 3)])
+def test_cuda_core_kernel_between_one_block_per_sm_and_many(mode, head, users, hist, queries):
+    """Wide blocks beyond one per SM, chunks from 64 positions on and whole histories, as the estimate chooses."""
+    w = _workload(mode=mode, dtype="f32", head=head, users=users, hist=hist, queries=queries)
+    _attend_matches(w, synth.generate(w), want_kernel=1)
+
+
+@pytest.mark.parametrize("mode", ["softmax", "silu_over_l"])
+@pytest.mark.parametrize("head", [(14, 2), (30, 2), (60, 4), (120, 8)], ids=["d16", "d32", "d64", "d128"])
 @pytest.mark.parametrize("chunks", [2, 8, 9, 40])
 def test_merge_of_chunks(mode, head, chunks):
     """The merge kernel requests eight chunks at a time."""

@@ -41,6 +41,7 @@ def lib(objects, tmp_path_factory):
                    check=True)
     lib = C.CDLL(so)
     lib.fake_count.restype = C.c_long
+    lib.fake_launched.restype = C.POINTER(C.c_long)
     return lib
 
 
@@ -155,4 +156,28 @@ def test_a_threads_first_call_may_need_a_tensor_map(lib):
     assert put(lib, ctx, block, users, np.full(300, 40), d_user=4) == 0
     assert lib.ckv_set_option(ctx, b"mma_loader", C.c_int64(2)) == 0
     assert lib.ckv_attend(ctx, 300, ptr(users), ptr(np.arange(301, dtype=np.int32)), block, block, None) == 0
+    lib.ckv_destroy(ctx)
+
+
+# 2 users: kept whole (the list travels as a kernel argument).  207 users of one query: wide blocks of 16 warps although there
+# are more than SMs.  75 ragged users of up to 16 queries: cut.  500 short histories: blocks enough.
+@pytest.mark.parametrize("users,lo,hi,queries,threads,cut", [(2, 1000, 1000, 5, 256, False), (207, 745, 745, 1, 512, False),
+                                                             (75, 50, 1000, 16, 128, True), (500, 100, 100, 1, 128, False)])
+def test_cuda_core_lists_of_a_few_hundred_blocks(lib, users, lo, hi, queries, threads, cut):
+    """Chunks and block size of the CUDA-core kernel (fp32, 2 groups of 32-wide heads, 148 SMs)."""
+    ctx = C.c_void_p()
+    assert lib.ckv_create(C.byref(Config(2, 32, 0, 0, 0, 0.0, 0)), C.byref(ctx)) == 0
+    block = device_block(lib, 2 * 1024 * 32 * 4)
+    assert lib.ckv_pool_load(ctx, block, block, 1024, 30, None) == 0
+    ids = np.arange(users, dtype=np.int64)
+    lens = np.random.default_rng(0).permutation(np.linspace(lo, hi, users).round().astype(np.int64))
+    assert put(lib, ctx, block, ids, lens, d_user=2) == 0
+    q_off = np.concatenate([[0], np.cumsum(np.arange(users) % queries + 1 if cut else np.full(users, queries))]).astype(np.int32)
+    assert lib.ckv_attend(ctx, users, ptr(ids), ptr(q_off), block, block, None) == 0
+    launched = np.ctypeslib.as_array(lib.fake_launched(), (6,))
+    split = C.c_int64()
+    assert lib.ckv_last_stat(ctx, b"split_items", C.byref(split)) == 0
+    assert (split.value > 0) == cut
+    if not cut:  # (otherwise the last launch is the merge)
+        assert launched[3] == threads
     lib.ckv_destroy(ctx)
