@@ -587,7 +587,7 @@ inline int64_t mma_blocks(uint32_t M, int qpw) { return qpw == 16 ? (M + 15) / 1
 struct ListShape {
     const int qpw_wide;                 // queries of a warp that holds several tiles of them
     int32_t max_M = 0, min_M = INT32_MAX, max_L = 0, min_L = INT32_MAX;  // of requests with a query
-    int64_t active = 0, positions = 0;  // how many have one, their history lengths in all
+    int64_t active = 0, positions = 0, rows = 0;  // how many have one, their history lengths and query rows in all
     int64_t blocks128 = 0, tiles64 = 0; // blocks of 128 queries, and (block, 64 positions) tiles
     int64_t units16 = 0, tiles16 = 0, units_wide = 0, tiles_wide = 0;  // MmaWork of unchunked histories
     int64_t passes = 0, pass_positions = 0;  // of the CUDA-core kernel, four queries at a time; their history lengths in all
@@ -602,6 +602,7 @@ struct ListShape {
         max_L = std::max(max_L, length);
         min_L = std::min(min_L, length);
         positions += L;
+        rows += M;
         const int64_t b = (M + 127) / 128, b16 = mma_blocks(M, 16), bw = mma_blocks(M, qpw_wide), t = (L + 31) / 32, p = (M + 3) / 4;
         passes += p;
         pass_positions += p * L;
@@ -706,13 +707,16 @@ int choose_family(const ckv_ctx* ctx, bool with_vis, const ListShape& s)
     // tcgen05 from three 16-query blocks on, else the warp-level tensor-core kernel (faster than the CUDA-core
     // kernel from a single query on); the CUDA-core kernel serves what neither supports.  Up to six blocks the
     // warp-level kernel also takes lists too small to fill the tcgen05 kernel's workers (measured: 1.2 us per tile time of
-    // its resident warps and 4 us besides).
+    // its resident warps and 4 us besides), and for self-attention, as many queries as positions with visible lengths, lists of
+    // any number: half of their pairs count, and the tcgen05 kernel needs a plan and a launch for the limits, 5 us, whatever the
+    // list.  (The estimates are of whole histories, the limits may be on the device.  7 causal self-attentions of 556
+    // positions, 2 groups: 22.7 us there, 11.0 here; one of 50 12.4 and 4.3; eight of 500, 8 groups, 22.7 and 23.7.)
     bool few = false;
-    if (can_umma && can_mma && !with_vis && max_M >= 48 && max_M <= 96 && n_active > 0) {
+    if (can_umma && can_mma && max_M >= 48 && (max_M <= 96 || (with_vis && s.rows >= total_pos)) && n_active > 0) {
         double tile_times, t_umma;
         mma_parts(ctx, s.mma(16), 16, &tile_times);
         umma_chunk(ctx, s, &t_umma);
-        few = 4 + 1.2 * tile_times < t_umma;
+        few = 4 + 1.2 * tile_times < t_umma + (with_vis ? 5 : 0);
     }
     // One query per user: the pool-side factorisation trades the row gathers for two tables per (user, group).
     const bool can_fact = plain && s.single() &&

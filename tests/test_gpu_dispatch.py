@@ -5,6 +5,7 @@ import torch
 
 import synth
 from ckv_testlib import assert_close, gpu_attend, make_session, oracle_attend, to_dev
+from oracle import ckv_oracle as O
 from test_route import _bf16, _check, _gpu_route
 
 pytestmark = pytest.mark.gpu
@@ -166,3 +167,28 @@ def test_router_bias_keeps_its_32_bits():
     bias[0, 217] = np.nextafter(bias[0, 0], np.float32(2), dtype=np.float32)
     x, W = _bf16(np.zeros((5, d_in))), _bf16(np.zeros((1, m, d_in)))
     assert (_gpu_route(x, W, bias, 2) == 217).all()
+
+
+@pytest.mark.parametrize("mode", ["softmax", "silu_over_l"])
+@pytest.mark.parametrize("hist,users", [((48, 52), 1), ((17, 300), 5), ((129, 129), 9), ((700, 700), 2)])
+def test_causal_self_attention_of_few_users(mode, hist, users):
+    """As many queries as positions, each seeing those up to its own: the warp-level kernel, whatever the number."""
+    w = _workload(mode=mode, users=users, hist=hist, queries=1)
+    d = synth.generate(w)
+    lens = np.diff(d["hist_off"])
+    vis = np.concatenate([np.arange(1, n + 1) for n in lens]).astype(np.int32)
+    d["q_off"] = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    rng = np.random.default_rng(3)
+    d["queries"] = synth.f32_to_bf16_bits(rng.standard_normal((int(lens.sum()), w.n_groups, w.head_dim)).astype(np.float32))
+    s = make_session(w, d)
+    out = s.attend_visible(d["users"], d["q_off"], vis, to_dev(d["queries"], "bf16"))
+    got = out.float().cpu().numpy().astype(np.float64)
+    assert s.stat("kernel") == 2 and s.stat("device_errors") == 0
+    s.close()
+    want = O.attend_variants("bf16", mode, w.default_scale, w.head_dim, d["pool_K"], d["pool_V"], d["hist_off"], d["idx_K"],
+                             d["idx_V"], d["user_K"], d["user_V"], d["q_off"], d["queries"], vis=vis)
+    # (a SiLU row that sees a few positions is a sum of a few terms: its small values are compared with the largest of all)
+    if mode == "softmax":
+        assert_close(got, want, "bf16", f"{hist} {users}")
+    else:
+        assert np.abs(got - want).max() <= 1e-2 * np.abs(want).max()

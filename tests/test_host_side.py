@@ -181,3 +181,18 @@ def test_cuda_core_lists_of_a_few_hundred_blocks(lib, users, lo, hi, queries, th
     if not cut:  # (otherwise the last launch is the merge)
         assert launched[3] == threads
     lib.ckv_destroy(ctx)
+
+
+# (users, positions, queries, kernel family): few and short self-attentions go to the warp-level kernel, many and long ones
+# and tails of longer histories to the tcgen05 kernel
+@pytest.mark.parametrize("users,length,queries,family", [(7, 556, 556, 2), (1, 50, 50, 2), (1, 1500, 1500, 2), (20, 1500, 1500, 3),
+                                                         (64, 300, 300, 3), (8, 500, 60, 2), (3, 1500, 128, 3)])
+def test_kernel_of_lists_with_visible_lengths(lib, users, length, queries, family):
+    ctx, block = context(lib, G=2, D=32, d_user=2)
+    ids = np.arange(users, dtype=np.int64)
+    assert put(lib, ctx, block, ids, np.full(users, length), d_user=2) == 0
+    q_off = (np.arange(users + 1) * queries).astype(np.int32)
+    assert lib.ckv_attend_visible(ctx, users, ptr(ids), ptr(q_off), block, block, block, None) == 0
+    kernel = C.c_int64()
+    assert lib.ckv_last_stat(ctx, b"kernel", C.byref(kernel)) == 0 and kernel.value == family
+    lib.ckv_destroy(ctx)
