@@ -585,13 +585,11 @@ inline int64_t mma_blocks(uint32_t M, int qpw) { return qpw == 16 ? (M + 15) / 1
 // needs: next to the look-ups the sums cost 17 ns a request instead of 3 (a look-up is a cache miss, and fewer of them are
 // in flight with more work between them), and a walk per estimate another 3 each.
 struct ListShape {
-    const int qpw_wide;                 // queries of a warp that holds several tiles of them
     int32_t max_M = 0, min_M = INT32_MAX, max_L = 0, min_L = INT32_MAX;  // of requests with a query
     int64_t active = 0, positions = 0, rows = 0;  // how many have one, their history lengths and query rows in all
     int64_t blocks128 = 0, tiles64 = 0; // blocks of 128 queries, and (block, 64 positions) tiles
-    int64_t units16 = 0, tiles16 = 0, units_wide = 0, tiles_wide = 0;  // MmaWork of unchunked histories
+    int64_t units[3] = {}, tiles[3] = {};    // MmaWork of unchunked histories, for 16, 32 and 48 queries per warp
     int64_t passes = 0, pass_positions = 0;  // of the CUDA-core kernel, four queries at a time; their history lengths in all
-    explicit ListShape(int head_dim) : qpw_wide(mma_wide_queries(head_dim)) {}
     void add(int32_t length, int32_t queries)
     {
         if (queries <= 0) return;
@@ -603,24 +601,25 @@ struct ListShape {
         min_L = std::min(min_L, length);
         positions += L;
         rows += M;
-        const int64_t b = (M + 127) / 128, b16 = mma_blocks(M, 16), bw = mma_blocks(M, qpw_wide), t = (L + 31) / 32, p = (M + 3) / 4;
+        const int64_t b = (M + 127) / 128, t = (L + 31) / 32, p = (M + 3) / 4;
         passes += p;
         pass_positions += p * L;
         blocks128 += b;
         tiles64 += b * ((L + 63) / 64);
-        units16 += b16;
-        tiles16 += b16 * t;
-        units_wide += bw;
-        tiles_wide += bw * t;
+        for (int i = 0; i < 3; ++i) {
+            const int64_t u = mma_blocks(M, 16 * (i + 1));
+            units[i] += u;
+            tiles[i] += u * t;
+        }
     }
     bool same_M() const { return min_M == max_M || active == 0; }
     bool single() const { return active > 0 && max_M == 1; }  // one query each
-    MmaWork mma(int qpw) const  // unchunked, qpw = 16 or qpw_wide
+    MmaWork mma(int qpw) const  // unchunked
     {
         MmaWork w;
         if (active == 0) return w;
-        w.units = qpw == 16 ? units16 : units_wide;
-        w.tiles = qpw == 16 ? tiles16 : tiles_wide;
+        w.units = units[qpw / 16 - 1];
+        w.tiles = tiles[qpw / 16 - 1];
         w.min_tiles = (min_L + 31) / 32;
         w.max_tiles = (max_L + 31) / 32;
         w.alike = same_M();
@@ -631,12 +630,13 @@ struct ListShape {
 int mma_qpw(const ckv_ctx* ctx, const ListShape& s)
 {
     const int D = ctx->cfg.head_dim;
-    return mma_queries_per_warp(D, s.max_M, s.tiles16 * ctx->cfg.n_groups >= (int64_t)20 * ctx->n_sms * mma_warps_per_sm(D, 16));
+    return mma_queries_per_warp(D, s.max_M, s.tiles[0] * ctx->cfg.n_groups >= (int64_t)20 * ctx->n_sms * mma_warps_per_sm(D, 16));
 }
 
 // Queries per warp and warps per unit of histories cut into chunks of `chunk`; `each(add)` calls add(L, M) for every request
 // with a query.  Holding more queries per warp saves gathers and lengthens a tile (measured 1.45 times for 32 queries at
-// head_dim 64, 1.3 for 48 at 32), but leaves fewer units to spread: lists of few long histories are better off with 16.
+// head_dim 64; at 32 by how many 16-query tiles of a unit hold queries, see `longer`), but leaves fewer units to spread:
+// lists of few long histories are better off with 16.
 template <typename F>
 void mma_shape(const ckv_ctx* ctx, const ListShape& s, int64_t chunk, F&& each, int& qpw, int& parts)
 {
@@ -651,7 +651,14 @@ void mma_shape(const ckv_ctx* ctx, const ListShape& s, int64_t chunk, F&& each, 
     qpw = mma_qpw(ctx, s);
     const double t = estimate(qpw, parts);
     int p16;
-    if (qpw > 16 && estimate(16, p16) < (qpw == 32 ? 1.45 : 1.3) * t) {
+    if (qpw == 16) return;
+    const bool softmax = ctx->cfg.mode == CKV_SOFTMAX;
+    // the tiles of a unit that hold queries, on the average of many units per warp; of few the fullest set the pace
+    const double units = (double)s.units[qpw / 16 - 1], warps = (double)ctx->n_sms * mma_warps_per_sm(ctx->cfg.head_dim, qpw);
+    const double used = units * ctx->cfg.n_groups >= 8 * warps ? (double)s.units[0] / units : qpw / 16;
+    const double longer = ctx->cfg.head_dim == 64 ? 1.45 : qpw == 32 ? (softmax ? 0.65 + 0.42 * used : 0.72 + 0.31 * used)
+                                                                    : (softmax ? 0.27 + 0.42 * used : 0.29 + 0.34 * used);
+    if (estimate(16, p16) < longer * t) {
         qpw = 16;
         parts = p16;
     }
@@ -883,7 +890,7 @@ ckv_status build_plan(ckv_ctx* ctx, Plan& pl, int32_t n, const int64_t* users, c
         r.part0 = -1;
         r.n_chunks = 1;
     }
-    ListShape shape(ctx->cfg.head_dim);
+    ListShape shape;
     for (const Req& r : reqs) shape.add(r.L, r.M);
     pl.max_M = shape.max_M;
     pl.n_req = n;
@@ -1601,7 +1608,7 @@ struct InlineList {
 ckv_status inline_list(ckv_ctx* ctx, int32_t n, const int64_t* users, const int32_t* q_off, bool with_vis, InlineList& x)
 {
     if (n > kInlineReqs || ctx->opt_split > 0 || ctx->opt_kernel > 2 || ctx->opt_loader == 2) return CKV_OK;
-    ListShape shape(ctx->cfg.head_dim);
+    ListShape shape;
     for (int32_t k = 0; k < n; ++k) {
         const UserEntry* f = ctx->users.find(users[k]);
         if (!f) return CKV_ERR_UNKNOWN_USER;
@@ -2207,7 +2214,7 @@ extern "C" ckv_status ckv_attend_static(ckv_ctx* ctx, int32_t n, const int64_t* 
     // the plan, in fixed-size host arrays; nothing is enqueued before the request is known to fit
     StaticRow rows[kStaticMaxReqs];
     const int D = ctx->cfg.head_dim, G = ctx->cfg.n_groups;
-    ListShape shape(ctx->cfg.head_dim);
+    ListShape shape;
     for (int32_t k = 0; k < n; ++k) {
         const UserEntry* f = ctx->users.find(users[k]);
         if (!f) return CKV_ERR_UNKNOWN_USER;

@@ -116,7 +116,9 @@ struct MmaCfg {
     static constexpr int WARPS = 4;
     // TMA: tiles on 1024-byte boundaries (the swizzle pattern follows the address), then one mbarrier per slot
     static constexpr int SMEM = WARPS * NST * 2 * TILE_B + (TMA ? 1024 + WARPS * NST * 8 : 0);
-    static constexpr int MIN_BLOCKS = MT == 1 ? (D == 64 ? (TMA ? 3 : 2) : 4) : 1;
+    // (two query tiles, 32-wide: 168 registers and some spills outside the loop; left to itself the compiler takes 200 to 240
+    // and a third of the warps goes, 134 us instead of 117 for 3000 users x 300 positions x 20..32 queries, SiLU)
+    static constexpr int MIN_BLOCKS = MT == 1 ? (D == 64 ? (TMA ? 3 : 2) : 4) : D == 32 && MT == 2 ? 3 : 1;
 };
 
 enum { ERR_MMA_LOAD = 16 };  // a bounded wait for a TMA tile ran out
@@ -732,13 +734,14 @@ template <int D, int MT>
 cudaError_t launch_mma(const AttendArgs& a, int n_mb, int parts, const InlineTable* tab, const CUtensorMap* maps,
                        int* err_flag, const Launch& l)
 {
+    constexpr bool HAS_TMA = D != 32 || MT != 2;  // (never asked for with the other)
     const bool i16 = a.cv.idx_bytes == 2;
     const bool var = a.vis != nullptr || a.cv.full_k || a.cv.full_v;  // the TMA loader is never asked for with these
 #define CKV_MMA_ONE(MODE, I16, TMA, VAR)                                                                   \
     (parts > 1 ? launch_mma_one<D, MT, MODE, I16, TMA, VAR, true>(a, n_mb, parts, tab, maps, err_flag, l)  \
                : launch_mma_one<D, MT, MODE, I16, TMA, VAR, false>(a, n_mb, parts, tab, maps, err_flag, l))
 #define CKV_MMA_GO(MODE, I16)                                                                              \
-    (maps  ? CKV_MMA_ONE(MODE, I16, true, false)                                                           \
+    (maps  ? CKV_MMA_ONE(MODE, I16, HAS_TMA, false)                                                        \
      : var ? CKV_MMA_ONE(MODE, I16, false, true)                                                           \
            : CKV_MMA_ONE(MODE, I16, false, false))
     if (a.mode == CKV_SOFTMAX) return i16 ? CKV_MMA_GO(CKV_SOFTMAX, true) : CKV_MMA_GO(CKV_SOFTMAX, false);

@@ -236,7 +236,6 @@ cudaError_t launch_combine(int D, int max_M, const AttendArgs& a, const int32_t*
 bool mma_supported(int dtype, int head_dim, int d_user);  // d_user of the shared side(s)
 // big: every resident warp has some twenty tiles of 32 positions x 16 queries to do
 int mma_queries_per_warp(int head_dim, int max_M, bool big);
-inline int mma_wide_queries(int head_dim) { return head_dim == 64 ? 32 : 48; }  // what it answers if not 16
 // tensor_maps: null = fill the staging ring with cp.async copies; else the two maps of make_pool_tensor_maps =
 // fill it with TMA gathers (err_flag: device int, OR-ed with a code if a bounded wait for a tile ran out).
 // parts: warps that share one (item, group, query block), a power of two up to kMmaMaxParts; more than four lie in a

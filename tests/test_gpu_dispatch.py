@@ -47,9 +47,9 @@ def test_warps_sharing_one_unit(mode, head, length):
 
 
 @pytest.mark.parametrize("mode", ["softmax", "silu_over_l"])
-@pytest.mark.parametrize("head,queries", [((31, 1), 33), ((31, 1), 47), ((60, 4), 17), ((60, 4), 40)])
+@pytest.mark.parametrize("head,queries", [((31, 1), 17), ((31, 1), 32), ((31, 1), 33), ((31, 1), 47), ((60, 4), 17), ((60, 4), 40)])
 def test_several_query_tiles_per_warp(mode, head, queries):
-    """Enough work for every resident warp: a warp holds 48 (32-wide heads) or 32 queries (64-wide)."""
+    """Enough work for every resident warp: a warp holds 32 or 48 queries (32-wide heads) or 32 (64-wide)."""
     w = _workload(mode=mode, head=head, groups=4, users=450, hist=(400, 430), queries=queries)
     d = synth.generate(w)
     sel = np.arange(0, w.n_users, 37)
