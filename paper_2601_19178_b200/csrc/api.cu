@@ -585,11 +585,13 @@ inline int64_t mma_blocks(uint32_t M, int qpw) { return qpw == 16 ? (M + 15) / 1
 // needs: next to the look-ups the sums cost 17 ns a request instead of 3 (a look-up is a cache miss, and fewer of them are
 // in flight with more work between them), and a walk per estimate another 3 each.
 struct ListShape {
+    const bool tensor;                  // a tensor-core family can run: what only those want is gathered too
     int32_t max_M = 0, min_M = INT32_MAX, max_L = 0, min_L = INT32_MAX;  // of requests with a query
     int64_t active = 0, positions = 0, rows = 0;  // how many have one, their history lengths and query rows in all
     int64_t blocks128 = 0, tiles64 = 0; // blocks of 128 queries, and (block, 64 positions) tiles
     int64_t units[3] = {}, tiles[3] = {};    // MmaWork of unchunked histories, for 16, 32 and 48 queries per warp
     int64_t passes = 0, pass_positions = 0;  // of the CUDA-core kernel, four queries at a time; their history lengths in all
+    explicit ListShape(const ckv_ctx* ctx) : tensor(ctx->has_mma || ctx->has_umma) {}
     void add(int32_t length, int32_t queries)
     {
         if (queries <= 0) return;
@@ -601,9 +603,11 @@ struct ListShape {
         min_L = std::min(min_L, length);
         positions += L;
         rows += M;
-        const int64_t b = (M + 127) / 128, t = (L + 31) / 32, p = (M + 3) / 4;
+        const int64_t p = (M + 3) / 4;
         passes += p;
         pass_positions += p * L;
+        if (!tensor) return;
+        const int64_t b = (M + 127) / 128, t = (L + 31) / 32;
         blocks128 += b;
         tiles64 += b * ((L + 63) / 64);
         for (int i = 0; i < 3; ++i) {
@@ -816,7 +820,8 @@ int64_t simt_shape(const ckv_ctx* ctx, const ListShape& s, bool* wide)
         consider(INT32_MAX, false);
         consider(INT32_MAX, true);
     }
-    for (int64_t c = 64; c <= 4096 && c < s.max_L; c *= 2) consider(c, false);
+    if (best_t > 8.5 + plan)  // (what any cut costs)
+        for (int64_t c = 64; c <= 4096 && c < s.max_L; c *= 2) consider(c, false);
     return best;
 }
 
@@ -890,7 +895,7 @@ ckv_status build_plan(ckv_ctx* ctx, Plan& pl, int32_t n, const int64_t* users, c
         r.part0 = -1;
         r.n_chunks = 1;
     }
-    ListShape shape;
+    ListShape shape(ctx);
     for (const Req& r : reqs) shape.add(r.L, r.M);
     pl.max_M = shape.max_M;
     pl.n_req = n;
@@ -1608,7 +1613,7 @@ struct InlineList {
 ckv_status inline_list(ckv_ctx* ctx, int32_t n, const int64_t* users, const int32_t* q_off, bool with_vis, InlineList& x)
 {
     if (n > kInlineReqs || ctx->opt_split > 0 || ctx->opt_kernel > 2 || ctx->opt_loader == 2) return CKV_OK;
-    ListShape shape;
+    ListShape shape(ctx);
     for (int32_t k = 0; k < n; ++k) {
         const UserEntry* f = ctx->users.find(users[k]);
         if (!f) return CKV_ERR_UNKNOWN_USER;
@@ -2214,7 +2219,7 @@ extern "C" ckv_status ckv_attend_static(ckv_ctx* ctx, int32_t n, const int64_t* 
     // the plan, in fixed-size host arrays; nothing is enqueued before the request is known to fit
     StaticRow rows[kStaticMaxReqs];
     const int D = ctx->cfg.head_dim, G = ctx->cfg.n_groups;
-    ListShape shape;
+    ListShape shape(ctx);
     for (int32_t k = 0; k < n; ++k) {
         const UserEntry* f = ctx->users.find(users[k]);
         if (!f) return CKV_ERR_UNKNOWN_USER;
