@@ -9,7 +9,8 @@
 // with shuffles, the softmax is the running-max form, and partial results of the
 // sub-warps / warps / history chunks are merged with the usual (m, l, acc) rule.
 // Two block sizes: 4 warps when there are blocks enough for every SM, 16 (8 with several queries per user) when there
-// are not: a small call is a chain of dependent loads per step, so it wants few steps per warp.
+// are not: a small call is a chain of dependent loads per step, so it wants few steps per warp.  The host's estimate of
+// the run chooses (simt_shape), and whether histories are cut into chunks instead.
 // A side that is not shared (sharing only keys or only values) has its full-width rows in the
 // arena: they are read in place of the pool rows, coalesced, and nothing is patched.  With
 // visible lengths a query row only takes the positions before its own limit.
