@@ -722,8 +722,10 @@ int choose_family(const ckv_ctx* ctx, bool with_vis, const ListShape& s)
     // any number: half of their pairs count, and the tcgen05 kernel needs a plan and a launch for the limits, 5 us, whatever the
     // list.  (The estimates are of whole histories, the limits may be on the device.  7 causal self-attentions of 556
     // positions, 2 groups: 22.7 us there, 11.0 here; one of 50 12.4 and 4.3; eight of 500, 8 groups, 22.7 and 23.7.)
+    // (not where the option asks for the TMA loader, which takes neither limits nor sides that are not shared)
     bool few = false;
-    if (can_umma && can_mma && max_M >= 48 && (max_M <= 96 || (with_vis && s.rows >= total_pos)) && n_active > 0) {
+    const bool loads = ctx->opt_loader != 2 || (plain && ctx->has_tma);
+    if (can_umma && can_mma && loads && max_M >= 48 && (max_M <= 96 || (with_vis && s.rows >= total_pos)) && n_active > 0) {
         double tile_times, t_umma;
         mma_parts(ctx, s.mma(16), 16, &tile_times);
         umma_chunk(ctx, s, &t_umma);

@@ -196,3 +196,24 @@ def test_kernel_of_lists_with_visible_lengths(lib, users, length, queries, famil
     kernel = C.c_int64()
     assert lib.ckv_last_stat(ctx, b"kernel", C.byref(kernel)) == 0 and kernel.value == family
     lib.ckv_destroy(ctx)
+
+
+def test_tma_loader_option_leaves_the_tcgen05_kernel_its_lists(lib):
+    """The warp-level kernel's TMA loader takes neither visible lengths nor sides that are not shared: with that option set,
+    short lists with either stay with the tcgen05 kernel, which has no such option, instead of being refused."""
+    for sides, vis, queries in (((30, 30), True, 500), ((30, 30), True, 60), ((30, 0), False, 60), ((0, 30), False, 60)):
+        ctx = C.c_void_p()
+        assert lib.ckv_create(C.byref(Config(2, 32, 1, 1, 0, 0.0, 0)), C.byref(ctx)) == 0
+        block = device_block(lib, 1 << 20)
+        assert lib.ckv_pool_load_sides(ctx, block, block, 1000, *sides, None) == 0
+        ids = np.arange(2, dtype=np.int64)
+        assert put(lib, ctx, block, ids, np.full(2, 500), d_user=2) == 0
+        q_off = (np.arange(3) * queries).astype(np.int32)
+        call = [ctx, 2, ptr(ids), ptr(q_off)] + ([block] if vis else []) + [block, block, None]
+        attend = lib.ckv_attend_visible if vis else lib.ckv_attend
+        kernel = C.c_int64()
+        for loader, family in ((1, 2), (2, 3)):
+            assert lib.ckv_set_option(ctx, b"mma_loader", C.c_int64(loader)) == 0
+            assert attend(*call) == 0
+            assert lib.ckv_last_stat(ctx, b"kernel", C.byref(kernel)) == 0 and kernel.value == family
+        lib.ckv_destroy(ctx)
