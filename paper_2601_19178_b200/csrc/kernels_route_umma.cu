@@ -1,21 +1,24 @@
 // Prefill router (Sec. 4.3) on the tcgen05 tensor cores: I[i][g] = lowest j maximising x_i . W_g[j] + b_g[j].
 //
-// One CTA owns 256 positions of one group, as two blocks of 128, and every S-th share of the group's entries (S CTAs in
+// One CTA owns 384 positions of one group, as three blocks of 128, and every S-th share of the group's entries (S CTAs in
 // a cluster share the positions when there are too few of them to fill the SMs).  The positions' inputs sit in TMEM
 // (A operand, lane = position); the group's weight rows stream through a ring of shared-memory stages in tiles of 128
-// entries (B operand, one swizzled TMA box per tile), and every tile is multiplied with both blocks.  The bias is one
-// more K = 16 step of the product, ones times the bias cut into three bf16 parts whose sum is the fp32 bias exactly (below
-// 2^-100 the parts are those of 2^100 times the bias and meet 2^-100: bf16 has no room for the last of them there), so
-// the read-out touches no shared memory.  One thread per block issues the products into three 128-column TMEM
-// accumulators in turn; two groups of four warps, one per block (thread = position = TMEM lane), fetch their accumulator
-// into registers, release it at once, and keep a running (best score, entry); the score matrix never leaves the SM.
-// What bounds it: a product takes 64 clocks (five per block and tile at d_in = 64), but every barrier operation next to
-// running products takes its thread about 200, so an issuing thread spends 1150 clocks on a step (225 on the stage, 340 on
-// the accumulator, 430 in the products, 130 in the commits), and two of them set the pace.  Measured on 131072 positions
-// x 16384 entries x 4 groups, d_in = 64: 1.23 ms (895 TFLOP/s), with one issuing thread 1.73; with A and the bias in
-// shared memory, whose fetch competed with the B operand for its 128 bytes per clock, 2.04.  Four issuing threads leave
-// the read-out 128 registers (spills: 1.34 ms); four accumulators of 96 columns, each with its own issuing thread and
-// read-out group: 1.41.
+// entries (96 at d_in = 128; B operand, one swizzled TMA box per 64 inputs), and every tile is multiplied with all three
+// blocks.  The bias is one more K = 16 step of the product, ones times the bias cut into three bf16 parts whose sum is the
+// fp32 bias exactly (below 2^-100 the parts are those of 2^100 times the bias and meet 2^-100: bf16 has no room for the last
+// of them there), so the read-out touches no shared memory for it.  A block has four read-out warps (thread = position =
+// TMEM lane), an issuing warp and two accumulators of 64 columns (one of 96 at d_in = 128) of its own.  The read-out fetches
+// an accumulator into registers, releases it at once, and keeps a running (best score, entry); the score matrix never
+// leaves the SM.
+// What bounds it: the turn of an accumulator, products -> commit -> read-out -> release -> products, some 800 to 1000
+// clocks of latency of which the products are 160, and TMEM, which holds 384 columns of accumulators in turn; with that the
+// tensor core is 95 % busy with bias and products at d_in = 64.  So the turn is kept short: the release is a named
+// barrier of five warps (an mbarrier cost 340 clocks next to running products), the issuing warp waits for its tile
+// before it, the products are issued under elect.sync from values known to be uniform (under "lane 0" the five of them
+// took 380 clocks, now 200).  131072 positions x 16384 entries x 4 groups, d_in 64: 1250 us -> 893 (1232 TFLOP/s; 1197 with
+// three blocks alone, 953 with the elected issue, 930 with accumulators of 128 columns and 152 registers a read-out
+// thread instead of two of 64); d_in 32: 1170 -> 800; 10000 x 16384 x 2: 140 -> 76.  Three blocks and not two: a weight tile
+// is fetched from L2 once for all of a CTA's positions, and three turns overlap.
 // Every wait is bounded: a time-out raises the CTA's abort flag, the CTA drains, frees its TMEM and reports through
 // the error word.  The call then returns an error and its whole output is not valid: the CTA itself writes none, but others
 // have, among them the first of its cluster, which takes the best entries of all of them as they stand.
@@ -28,18 +31,17 @@
 namespace ckv {
 namespace {
 
-constexpr int kRows = 256, kTileN = 128, kAcc = 3;
-constexpr int kEpiWarps = 8, kIssueWarp = kEpiWarps, kIssuers = 2, kLoadWarp = kIssueWarp + kIssuers, kBiasWarp = kLoadWarp + 1;
-constexpr int kThreadsRU = (kBiasWarp + 1) * 32;  // twelve warps: 168 registers for a read-out thread's 128 columns
+constexpr int kBlocks = 3, kRows = 128 * kBlocks;
+constexpr int kEpiWarps = 4 * kBlocks, kIssueWarp = kEpiWarps, kLoadWarp = kIssueWarp + kBlocks;
+constexpr int kThreadsRU = (kLoadWarp + 1) * 32;  // sixteen warps: 128 registers a thread
 constexpr int kMaxClusterRU = 8;
 constexpr uint32_t kSpin = 1u << 18, kSuspend = 4000;
 constexpr float kTinyBias = 0x1p-100f;  // 0x0d80 in bf16
 enum { ERR_ROUTE = 64 };
 
-// A step k is (tile, block); it uses accumulator k mod 3.  With two blocks an accumulator goes from one block to the
-// other, so that its uses are told apart by barriers per step mod 6: each has one waiting role, which meets every phase.
-constexpr int kMaxStages = 8, kAccBars = 2 * kAcc;
-enum Bar { B_FULL = 0, B_EMPTY = kMaxStages, B_AFULL = 2 * kMaxStages, B_AEMPTY = B_AFULL + kAccBars, B_DRAIN = B_AEMPTY + kAccBars, B_COUNT };
+constexpr int kMaxStages = 8;
+constexpr int kMaxAcc = 2;  // accumulators of a block
+enum Bar { B_FULL = 0, B_EMPTY = kMaxStages, B_AFULL = 2 * kMaxStages, B_DRAIN = B_AFULL + kBlocks * kMaxAcc, B_COUNT };
 
 __device__ __forceinline__ uint32_t s_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void bar_init(uint32_t bar, uint32_t count)
@@ -50,7 +52,7 @@ __device__ __forceinline__ void bar_arrive(uint32_t bar)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
-__device__ __noinline__ bool bar_wait(uint32_t bar, uint32_t parity, const volatile int* abort_flag)
+__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, const volatile int* abort_flag)
 {
     for (uint32_t i = 0; i < kSpin; ++i) {
         uint32_t ok;
@@ -66,20 +68,24 @@ __device__ __noinline__ bool bar_wait(uint32_t bar, uint32_t parity, const volat
     }
     return false;
 }
+// Named barrier of an accumulator, for its block's four read-out warps and its issuing warp: "it has been read".  The read-out arrives
+// and runs on; once a wait has run out it takes part as the issuing warp does, so that no step is passed twice.
+__device__ __forceinline__ void acc_arrive(int acc) { asm volatile("bar.arrive %0, 160;" ::"r"(1 + acc) : "memory"); }
+__device__ __forceinline__ void acc_sync(int acc) { asm volatile("bar.sync %0, 160;" ::"r"(1 + acc) : "memory"); }
+// One thread of the (converged) warp.  The issuing code stands under this and not under "lane 0", and depends on a warp number
+// that is known to be uniform: the tensor-core instructions take their operands from uniform registers.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(p)::"memory");
+    return p != 0;
+}
 __device__ __forceinline__ void fence_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tc_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_commit_to(uint32_t bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t acc)
-{
-    asm volatile(
-        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(acc)
-        : "memory");
 }
 __device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t acc)
 {
@@ -134,6 +140,12 @@ __device__ __forceinline__ void st16(uint32_t taddr, const uint32_t* r)
         "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
         : "memory");
 }
+__device__ __forceinline__ void st8(uint32_t taddr, const uint32_t (&r)[8])
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(r[0]), "r"(r[1]),
+                 "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+                 : "memory");
+}
 __device__ __forceinline__ float max3f(float a, float b, float c)
 {
     float r;
@@ -142,18 +154,23 @@ __device__ __forceinline__ float max3f(float a, float b, float c)
 }
 template <int DIN>
 struct RU {
+    static constexpr int AN = DIN == 128 ? 96 : 64;        // columns of an accumulator
+    static constexpr int ACCS = DIN == 128 ? 1 : 2;        // accumulators of a block
+    static constexpr int TN = ACCS * AN;                   // entries per tile
     static constexpr int ROWB = DIN >= 64 ? 128 : 64;      // bytes of a row inside a TMA box = its swizzle span
     static constexpr int BOXES = DIN == 128 ? 2 : 1;       // boxes (of 64 inputs) per tile
-    static constexpr int BOX = kTileN * ROWB;              // bytes of a box
+    static constexpr int BOX = TN * ROWB;                  // bytes of a box
     static constexpr int TILE = BOXES * BOX;               // bytes of a weight tile
-    static constexpr int STAGES = DIN == 128 ? 5 : 8;
-    static constexpr int BIAS = kTileN * 32;               // bytes of a tile's bias step (16 bf16 per entry)
-    static constexpr int OFF_W = 0, OFF_BIAS = STAGES * TILE, OFF_ONES = OFF_BIAS + STAGES * BIAS,
-                         OFF_BEST = OFF_ONES + 128 * 32,   // [kRows] (score, entry), read by the cluster's first CTA
-                         OFF_BAR = OFF_BEST + kRows * 8, OFF_ABORT = OFF_BAR + B_COUNT * 8, SMEM = OFF_ABORT + 16;
-    static_assert(STAGES <= kMaxStages && SMEM <= 226 * 1024, "shared memory");
-    static constexpr uint32_t COL_A = kAcc * kTileN;       // TMEM columns of the inputs, DIN / 2 per block
-    static_assert(COL_A + 2 * (DIN / 2) <= 512, "TMEM columns");
+    static constexpr int STAGES = DIN == 128 ? 6 : 8;
+    static constexpr int BIAS = TN * 32;                   // bytes of a tile's bias step (16 bf16 per entry)
+    static constexpr int OFF_W = 0, OFF_BIAS = STAGES * TILE,
+                         OFF_BEST = OFF_BIAS + STAGES * BIAS,  // [kRows] (score, entry), read by the cluster's first CTA
+                         OFF_KEPT = OFF_BEST + kRows * 8,      // [8][kRows] four scores of a position's best chunk
+                         OFF_BAR = OFF_KEPT + kRows * 128, OFF_ABORT = OFF_BAR + B_COUNT * 8, SMEM = OFF_ABORT + 16;
+    static_assert(STAGES <= kMaxStages && SMEM <= 226 * 1024 && BOX % 1024 == 0, "shared memory");
+    // TMEM: an accumulator per block, the inputs of each block (two per column), the ones of the bias step
+    static constexpr uint32_t COL_A = kBlocks * TN, COL_ONES = COL_A + kBlocks * (DIN / 2);
+    static_assert(COL_ONES + 8 <= 512, "TMEM columns");
 };
 // Swizzled K-major operand (TMA box of ROWB-byte rows, groups of eight rows ROWB * 8 bytes apart).
 template <int DIN>
@@ -174,32 +191,30 @@ __global__ void __launch_bounds__(kThreadsRU, 1)
                       int n, int m, int G, int32_t* __restrict__ out, int* flags, int slot, int n_split)
 {
     using L = RU<DIN>;
+    constexpr int TN = L::TN, AN = L::AN, ACCS = L::ACCS;
     extern __shared__ __align__(1024) unsigned char usm[];
     __shared__ uint32_t tmem_slot;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const uint32_t sb = s_u32(usm);
     auto bar = [&](int i) { return sb + L::OFF_BAR + 8u * (uint32_t)i; };
     volatile int* abort_flag = reinterpret_cast<volatile int*>(usm + L::OFF_ABORT);
     const int grp = blockIdx.y, split = (int)(blockIdx.x % (uint32_t)n_split);
     const int64_t row0 = (int64_t)(blockIdx.x / (uint32_t)n_split) * kRows;
-    const int n_blocks = n - row0 > 128 ? 2 : 1;
+    const int n_blocks = (int)min((n - row0 + 127) / 128, (int64_t)kBlocks);
     const float* bg = bias ? bias + (int64_t)grp * m : nullptr;
     // this CTA's tiles of the group's entries
-    const int all_tiles = (m + kTileN - 1) / kTileN;
+    const int all_tiles = (m + TN - 1) / TN;
     const int tile0 = (int)((int64_t)all_tiles * split / n_split), n_tiles = (int)((int64_t)all_tiles * (split + 1) / n_split) - tile0;
     // a tile needs the bias step if there is a bias, or entries past the last one to rule out
-    auto biased = [&](int t) { return bg != nullptr || (tile0 + t + 1) * kTileN > m; };
+    auto biased = [&](int t) { return bg != nullptr || (tile0 + t + 1) * TN > m; };
 
     if (tid == 0) {
         for (int s = 0; s < L::STAGES; ++s) {
-            bar_init(bar(B_FULL + s), 2);  // the loading thread (with the box's bytes) and the bias warp
+            bar_init(bar(B_FULL + s), 2);  // the loading warp, with the box's bytes and behind the bias step
             bar_init(bar(B_EMPTY + s), (uint32_t)n_blocks);
         }
-        for (int e = 0; e < kAccBars; ++e) {
-            bar_init(bar(B_AFULL + e), 1);
-            bar_init(bar(B_AEMPTY + e), 128);
-        }
-        bar_init(bar(B_DRAIN), kIssuers);
+        for (int e = 0; e < kBlocks * L::ACCS; ++e) bar_init(bar(B_AFULL + e), 1);
+        bar_init(bar(B_DRAIN), kBlocks);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -208,14 +223,8 @@ __global__ void __launch_bounds__(kThreadsRU, 1)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    if (warp == kBiasWarp) {
-        // A operand of the bias step: three ones and three times kTinyBias per position; and the second chunk of every
-        // bias slot stays zero
-        for (int r = lane; r < 128; r += 32) {
-            *reinterpret_cast<uint4*>(usm + L::OFF_ONES + step_off(r, 0)) = make_uint4(0x3f803f80u, 0x0d803f80u, 0x0d800d80u, 0);
-            *reinterpret_cast<uint4*>(usm + L::OFF_ONES + step_off(r, 1)) = make_uint4(0, 0, 0, 0);
-        }
-        for (int r = lane; r < kTileN * L::STAGES; r += 32)  // (slots are whole groups of eight rows, one behind the other)
+    if (warp == kLoadWarp) {  // the second chunk of every bias slot stays zero (slots are whole groups of eight rows)
+        for (int r = lane; r < TN * L::STAGES; r += 32)
             *reinterpret_cast<uint4*>(usm + L::OFF_BIAS + step_off(r, 1)) = make_uint4(0, 0, 0, 0);
         fence_async();
     }
@@ -227,7 +236,7 @@ __global__ void __launch_bounds__(kThreadsRU, 1)
     float best = -CUDART_INF_F;
     int arg = 0;
 
-    // four read-out warps and one issuing thread per block of positions
+    // four read-out warps and one issuing warp per block of positions
     const int e = warp >> 2;
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
     const int row = 128 * e + (warp & 3) * 32 + lane;  // this read-out thread's position
@@ -245,6 +254,10 @@ __global__ void __launch_bounds__(kThreadsRU, 1)
             }
             st16(tmem + lane_base + L::COL_A + e * (DIN / 2) + 16 * h, v);
         }
+        if (e == 0) {  // A operand of the bias step: three ones and three times kTinyBias per position
+            const uint32_t ones[8] = {0x3f803f80u, 0x0d803f80u, 0x0d800d80u, 0, 0, 0, 0, 0};
+            st8(tmem + lane_base + L::COL_ONES, ones);
+        }
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
     }
     tc_before();
@@ -253,127 +266,145 @@ __global__ void __launch_bounds__(kThreadsRU, 1)
 
     if (warp < kEpiWarps) {
         // ------------------------------------------------------------ running arg-max, thread = position
+        // Only the maximum of 32 columns is compared with the running best; a chunk that has a new best is kept as it is
+        // in shared memory (four scores of a thread per 16-byte word, threads side by side), and the one that is left at
+        // the end is searched for its first maximal column: the search in place took the ALU pipe from 45 to 67 % (1.29 ->
+        // 1.20 ms of the case above).  Chunks come in increasing order of the entries and the comparison is strict, so the lowest entry wins
+        // among equals; past the last entry the bias is -inf.
+        uint4* const kept = reinterpret_cast<uint4*>(usm + L::OFF_KEPT) + row;
+        auto look = [&](const uint32_t (&v)[32], int j0) {
+            float m0 = __uint_as_float(v[0]), m1 = __uint_as_float(v[1]);
+#pragma unroll
+            for (int q = 2; q < 30; q += 4) {
+                m0 = max3f(m0, __uint_as_float(v[q]), __uint_as_float(v[q + 1]));
+                m1 = max3f(m1, __uint_as_float(v[q + 2]), __uint_as_float(v[q + 3]));
+            }
+            const float mx = max3f(fmaxf(m0, m1), __uint_as_float(v[30]), __uint_as_float(v[31]));
+            if (mx > best) {
+                best = mx;
+                arg = j0;
+#pragma unroll
+                for (int q = 0; q < 8; ++q) kept[q * kRows] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+            }
+        };
+        const uint32_t tacc = tmem + lane_base + (uint32_t)(TN * e);
         for (int t = 0; e < n_blocks && t < n_tiles; ++t) {
-            const int k = n_blocks * t + e, b = k % kAccBars;
-            ok = bar_wait(bar(B_AFULL + b), (k / kAccBars) & 1, abort_flag);
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
-            tc_after();
-            const uint32_t tacc = tmem + lane_base + (uint32_t)(kTileN * (k % kAcc));
-            const int j0 = (tile0 + t) * kTileN;
-            // the whole accumulator into registers, so that it is free again before it is looked at
-            uint32_t v[kTileN / 32][32];
 #pragma unroll
-            for (int c = 0; c < kTileN / 32; ++c) ld32(tacc + 32 * c, v[c]);
-#pragma unroll
-            for (int c = 0; c < kTileN / 32; ++c) wait_ld32(v[c]);
-            tc_before();
-            bar_arrive(bar(B_AEMPTY + b));
-            // Only the maximum of 32 columns is compared with the running best (a new best gets rare quickly); they are
-            // searched for their first maximal column only then.  Entries come in increasing order and the comparison
-            // is strict, so the lowest entry wins among equals; past the last entry the bias is -inf.
-#pragma unroll
-            for (int c = 0; c < kTileN / 32; ++c) {
-                float m0 = __uint_as_float(v[c][0]), m1 = __uint_as_float(v[c][1]);
-#pragma unroll
-                for (int q = 2; q < 30; q += 4) {
-                    m0 = max3f(m0, __uint_as_float(v[c][q]), __uint_as_float(v[c][q + 1]));
-                    m1 = max3f(m1, __uint_as_float(v[c][q + 2]), __uint_as_float(v[c][q + 3]));
+            for (int h = 0; h < ACCS; ++h) {
+                const int acc = ACCS * e + h;
+                if (ok) {
+                    ok = bar_wait(bar(B_AFULL + acc), t & 1, abort_flag);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) *abort_flag = 1;
                 }
-                const float mx = max3f(fmaxf(m0, m1), __uint_as_float(v[c][30]), __uint_as_float(v[c][31]));
-                if (mx > best) {
-                    best = mx;
-                    int first = 31;
-#pragma unroll
-                    for (int q = 30; q >= 0; --q) first = __uint_as_float(v[c][q]) == mx ? q : first;
-                    arg = j0 + 32 * c + first;
+                if (!ok) {
+                    if (t + 1 < n_tiles) acc_sync(acc);
+                    continue;
                 }
+                tc_after();
+                // the whole accumulator into registers, so that it is free again before it is looked at
+                uint32_t v[AN / 32][32];
+#pragma unroll
+                for (int c = 0; c < AN / 32; ++c) ld32(tacc + AN * h + 32 * c, v[c]);
+#pragma unroll
+                for (int c = 0; c < AN / 32; ++c) wait_ld32(v[c]);
+                tc_before();
+                if (t + 1 < n_tiles) acc_arrive(acc);
+#pragma unroll
+                for (int c = 0; c < AN / 32; ++c) look(v[c], (tile0 + t) * TN + AN * h + 32 * c);
             }
         }
-        if (!ok) *abort_flag = 1;
-    } else if (warp < kIssueWarp + kIssuers) {
-        // ------------------------------------------------------------ MMA issue, one thread per block
-        if (lane == 0) {
-            constexpr uint32_t idesc = idesc_bf16(128, kTileN);
-            const uint64_t ones = mat_desc(sb + L::OFF_ONES, 128, 256);
-            const int blk = warp - kIssueWarp;
-            for (int t = 0; blk < n_blocks && t < n_tiles; ++t) {
-                const int k = n_blocks * t + blk, s = t % L::STAGES, kp = k - kAcc;  // kp: the accumulator's use before
-                ok = bar_wait(bar(B_FULL + s), (t / L::STAGES) & 1, abort_flag) &&
-                     (kp < 0 || bar_wait(bar(B_AEMPTY + kp % kAccBars), (kp / kAccBars) & 1, abort_flag));
-                if (!ok) break;
-                tc_after();
-                const uint64_t w = swz_desc<DIN>(sb + L::OFF_W + s * L::TILE);
-                const uint32_t d = tmem + (uint32_t)(kTileN * (k % kAcc)), at = tmem + L::COL_A + blk * (DIN / 2);
+        if (best > -CUDART_INF_F) {
+            int first = 0;
 #pragma unroll
-                for (int ks = 0; ks < DIN / 16; ++ks)
-                    mma_ts(d, at + 8 * ks, w + (uint64_t)(((ks & 3) * 32 + (ks >> 2) * L::BOX) >> 4), idesc, ks > 0);
-                if (biased(t)) mma_ss(d, ones, mat_desc(sb + L::OFF_BIAS + s * L::BIAS, 128, 256), idesc, 1u);
-                tc_commit_to(bar(B_AFULL + k % kAccBars));
-                tc_commit_to(bar(B_EMPTY + s));
+            for (int q = 7; q >= 0; --q) {
+                const uint4 w = kept[q * kRows];
+                if (__uint_as_float(w.w) == best) first = 4 * q + 3;
+                if (__uint_as_float(w.z) == best) first = 4 * q + 2;
+                if (__uint_as_float(w.y) == best) first = 4 * q + 1;
+                if (__uint_as_float(w.x) == best) first = 4 * q;
             }
-            if (!ok) *abort_flag = 1;
+            arg += first;
+        }
+    } else if (warp < kIssueWarp + kBlocks) {
+        // ------------------------------------------------------------ MMA issue, one warp per block
+        constexpr uint32_t idesc = idesc_bf16(128, AN);
+        const int blk = warp - kIssueWarp;
+        const uint32_t d = tmem + (uint32_t)(TN * blk), at = tmem + L::COL_A + blk * (DIN / 2), ones = tmem + L::COL_ONES;
+        int s = 0;
+        uint32_t par = 0;
+        for (int t = 0; blk < n_blocks && t < n_tiles; ++t) {
+            if (ok) {  // (the tile has usually been there for long: this wait lies before the one that paces the block)
+                ok = bar_wait(bar(B_FULL + s), par, abort_flag);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) *abort_flag = 1;
+            }
+#pragma unroll
+            for (int h = 0; h < ACCS; ++h) {
+                if (t > 0) acc_sync(ACCS * blk + h);
+                if (ok && elect_one()) {
+                    tc_after();
+                    // (entries AN h and up of the tile: whole groups of eight rows further on)
+                    const uint64_t w = swz_desc<DIN>(sb + L::OFF_W + s * L::TILE + AN * h * L::ROWB);
+#pragma unroll
+                    for (int ks = 0; ks < DIN / 16; ++ks)
+                        mma_ts(d + AN * h, at + 8 * ks, w + (uint64_t)(((ks & 3) * 32 + (ks >> 2) * L::BOX) >> 4), idesc, ks > 0);
+                    if (biased(t)) mma_ts(d + AN * h, ones, mat_desc(sb + L::OFF_BIAS + s * L::BIAS + AN * h * 32, 128, 256), idesc, 1u);
+                    tc_commit_to(bar(B_AFULL + ACCS * blk + h));
+                    if (h == ACCS - 1) tc_commit_to(bar(B_EMPTY + s));
+                }
+                __syncwarp();
+            }
+            if (++s == L::STAGES) {
+                s = 0;
+                par ^= 1;
+            }
+        }
+        if (lane == 0) {
             // nothing of this CTA may still run on the tensor core at teardown
             tc_commit_to(bar(B_DRAIN));
             volatile int never = 0;
             if (!bar_wait(bar(B_DRAIN), 0, &never)) *abort_flag = 1;
         }
         __syncwarp();
-    } else if (warp == kLoadWarp) {
-        // ------------------------------------------------------------ weight tiles
-        if (lane == 0) {
-            int s = 0, issued = 0;
-            uint32_t pe = 1;
-            for (int t = 0; t < n_tiles; ++t) {
-                ok = bar_wait(bar(B_EMPTY + s), pe, abort_flag);
-                if (!ok) break;
-                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar(B_FULL + s)), "r"(L::TILE)
-                             : "memory");
-#pragma unroll
-                for (int h = 0; h < L::BOXES; ++h)
-                    asm volatile(
-                        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
-                        "[%4];" ::"r"(sb + L::OFF_W + s * L::TILE + h * L::BOX),
-                        "l"(&tmW), "r"(64 * h), "r"(grp * m + (tile0 + t) * kTileN), "r"(bar(B_FULL + s))
-                        : "memory");
-                ++issued;
-                if (++s == L::STAGES) {
-                    s = 0;
-                    pe ^= 1;
-                }
-            }
-            if (!ok) {
-                *abort_flag = 1;
-                // the copies in flight land before the CTA ends: every stage's last fill has its bytes (a stage whose
-                // bias arrival is missing times out here, with its bytes long there)
-                volatile int never = 0;
-                for (int k = issued > L::STAGES ? issued - L::STAGES : 0; k < issued; ++k)
-                    bar_wait(bar(B_FULL + k % L::STAGES), (k / L::STAGES) & 1, &never);
-            }
-        }
-        __syncwarp();
     } else {
-        // ------------------------------------------------------------ bias steps: b = hi + mid + lo, bf16 each, exactly
-        // two tiles at a time: the wait, the fence and the hand-over are a chain, and one per tile would set the pace
-        constexpr int kPer = kTileN / 32;
+        // ------------------------------------------------------------ weight tiles, and their bias steps
+        // b = hi + mid + lo, bf16 each, exactly.  Two tiles at a time: the waits, the fence and the hand-over are a chain.
+        constexpr int kPer = TN / 32;
         auto load_bias = [&](int t, float (&b)[2 * kPer]) {
 #pragma unroll
             for (int i = 0; i < 2 * kPer; ++i) {
-                const int j = (tile0 + t) * kTileN + 32 * i + lane;
+                const int j = (tile0 + t) * TN + 32 * i + lane;
                 b[i] = j < m ? (bg ? __ldg(bg + j) : 0.f) : -CUDART_INF_F;
             }
         };
         float nxt[2 * kPer];
         load_bias(0, nxt);
+        int issued = 0, handed = 0;  // tiles whose copies have been issued / that have been handed over
         for (int t = 0; t < n_tiles; t += 2) {
             float cur[2 * kPer];
 #pragma unroll
             for (int i = 0; i < 2 * kPer; ++i) cur[i] = nxt[i];
             load_bias(t + 2, nxt);
             const int n_t = min(2, n_tiles - t);
-            for (int h = 0; h < n_t; ++h)
-                ok = ok && bar_wait(bar(B_EMPTY + (t + h) % L::STAGES), (((t + h) / L::STAGES) & 1) ^ 1, abort_flag);
-            ok = __all_sync(0xffffffffu, ok);
+            for (int h = 0; h < n_t; ++h) {
+                const int s = (t + h) % L::STAGES;
+                ok = bar_wait(bar(B_EMPTY + s), (((t + h) / L::STAGES) & 1) ^ 1, abort_flag);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                if (lane == 0) {
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar(B_FULL + s)), "r"(L::TILE)
+                                 : "memory");
+#pragma unroll
+                    for (int i = 0; i < L::BOXES; ++i)
+                        asm volatile(
+                            "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, "
+                            "%3}], [%4];" ::"r"(sb + L::OFF_W + s * L::TILE + i * L::BOX),
+                            "l"(&tmW), "r"(64 * i), "r"(grp * m + (tile0 + t + h) * TN), "r"(bar(B_FULL + s))
+                            : "memory");
+                }
+                ++issued;
+            }
             if (!ok) break;
             if (biased(t + n_t - 1)) {
 #pragma unroll
@@ -392,8 +423,17 @@ __global__ void __launch_bounds__(kThreadsRU, 1)
             }
             __syncwarp();
             if (lane < n_t) bar_arrive(bar(B_FULL + (t + lane) % L::STAGES));
+            handed += n_t;
         }
-        if (!ok) *abort_flag = 1;
+        if (!ok && lane == 0) {
+            *abort_flag = 1;
+            // the copies in flight land before the CTA ends
+            volatile int never = 0;
+            for (int k = handed; k < issued; ++k) bar_arrive(bar(B_FULL + k % L::STAGES));
+            for (int k = issued > L::STAGES ? issued - L::STAGES : 0; k < issued; ++k)
+                bar_wait(bar(B_FULL + k % L::STAGES), (k / L::STAGES) & 1, &never);
+        }
+        __syncwarp();
     }
 
     tc_before();
@@ -432,10 +472,10 @@ __global__ void __launch_bounds__(kThreadsRU, 1)
     if (slot >= 0) report_done(Report{flags, flags + 1, &route_count[slot]}, gridDim.x * gridDim.y);
 }
 
-// The weights as rows of `d_in` inputs, boxes of 128 rows and at most 64 inputs.
-bool make_weight_map(int d_in, int64_t rows, const void* W, CUtensorMap* map)
+// The weights as rows of `d_in` inputs, boxes of a tile's rows and at most 64 inputs.
+bool make_weight_map(int d_in, int64_t rows, int tile_rows, const void* W, CUtensorMap* map)
 {
-    return encode_rows(map, W, d_in, rows, d_in < 64 ? d_in : 64, kTileN, d_in < 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+    return encode_rows(map, W, d_in, rows, d_in < 64 ? d_in : 64, tile_rows, d_in < 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
                        CU_TENSOR_MAP_L2_PROMOTION_L2_128B);
 }
 
@@ -444,17 +484,18 @@ cudaError_t launch_t(const void* x, const void* W, const float* bias, int n, int
                      int slot, cudaStream_t s)
 {
     CUtensorMap map;
-    if (!make_weight_map(DIN, (int64_t)G * m, W, &map)) return cudaErrorInvalidValue;
-    // CTAs per position block: as many as shorten the run most, counting whole waves of CTAs over the SMs and about
-    // four tiles' time for setting one up
+    if (!make_weight_map(DIN, (int64_t)G * m, RU<DIN>::TN, W, &map)) return cudaErrorInvalidValue;
+    // CTAs that share a block of positions: as many as shorten the run most, counting whole waves of CTAs over the SMs and
+    // fourteen tiles' time per CTA: 5 us until the first product is there and for the end, and as much for the first
+    // tiles, in which most chunks bring a new best (40 000 positions x 4096 entries x 4 groups: 106 us; 119 by four tiles)
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t ctas = (int64_t)((n + kRows - 1) / kRows) * G, tiles = (m + kTileN - 1) / kTileN;
+    const int64_t ctas = (int64_t)((n + kRows - 1) / kRows) * G, tiles = (m + RU<DIN>::TN - 1) / RU<DIN>::TN;
     int split = 1;
     int64_t best = INT64_MAX;
     for (int sp = 1; sp <= kMaxClusterRU && sp <= tiles; sp *= 2) {
-        const int64_t cost = (ctas * sp + sms - 1) / sms * ((tiles + sp - 1) / sp + 4);
+        const int64_t cost = (ctas * sp + sms - 1) / sms * ((tiles + sp - 1) / sp + 14);
         if (cost < best) {
             best = cost;
             split = sp;

@@ -250,3 +250,22 @@ def test_gpu_route_biases_out_of_the_ordinary(n, G, d, m, variant):
         for g in range(G):
             want[g] = 1 if winner[g] == 0 else 0
         assert (_gpu_route(x, zero, b, variant) == want[None]).all(), -low
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("d_in", [32, 64, 128])
+@pytest.mark.parametrize("n,m", [(128, 64), (129, 65), (257, 96), (384, 97), (385, 128), (383, 129), (769, 193), (64, 2500)])
+def test_gpu_router_at_the_edges_of_blocks_and_tiles(d_in, n, m):
+    """Whole blocks of 128 positions and one more or less, accumulators and tiles that are full, begun or missing; every
+    position's best entry planted, so that each column of a tile is the answer of some position, bit for bit."""
+    rng = np.random.default_rng(n * m)
+    x = _bf16(rng.standard_normal((n, d_in)) / np.sqrt(d_in))
+    W = _bf16(rng.standard_normal((2, m, d_in)))
+    bias = (0.1 * rng.standard_normal((2, m))).astype(np.float32)
+    _check(x, W, bias, f"d_in={d_in} n={n} m={m}")
+    # weights zero: the score is the bias, and a position's choice the largest bias, the first of two equal ones
+    for j in {0, 31, 32, 63, 64, 95, 96, 127, 128, m - 1} & set(range(m)):
+        b = np.zeros((2, m), np.float32)
+        b[0, j] = b[1, j] = 1.0
+        b[1, m - 1] = 1.0
+        assert (_gpu_route(x, np.zeros_like(W), b) == j).all(), j
