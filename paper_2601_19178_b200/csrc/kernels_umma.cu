@@ -4,7 +4,7 @@
 // units, where a unit is (work item = history chunk of one user, group, block of up to 128 queries).  The history chunk
 // is processed in tiles of 64 positions.  A worker is (warp-specialised, 6 warps of the CTA's 18)
 //   four normalisation warps: thread i owns query row i = TMEM lane i
-//   one issuing thread: the score MMAs and the weighted-sum MMAs
+//   one issuing warp: the score MMAs and the weighted-sum MMAs
 //   one producer warp: gathers pool rows into the worker's ring of shared-memory stages with 16-byte cp.async, patches
 //     the user-specific leading elements (Eq. K), publishes the tile one tile later, and stages Q with a unit's first
 //     tile.  (A side that is not shared -- sharing only keys or only values -- is copied from the user's full-width
@@ -28,7 +28,9 @@
 // 32-column chunk of scores at a time) and TMEM (3 x (2 x 64 + 32) = 480 columns) admit no fourth.  With the three groups
 // on one unit instead (its tiles dealt out in turn, accumulators merged through shared memory at its end) a unit cost
 // 5 us plus 0.45 us per 128 positions; now an SM of busy workers takes 0.4 us per 64 positions and 1.5 us per unit, the
-// special-function unit busy 70 % of the time.  1024 users x 1024 positions x 100 queries x 8 groups 490 -> 385 us, 2048
+// special-function unit busy 70 % of the time.  The issuing warp walks its loop as a whole and an elected thread issues, with
+// operands known to be uniform: under "lane 0" each product and commit waited for its operands' way into uniform registers
+// (the three cases below 386 -> 357 us, 2.57 -> 2.47 ms, 148 -> 127 us).  1024 users x 1024 positions x 100 queries x 8 groups 490 -> 385 us, 2048
 // users x 4096 x 128 (SiLU) 2.88 -> 2.57 ms, 64 causal self-attentions of 200..1500 positions 283 -> 147 us.
 //
 // Softmax bookkeeping.  The reference maximum m of a row is the largest of the first 32 scores of the unit's
@@ -159,6 +161,13 @@ __device__ __forceinline__ void cp_async16_once(uint32_t dst, const void* src, u
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+// One thread of the (converged) warp.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(p)::"memory");
+    return p != 0;
+}
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -589,7 +598,8 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma_kernel(const AttendAr
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ uint32_t tmem_base_slot;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // (the warp number as a value known to be uniform: tensor-core and TMEM instructions take theirs from uniform registers)
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const uint32_t sbase = smem_u32(smem);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::ABORT);
     const int G = a.cv.n_groups;
@@ -761,70 +771,81 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma_kernel(const AttendAr
         }
     } else if (warp < kProducerWarp0) {
         // --------------------------------------------------------------------- MMA issue
-        // One thread, and its loop paces the worker: it is a chain of dependent instructions, so everything that can be
-        // kept out of it is (descriptors are a constant plus an offset, waits poll once inline before they call).
-        if (lane == 0) {
-            constexpr uint32_t idesc_s = make_idesc(128, TH, false), idesc_pv = make_idesc(128, D, true);
-            const uint64_t dq0 = smem_desc(wbase + L::Q, 128, 512), dk0 = smem_desc(wbase + L::K, 128, 512),
-                           dv0 = smem_desc(wbase + L::V, kVGroup, 128);
-            auto at = [](uint64_t d, uint32_t byte_off) { return d + (uint64_t)(byte_off >> 4); };  // no carry out of the address field
-            Units<false, VIS> un;
-            un.init(a, n_work, b);
-            int cnt = 0, done = 0;    // steps whose scores / weighted sum have been issued; at most two apart
-            int s = 0, par = 0;       // stage of step cnt and the phase parity of its tile
-            int pv_s = 0;             // stage of step `done`
-            uint32_t acc0 = 0, acc1 = 0;  // of the steps in flight, oldest first: O already holds earlier tiles of the unit
-            int useq = 0;             // units begun
-            bool ok = true;
-            // O += P_i V for step `done`, once the normalisation warps have written P_i
-            auto issue_pv = [&]() {
-                const int i = done & 1;
-                if (!mbar_wait_fast(bar(BAR_PREADY + i), (done >> 1) & 1, abort_flag, SITE_PREADY)) return false;
+        // One warp, and its loop paces the worker: it is a chain of dependent instructions, so everything that can be
+        // kept out of it is (descriptors are a constant plus an offset, waits poll once inline before they call).  The
+        // whole warp walks it and an elected thread issues.
+        constexpr uint32_t idesc_s = make_idesc(128, TH, false), idesc_pv = make_idesc(128, D, true);
+        const uint64_t dq0 = smem_desc(wbase + L::Q, 128, 512), dk0 = smem_desc(wbase + L::K, 128, 512),
+                       dv0 = smem_desc(wbase + L::V, kVGroup, 128);
+        auto at = [](uint64_t d, uint32_t byte_off) { return d + (uint64_t)(byte_off >> 4); };  // no carry out of the address field
+        auto arrived = [&](uint32_t bar, uint32_t parity, int site) {
+            const bool here = mbar_wait_fast(bar, parity, abort_flag, site);
+            return __all_sync(0xffffffffu, here) != 0;
+        };
+        Units<false, VIS> un;
+        un.init(a, n_work, b);
+        int cnt = 0, done = 0;    // steps whose scores / weighted sum have been issued; at most two apart
+        int s = 0, par = 0;       // stage of step cnt and the phase parity of its tile
+        int pv_s = 0;             // stage of step `done`
+        uint32_t acc0 = 0, acc1 = 0;  // of the steps in flight, oldest first: O already holds earlier tiles of the unit
+        int useq = 0;             // units begun
+        bool ok = true;
+        // O += P_i V for step `done`, once the normalisation warps have written P_i
+        auto issue_pv = [&]() {
+            const int i = done & 1;
+            if (!arrived(bar(BAR_PREADY + i), (done >> 1) & 1, SITE_PREADY)) return false;
+            if (elect_one()) {
                 tc_fence_after();
                 const uint64_t dv = at(dv0, (uint32_t)pv_s * kTileV);
 #pragma unroll
                 for (int kk = 0; kk < TH / 16; ++kk)  // sixteen positions per instruction
                     umma_ts(tO0, tS0 + (uint32_t)TH * i + 8 * kk, at(dv, kk * 2 * kVGroup), idesc_pv, kk > 0 ? 1u : acc0);
                 tc_commit(bar(BAR_EMPTY + pv_s));
-                acc0 = acc1;
-                if (++pv_s == NS) pv_s = 0;
-                ++done;
-                return true;
-            };
-            for (; ok && un.valid; un.next(), ++useq) {
-                const uint64_t dq = at(dq0, (uint32_t)(useq & 1) * kTileQ);
-                for (int j = 0; j < un.u.n_tiles; ++j) {
-                    // buffer i still holds the weights of step cnt - 2: its weighted sum goes first (and before the wait
-                    // for the tile: at a unit's end the normalisation warps wait for exactly this weighted sum).  The tensor
-                    // core runs this thread's instructions in order, so the scores below need not wait for it to finish.
-                    if (cnt - done == 2) ok = issue_pv();
-                    if (ok) ok = mbar_wait_fast(bar(BAR_FULL + s), par, abort_flag, SITE_TILE);
-                    if (!ok) break;
+            }
+            __syncwarp();
+            acc0 = acc1;
+            if (++pv_s == NS) pv_s = 0;
+            ++done;
+            return true;
+        };
+        for (; ok && un.valid; un.next(), ++useq) {
+            const uint64_t dq = at(dq0, (uint32_t)(useq & 1) * kTileQ);
+            const int n_tiles = __shfl_sync(0xffffffffu, un.u.n_tiles, 0);
+            for (int j = 0; j < n_tiles; ++j) {
+                // buffer i still holds the weights of step cnt - 2: its weighted sum goes first (and before the wait
+                // for the tile: at a unit's end the normalisation warps wait for exactly this weighted sum).  The tensor
+                // core runs this warp's instructions in order, so the scores below need not wait for it to finish.
+                if (cnt - done == 2) ok = issue_pv();
+                if (ok) ok = arrived(bar(BAR_FULL + s), par, SITE_TILE);
+                if (!ok) break;
+                const int i = cnt & 1;
+                if (elect_one()) {
                     tc_fence_after();
-                    const int i = cnt & 1;
                     const uint64_t dk = at(dk0, (uint32_t)s * kTileK);
 #pragma unroll
                     for (int ks = 0; ks < D / 16; ++ks)
                         umma_ss(tS0 + (uint32_t)TH * i, at(dq, ks * 256), at(dk, ks * 256), idesc_s, ks > 0 ? 1u : 0u);
                     tc_commit(bar(BAR_SFULL + i));
-                    (cnt == done ? acc0 : acc1) = j > 0 ? 1u : 0u;
-                    if (++s == NS) {
-                        s = 0;
-                        par ^= 1;
-                    }
-                    ++cnt;
+                    if (j == n_tiles - 1) tc_commit(bar(BAR_QEMPTY + (useq & 1)));
                 }
-                if (ok) tc_commit(bar(BAR_QEMPTY + (useq & 1)));
+                __syncwarp();
+                (cnt == done ? acc0 : acc1) = j > 0 ? 1u : 0u;
+                if (++s == NS) {
+                    s = 0;
+                    par ^= 1;
+                }
+                ++cnt;
             }
-            while (ok && done < cnt) ok = issue_pv();
-            if (!ok) {
-                *abort_flag = 1;
-                atomicOr(err_flag, ERR_MMA);
-            }
-            // nothing of this worker may still be running on the tensor core at teardown
-            tc_commit(bar(BAR_DRAIN));
-            if (!mbar_wait(bar(BAR_DRAIN), 0, abort_flag + 2, SITE_DRAIN)) atomicOr(err_flag, ERR_DRAIN);
         }
+        while (ok && done < cnt) ok = issue_pv();
+        if (lane == 0 && !ok) {
+            *abort_flag = 1;
+            atomicOr(err_flag, ERR_MMA);
+        }
+        __syncwarp();
+        // nothing of this worker may still be running on the tensor core at teardown
+        if (elect_one()) tc_commit(bar(BAR_DRAIN));
+        if (!mbar_wait(bar(BAR_DRAIN), 0, abort_flag + 2, SITE_DRAIN)) atomicOr(err_flag, ERR_DRAIN);
         __syncwarp();
     } else {
         // --------------------------------------------------------------------- producer
