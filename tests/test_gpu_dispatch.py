@@ -192,3 +192,33 @@ def test_causal_self_attention_of_few_users(mode, hist, users):
         assert_close(got, want, "bf16", f"{hist} {users}")
     else:
         assert np.abs(got - want).max() <= 1e-2 * np.abs(want).max()
+
+
+@pytest.mark.parametrize("mode", ["softmax", "silu_over_l"])
+@pytest.mark.parametrize("queries", [1, 31, 33, 64, 65, 96, 97, 129, 161, 225])
+def test_tcgen05_kernel_with_warps_without_a_row(mode, queries):
+    """Blocks of 1 to 128 query rows, several units per worker (rows turn by 32 from unit to unit), histories that end in
+    the first or the second half of a tile."""
+    w = _workload(mode=mode, groups=8, users=150, hist=(17, 200), queries=queries)
+    _attend_matches(w, synth.generate(w), want_kernel=3, kernel=3)
+
+
+@pytest.mark.parametrize("mode", ["softmax", "silu_over_l"])
+@pytest.mark.parametrize("queries", [40, 97, 260])
+def test_tcgen05_kernel_rows_that_see_parts_of_a_tile(mode, queries):
+    """Visible lengths around the 32-position chunks of a tile, whole warps and single rows that see nothing of one."""
+    w = _workload(mode=mode, groups=4, users=60, hist=(60, 300), queries=queries)
+    d = synth.generate(w)
+    rng = np.random.default_rng(queries)
+    lens = np.diff(d["hist_off"])
+    vis = np.concatenate([np.clip(32 * rng.integers(0, 11, queries) + rng.integers(-1, 2, queries), 0, L) if u % 2 else
+                          np.full(queries, min(32 * (u % 9), L)) for u, L in enumerate(lens)]).astype(np.int32)
+    vis[vis == 1] = 0
+    s = make_session(w, d, kernel=3)
+    out = s.attend_visible(d["users"], d["q_off"], torch.from_numpy(vis).cuda(), to_dev(d["queries"], w.dtype))
+    torch.cuda.synchronize()
+    assert s.stat("kernel") == 3 and s.stat("device_errors") == 0
+    s.close()
+    want = O.attend_variants(w.dtype, w.mode, w.default_scale, w.head_dim, d["pool_K"], d["pool_V"], d["hist_off"], d["idx_K"],
+                             d["idx_V"], d["user_K"], d["user_V"], d["q_off"], d["queries"], vis=vis)
+    assert_close(out.float().cpu().numpy().astype(np.float64), want, "bf16", f"{mode} {queries}")
