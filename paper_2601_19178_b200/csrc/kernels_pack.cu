@@ -63,20 +63,20 @@ __device__ __forceinline__ void copy_user(E* dst, const E* src, int width, int v
     for (int c = 0; c < width; ++c) dst[c] = real ? __ldg(src + c) : E(0);
 }
 
+// Returns whether the index was out of range (an entry of the pool is stored in its place).
 template <typename E, typename I>
-__device__ __forceinline__ void store_unit(const SideDst& d, int64_t dst, const int32_t* idx_src, const E* user_src,
-                                           int64_t src, bool real, int n_entries, int* bad_flag)
+__device__ __forceinline__ bool store_unit(const SideDst& d, int64_t dst, const int32_t* idx_src, const E* user_src,
+                                           int64_t src, bool real, int n_entries)
 {
+    bool bad = false;
     int32_t j = d.idx && real ? __ldg(idx_src + src) : 0;
     if (d.width > 0)
         copy_user<E>(reinterpret_cast<E*>(d.user) + dst * d.width, user_src + src * d.width, d.width, d.vec, real);
     if (d.idx) {  // padding: a valid row index (and zeros)
-        if (j < 0 || j >= n_entries) {
-            *reinterpret_cast<volatile int*>(bad_flag) = 1;  // host memory: written in the error case alone
-            j = 0;
-        }
-        reinterpret_cast<I*>(d.idx)[dst] = (I)j;
+        bad = j < 0 || j >= n_entries;
+        reinterpret_cast<I*>(d.idx)[dst] = (I)(bad ? 0 : j);
     }
+    return bad;
 }
 
 // One warp per tile of 32 positions of one user, every group of them: the inputs are [position][group], the arena is
@@ -101,6 +101,7 @@ __global__ void __launch_bounds__(256) pack_kernel(int G, int n_entries, int n_u
         if (tab[mid].tile0 <= t0) u = mid; else hi = mid;
     }
     PutUser e = tab[u];
+    bool bad = false;
     for (int64_t t = t0; t < t1; ++t) {
         while (u + 1 < n_users && tab[u + 1].tile0 <= t) e = tab[++u];
         const int i = (int)(32 * (t - e.tile0)) + lane, Lpad = (e.L + 31) & ~31;
@@ -108,11 +109,11 @@ __global__ void __launch_bounds__(256) pack_kernel(int G, int n_entries, int n_u
         const bool real = i < e.L;
 #pragma unroll 4
         for (int g = 0; g < G; ++g) {
-            store_unit<E, I>(dK, dst + (int64_t)g * Lpad, idxK, userK, src + g, real, n_entries, report.bad);
-            store_unit<E, I>(dV, dst + (int64_t)g * Lpad, idxV, userV, src + g, real, n_entries, report.bad);
+            bad |= store_unit<E, I>(dK, dst + (int64_t)g * Lpad, idxK, userK, src + g, real, n_entries);
+            bad |= store_unit<E, I>(dV, dst + (int64_t)g * Lpad, idxV, userV, src + g, real, n_entries);
         }
     }
-    report_done(report, gridDim.x);
+    report_outcome(report, bad, gridDim.x);
 }
 
 template <typename E, typename I>
@@ -134,6 +135,7 @@ __global__ void append_kernel(int G, int n_entries, int64_t old_base, int L_old,
 {
     const int first = dst_base == old_base ? L_old : 0, n = Lpad_tot - first;
     const int64_t total = (int64_t)G * n;
+    bool bad = false;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
         const int g = (int)(t / n);
         const int i = first + (int)(t - (int64_t)g * n);
@@ -145,11 +147,11 @@ __global__ void append_kernel(int G, int n_entries, int64_t old_base, int L_old,
         } else {
             const int64_t src = (int64_t)(i - L_old) * G + g;
             const bool real = i < L_old + L_new;
-            store_unit<E, I>(dK, dst, idxK, userK, src, real, n_entries, report.bad);
-            store_unit<E, I>(dV, dst, idxV, userV, src, real, n_entries, report.bad);
+            bad |= store_unit<E, I>(dK, dst, idxK, userK, src, real, n_entries);
+            bad |= store_unit<E, I>(dV, dst, idxV, userV, src, real, n_entries);
         }
     }
-    report_done(report, gridDim.x);
+    report_outcome(report, bad, gridDim.x);
 }
 
 template <typename E, typename I>
