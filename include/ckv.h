@@ -259,12 +259,13 @@ CKV_API ckv_status ckv_materialize(ckv_ctx* ctx, int64_t user, void* K_out, void
  *   W        device, bf16 [n_groups][n_entries][d_in]   router weights, an entry's weights contiguous
  *   bias     device, fp32 [n_groups][n_entries], or NULL for none
  *   idx_out  device, int32 [n][n_groups]        what ckv_cache_put takes as idx_K / idx_V
- *   variant  0 = default (tcgen05 kernel), 1 = warp-level tensor-core kernel, 2 = tcgen05 kernel
+ *   variant  0 = default (the tcgen05 kernel, or, for few positions, a warp-level tensor-core kernel that shares the
+ *            entries), 1 = warp-level tensor-core kernel, 2 = tcgen05 kernel
  * Products are exact, sums fp32; scores equal in that arithmetic resolve to the lowest index.  The bias
- * is one of the summands, unrounded: the tensor cores add it with the products (variant 1: it is added
- * behind them), so scores no further apart than the rounding of such a sum may resolve differently in
- * the two variants.  The tcgen05 kernel's waits are bounded; the call reads its error word and
- * therefore waits for the kernel (variant 1 is only stream-ordered).
+ * is one of the summands, unrounded: the tcgen05 kernel adds it with the products (the others: behind
+ * them), so scores no further apart than the rounding of such a sum may resolve differently from one
+ * kernel to the other.  The tcgen05 kernel's waits are bounded and the call reads its error word;
+ * variants 0 and 2 wait for their kernel, whichever it is (variant 1 is only stream-ordered).
  * Errors: INVALID_ARG (sizes, null or host pointers), UNSUPPORTED (d_in), OOM, CUDA (also: a wait
  * inside the kernel ran out; idx_out is not valid then).
  */

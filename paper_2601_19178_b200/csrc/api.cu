@@ -1999,7 +1999,8 @@ ckv_status ckv_route(int32_t device, int32_t n, int32_t n_groups, int32_t d_in, 
     } else {
         HostFlag flag(HostFlag::kRoute);
         if (!flag.p) return CKV_ERR_OOM;
-        e = launch_route_umma(d_in, x, W, bias, n, n_entries, n_groups, idx_out, flag.p, flag.slot(), s);
+        e = (variant == 0 && route_few(d_in, x, W, n, n_entries, n_groups) ? launch_route_few : launch_route_umma)(
+            d_in, x, W, bias, n, n_entries, n_groups, idx_out, flag.p, flag.slot(), s);
         if (e == cudaSuccess) e = wait_done(flag.p + 1, s);
         // a bounded wait inside the kernel ran out: the output is not valid
         if (e == cudaSuccess && *(volatile int*)flag.p) return CKV_ERR_CUDA;

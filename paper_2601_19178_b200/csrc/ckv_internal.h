@@ -288,6 +288,12 @@ constexpr int kRouteSlots = 64;
 cudaError_t launch_route_umma(int d_in, const void* x, const void* W, const float* bias, int n, int n_entries, int G,
                               int32_t* out, int* flags, int slot, cudaStream_t s);
 
+// kernels_route.cu, the same for few positions (route_few says which calls that is): the entries shared by the warps of a
+// cluster.  flags, slot: as above, flags[0] stays 0.
+bool route_few(int d_in, const void* x, const void* W, int n, int n_entries, int G);
+cudaError_t launch_route_few(int d_in, const void* x, const void* W, const float* bias, int n, int n_entries, int G,
+                             int32_t* out, int* flags, int slot, cudaStream_t s);
+
 // out[i][g][c] = x_i . W[g][c] + bias[g][c] (bf16 in and out, fp32 sums); W [G][d_out][d_in], bias [G][d_out] or null.
 bool project_supported(int d_in, int d_out, int n_groups);
 cudaError_t launch_project(int d_in, int d_out, int G, const void* x, const void* W, const float* bias, int64_t n,

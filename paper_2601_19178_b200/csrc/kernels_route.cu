@@ -167,6 +167,173 @@ cudaError_t launch_route_t(const void* x, const void* W, const float* bias, int 
     return cudaGetLastError();
 }
 
+// Few positions: 32 per block, and its eight warps (of up to eight blocks of a cluster) share the entries, each a run of
+// consecutive tiles of eight.  Entry rows go from L2 into the B fragments by 16-byte loads, no shared memory: lane (g, t)
+// holds pieces t, t + 4, ... of entry g's row, so that the feature order of the dot product is permuted, in both operands
+// alike.  The next four tiles are requested before the four at hand are worked on.  What bounds it is latency, a launch and
+// the report to the host included (the tcgen05 kernel has TMEM, barriers, tensor maps and a pipeline to set up first), and
+// with more positions the weights, which every block of 32 reads from L2 for itself.
+constexpr int kFewRows = 32, kFewWarps = 8, kFewMaxSplit = 8, kFewBatch = 4;
+
+__device__ unsigned few_count[kRouteSlots];  // finished blocks of the launch that holds the slot, zero between launches
+
+template <int DIN>
+__global__ void __launch_bounds__(kFewWarps * 32, DIN == 128 ? 1 : 2)
+    route_few_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ W, const float* __restrict__ bias, int n,
+                     int m, int G, int32_t* __restrict__ out, int* flags, int slot, int n_split)
+{
+    constexpr int PIECES = DIN / 32, MT = kFewRows / 16, B = kFewBatch;
+    __shared__ float2 found[kFewWarps][kFewRows];  // (score, entry) of a warp; row 0: of the block
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int grp = blockIdx.y, split = (int)(blockIdx.x % (uint32_t)n_split);
+    const int64_t row0 = (int64_t)(blockIdx.x / (uint32_t)n_split) * kFewRows;
+    const uint16_t* Wg = W + (int64_t)grp * m * DIN;
+    const float* bg = bias ? bias + (int64_t)grp * m : nullptr;
+    const int tiles = (m + 7) / 8, parts = kFewWarps * n_split, part = split * kFewWarps + warp;
+    const int first = (int)((int64_t)tiles * part / parts), end = (int)((int64_t)tiles * (part + 1) / parts);
+
+    uint4 w[B][PIECES];
+    float b0[B], b1[B];
+    auto fetch = [&](int tile) {  // tiles `tile` .. + B - 1 (past the last entry: the last row, bias -inf)
+#pragma unroll
+        for (int i = 0; i < B; ++i) {
+            const int j = min(8 * (tile + i) + g, m - 1), c = 8 * (tile + i) + 2 * t;
+#pragma unroll
+            for (int q = 0; q < PIECES; ++q) w[i][q] = __ldg(reinterpret_cast<const uint4*>(Wg + (int64_t)j * DIN) + t + 4 * q);
+            b0[i] = c < m ? (bg ? __ldg(bg + c) : 0.f) : -CUDART_INF_F;
+            b1[i] = c + 1 < m ? (bg ? __ldg(bg + c + 1) : 0.f) : -CUDART_INF_F;
+        }
+    };
+    if (first < end) fetch(first);
+    uint4 xa[MT][2][PIECES];  // rows g and g + 8 of each tile of sixteen positions
+#pragma unroll
+    for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int64_t r = row0 + 16 * mt + 8 * h + g;
+#pragma unroll
+            for (int q = 0; q < PIECES; ++q)
+                xa[mt][h][q] = r < n ? __ldg(reinterpret_cast<const uint4*>(x + r * DIN) + t + 4 * q) : make_uint4(0, 0, 0, 0);
+        }
+    float bv[MT][2];
+    int bi[MT][2];
+#pragma unroll
+    for (int mt = 0; mt < MT; ++mt) {
+        bv[mt][0] = bv[mt][1] = -CUDART_INF_F;
+        bi[mt][0] = bi[mt][1] = 0;
+    }
+    for (int tile = first; tile < end; tile += B) {
+        uint4 cw[B][PIECES];
+        float c0[B], c1[B];
+#pragma unroll
+        for (int i = 0; i < B; ++i) {
+#pragma unroll
+            for (int q = 0; q < PIECES; ++q) cw[i][q] = w[i][q];
+            c0[i] = b0[i];
+            c1[i] = b1[i];
+        }
+        if (tile + B < end) fetch(tile + B);
+#pragma unroll
+        for (int i = 0; i < B; ++i) {
+            if (tile + i >= end) break;
+            const int j = 8 * (tile + i) + 2 * t;  // entries of this lane's two accumulator columns
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt) {
+                float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int q = 0; q < PIECES; ++q) {
+                    const uint4 lo = xa[mt][0][q], hi = xa[mt][1][q];
+                    const uint32_t a0[4] = {lo.x, hi.x, lo.y, hi.y}, a1[4] = {lo.z, hi.z, lo.w, hi.w};
+                    mma_bf16(acc, a0, cw[i][q].x, cw[i][q].y);
+                    mma_bf16(acc, a1, cw[i][q].z, cw[i][q].w);
+                }
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    // entries come in increasing order: a strict comparison keeps the lowest among equals, and a score that
+                    // is not a number is never taken
+                    const float v0 = acc[2 * h] + c0[i], v1 = acc[2 * h + 1] + c1[i];
+                    if (v0 > bv[mt][h]) {
+                        bv[mt][h] = v0;
+                        bi[mt][h] = j;
+                    }
+                    if (v1 > bv[mt][h]) {
+                        bv[mt][h] = v1;
+                        bi[mt][h] = j + 1;
+                    }
+                }
+            }
+        }
+    }
+    // the lanes of a row, the warps of the block and the blocks of the cluster hold disjoint entries: the best of them, the
+    // lowest entry among equals
+    auto better = [](float v2, int i2, float v, int i) { return v2 > v || (v2 == v && i2 < i); };
+#pragma unroll
+    for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            float v = bv[mt][h];
+            int i = bi[mt][h];
+#pragma unroll
+            for (int o = 1; o <= 2; o <<= 1) {
+                const float v2 = __shfl_xor_sync(0xffffffffu, v, o);
+                const int i2 = __shfl_xor_sync(0xffffffffu, i, o);
+                if (better(v2, i2, v, i)) {
+                    v = v2;
+                    i = i2;
+                }
+            }
+            if (t == 0) found[warp][16 * mt + 8 * h + g] = make_float2(v, __int_as_float(i));
+        }
+    __syncthreads();
+    float v = 0.f;
+    int i = 0;
+    if (warp == 0) {
+        v = found[0][lane].x;
+        i = __float_as_int(found[0][lane].y);
+#pragma unroll
+        for (int k = 1; k < kFewWarps; ++k) {
+            const float2 f = found[k][lane];
+            if (better(f.x, __float_as_int(f.y), v, i)) {
+                v = f.x;
+                i = __float_as_int(f.y);
+            }
+        }
+        found[0][lane] = make_float2(v, __int_as_float(i));
+    }
+    if (n_split > 1) {
+        asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (split == 0 && warp == 0) {
+            for (int r = 1; r < n_split; ++r) {
+                uint32_t remote;
+                float v2, i2;
+                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_u32(&found[0][lane])), "r"(r));
+                asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v2), "=f"(i2) : "r"(remote) : "memory");
+                if (better(v2, __float_as_int(i2), v, i)) {
+                    v = v2;
+                    i = __float_as_int(i2);
+                }
+            }
+        }
+        asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+    if (warp == 0 && split == 0 && row0 + lane < n) out[(row0 + lane) * G + grp] = i;
+    if (slot >= 0 && split == 0) report_done(Report{flags, flags + 1, &few_count[slot]}, gridDim.x / (unsigned)n_split * gridDim.y);
+}
+
+template <int DIN>
+cudaError_t launch_route_few_t(const void* x, const void* W, const float* bias, int n, int m, int G, int32_t* out, int* flags,
+                               int slot, cudaStream_t s)
+{
+    const int64_t blocks = (int64_t)((n + kFewRows - 1) / kFewRows) * G;
+    const int tiles = (m + 7) / 8;
+    // a cluster's blocks share the entries as long as there are SMs for them and each warp keeps two batches
+    int split = 1;
+    while (split < kFewMaxSplit && blocks * split * 2 <= (DIN == 128 ? 148 : 2 * 148) && tiles >= 2 * split * kFewWarps * 2 * kFewBatch) split *= 2;
+    const dim3 grid((unsigned)((n + kFewRows - 1) / kFewRows * split), (unsigned)G);
+    return launch_kernel(Launch{s, nullptr, nullptr}, route_few_kernel<DIN>, grid, kFewWarps * 32, 0, split, (const uint16_t*)x,
+                         (const uint16_t*)W, bias, n, m, G, out, flags, slot, split);
+}
+
 // User-specific low-dimensional projection of the prefill (Sec. 4.2): y[i][g][c] = x_i . W[g][c] + b[g][c],
 // d_out <= 16 outputs per group.  Memory-bound: one thread per output element, the weights in shared memory
 // (rows padded by 16 bytes against bank conflicts), 16-byte loads of the input row, fp32 sums, bf16 result.
@@ -212,6 +379,25 @@ cudaError_t launch_route(int d_in, const void* x, const void* W, const float* bi
         case 32: return launch_route_t<32>(x, W, bias, n, n_entries, G, out, s);
         case 64: return launch_route_t<64>(x, W, bias, n, n_entries, G, out, s);
         default: return launch_route_t<128>(x, W, bias, n, n_entries, G, out, s);
+    }
+}
+
+// Up to 1.1e9 products: 500 positions x 16384 entries x 2 groups (d_in 64, 1.05e9) 37 us against 42 with the tcgen05 kernel,
+// 1000 x 4096 x 4 27 / 32, 2000 x 4096 x 4 (d_in 32) 29 / 34; at 1.3e9 33 / 32 and 39 / 34, at 2.1e9 40 / 42 and 47 / 40 (a call
+// and a wait for the stream, before the report; without that wait the line lies in the same place).
+bool route_few(int d_in, const void* x, const void* W, int n, int n_entries, int G)
+{
+    if (((uintptr_t)x | (uintptr_t)W) & 15) return false;  // rows are read sixteen bytes at a time
+    return (double)n * n_entries * G * d_in <= 1.1e9;
+}
+
+cudaError_t launch_route_few(int d_in, const void* x, const void* W, const float* bias, int n, int n_entries, int G,
+                             int32_t* out, int* flags, int slot, cudaStream_t s)
+{
+    switch (d_in) {
+        case 32: return launch_route_few_t<32>(x, W, bias, n, n_entries, G, out, flags, slot, s);
+        case 64: return launch_route_few_t<64>(x, W, bias, n, n_entries, G, out, flags, slot, s);
+        default: return launch_route_few_t<128>(x, W, bias, n, n_entries, G, out, flags, slot, s);
     }
 }
 

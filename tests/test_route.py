@@ -269,3 +269,22 @@ def test_gpu_router_at_the_edges_of_blocks_and_tiles(d_in, n, m):
         b[0, j] = b[1, j] = 1.0
         b[1, m - 1] = 1.0
         assert (_gpu_route(x, np.zeros_like(W), b) == j).all(), j
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("d_in,n,m,G", [(32, 1, 1, 1), (32, 33, 7, 2), (64, 32, 9, 1), (64, 31, 257, 3), (128, 65, 4096, 1),
+                                        (64, 200, 16384, 1), (32, 1000, 2048, 2), (64, 1072, 8000, 2), (64, 1075, 8000, 2)])
+def test_gpu_router_for_few_positions(d_in, n, m, G):
+    """The kernel that shares the entries among warps and clusters: blocks of 32 positions, tiles of eight entries, begun ones,
+    warps without a tile, and both sides of the line (1.1e9 products) beyond which the tcgen05 kernel takes over."""
+    rng = np.random.default_rng(n + m)
+    x = _bf16(rng.standard_normal((n, d_in)) / np.sqrt(d_in))
+    W = rng.standard_normal((G, m, d_in)).astype(np.float32)
+    bias = (0.1 * rng.standard_normal((G, m))).astype(np.float32)
+    _check(x, _bf16(W), bias, f"d_in={d_in} n={n} m={m} G={G}")
+    _check(x, _bf16(W), None, f"no bias d_in={d_in} n={n} m={m} G={G}")
+    # every entry there twice: the same sums, so the first one of the two, whichever warp or block holds it
+    half = (m + 1) // 2
+    W[:, half:] = W[:, :m - half]
+    bias[:, half:] = bias[:, :m - half]
+    assert _gpu_route(x, _bf16(W), bias).max() < half
