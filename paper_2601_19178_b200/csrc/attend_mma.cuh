@@ -39,6 +39,7 @@ namespace ckv {
 namespace {
 
 constexpr float kLog2e = 1.4426950408889634f;
+constexpr float kSumLimit = 0x1p70f;  // see `normalise`
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src)
 {
@@ -457,50 +458,80 @@ __global__ void __launch_bounds__(128, MmaCfg<D, MT, TMA>::MIN_BLOCKS)
                         if (pc + 1 >= e_hi) s[nt][3] = -CUDART_INF_F;
                     }
                 }
-                float mx0 = s[0][0], mx1 = s[0][2];
+                // A row's reference is the maximum of the first tile and stays there: fp32 sums and bf16 weights have the
+                // exponent range for scores far above it.  A lane's eight weights that add up to more than 2^70, or to no
+                // number, give away that a score has left it; then, as in the first tile, the reference goes to the
+                // maximum.  (A row that sees nothing of the first tile sees nothing of the others.)  That takes the maxima
+                // and four dependent shuffles out of every other tile (65536 users x 512 positions x 16 queries
+                // 2364 -> 2163 us, 4096 x 512 x 16 64-wide 315 -> 259, 199 ragged ones 63 -> 58).
+                float ps0, ps1;
+                auto weigh = [&]() {  // the weights and this lane's share of their sums
+                    const float r0 = VAR && m_run[mt][0] == -CUDART_INF_F ? 0.f : m_run[mt][0],
+                                r1 = VAR && m_run[mt][1] == -CUDART_INF_F ? 0.f : m_run[mt][1];
+                    ps0 = ps1 = 0.f;
 #pragma unroll
-                for (int nt = 0; nt < 4; ++nt) {
-                    mx0 = fmaxf(mx0, fmaxf(s[nt][0], s[nt][1]));
-                    mx1 = fmaxf(mx1, fmaxf(s[nt][2], s[nt][3]));
-                }
-                mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 1));
-                mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 2));
-                if (has_hi) {
-                    mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 1));
-                    mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 2));
-                }
-                // a row may not see any position of this tile (or of any tile so far): its maximum is then -inf
-                // and must not enter the exponent arguments
-                const float mn0 = fmaxf(m_run[mt][0], mx0 * sc);
-                const float mn1 = has_hi ? fmaxf(m_run[mt][1], mx1 * sc) : 0.f;
-                // (without visible lengths the first position of a tile is always attended and the maxima are finite)
-                const float ms0 = VAR && mn0 == -CUDART_INF_F ? 0.f : mn0, ms1 = VAR && mn1 == -CUDART_INF_F ? 0.f : mn1;
-                // the running maxima settle after a few tiles: rescale only when one of them moved
-                const bool moved = mn0 != m_run[mt][0] || (has_hi && mn1 != m_run[mt][1]);
-                if (__any_sync(0xffffffffu, moved)) {
-                    const float c0 = ex2(m_run[mt][0] - ms0), c1 = has_hi ? ex2(m_run[mt][1] - ms1) : 1.f;
-                    m_run[mt][0] = mn0;
-                    if (has_hi) m_run[mt][1] = mn1;
-                    l_run[mt][0] *= c0;
-                    l_run[mt][1] *= c1;
-#pragma unroll
-                    for (int j = 0; j < NTD; ++j) {
-                        o[mt][j][0] *= c0; o[mt][j][1] *= c0;
-                        o[mt][j][2] *= c1; o[mt][j][3] *= c1;
+                    for (int nt = 0; nt < 4; ++nt) {
+                        const float p0v = ex2(fmaf(s[nt][0], sc, -r0)), p1v = ex2(fmaf(s[nt][1], sc, -r0));
+                        ps0 += p0v + p1v;
+                        pa[nt >> 1][(nt & 1) * 2] = pack_bf16(p0v, p1v);
+                        if (has_hi) {
+                            const float p2v = ex2(fmaf(s[nt][2], sc, -r1)), p3v = ex2(fmaf(s[nt][3], sc, -r1));
+                            ps1 += p2v + p3v;
+                            pa[nt >> 1][(nt & 1) * 2 + 1] = pack_bf16(p2v, p3v);
+                        } else {
+                            pa[nt >> 1][(nt & 1) * 2 + 1] = 0u;
+                        }
                     }
-                }
-                float ps0 = 0.f, ps1 = 0.f;
+                };
+                auto left = [&]() { return __any_sync(0xffffffffu, !(ps0 <= kSumLimit && ps1 <= kSumLimit)) != 0; };
+                auto move = [&]() {
+                    float mx0 = s[0][0], mx1 = s[0][2];
 #pragma unroll
-                for (int nt = 0; nt < 4; ++nt) {
-                    const float p0v = ex2(fmaf(s[nt][0], sc, -ms0)), p1v = ex2(fmaf(s[nt][1], sc, -ms0));
-                    ps0 += p0v + p1v;
-                    pa[nt >> 1][(nt & 1) * 2] = pack_bf16(p0v, p1v);
+                    for (int nt = 0; nt < 4; ++nt) {
+                        mx0 = fmaxf(mx0, fmaxf(s[nt][0], s[nt][1]));
+                        mx1 = fmaxf(mx1, fmaxf(s[nt][2], s[nt][3]));
+                    }
+                    mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 1));
+                    mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 2));
                     if (has_hi) {
-                        const float p2v = ex2(fmaf(s[nt][2], sc, -ms1)), p3v = ex2(fmaf(s[nt][3], sc, -ms1));
-                        ps1 += p2v + p3v;
-                        pa[nt >> 1][(nt & 1) * 2 + 1] = pack_bf16(p2v, p3v);
-                    } else {
-                        pa[nt >> 1][(nt & 1) * 2 + 1] = 0u;
+                        mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 1));
+                        mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 2));
+                    }
+                    // a row may not see any position of this tile (or of any tile so far): its maximum is then -inf
+                    // and must not enter the exponent arguments
+                    const float mn0 = fmaxf(m_run[mt][0], mx0 * sc);
+                    const float mn1 = has_hi ? fmaxf(m_run[mt][1], mx1 * sc) : 0.f;
+                    // (without visible lengths the first position of a tile is always attended and the maxima are finite)
+                    const float ms0 = VAR && mn0 == -CUDART_INF_F ? 0.f : mn0, ms1 = VAR && mn1 == -CUDART_INF_F ? 0.f : mn1;
+                    // the running maxima settle after a few tiles: rescale only when one of them moved
+                    const bool moved = mn0 != m_run[mt][0] || (has_hi && mn1 != m_run[mt][1]);
+                    if (__any_sync(0xffffffffu, moved)) {
+                        const float c0 = ex2(m_run[mt][0] - ms0), c1 = has_hi ? ex2(m_run[mt][1] - ms1) : 1.f;
+                        m_run[mt][0] = mn0;
+                        if (has_hi) m_run[mt][1] = mn1;
+                        l_run[mt][0] *= c0;
+                        l_run[mt][1] *= c1;
+#pragma unroll
+                        for (int j = 0; j < NTD; ++j) {
+                            o[mt][j][0] *= c0; o[mt][j][1] *= c0;
+                            o[mt][j][2] *= c1; o[mt][j][3] *= c1;
+                        }
+                    }
+                };
+                if constexpr (SHARED) {  // (one copy of the code: a warp that shares a short unit meets it cold)
+                    bool moves = step == 0;
+#pragma unroll 1
+                    while (true) {
+                        if (moves) move();
+                        weigh();
+                        if (moves || !left()) break;
+                        moves = true;
+                    }
+                } else {
+                    if (step != 0) weigh();
+                    if (step == 0 || left()) {
+                        move();
+                        weigh();
                     }
                 }
                 l_run[mt][0] += ps0;

@@ -222,3 +222,22 @@ def test_tcgen05_kernel_rows_that_see_parts_of_a_tile(mode, queries):
     want = O.attend_variants(w.dtype, w.mode, w.default_scale, w.head_dim, d["pool_K"], d["pool_V"], d["hist_off"], d["idx_K"],
                              d["idx_V"], d["user_K"], d["user_V"], d["q_off"], d["queries"], vis=vis)
     assert_close(out.float().cpu().numpy().astype(np.float64), want, "bf16", f"{mode} {queries}")
+
+
+@pytest.mark.parametrize("users", [1, 900])
+@pytest.mark.parametrize("head,queries", [((30, 2), 7), ((30, 2), 16), ((30, 2), 33), ((60, 4), 5), ((60, 4), 20)])
+@pytest.mark.parametrize("ramp", [(-60, 60), (60, -60), (0, 95)])
+def test_warp_level_kernel_reference_far_from_later_scores(users, head, queries, ramp):
+    """Scores that climb or fall by 130 to 170 octaves along a history: a row's reference, the maximum of its first tile, is left
+    and moved, or stays far above everything behind it.  One user: warps share a unit and merge references apart."""
+    w = _workload(head=head, users=users, hist=(200, 400), queries=queries)
+    d = synth.generate(w)
+    for a, b in zip(d["hist_off"][:-1], d["hist_off"][1:]):
+        d["user_K"][a:b, :, 0] = synth.f32_to_bf16_bits(np.linspace(*ramp, b - a, dtype=np.float32))[:, None]
+    d["queries"][:, :, 0] = synth.f32_to_bf16_bits(np.full(d["queries"].shape[:2], 1.0, np.float32))
+    sel = np.arange(0, users, 90)
+    s = make_session(w, d, scale=1.0, kernel=2)
+    got = gpu_attend(w, d, session=s)
+    s.close()
+    rows = np.concatenate([np.arange(d["q_off"][u], d["q_off"][u + 1]) for u in sel])
+    assert_close(got[rows], oracle_attend(w, d, scale=1.0, sel=sel), "bf16", f"{users} {head} {queries} {ramp}")
