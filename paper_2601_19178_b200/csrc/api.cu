@@ -642,7 +642,7 @@ int mma_qpw(const ckv_ctx* ctx, const ListShape& s)
 // head_dim 64; at 32 by how many 16-query tiles of a unit hold queries, see `longer`), but leaves fewer units to spread:
 // lists of few long histories are better off with 16.
 template <typename F>
-void mma_shape(const ckv_ctx* ctx, const ListShape& s, int64_t chunk, F&& each, int& qpw, int& parts)
+void mma_shape(const ckv_ctx* ctx, const ListShape& s, int64_t chunk, F&& each, int& qpw, int& parts, double* tile_times = nullptr)
 {
     auto estimate = [&](int q, int& p) {
         MmaWork w;
@@ -654,6 +654,7 @@ void mma_shape(const ckv_ctx* ctx, const ListShape& s, int64_t chunk, F&& each, 
     };
     qpw = mma_qpw(ctx, s);
     const double t = estimate(qpw, parts);
+    if (tile_times) *tile_times = t;
     int p16;
     if (qpw == 16) return;
     const bool softmax = ctx->cfg.mode == CKV_SOFTMAX;
@@ -662,21 +663,26 @@ void mma_shape(const ckv_ctx* ctx, const ListShape& s, int64_t chunk, F&& each, 
     const double used = units * ctx->cfg.n_groups >= 8 * warps ? (double)s.units[0] / units : qpw / 16;
     const double longer = ctx->cfg.head_dim == 64 ? 1.45 : qpw == 32 ? (softmax ? 0.65 + 0.42 * used : 0.72 + 0.31 * used)
                                                                     : (softmax ? 0.27 + 0.42 * used : 0.29 + 0.34 * used);
-    if (estimate(16, p16) < longer * t) {
+    const double t16 = estimate(16, p16);
+    if (t16 < longer * t) {
         qpw = 16;
         parts = p16;
+        if (tile_times) *tile_times = t16;
     }
 }
 
 // Chunk length of the tcgen05 kernel: the one with the shortest estimated run, in microseconds.  Three persistent workers
-// per SM walk a (chunk, group, 128 queries) unit alone; measured, a worker takes 1 us per 64 positions when it has the SM
-// to itself and 1.4 next to two others, 1.5 per unit, the launch 6, and merging chunks 6 and 0.007 per chunk.  Units of one size
-// run in whole rounds; mixed ones are dealt out longest first, and only the longest of them bounds the run from below.
+// per SM walk a (chunk, group, 128 queries) unit alone; a worker takes 0.68 us per 64 positions when it has the SM
+// to itself and 1.2 next to two others (0.77 if one of its four warps has rows), 1.2 per unit, the launch 6.6, and merging
+// chunks 6 and 0.007 per chunk.  Units of one size run in whole rounds; mixed ones are dealt out longest first, and only the
+// longest of them bounds the run from below.  (Fitted to 244 lists of 4..3900 users, 32..3000 positions, 1..93 queries: 10 %.)
 int64_t umma_chunk(const ckv_ctx* ctx, const ListShape& s, double* time = nullptr)
 {
     const double workers = 3.0 * ctx->n_sms, G = ctx->cfg.n_groups;
     const MmaWork w16 = s.mma(16);
     const bool alike = w16.alike && w16.min_tiles == w16.max_tiles;
+    // warps of a block of 128 queries that have rows, of four (s.units[1]: blocks of 32 queries)
+    const double filled = s.blocks128 > 0 ? 0.26 + 0.185 * (double)s.units[1] / (double)s.blocks128 : 1;
     int64_t best = 16384;
     double best_t = 1e300;
     for (int64_t n = (s.max_L + 16383) / 16384, last = 0; n <= 512 && last != 256; n += (n + 15) / 16) {
@@ -687,15 +693,15 @@ int64_t umma_chunk(const ckv_ctx* ctx, const ListShape& s, double* time = nullpt
         const double cut = alike ? (double)((s.max_L + c - 1) / c) * s.blocks128 : s.tiles64 * 64.0 / c + (split ? 0.5 : 0) * s.blocks128;
         const double units = G * std::max<double>(cut, s.blocks128), tiles = c / 64;
         auto unit_us = [&](double n_tiles, double n) {  // of n units that run at a time
-            return n_tiles * (0.8 + 0.2 * std::min(3.0, std::max(1.0, n / ctx->n_sms))) + 1.5;
+            return n_tiles * (0.42 + 0.26 * filled * std::min(3.0, std::max(1.0, n / ctx->n_sms))) + 1.2;
         };
         const double longest = std::min<double>(tiles, (s.max_L + 63) / 64);
-        double t = 6 + (split ? 6 + 0.007 * units : 0);
+        double t = 6.6 + (split ? 6 + 0.007 * units : 0);
         if (alike) {
             const double full = std::floor(units / workers), rest = units - full * workers;
             t += full * unit_us(longest, workers) + (rest > 0 ? unit_us(longest, rest) : 0);
         } else
-            t += std::max(unit_us(longest, units), (unit_us(s.tiles64 * G, units) + 1.5 * (units - 1)) / workers);
+            t += std::max(unit_us(longest, units), (unit_us(s.tiles64 * G, units) + 1.2 * (units - 1)) / workers);
         if (t < best_t) {
             best_t = t;
             best = c;
@@ -715,21 +721,38 @@ int choose_family(const ckv_ctx* ctx, bool with_vis, const ListShape& s)
     // factorisation
     const bool plain = !with_vis && !ctx->full_k && !ctx->full_v;
     const bool can_umma = ctx->has_umma;
-    // tcgen05 from three 16-query blocks on, else the warp-level tensor-core kernel (faster than the CUDA-core
-    // kernel from a single query on); the CUDA-core kernel serves what neither supports.  Up to six blocks the
-    // warp-level kernel also takes lists too small to fill the tcgen05 kernel's workers (measured: 1.2 us per tile time of
-    // its resident warps and 4 us besides), and for self-attention, as many queries as positions with visible lengths, lists of
-    // any number: half of their pairs count, and the tcgen05 kernel needs a plan and a launch for the limits, 5 us, whatever the
-    // list.  (The estimates are of whole histories, the limits may be on the device.  7 causal self-attentions of 556
-    // positions, 2 groups: 22.7 us there, 11.0 here; one of 50 12.4 and 4.3; eight of 500, 8 groups, 22.7 and 23.7.)
-    // (not where the option asks for the TMA loader, which takes neither limits nor sides that are not shared)
-    bool few = false;
+    // The warp-level tensor-core kernel up to 16 queries per user, whose rows it gathers once; the tcgen05 kernel above 96; in
+    // between the shorter estimated run.  (The CUDA-core kernel serves what neither supports.)  The warp-level kernel's: 3.9
+    // us and a cost per tile time of its resident warps, by the queries a warp holds.  Below 48 queries a list that could
+    // travel as a kernel argument there has its planning for the tcgen05 kernel counted, 15 us and 0.16 per user of the host,
+    // which bound a caller with a new list on every call (199 users of 17..1999 positions, 1..40 queries: 47 us a call, the
+    // kernel 28, the warp-level one 35).  Of the 244 lists that umma_chunk is fitted to, most get the faster kernel; they lose
+    // 1.2 % in the mean, 36 % at most (with the tcgen05 kernel from 48 queries on alone 3.8 and 74).  24 queries, 250
+    // users of 100..1500 positions, 4 groups: 39.6 / 31.8 us; 40 queries, 1500 x 1000, 8 groups: 567 / 470; 20 x 2000: 23.2 / 27.3.
+    // For self-attention, as many queries as positions with visible lengths, lists of any number are compared: half of
+    // their pairs count, and the tcgen05 kernel needs a launch for the limits, 5 us, whatever the list.  (The estimates are of
+    // whole histories, the limits may be on the device.  7 causal self-attentions of 556 positions, 2 groups: 22.7 us there, 11.0
+    // here; one of 50 12.4 and 4.3; nine of 1150 25.1 and 39.3.)
+    // (Not compared where the option asks for the TMA loader, which takes neither limits nor sides that are not shared:
+    // the tcgen05 kernel from 48 queries on.)
     const bool loads = ctx->opt_loader != 2 || (plain && ctx->has_tma);
-    if (can_umma && can_mma && loads && max_M >= 48 && (max_M <= 96 || (with_vis && s.rows >= total_pos)) && n_active > 0) {
+    const bool self = with_vis && s.rows >= total_pos;
+    bool few = max_M < (can_mma && loads ? 17 : 48);
+    if (can_umma && can_mma && loads && !few && n_active > 0 && (max_M <= 96 || self)) {
+        int qpw, parts;
         double tile_times, t_umma;
-        mma_parts(ctx, s.mma(16), 16, &tile_times);
         umma_chunk(ctx, s, &t_umma);
-        few = 4 + 1.2 * tile_times < t_umma + (with_vis ? 5 : 0);
+        if (self) {
+            mma_parts(ctx, s.mma(16), 16, &tile_times);
+            few = 4 + 0.7 * tile_times < t_umma + 5;
+        } else {
+            mma_shape(ctx, s, INT32_MAX, [](auto&&) {}, qpw, parts, &tile_times);
+            const bool softmax = ctx->cfg.mode == CKV_SOFTMAX;
+            const double per_tile = qpw == 16 ? (softmax ? 0.99 : 0.87) : qpw == 32 ? (softmax ? 1.55 : 1.14) : (softmax ? 1.59 : 1.26);
+            if (with_vis) t_umma += 5;
+            if (max_M < 48 && n_active <= kInlineReqs) t_umma = std::max(t_umma, 15 + 0.16 * (double)n_active);
+            few = 3.9 + per_tile * tile_times < 1.05 * t_umma;
+        }
     }
     // One query per user: the pool-side factorisation trades the row gathers for two tables per (user, group).
     const bool can_fact = plain && s.single() &&
@@ -751,7 +774,7 @@ int choose_family(const ckv_ctx* ctx, bool with_vis, const ListShape& s)
         fact_pays = t_fact < t_gather;
     }
     switch (ctx->opt_kernel) {
-        case 0: return can_umma && max_M >= 48 && !few ? 3 : fact_pays ? 4 : can_mma ? 2 : 1;
+        case 0: return can_umma && !few ? 3 : fact_pays ? 4 : can_mma ? 2 : 1;
         case 1: return 1;
         case 2: return can_mma ? 2 : 0;
         case 3: return can_umma ? 3 : 0;
