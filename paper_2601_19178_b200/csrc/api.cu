@@ -154,6 +154,7 @@ struct Plan {
     Work* d_works = nullptr;
     int32_t n_items = 0, n_split = 0, split_items = 0, max_M = 0, n_req = 0, family = 1, n_works = 0;
     int32_t parts = 1, qpw = 16;  // family 2: warps that share a unit, queries a warp holds
+    bool dense = false;           // ... more resident warps with shallower rings
     bool wide = false;            // family 1: blocks of more warps
     int64_t part_rows = 0;
     uint64_t last_use = 0;
@@ -555,10 +556,10 @@ struct MmaWork {
 // about four tiles, across a cluster five (head_dim 64: six, with clusters of eight nine).  Units of one size run in whole
 // rounds; mixed ones, longest histories first, leave SMs idle for about three quarters of the longest.  (Fitted to sweeps of 1..32 warps over
 // 1..300 users of 200..16384 positions; within 15 % of most, and the number it picks within 6 % of the best.)
-int mma_parts(const ckv_ctx* ctx, const MmaWork& w, int qpw, double* tile_times)
+int mma_parts(const ckv_ctx* ctx, const MmaWork& w, int qpw, double* tile_times, bool dense = false)
 {
     const int D = ctx->cfg.head_dim;
-    const double warps = (double)ctx->n_sms * mma_warps_per_sm(D, qpw), G = ctx->cfg.n_groups;
+    const double warps = (double)ctx->n_sms * mma_warps_per_sm(D, qpw, dense), G = ctx->cfg.n_groups;
     int best = 1;
     double best_t = 1e300;
     for (int parts = 1; parts <= kMmaMaxParts && parts <= std::max<int64_t>(w.max_tiles, 1); parts *= 2) {
@@ -637,25 +638,46 @@ int mma_qpw(const ckv_ctx* ctx, const ListShape& s)
     return mma_queries_per_warp(D, s.max_M, s.tiles[0] * ctx->cfg.n_groups >= (int64_t)20 * ctx->n_sms * mma_warps_per_sm(D, 16));
 }
 
+constexpr double kDenseTile = 1.3;  // see mma_shape
+
 // Queries per warp and warps per unit of histories cut into chunks of `chunk`; `each(add)` calls add(L, M) for every request
 // with a query.  Holding more queries per warp saves gathers and lengthens a tile (measured 1.45 times for 32 queries at
 // head_dim 64; at 32 by how many 16-query tiles of a unit hold queries, see `longer`), but leaves fewer units to spread:
 // lists of few long histories are better off with 16.
+// `plain` (both sides shared, no visible lengths): 64-wide heads may also run `dense`, twelve resident warps with rings of two
+// slots instead of eight with three, whose tile times count kDenseTile times as long.  That is the ratio of a warp that
+// has latency to wait for and no others beside it; on full SMs the dense form is 6 to 15 % faster (199 ragged users 58.3 -> 50.3 us a
+// call, 4096 x 512 x 16 queries 259 -> 242, 2000 of 30..300 positions 47.8 -> 41.6), and 29 % where a list fits twelve
+// warps in one round and eight in two (220 users x 1000, 2 groups: 22.2 -> 15.7 us); of 56 lists none lost more than 4 %.  At 1.2
+// lists of a few ragged users lose up to 19 %.
 template <typename F>
-void mma_shape(const ckv_ctx* ctx, const ListShape& s, int64_t chunk, F&& each, int& qpw, int& parts, double* tile_times = nullptr)
+void mma_shape(const ckv_ctx* ctx, const ListShape& s, int64_t chunk, bool plain, F&& each, int& qpw, int& parts, bool& dense,
+               double* tile_times = nullptr)
 {
-    auto estimate = [&](int q, int& p) {
+    dense = false;
+    auto estimate = [&](int q, int& p, bool& d) {
         MmaWork w;
         if (chunk >= s.max_L) w = s.mma(q);
         else each([&](int32_t L, int32_t M) { w.add(L, mma_blocks(M, q), s.same_M(), chunk); });
         double t;
         p = mma_parts(ctx, w, q, &t);
+        d = false;
+        if (plain && ctx->cfg.head_dim == 64 && q == 16) {
+            double td;
+            const int pd = mma_parts(ctx, w, q, &td, true);
+            if (kDenseTile * td < t) {
+                t = kDenseTile * td;
+                p = pd;
+                d = true;
+            }
+        }
         return t;
     };
     qpw = mma_qpw(ctx, s);
-    const double t = estimate(qpw, parts);
+    const double t = estimate(qpw, parts, dense);
     if (tile_times) *tile_times = t;
     int p16;
+    bool d16;
     if (qpw == 16) return;
     const bool softmax = ctx->cfg.mode == CKV_SOFTMAX;
     // the tiles of a unit that hold queries, on the average of many units per warp; of few the fullest set the pace
@@ -663,10 +685,11 @@ void mma_shape(const ckv_ctx* ctx, const ListShape& s, int64_t chunk, F&& each, 
     const double used = units * ctx->cfg.n_groups >= 8 * warps ? (double)s.units[0] / units : qpw / 16;
     const double longer = ctx->cfg.head_dim == 64 ? 1.45 : qpw == 32 ? (softmax ? 0.65 + 0.42 * used : 0.72 + 0.31 * used)
                                                                     : (softmax ? 0.27 + 0.42 * used : 0.29 + 0.34 * used);
-    const double t16 = estimate(16, p16);
+    const double t16 = estimate(16, p16, d16);
     if (t16 < longer * t) {
         qpw = 16;
         parts = p16;
+        dense = d16;
         if (tile_times) *tile_times = t16;
     }
 }
@@ -746,7 +769,8 @@ int choose_family(const ckv_ctx* ctx, bool with_vis, const ListShape& s)
             mma_parts(ctx, s.mma(16), 16, &tile_times);
             few = 4 + 0.7 * tile_times < t_umma + 5;
         } else {
-            mma_shape(ctx, s, INT32_MAX, [](auto&&) {}, qpw, parts, &tile_times);
+            bool dense;
+            mma_shape(ctx, s, INT32_MAX, plain, [](auto&&) {}, qpw, parts, dense, &tile_times);
             const bool softmax = ctx->cfg.mode == CKV_SOFTMAX;
             const double per_tile = qpw == 16 ? (softmax ? 0.99 : 0.87) : qpw == 32 ? (softmax ? 1.55 : 1.14) : (softmax ? 1.59 : 1.26);
             if (with_vis) t_umma += 5;
@@ -766,7 +790,7 @@ int choose_family(const ckv_ctx* ctx, bool with_vis, const ListShape& s)
     if (can_fact) {
         const bool wide = ctx->cfg.head_dim == 64;
         const double a = wide ? 1.2 : 1.0, b = wide ? 0.00055 : 0.0005, c = wide ? 0.0010 : 0.0009,
-                     d = wide ? 0.0047 : 0.0027;
+                     d = wide ? 0.0041 : 0.0025;
         const double pairs = (double)n_active * ctx->cfg.n_groups, mean_L = (double)total_pos / (double)n_active;
         const double waves = std::ceil(pairs / ctx->n_sms);
         const double t_fact = 5.0 + waves * (a + b * ctx->n_entries + c * mean_L);
@@ -931,13 +955,14 @@ ckv_status build_plan(ckv_ctx* ctx, Plan& pl, int32_t n, const int64_t* users, c
                       : pl.family == 1                     ? simt_shape(ctx, shape, &pl.wide)
                                                            : auto_split_len(ctx, shape, pl.family);
     pl.parts = 1;
+    pl.dense = false;
     if (pl.family == 2) {
         if (ctx->opt_split > 0) pl.qpw = mma_qpw(ctx, shape);
         else
-            mma_shape(ctx, shape, C, [&](auto&& add) {
+            mma_shape(ctx, shape, C, !with_vis && !ctx->full_k && !ctx->full_v, [&](auto&& add) {
                 for (const Req& r : reqs)
                     if (r.M > 0) add(r.L, r.M);
-            }, pl.qpw, pl.parts);
+            }, pl.qpw, pl.parts, pl.dense);
     }
     std::vector<Item> items;
     std::vector<int32_t> split;
@@ -1591,14 +1616,14 @@ namespace {
 // on B200 a warp spends about 100 clocks per TMA gather instruction it issues, so with the compute warps doing
 // their own gathers the TMA loader measured slower (cfg4: 607 against 522 us; cfg5, Zipf indices that profit
 // from L1, which TMA bypasses: 5.07 against 2.37 ms).  Both loaders give the same bits.
-ckv_status run_mma(ckv_ctx* ctx, int D, int max_M, int qpw, int parts, const AttendArgs& a, const InlineTable* tab,
+ckv_status run_mma(ckv_ctx* ctx, int D, int max_M, int qpw, int parts, bool dense, const AttendArgs& a, const InlineTable* tab,
                    const Launch& l)
 {
     const int loader = ctx->opt_loader == 2 ? 2 : 1;
     // the TMA loader serves the plain form only (both sides shared, no visible lengths)
     if (loader == 2 && (!ctx->has_tma || a.cv.full_k || a.cv.full_v || a.vis)) return CKV_ERR_UNSUPPORTED;
     ctx->st_loader = loader;
-    CK(launch_attend_mma(D, max_M, qpw, parts, a, tab, loader == 2 ? ctx->tmaps : nullptr, ctx->d_err, l));
+    CK(launch_attend_mma(D, max_M, qpw, parts, dense, a, tab, loader == 2 ? ctx->tmaps : nullptr, ctx->d_err, l));
     return CKV_OK;
 }
 
@@ -1630,7 +1655,7 @@ cudaError_t pipe_prepare(ckv_ctx* ctx)
 struct InlineList {
     InlineTable tab;
     int32_t n = 0, max_M = 0, parts = 1, qpw = 16, family = 0;
-    bool wide = false;
+    bool wide = false, dense = false;
 };
 
 // Fills `x`; x.family stays 0 if the list has to go through a plan (too long, or a kernel family or a chunking that
@@ -1653,7 +1678,7 @@ ckv_status inline_list(ckv_ctx* ctx, int32_t n, const int64_t* users, const int3
         (family == 1 ? simt_shape(ctx, shape, &x.wide) : auto_split_len(ctx, shape, family)) < shape.max_L)
         return CKV_OK;
     if (family == 2)
-        mma_shape(ctx, shape, INT32_MAX, [](auto&&) {}, x.qpw, x.parts);
+        mma_shape(ctx, shape, INT32_MAX, !with_vis && !ctx->full_k && !ctx->full_v, [](auto&&) {}, x.qpw, x.parts, x.dense);
     // longest first, as in a plan: the tail of the grid is made of short ones
     if (shape.max_L != shape.min_L && (int64_t)x.n * ctx->cfg.n_groups > ctx->n_sms)
         std::sort(x.tab.r, x.tab.r + x.n, [](const InlineReq& a, const InlineReq& b) { return a.L > b.L; });
@@ -1700,7 +1725,7 @@ ckv_status launch_slice(ckv_ctx* ctx, const Plan* pl, AttendArgs a, int i0, int 
         } else if (pl->family == 3)
             CK(launch_attend_umma(a, ctx->n_sms, ctx->d_err, l));
         else if (pl->family == 2) {
-            ckv_status st2 = run_mma(ctx, D, pl->max_M, pl->qpw, pl->parts, a, nullptr, l);
+            ckv_status st2 = run_mma(ctx, D, pl->max_M, pl->qpw, pl->parts, pl->dense, a, nullptr, l);
             if (st2 != CKV_OK) return st2;
         } else
             CK(launch_attend_simt(ctx->cfg.dtype, D, pl->max_M,
@@ -1828,7 +1853,7 @@ ckv_status attend_impl(ckv_ctx* ctx, int32_t n, const int64_t* users, const int3
             Launch l = launch_on(ctx, s);
             l.early = true;
             st = timed(ctx, ctx->opt_time != 0, s, [&]() -> ckv_status {
-                if (x.family == 2) return run_mma(ctx, D, x.max_M, x.qpw, x.parts, a, &x.tab, l);
+                if (x.family == 2) return run_mma(ctx, D, x.max_M, x.qpw, x.parts, x.dense, a, &x.tab, l);
                 CK(launch_attend_simt(ctx->cfg.dtype, D, x.max_M, x.wide, a, &x.tab, l));
                 return CKV_OK;
             });
@@ -2322,7 +2347,7 @@ extern "C" ckv_status ckv_attend_static(ckv_ctx* ctx, int32_t n, const int64_t* 
     const Launch l{s, nullptr, &ctx->grants};
     if (n_items > 0) {
         if (family == 2)
-            CK(launch_attend_mma(D, max_M, 16, 1, a, nullptr, nullptr, ctx->d_err, l));
+            CK(launch_attend_mma(D, max_M, 16, 1, false, a, nullptr, nullptr, ctx->d_err, l));
         else
             CK(launch_attend_simt(ctx->cfg.dtype, D, max_M, simt_wide(ctx, n_items), a, nullptr, l));
     }

@@ -106,20 +106,23 @@ __device__ __forceinline__ void store_user_part(uint32_t addr, const uint4& r, i
     }
 }
 
-template <int D, int MT, bool TMA>
+// DENSE (64-wide heads, 16 queries a warp): a ring of two slots instead of three, which leaves room for three blocks per SM.
+// The deeper ring is the better one as long as the SMs are not full (see mma_shape in the host code).  (Twenty warps at
+// 32-wide heads spill: 143 -> 229 us for 4096 users x 512 positions x 16 queries; three slots there: 148.)
+template <int D, int MT, bool TMA, bool DENSE = false>
 struct MmaCfg {
     static constexpr int ROWB = D * 2;            // bytes per row
     static constexpr int CPR = ROWB / 16;         // 16-byte chunks per row
     static constexpr int RPI = 32 / CPR;          // rows one warp-wide copy instruction covers
     static constexpr int TILE_B = 32 * ROWB;      // one K or V tile of 32 positions
     // ring depth (more resident warps beat a deeper ring, except for cp.async with 128-byte rows)
-    static constexpr int NST = (D == 64 && !TMA) ? 3 : 2;
+    static constexpr int NST = (D == 64 && !TMA && !DENSE) ? 3 : 2;
     static constexpr int WARPS = 4;
     // TMA: tiles on 1024-byte boundaries (the swizzle pattern follows the address), then one mbarrier per slot
     static constexpr int SMEM = WARPS * NST * 2 * TILE_B + (TMA ? 1024 + WARPS * NST * 8 : 0);
     // (two query tiles, 32-wide: 168 registers and some spills outside the loop; left to itself the compiler takes 200 to 240
     // and a third of the warps goes, 134 us instead of 117 for 3000 users x 300 positions x 20..32 queries, SiLU)
-    static constexpr int MIN_BLOCKS = MT == 1 ? (D == 64 ? (TMA ? 3 : 2) : 4) : D == 32 && MT == 2 ? 3 : 1;
+    static constexpr int MIN_BLOCKS = MT == 1 ? (D == 64 ? (TMA || DENSE ? 3 : 2) : 4) : D == 32 && MT == 2 ? 3 : 1;
 };
 
 enum { ERR_MMA_LOAD = 16 };  // a bounded wait for a TMA tile ran out
@@ -164,12 +167,12 @@ struct TmaMaps {
 
 // VAR = false: both sides shared and no visible lengths (the hot configurations); the code for the variants is
 // compiled out.  SHARED = false: one warp per unit.
-template <int D, int MT, int MODE, bool IDX16, bool TMA, bool VAR, bool SHARED>
-__global__ void __launch_bounds__(128, MmaCfg<D, MT, TMA>::MIN_BLOCKS)
+template <int D, int MT, int MODE, bool IDX16, bool TMA, bool VAR, bool SHARED, bool DENSE = false>
+__global__ void __launch_bounds__(128, MmaCfg<D, MT, TMA, DENSE>::MIN_BLOCKS)
     attend_mma_kernel(const __grid_constant__ AttendArgs a, int n_mb, int log_wpu, int n_cta, int* err_flag,
                       const __grid_constant__ std::conditional_t<TMA, TmaMaps, InlineTable> tab)
 {
-    using C = MmaCfg<D, MT, TMA>;
+    using C = MmaCfg<D, MT, TMA, DENSE>;
     constexpr int NTD = D / 8, KS = D / 16, ROWB = C::ROWB, CPR = C::CPR, RPI = C::RPI, NST = C::NST;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -737,11 +740,11 @@ __global__ void __launch_bounds__(128, MmaCfg<D, MT, TMA>::MIN_BLOCKS)
     }
 }
 
-template <int D, int MT, int MODE, bool IDX16, bool TMA, bool VAR, bool SHARED>
+template <int D, int MT, int MODE, bool IDX16, bool TMA, bool VAR, bool SHARED, bool DENSE>
 cudaError_t launch_mma_one(const AttendArgs& a, int n_mb, int parts, const InlineTable* tab, const CUtensorMap* maps,
                            int* err_flag, const Launch& l)
 {
-    using C = MmaCfg<D, MT, TMA>;
+    using C = MmaCfg<D, MT, TMA, DENSE>;
     int log_wpu = 0;
     while (log_wpu < 2 && (1 << log_wpu) < parts) ++log_wpu;
     const int n_cta = parts >> log_wpu;
@@ -752,7 +755,7 @@ cudaError_t launch_mma_one(const AttendArgs& a, int n_mb, int parts, const Inlin
                              log_wpu, n_cta, err_flag, TmaMaps{maps[0], maps[1]});
     } else {
         static const InlineTable none{};
-        return launch_kernel(l, attend_mma_kernel<D, MT, MODE, IDX16, false, VAR, SHARED>, grid, 128, C::SMEM, n_cta, a, n_mb,
+        return launch_kernel(l, attend_mma_kernel<D, MT, MODE, IDX16, false, VAR, SHARED, DENSE>, grid, 128, C::SMEM, n_cta, a, n_mb,
                              log_wpu, n_cta, err_flag, tab ? *tab : none);
     }
 }
@@ -760,21 +763,21 @@ cudaError_t launch_mma_one(const AttendArgs& a, int n_mb, int parts, const Inlin
 }  // namespace
 
 // Instantiated for each (head_dim, query tiles of a warp) in a file of its own, kernels_mma_*.cu: the forms of the kernel take a
-// minute to compile in one.
-template <int D, int MT>
+// minute to compile in one.  DENSE: the plain form with cp.async alone (maps null, both sides shared, no visible lengths).
+template <int D, int MT, bool DENSE>
 cudaError_t launch_mma(const AttendArgs& a, int n_mb, int parts, const InlineTable* tab, const CUtensorMap* maps,
                        int* err_flag, const Launch& l)
 {
-    constexpr bool HAS_TMA = D != 32 || MT != 2;  // (never asked for with the other)
+    constexpr bool HAS_TMA = !DENSE && (D != 32 || MT != 2);  // (never asked for with the others)
     const bool i16 = a.cv.idx_bytes == 2;
-    const bool var = a.vis != nullptr || a.cv.full_k || a.cv.full_v;  // the TMA loader is never asked for with these
-#define CKV_MMA_ONE(MODE, I16, TMA, VAR)                                                                   \
-    (parts > 1 ? launch_mma_one<D, MT, MODE, I16, TMA, VAR, true>(a, n_mb, parts, tab, maps, err_flag, l)  \
-               : launch_mma_one<D, MT, MODE, I16, TMA, VAR, false>(a, n_mb, parts, tab, maps, err_flag, l))
+    const bool var = !DENSE && (a.vis != nullptr || a.cv.full_k || a.cv.full_v);  // the TMA loader is never asked for with these
+#define CKV_MMA_ONE(MODE, I16, TMA, VAR)                                                                          \
+    (parts > 1 ? launch_mma_one<D, MT, MODE, I16, TMA, VAR, true, DENSE>(a, n_mb, parts, tab, maps, err_flag, l)  \
+               : launch_mma_one<D, MT, MODE, I16, TMA, VAR, false, DENSE>(a, n_mb, parts, tab, maps, err_flag, l))
 #define CKV_MMA_GO(MODE, I16)                                                                              \
-    (maps  ? CKV_MMA_ONE(MODE, I16, HAS_TMA, false)                                                        \
-     : var ? CKV_MMA_ONE(MODE, I16, false, true)                                                           \
-           : CKV_MMA_ONE(MODE, I16, false, false))
+    (HAS_TMA && maps ? CKV_MMA_ONE(MODE, I16, HAS_TMA, false)                                              \
+     : var           ? CKV_MMA_ONE(MODE, I16, false, !DENSE)                                               \
+                     : CKV_MMA_ONE(MODE, I16, false, false))
     if (a.mode == CKV_SOFTMAX) return i16 ? CKV_MMA_GO(CKV_SOFTMAX, true) : CKV_MMA_GO(CKV_SOFTMAX, false);
     return i16 ? CKV_MMA_GO(CKV_SILU_OVER_L, true) : CKV_MMA_GO(CKV_SILU_OVER_L, false);
 #undef CKV_MMA_GO

@@ -260,11 +260,12 @@ int mma_queries_per_warp(int head_dim, int max_M, bool big);
 // tensor_maps: null = fill the staging ring with cp.async copies; else the two maps of make_pool_tensor_maps =
 // fill it with TMA gathers (err_flag: device int, OR-ed with a code if a bounded wait for a tile ran out).
 // parts: warps that share one (item, group, query block), a power of two up to kMmaMaxParts; more than four lie in a
-// cluster of thread blocks.  tab: the requests when a.inl is set (cp.async loader only).
+// cluster of thread blocks.  tab: the requests when a.inl is set (cp.async loader only).  dense: more resident warps with
+// shallower rings (head_dim 64, 16 queries a warp, the plain form with cp.async; ignored elsewhere).
 constexpr int kMmaMaxParts = 32;
-cudaError_t launch_attend_mma(int head_dim, int max_M, int queries_per_warp, int parts, const AttendArgs& a, const InlineTable* tab,
+cudaError_t launch_attend_mma(int head_dim, int max_M, int queries_per_warp, int parts, bool dense, const AttendArgs& a, const InlineTable* tab,
                               const void* tensor_maps, int* err_flag, const Launch& l);
-int mma_warps_per_sm(int head_dim, int queries_per_warp);
+int mma_warps_per_sm(int head_dim, int queries_per_warp, bool dense = false);
 bool make_pool_tensor_maps(int head_dim, int64_t rows, const void* poolK, const void* poolV, void* maps_out);
 
 // ---- kernels_fact.cu : pool-side factorisation for one query per user (bf16, head_dim 32 or 64, d_user <= 8)

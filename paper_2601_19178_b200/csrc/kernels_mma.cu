@@ -4,7 +4,7 @@
 
 namespace ckv {
 
-template <int D, int MT>
+template <int D, int MT, bool DENSE>
 cudaError_t launch_mma(const AttendArgs& a, int n_mb, int parts, const InlineTable* tab, const CUtensorMap* maps,
                        int* err_flag, const Launch& l);
 
@@ -25,24 +25,28 @@ int mma_queries_per_warp(int D, int max_M, bool big)
 }
 
 // warps of the kernel that are resident on an SM
-int mma_warps_per_sm(int D, int queries_per_warp)
+int mma_warps_per_sm(int D, int queries_per_warp, bool dense)
 {
+    if (dense) return 12;
     return D == 64 ? 8 : queries_per_warp == 16 ? 16 : queries_per_warp == 32 ? 12 : 8;
 }
 
-cudaError_t launch_attend_mma(int D, int max_M, int queries_per_warp, int parts, const AttendArgs& a, const InlineTable* tab,
+cudaError_t launch_attend_mma(int D, int max_M, int queries_per_warp, int parts, bool dense, const AttendArgs& a, const InlineTable* tab,
                               const void* tensor_maps, int* err_flag, const Launch& l)
 {
     if (a.n_items == 0) return cudaSuccess;
     const CUtensorMap* maps = reinterpret_cast<const CUtensorMap*>(tensor_maps);
     if (maps && D == 32 && queries_per_warp == 32) queries_per_warp = 16;  // (no such form with the TMA loader; the same bits)
     const int n_mb = (max_M + queries_per_warp - 1) / queries_per_warp;
-    if (D == 64)
-        return queries_per_warp == 16 ? launch_mma<64, 1>(a, n_mb, parts, tab, maps, err_flag, l)
-                                      : launch_mma<64, 2>(a, n_mb, parts, tab, maps, err_flag, l);
-    return queries_per_warp == 16   ? launch_mma<32, 1>(a, n_mb, parts, tab, maps, err_flag, l)
-           : queries_per_warp == 32 ? launch_mma<32, 2>(a, n_mb, parts, tab, maps, err_flag, l)
-                                    : launch_mma<32, 3>(a, n_mb, parts, tab, maps, err_flag, l);
+    if (D == 64) {
+        if (dense && queries_per_warp == 16 && !maps && !a.vis && !a.cv.full_k && !a.cv.full_v)
+            return launch_mma<64, 1, true>(a, n_mb, parts, tab, maps, err_flag, l);
+        return queries_per_warp == 16 ? launch_mma<64, 1, false>(a, n_mb, parts, tab, maps, err_flag, l)
+                                      : launch_mma<64, 2, false>(a, n_mb, parts, tab, maps, err_flag, l);
+    }
+    return queries_per_warp == 16   ? launch_mma<32, 1, false>(a, n_mb, parts, tab, maps, err_flag, l)
+           : queries_per_warp == 32 ? launch_mma<32, 2, false>(a, n_mb, parts, tab, maps, err_flag, l)
+                                    : launch_mma<32, 3, false>(a, n_mb, parts, tab, maps, err_flag, l);
 }
 
 // Tensor maps of the K and the V pool ([n_groups * n_entries] rows of head_dim bf16) for tile::gather4: a box of

@@ -2,5 +2,5 @@
 #include "attend_mma.cuh"
 
 namespace ckv {
-template cudaError_t launch_mma<32, 1>(const AttendArgs&, int, int, const InlineTable*, const CUtensorMap*, int*, const Launch&);
+template cudaError_t launch_mma<32, 1, false>(const AttendArgs&, int, int, const InlineTable*, const CUtensorMap*, int*, const Launch&);
 }  // namespace ckv

@@ -241,3 +241,21 @@ def test_warp_level_kernel_reference_far_from_later_scores(users, head, queries,
     s.close()
     rows = np.concatenate([np.arange(d["q_off"][u], d["q_off"][u + 1]) for u in sel])
     assert_close(got[rows], oracle_attend(w, d, scale=1.0, sel=sel), "bf16", f"{users} {head} {queries} {ramp}")
+
+
+@pytest.mark.parametrize("mode", ["softmax", "silu_over_l"])
+@pytest.mark.parametrize("users,hist,queries,groups,pool", [(220, (1000, 1000), 3, 2, 500), (700, (1, 300), 16, 3, 500),
+                                                            (700, (1, 300), 20, 3, 500), (225, (31, 65), 1, 9, 66000)])
+def test_more_resident_warps_at_64_wide_heads(mode, users, hist, queries, groups, pool):
+    """Lists that fill the SMs run with rings of two slots and twelve warps per SM: warps that share a unit and whole units, 16-
+    and 32-bit indices, histories from one position on."""
+    w = _workload(mode=mode, head=(60, 4), groups=groups, users=users, hist=hist, queries=queries, pool=pool)
+    if mode != "softmax":
+        w = synth.scaled(w, hist_len=(max(hist[0], 17), hist[1]))
+    d = synth.generate(w)
+    sel = np.arange(0, users, 23)
+    s = make_session(w, d, kernel=2)
+    got = gpu_attend(w, d, session=s)
+    s.close()
+    rows = np.concatenate([np.arange(d["q_off"][u], d["q_off"][u + 1]) for u in sel])
+    assert_close(got[rows], oracle_attend(w, d, sel=sel), "bf16", f"{users} {hist} {queries}")
