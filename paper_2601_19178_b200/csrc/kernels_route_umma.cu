@@ -15,9 +15,10 @@
 // tensor core is 95 % busy with bias and products at d_in = 64.  So the turn is kept short: the release is a named
 // barrier of five warps (an mbarrier cost 340 clocks next to running products), the issuing warp waits for its tile
 // before it, the products are issued under elect.sync from values known to be uniform (under "lane 0" the five of them
-// took 380 clocks, now 200).  131072 positions x 16384 entries x 4 groups, d_in 64: 1250 us -> 893 (1232 TFLOP/s; 1197 with
+// took 380 clocks, now 200).  131072 positions x 16384 entries x 4 groups, d_in 64: 1250 us -> 880 (1250 TFLOP/s; 1197 with
 // three blocks alone, 953 with the elected issue, 930 with accumulators of 128 columns and 152 registers a read-out
-// thread instead of two of 64); d_in 32: 1170 -> 800; 10000 x 16384 x 2: 140 -> 76.  Three blocks and not two: a weight tile
+// thread instead of two of 64, 891 with the first tiles requested behind the inputs instead of beside them); d_in 32: 1165 ->
+// 795; 10000 x 16384 x 2: 140 -> 71.  Three blocks and not two: a weight tile
 // is fetched from L2 once for all of a CTA's positions, and three turns overlap.
 // Every wait is bounded: a time-out raises the CTA's abort flag, the CTA drains, frees its TMEM and reports through
 // the error word.  The call then returns an error and its whole output is not valid: the CTA itself writes none, but others
@@ -208,6 +209,18 @@ __global__ void __launch_bounds__(kThreadsRU, 1)
     // a tile needs the bias step if there is a bias, or entries past the last one to rule out
     auto biased = [&](int t) { return bg != nullptr || (tile0 + t + 1) * TN > m; };
 
+    // four read-out warps and one issuing warp per block of positions
+    const int e = warp >> 2;
+    const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
+    const int row = 128 * e + (warp & 3) * 32 + lane;  // this read-out thread's position
+    // its inputs are requested before anything is set up (zero rows past the end)
+    uint4 xin[DIN / 8];
+    if (warp < 4 * n_blocks) {
+        const uint4* xr = reinterpret_cast<const uint4*>(x + (row0 + row) * DIN);
+        const bool in = row0 + row < n;
+#pragma unroll
+        for (int q = 0; q < DIN / 8; ++q) xin[q] = in ? __ldg(xr + q) : make_uint4(0, 0, 0, 0);
+    }
     if (tid == 0) {
         for (int s = 0; s < L::STAGES; ++s) {
             bar_init(bar(B_FULL + s), 2);  // the loading warp, with the box's bytes and behind the bias step
@@ -236,20 +249,14 @@ __global__ void __launch_bounds__(kThreadsRU, 1)
     float best = -CUDART_INF_F;
     int arg = 0;
 
-    // four read-out warps and one issuing warp per block of positions
-    const int e = warp >> 2;
-    const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-    const int row = 128 * e + (warp & 3) * 32 + lane;  // this read-out thread's position
     if (warp < 4 * n_blocks) {
-        // the positions' inputs, once: two bf16 per column (zero rows past the end)
-        const uint4* xr = reinterpret_cast<const uint4*>(x + (row0 + row) * DIN);
-        const bool in = row0 + row < n;
+        // the positions' inputs, once: two bf16 per column
 #pragma unroll
         for (int h = 0; h < DIN / 32; ++h) {
             uint32_t v[16];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const uint4 w = in ? __ldg(xr + 4 * h + q) : make_uint4(0, 0, 0, 0);
+                const uint4 w = xin[4 * h + q];
                 v[4 * q] = w.x; v[4 * q + 1] = w.y; v[4 * q + 2] = w.z; v[4 * q + 3] = w.w;
             }
             st16(tmem + lane_base + L::COL_A + e * (DIN / 2) + 16 * h, v);
@@ -260,9 +267,11 @@ __global__ void __launch_bounds__(kThreadsRU, 1)
         }
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
     }
-    tc_before();
-    __syncthreads();
-    tc_after();
+    if (warp < kLoadWarp) {  // (the loading warp is on its way: the first tiles travel meanwhile)
+        tc_before();
+        asm volatile("bar.sync 15, %0;" ::"n"(kLoadWarp * 32) : "memory");
+        tc_after();
+    }
 
     if (warp < kEpiWarps) {
         // ------------------------------------------------------------ running arg-max, thread = position
@@ -486,7 +495,7 @@ cudaError_t launch_t(const void* x, const void* W, const float* bias, int n, int
     CUtensorMap map;
     if (!make_weight_map(DIN, (int64_t)G * m, RU<DIN>::TN, W, &map)) return cudaErrorInvalidValue;
     // CTAs that share a block of positions: as many as shorten the run most, counting whole waves of CTAs over the SMs and
-    // fourteen tiles' time per CTA: 5 us until the first product is there and for the end, and as much for the first
+    // fourteen tiles' time per CTA: 4 us until the first product is there and for the end, and more for the first
     // tiles, in which most chunks bring a new best (40 000 positions x 4096 entries x 4 groups: 106 us; 119 by four tiles)
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
