@@ -62,15 +62,16 @@ struct __align__(16) PairRec {
     uint4 q_head;     // the query's first eight elements (the user part meets them), bf16
 };
 
-// Rows of the tables follow the items: row = item * G + group.
+// Rows of the tables follow the items: row = item * G + group.  The rows of the first items are written last, those of all groups
+// together: the main kernel begins with them and finds them in L2 (512 users x 4 groups x 16384 entries 195 -> 192 us).
 template <int D>
 __global__ void __launch_bounds__(128)
     fact_table_kernel(const __grid_constant__ AttendArgs a, float* __restrict__ tw, PairRec* __restrict__ recs)
 {
     constexpr int KS = D / 16, MT = kTableMT;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gl = lane >> 2, t = lane & 3;
-    const int m = a.cv.n_entries, G = a.cv.n_groups, grp = blockIdx.z;
-    const int j0 = blockIdx.x * 256 + warp * 64, r0 = blockIdx.y * (16 * MT);
+    const int m = a.cv.n_entries, G = a.cv.n_groups, grp = blockIdx.y;
+    const int j0 = blockIdx.x * 256 + warp * 64, r0 = (gridDim.z - 1 - blockIdx.z) * (16 * MT);
     if (blockIdx.x == 0 && threadIdx.x < 16 * MT && r0 + (int)threadIdx.x < a.n_items) {
         const Req rq = a.reqs[a.items[r0 + threadIdx.x].req];
         PairRec rec;
@@ -590,7 +591,7 @@ cudaError_t launch_slab(const AttendArgs& a, int n_sms, float* tw, float* aux, c
     const int m = a.cv.n_entries, G = a.cv.n_groups, n_pairs = a.n_items * G;
     PairRec* recs = reinterpret_cast<PairRec*>(aux + (size_t)n_pairs * kAux);
     cudaError_t e = launch_kernel(l, fact_table_kernel<D>,
-                                  dim3((m + 255) / 256, (a.n_items + 16 * kTableMT - 1) / (16 * kTableMT), G), 128, 0, 1, a, tw, recs);
+                                  dim3((m + 255) / 256, G, (a.n_items + 16 * kTableMT - 1) / (16 * kTableMT)), 128, 0, 1, a, tw, recs);
     if (e != cudaSuccess) return e;
     // two table buffers if they fit next to the histogram; two CTAs of half the threads per SM if that leaves room for both
     const size_t table = (size_t)row_floats(m) * sizeof(float);
