@@ -13,6 +13,11 @@
 // arena; they are copied into the ring in place of pool rows (cp.async loader only) and nothing is
 // patched.  With visible lengths a query row only takes the positions before its own limit.
 //
+// What bounds it is the latency of a warp's chain, index -> row -> product -> weights -> product, against the warps that
+// registers and rings admit; the L1 / shared-memory data pipe, which every gathered row crosses on the way into the ring and
+// out of it, is 82 to 90 % busy with 32-wide heads, but a form that kept a group's K rows in shared memory (65 %) was 4 to 13
+// % slower all the same, with 16, 20 or 24 warps.
+//
 // Several warps may share one (item, group, query block): `parts` of them, a power of two, take its 32-position
 // tiles in turn and merge their (m, l, O) at the end, through shared memory inside a block and through distributed
 // shared memory between the blocks of a cluster.  What bounds a small call is the chain index -> row -> product of

@@ -3,7 +3,7 @@
 // Persistent: one CTA per SM holds three workers, and every worker walks its own static round-robin share of the work
 // units, where a unit is (work item = history chunk of one user, group, block of up to 128 queries).  The history chunk
 // is processed in tiles of 64 positions.  A worker is (warp-specialised, 6 warps of the CTA's 18)
-//   four normalisation warps: thread i owns query row i = TMEM lane i
+//   four normalisation warps: thread i owns TMEM lane i, query row i of the block (turned by whole warps, see block_turn)
 //   one issuing warp: the score MMAs and the weighted-sum MMAs
 //   one producer warp: gathers pool rows into the worker's ring of shared-memory stages with 16-byte cp.async, patches
 //     the user-specific leading elements (Eq. K), publishes the tile one tile later, and stages Q with a unit's first
@@ -23,15 +23,20 @@
 //
 // What bounds it: the special-function unit (one ex2 or tanh per score, 16 per clock per SM).  The normalisation of a
 // tile is a chain of dependent work for its warp (wait for the scores, TMEM load, arithmetic, TMEM store, publish; at a
-// unit's end the last weighted sum, the accumulator read-out, the store) during most of which that unit is idle on the
-// warp's sub-partition; three workers fill each other's gaps.  Registers (65536 / 20 warps = 96 a thread, enough for one
-// 32-column chunk of scores at a time) and TMEM (3 x (2 x 64 + 32) = 480 columns) admit no fourth.  With the three groups
-// on one unit instead (its tiles dealt out in turn, accumulators merged through shared memory at its end) a unit cost
-// 5 us plus 0.45 us per 128 positions; now an SM of busy workers takes 0.4 us per 64 positions and 1.5 us per unit, the
-// special-function unit busy 70 % of the time.  The issuing warp walks its loop as a whole and an elected thread issues, with
-// operands known to be uniform: under "lane 0" each product and commit waited for its operands' way into uniform registers
-// (the three cases below 386 -> 357 us, 2.57 -> 2.47 ms, 148 -> 127 us).  1024 users x 1024 positions x 100 queries x 8 groups 490 -> 385 us, 2048
-// users x 4096 x 128 (SiLU) 2.88 -> 2.57 ms, 64 causal self-attentions of 200..1500 positions 283 -> 147 us.
+// unit's end the last weighted sum, the accumulator read-out, the store), and three workers fill each other's gaps: of the
+// 1900 clocks of a tile (SiLU; 2150 softmax) a warp spends 1530 in the arithmetic, whose share of the unit is 512, 105 on
+// the wait for the scores, 120 on the TMEM loads.  Registers (65536 / 20 warps = 96 a thread, enough for one
+// 32-column chunk of scores at a time) and TMEM (3 x (2 x 64 + 32) = 480 columns) admit no fourth.  An SM of busy
+// workers takes 0.36 us per 64 positions and 1.2 us per unit, the special-function unit busy 79 % of the time.
+// With the three groups on one unit instead (its tiles dealt out in turn, accumulators merged through shared memory at its
+// end) a unit cost 5 us plus 0.45 us per 128 positions; three workers took 1024 users x 1024 positions x 100 queries x 8 groups
+// from 490 to 386 us, 2048 users x 4096 x 128 (SiLU) from 2.88 to 2.57 ms, 64 causal self-attentions of 200..1500 positions from
+// 283 to 148 us.  The issuing warp walks its loop as a whole and an elected thread issues, with operands known to be
+// uniform: under "lane 0" each product and commit waited for its operands' way into uniform registers (357 us, 2.47 ms, 127
+// us).  With the swizzled tiles and the arithmetic left out that no row needs, both below, 354 us, 2.43 ms, 107 us.
+// (Measured and not kept: scores in pieces of sixteen columns with the next tile's requested ahead, and a unit's read-out put
+// off behind the next unit's first tile, 548 us and 3.27 ms: with the registers that takes the arithmetic no longer
+// overlaps itself.)
 //
 // Softmax bookkeeping.  The reference maximum m of a row is the largest of the first 32 scores of the unit's
 // first tile and stays fixed: later scores may exceed it by up to 2^64 (fp32 accumulators and bf16
