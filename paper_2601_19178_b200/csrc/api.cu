@@ -588,6 +588,7 @@ inline int64_t mma_blocks(uint32_t M, int qpw) { return qpw == 16 ? (M + 15) / 1
 struct ListShape {
     const bool tensor;                  // a tensor-core family can run: what only those want is gathered too
     int32_t max_M = 0, min_M = INT32_MAX, max_L = 0, min_L = INT32_MAX;  // of requests with a query
+    int64_t listed = 0;                 // requests, with or without one
     int64_t active = 0, positions = 0, rows = 0;  // how many have one, their history lengths and query rows in all
     int64_t blocks128 = 0, tiles64 = 0; // blocks of 128 queries, and (block, 64 positions) tiles
     int64_t units[3] = {}, tiles[3] = {};    // MmaWork of unchunked histories, for 16, 32 and 48 queries per warp
@@ -595,6 +596,7 @@ struct ListShape {
     explicit ListShape(const ckv_ctx* ctx) : tensor(ctx->has_mma || ctx->has_umma) {}
     void add(int32_t length, int32_t queries)
     {
+        ++listed;
         if (queries <= 0) return;
         const uint32_t L = (uint32_t)length, M = (uint32_t)queries;
         ++active;
@@ -694,18 +696,28 @@ void mma_shape(const ckv_ctx* ctx, const ListShape& s, int64_t chunk, bool plain
     }
 }
 
+// Costs of the tcgen05 kernel in microseconds, see umma_chunk.
+struct UmmaCost {
+    double tile, shared;      // 64 positions of a worker: alone on its SM, and more per worker there
+    double filled0, filled1;  // that part's share for a block's warps that have rows, 0 to 4
+    double unit, launch;
+};
+constexpr UmmaCost kUmmaCost = {0.42, 0.26, 0.26, 0.185, 1.2, 6.6};
+// The line for lists that can travel as a kernel argument, see choose_family.
+constexpr UmmaCost kUmmaCostPlanned = {0.8, 0.2, 1, 0, 1.5, 6};
+
 // Chunk length of the tcgen05 kernel: the one with the shortest estimated run, in microseconds.  Three persistent workers
 // per SM walk a (chunk, group, 128 queries) unit alone; a worker takes 0.68 us per 64 positions when it has the SM
 // to itself and 1.2 next to two others (0.77 if one of its four warps has rows), 1.2 per unit, the launch 6.6, and merging
 // chunks 6 and 0.007 per chunk.  Units of one size run in whole rounds; mixed ones are dealt out longest first, and only the
 // longest of them bounds the run from below.  (Fitted to 244 lists of 4..3900 users, 32..3000 positions, 1..93 queries: 10 %.)
-int64_t umma_chunk(const ckv_ctx* ctx, const ListShape& s, double* time = nullptr)
+int64_t umma_chunk(const ckv_ctx* ctx, const ListShape& s, double* time = nullptr, const UmmaCost& cost = kUmmaCost)
 {
     const double workers = 3.0 * ctx->n_sms, G = ctx->cfg.n_groups;
     const MmaWork w16 = s.mma(16);
     const bool alike = w16.alike && w16.min_tiles == w16.max_tiles;
     // warps of a block of 128 queries that have rows, of four (s.units[1]: blocks of 32 queries)
-    const double filled = s.blocks128 > 0 ? 0.26 + 0.185 * (double)s.units[1] / (double)s.blocks128 : 1;
+    const double filled = s.blocks128 > 0 ? cost.filled0 + cost.filled1 * (double)s.units[1] / (double)s.blocks128 : 1;
     int64_t best = 16384;
     double best_t = 1e300;
     for (int64_t n = (s.max_L + 16383) / 16384, last = 0; n <= 512 && last != 256; n += (n + 15) / 16) {
@@ -716,15 +728,15 @@ int64_t umma_chunk(const ckv_ctx* ctx, const ListShape& s, double* time = nullpt
         const double cut = alike ? (double)((s.max_L + c - 1) / c) * s.blocks128 : s.tiles64 * 64.0 / c + (split ? 0.5 : 0) * s.blocks128;
         const double units = G * std::max<double>(cut, s.blocks128), tiles = c / 64;
         auto unit_us = [&](double n_tiles, double n) {  // of n units that run at a time
-            return n_tiles * (0.42 + 0.26 * filled * std::min(3.0, std::max(1.0, n / ctx->n_sms))) + 1.2;
+            return n_tiles * (cost.tile + cost.shared * filled * std::min(3.0, std::max(1.0, n / ctx->n_sms))) + cost.unit;
         };
         const double longest = std::min<double>(tiles, (s.max_L + 63) / 64);
-        double t = 6.6 + (split ? 6 + 0.007 * units : 0);
+        double t = cost.launch + (split ? 6 + 0.007 * units : 0);
         if (alike) {
             const double full = std::floor(units / workers), rest = units - full * workers;
             t += full * unit_us(longest, workers) + (rest > 0 ? unit_us(longest, rest) : 0);
         } else
-            t += std::max(unit_us(longest, units), (unit_us(s.tiles64 * G, units) + 1.2 * (units - 1)) / workers);
+            t += std::max(unit_us(longest, units), (unit_us(s.tiles64 * G, units) + cost.unit * (units - 1)) / workers);
         if (t < best_t) {
             best_t = t;
             best = c;
@@ -746,12 +758,14 @@ int choose_family(const ckv_ctx* ctx, bool with_vis, const ListShape& s)
     const bool can_umma = ctx->has_umma;
     // The warp-level tensor-core kernel up to 16 queries per user, whose rows it gathers once; the tcgen05 kernel above 96; in
     // between the shorter estimated run.  (The CUDA-core kernel serves what neither supports.)  The warp-level kernel's: 3.9
-    // us and a cost per tile time of its resident warps, by the queries a warp holds.  Below 48 queries a list that could
-    // travel as a kernel argument there has its planning for the tcgen05 kernel counted, 15 us and 0.16 per user of the host,
-    // which bound a caller with a new list on every call (199 users of 17..1999 positions, 1..40 queries: 47 us a call, the
-    // kernel 28, the warp-level one 35).  Of the 244 lists that umma_chunk is fitted to, most get the faster kernel; they lose
-    // 1.2 % in the mean, 36 % at most (with the tcgen05 kernel from 48 queries on alone 3.8 and 74).  24 queries, 250
-    // users of 100..1500 positions, 4 groups: 39.6 / 31.8 us; 40 queries, 1500 x 1000, 8 groups: 567 / 470; 20 x 2000: 23.2 / 27.3.
+    // us and a cost per tile time of its resident warps, by the queries a warp holds.  Of the 244 lists that umma_chunk is
+    // fitted to, most get the faster kernel; they lose 1.2 % in the mean, 36 % at most (with the tcgen05 kernel from 48
+    // queries on alone 3.8 and 74).  24 queries, 3643 users of 531 positions, 2 groups: 142 / 131 us; 40 queries, 1500 x 1000, 8
+    // groups: 567 / 470.
+    // A list that can travel as a kernel argument to the warp-level kernel is one launch there, under stream capture too; the
+    // tcgen05 kernel has to have it planned, 15 us and 0.16 per user of the host, which bound a caller with a new list
+    // on every call (199 users of 17..1999 positions, 1..40 queries: 47 us a call, the kernel 28, the warp-level one 35).  Such a
+    // list goes there from 48 queries on, and only if it pays at costs that are 1.2 to 1.9 times as high as well.
     // For self-attention, as many queries as positions with visible lengths, lists of any number are compared: half of
     // their pairs count, and the tcgen05 kernel needs a launch for the limits, 5 us, whatever the list.  (The estimates are of
     // whole histories, the limits may be on the device.  7 causal self-attentions of 556 positions, 2 groups: 22.7 us there, 11.0
@@ -759,23 +773,27 @@ int choose_family(const ckv_ctx* ctx, bool with_vis, const ListShape& s)
     // (Not compared where the option asks for the TMA loader, which takes neither limits nor sides that are not shared:
     // the tcgen05 kernel from 48 queries on.)
     const bool loads = ctx->opt_loader != 2 || (plain && ctx->has_tma);
-    const bool self = with_vis && s.rows >= total_pos;
-    bool few = max_M < (can_mma && loads ? 17 : 48);
+    const bool self = with_vis && s.rows >= total_pos, short_list = s.listed <= kInlineReqs;
+    bool few = max_M < (can_mma && loads && !short_list ? 17 : 48);
     if (can_umma && can_mma && loads && !few && n_active > 0 && (max_M <= 96 || self)) {
-        int qpw, parts;
-        double tile_times, t_umma;
+        const double limits = with_vis ? 5 : 0;
+        double tiles16, t_umma;
+        mma_parts(ctx, s.mma(16), 16, &tiles16);
         umma_chunk(ctx, s, &t_umma);
         if (self) {
-            mma_parts(ctx, s.mma(16), 16, &tile_times);
-            few = 4 + 0.7 * tile_times < t_umma + 5;
+            few = 4 + 0.7 * tiles16 < t_umma + limits;
         } else {
+            int qpw, parts;
             bool dense;
+            double tile_times;
             mma_shape(ctx, s, INT32_MAX, plain, [](auto&&) {}, qpw, parts, dense, &tile_times);
             const bool softmax = ctx->cfg.mode == CKV_SOFTMAX;
             const double per_tile = qpw == 16 ? (softmax ? 0.99 : 0.87) : qpw == 32 ? (softmax ? 1.55 : 1.14) : (softmax ? 1.59 : 1.26);
-            if (with_vis) t_umma += 5;
-            if (max_M < 48 && n_active <= kInlineReqs) t_umma = std::max(t_umma, 15 + 0.16 * (double)n_active);
-            few = 3.9 + per_tile * tile_times < 1.05 * t_umma;
+            few = 3.9 + per_tile * tile_times < 1.05 * (t_umma + limits);
+        }
+        if (!few && short_list) {
+            umma_chunk(ctx, s, &t_umma, kUmmaCostPlanned);
+            few = 4 + 1.2 * tiles16 < t_umma + limits;
         }
     }
     // One query per user: the pool-side factorisation trades the row gathers for two tables per (user, group).

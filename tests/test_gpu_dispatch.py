@@ -259,3 +259,33 @@ def test_more_resident_warps_at_64_wide_heads(mode, users, hist, queries, groups
     s.close()
     rows = np.concatenate([np.arange(d["q_off"][u], d["q_off"][u + 1]) for u in sel])
     assert_close(got[rows], oracle_attend(w, d, sel=sel), "bf16", f"{users} {hist} {queries}")
+
+
+@pytest.mark.parametrize("queries", [5, 24, 47])
+def test_short_lists_under_stream_capture(queries):
+    """A list that travels as a kernel argument is captured as it is: replays do not depend on plans of other lists."""
+    w = _workload(groups=8, users=200, hist=(100, 900), queries=queries)
+    d = synth.generate(w)
+    s = make_session(w, d)
+    q = to_dev(d["queries"], w.dtype)
+    want = s.attend(d["users"], d["q_off"], q).clone()
+    out = torch.zeros_like(want)
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(stream):
+        s.attend(d["users"], d["q_off"], q, out)
+    torch.cuda.current_stream().wait_stream(stream)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        s.attend(d["users"], d["q_off"], q, out)
+    for k in range(6):  # other lists, planned ones
+        users = np.concatenate([np.roll(d["users"], k), d["users"][:30]])
+        q_off = (np.arange(len(users) + 1) * queries).astype(np.int32)
+        s.attend(users, q_off, torch.cat([q, q[:30 * queries]]))
+    out.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, want)
+    del graph
+    s.close()
