@@ -325,7 +325,8 @@ def ckv_version() -> int:
 def ckv_route(device: int, n: int, n_groups: int, d_in: int, n_entries: int, x, W, bias, idx_out, variant: int = 0,
               stream=None) -> None:
     """Router indices of n positions: x [n][d_in], W [G][n_entries][d_in] (bf16, device), bias [G][n_entries] fp32
-    or None, idx_out [n][G] int32 (device); variant 0 / 2 = tcgen05 kernel, 1 = warp-level tensor-core kernel."""
+    or None, idx_out [n][G] int32 (device); variant 0 = the library's choice, 1 = warp-level
+    tensor-core kernel, 2 = tcgen05 kernel."""
     stream = _stream(stream)
     st = _pycall.prefill(_ROUTE, device, n, n_groups, d_in, n_entries, x, W, bias, idx_out, int(variant), stream or 0)
     if st is not None:

@@ -317,15 +317,18 @@ struct ckv_ctx {
 
 namespace {
 
-bool is_device_ptr(const void* p)
+// Whose memory `p` points to: a device's (its ordinal), managed, or neither.
+enum { kManagedMemory = -1, kNoDeviceMemory = -2 };
+int memory_of(const void* p)
 {
     cudaPointerAttributes at;
     if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
         cudaGetLastError();
-        return false;
+        return kNoDeviceMemory;
     }
-    return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
+    return at.type == cudaMemoryTypeDevice ? at.device : at.type == cudaMemoryTypeManaged ? kManagedMemory : kNoDeviceMemory;
 }
+bool is_device_ptr(const void* p) { return memory_of(p) != kNoDeviceMemory; }
 
 cudaError_t grow(DevBuf& b, size_t bytes, int64_t* allocs = nullptr)
 {
@@ -2056,7 +2059,8 @@ ckv_status ckv_route(int32_t device, int32_t n, int32_t n_groups, int32_t d_in, 
     if (!x || !W || !idx_out) return CKV_ERR_INVALID_ARG;
     DeviceGuard dg(device);
     if (!dg.ok) return CKV_ERR_CUDA;
-    if (!is_device_ptr(x) || !is_device_ptr(W) || !is_device_ptr(idx_out) || (bias && !is_device_ptr(bias)))
+    const int out_at = memory_of(idx_out);
+    if (!is_device_ptr(x) || !is_device_ptr(W) || out_at == kNoDeviceMemory || (bias && !is_device_ptr(bias)))
         return CKV_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     cudaError_t e;
@@ -2065,9 +2069,12 @@ ckv_status ckv_route(int32_t device, int32_t n, int32_t n_groups, int32_t d_in, 
     } else {
         HostFlag flag(HostFlag::kRoute);
         if (!flag.p) return CKV_ERR_OOM;
+        // (a kernel's report covers what it has written to this GPU's own memory; for managed memory and a peer's the call
+        // waits for the stream)
+        const int slot = out_at == device ? flag.slot() : -1;
         e = (variant == 0 && route_few(d_in, x, W, n, n_entries, n_groups) ? launch_route_few : launch_route_umma)(
-            d_in, x, W, bias, n, n_entries, n_groups, idx_out, flag.p, flag.slot(), s);
-        if (e == cudaSuccess) e = wait_done(flag.p + 1, s);
+            d_in, x, W, bias, n, n_entries, n_groups, idx_out, flag.p, slot, s);
+        if (e == cudaSuccess) e = slot >= 0 ? wait_done(flag.p + 1, s) : cudaStreamSynchronize(s);
         // a bounded wait inside the kernel ran out: the output is not valid
         if (e == cudaSuccess && *(volatile int*)flag.p) return CKV_ERR_CUDA;
     }

@@ -7,6 +7,7 @@
 #include <utility>
 
 #include "ckv.h"
+#include "report.cuh"
 
 namespace ckv {
 
@@ -181,49 +182,6 @@ constexpr int kInlinePuts = 224;  // users whose table travels as a kernel argum
 struct PutTable {
     PutUser u[kInlinePuts];
 };
-// How a kernel reports to the host, in host-mapped memory: *bad becomes 1 on a bad index, and *done (if not null; the word
-// behind *bad, the two eight-byte aligned) at its end, which the host sees some microseconds before a stream synchronise
-// returns.  `count` is a device counter, zero between launches, used by one launch at a time.
-struct Report {
-    int* bad = nullptr;
-    int* done = nullptr;
-    unsigned* count = nullptr;
-};
-#ifdef __CUDACC__
-// The end of a kernel that reports, reached by all threads of the n_blocks blocks that take part: every thread's accesses to
-// this GPU's memory lie before *done.
-__device__ __forceinline__ void report_done(const Report& r, unsigned n_blocks)
-{
-    if (!r.done) return;
-    __syncthreads();
-    if (threadIdx.x != 0) return;
-    __threadfence();
-    unsigned before;  // (acquires what the other blocks' fences released; system-wide fences here cost 3 us more)
-    asm volatile("atom.acquire.gpu.global.add.u32 %0, [%1], 1;" : "=r"(before) : "l"(r.count) : "memory");
-    if (before != n_blocks - 1) return;
-    *r.count = 0;
-    *reinterpret_cast<volatile int*>(r.done) = 1;
-}
-// The same where the host asks for nothing but the outcome, `bad` of some thread, and takes the rest in stream order (at most
-// 65535 blocks): the outcome travels in the counter and in one word with *done, so that nothing waits for the kernel's
-// stores to arrive (two system-wide fences, 2 us of an append of 11).
-__device__ __forceinline__ void report_outcome(const Report& r, bool bad, unsigned n_blocks)
-{
-    if (!r.done) {
-        if (bad) *reinterpret_cast<volatile int*>(r.bad) = 1;
-        return;
-    }
-    bad = __syncthreads_or(bad);
-    if (threadIdx.x != 0) return;
-    if (n_blocks > 1) {
-        const unsigned before = atomicAdd(r.count, bad ? 0x10001u : 1u);
-        if ((before & 0xffffu) != n_blocks - 1) return;
-        bad |= before >> 16 != 0;
-        *r.count = 0;
-    }
-    *reinterpret_cast<volatile unsigned long long*>(r.bad) = (1ull << 32) | (bad ? 1u : 0u);
-}
-#endif
 // Packs n users' [P][G] indices and [P][G][d_user] user parts into arena units and validates the index range.  The users
 // come from `table` (device memory) or, if that is null, from *inl; the arena arrays and the sides' widths from `cv`
 // (head_dim D).
@@ -283,7 +241,7 @@ cudaError_t launch_route(int d_in, const void* x, const void* W, const float* bi
                          int32_t* out, cudaStream_t s);
 
 // ---- kernels_route_umma.cu : the same router on tcgen05 (TMEM accumulators, warp-specialised)
-// flags: two host-mapped ints.  flags[0] becomes a non-zero code if a bounded wait inside the kernel ran out (`out` is not
+// flags: two host-mapped ints.  flags[0] becomes non-zero if a bounded wait inside the kernel ran out (`out` is not
 // valid then, whether written or not); flags[1] becomes 1 at its end if slot is in [0, kRouteSlots) and no other launch uses it at the time.
 constexpr int kRouteSlots = 64;
 cudaError_t launch_route_umma(int d_in, const void* x, const void* W, const float* bias, int n, int n_entries, int G,

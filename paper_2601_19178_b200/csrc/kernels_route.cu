@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(kFewWarps * 32, DIN == 128 ? 1 : 2)
         asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     }
     if (warp == 0 && split == 0 && row0 + lane < n) out[(row0 + lane) * G + grp] = i;
-    if (slot >= 0 && split == 0) report_done(Report{flags, flags + 1, &few_count[slot]}, gridDim.x / (unsigned)n_split * gridDim.y);
+    if (slot >= 0 && split == 0) report_done(Report{flags, flags + 1, &few_count[slot]}, false, gridDim.x / (unsigned)n_split * gridDim.y);
 }
 
 template <int DIN>

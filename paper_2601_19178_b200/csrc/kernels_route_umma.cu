@@ -20,8 +20,8 @@
 // thread instead of two of 64, 891 with the first tiles requested behind the inputs instead of beside them); d_in 32: 1165 ->
 // 795; 10000 x 16384 x 2: 140 -> 71.  Three blocks and not two: a weight tile
 // is fetched from L2 once for all of a CTA's positions, and three turns overlap.
-// Every wait is bounded: a time-out raises the CTA's abort flag, the CTA drains, frees its TMEM and reports through
-// the error word.  The call then returns an error and its whole output is not valid: the CTA itself writes none, but others
+// Every wait is bounded: a time-out raises the CTA's abort flag, the CTA drains, frees its TMEM and reports to the
+// host.  The call then returns an error and its whole output is not valid: the CTA itself writes none, but others
 // have, among them the first of its cluster, which takes the best entries of all of them as they stand.
 #include <cuda_bf16.h>
 #include <math_constants.h>
@@ -38,7 +38,6 @@ constexpr int kThreadsRU = (kLoadWarp + 1) * 32;  // sixteen warps: 128 register
 constexpr int kMaxClusterRU = 8;
 constexpr uint32_t kSpin = 1u << 18, kSuspend = 4000;
 constexpr float kTinyBias = 0x1p-100f;  // 0x0d80 in bf16
-enum { ERR_ROUTE = 64 };
 
 constexpr int kMaxStages = 8;
 constexpr int kMaxAcc = 2;  // accumulators of a block
@@ -477,8 +476,7 @@ __global__ void __launch_bounds__(kThreadsRU, 1)
         asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     }
     if (warp < kEpiWarps && split == 0 && !*abort_flag && row0 + row < n) out[(row0 + row) * G + grp] = arg;
-    if (tid == 0 && *abort_flag) *reinterpret_cast<volatile int*>(flags) = ERR_ROUTE;
-    if (slot >= 0) report_done(Report{flags, flags + 1, &route_count[slot]}, gridDim.x * gridDim.y);
+    report_done(slot >= 0 ? Report{flags, flags + 1, &route_count[slot]} : Report{flags}, *abort_flag != 0, gridDim.x * gridDim.y);
 }
 
 // The weights as rows of `d_in` inputs, boxes of a tile's rows and at most 64 inputs.

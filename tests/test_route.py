@@ -288,3 +288,31 @@ def test_gpu_router_for_few_positions(d_in, n, m, G):
     W[:, half:] = W[:, :m - half]
     bias[:, half:] = bias[:, :m - half]
     assert _gpu_route(x, _bf16(W), bias).max() < half
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("variant", [0, 2])
+def test_indices_in_managed_memory_are_there_when_the_call_returns(variant):
+    """A kernel's report covers this GPU's own memory; output that the host can read has to be there when the call returns."""
+    import ctypes
+
+    import torch
+    import paper_2601_19178_b200 as ckv
+    from cuda.bindings import runtime as rt
+    n, G, d, m = 300, 2, 64, 1024
+    g = torch.Generator(device="cuda").manual_seed(5)
+    x = torch.randn((n, d), generator=g, device="cuda").bfloat16()
+    W = torch.randn((G, m, d), generator=g, device="cuda").bfloat16()
+    want = torch.empty((n, G), dtype=torch.int32, device="cuda")
+    ckv.ckv_route(0, n, G, d, m, x, W, None, want, variant)
+    want = want.cpu().numpy()
+    err, p = rt.cudaMallocManaged(n * G * 4, rt.cudaMemAttachGlobal)
+    assert err == rt.cudaError_t.cudaSuccess
+    out = np.ctypeslib.as_array(ctypes.cast(int(p), ctypes.POINTER(ctypes.c_int32)), (n, G))
+    for _ in range(50):
+        out[:] = -1
+        ckv.ckv_route(0, n, G, d, m, x, W, None, out, variant)
+        assert np.array_equal(out, want)
+    torch.cuda.synchronize()
+    del out
+    rt.cudaFree(p)
