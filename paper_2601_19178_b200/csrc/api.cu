@@ -379,8 +379,8 @@ cudaError_t run_checked(ckv_ctx* ctx, cudaStream_t s, bool* bad, F&& launch)
 
 constexpr size_t kKeepStaged = size_t(16) << 20;
 
-// A device copy of host input: in `keep` up to kKeepStaged bytes (the context's, for calls that wait for the stream
-// before they return), else in memory that the destructor frees.
+// A device copy of host input: in `keep` up to kKeepStaged bytes (the context's, for calls that wait for their
+// kernel), else in memory that the destructor frees.
 struct Staged {
     const void* dev = nullptr;
     void* owned = nullptr;

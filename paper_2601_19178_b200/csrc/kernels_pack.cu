@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(256) pack_kernel(int G, int n_entries, int n_u
             bad |= store_unit<E, I>(dV, dst + (int64_t)g * Lpad, idxV, userV, src + g, real, n_entries);
         }
     }
-    report_outcome(report, bad, gridDim.x);
+    report_done(report, bad, gridDim.x);
 }
 
 template <typename E, typename I>
@@ -151,7 +151,7 @@ __global__ void append_kernel(int G, int n_entries, int64_t old_base, int L_old,
             bad |= store_unit<E, I>(dV, dst, idxV, userV, src, real, n_entries);
         }
     }
-    report_outcome(report, bad, gridDim.x);
+    report_done(report, bad, gridDim.x);
 }
 
 template <typename E, typename I>
