@@ -27,6 +27,7 @@
 #include <math_constants.h>
 
 #include "ckv_internal.h"
+#include "ptx_helpers.cuh"
 #include "tensor_map.h"
 
 namespace ckv {
@@ -72,14 +73,6 @@ __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, const vo
 // and runs on; once a wait has run out it takes part as the issuing warp does, so that no step is passed twice.
 __device__ __forceinline__ void acc_arrive(int acc) { asm volatile("bar.arrive %0, 160;" ::"r"(1 + acc) : "memory"); }
 __device__ __forceinline__ void acc_sync(int acc) { asm volatile("bar.sync %0, 160;" ::"r"(1 + acc) : "memory"); }
-// One thread of the (converged) warp.  The issuing code stands under this and not under "lane 0", and depends on a warp number
-// that is known to be uniform: the tensor-core instructions take their operands from uniform registers.
-__device__ __forceinline__ bool elect_one()
-{
-    uint32_t p;
-    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(p)::"memory");
-    return p != 0;
-}
 __device__ __forceinline__ void fence_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tc_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -368,12 +361,10 @@ __global__ void __launch_bounds__(kThreadsRU, 1)
                 par ^= 1;
             }
         }
-        if (lane == 0) {
-            // nothing of this CTA may still run on the tensor core at teardown
-            tc_commit_to(bar(B_DRAIN));
-            volatile int never = 0;
-            if (!bar_wait(bar(B_DRAIN), 0, &never)) *abort_flag = 1;
-        }
+        // nothing of this CTA may still run on the tensor core at teardown
+        if (elect_one()) tc_commit_to(bar(B_DRAIN));
+        volatile int never = 0;
+        if (!bar_wait(bar(B_DRAIN), 0, &never)) *abort_flag = 1;
         __syncwarp();
     } else {
         // ------------------------------------------------------------ weight tiles, and their bias steps

@@ -40,6 +40,16 @@ __device__ __forceinline__ float tanh_fast(float x)
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// One thread of the (converged) warp, every time the same one.  Tensor-core instructions are issued under this and not under
+// "lane 0", and from a warp number that is known to be uniform: they take their operands from uniform registers.  A commit
+// covers what its own thread has issued, so it stands under this too, that of a kernel's end included.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(p)::"memory");
+    return p != 0;
+}
+
 // Programmatic launch (Launch::early): lets the stream's next kernel be set up, then waits until the previous one
 // has finished and its memory is visible.  Without that launch attribute both are no-ops.
 __device__ __forceinline__ void grid_dependency_wait()
