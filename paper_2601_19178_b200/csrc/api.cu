@@ -354,9 +354,10 @@ cudaError_t grow(DevBuf& b, size_t bytes, int64_t* allocs = nullptr)
 
 // Waits until the kernel just launched on `s` has written the host-mapped word `done`, which it writes last.  Short kernels
 // are over within microseconds of the launch, before a stream synchronise returns, so the word is watched first; after
-// that, and for every error, the stream is waited for.
+// that, and for every error, the stream is waited for.  done = null: the kernel does not report (as its launcher knows).
 cudaError_t wait_done(volatile int* done, cudaStream_t s)
 {
+    if (!done) return cudaStreamSynchronize(s);
     const auto t0 = std::chrono::steady_clock::now();
     while (!*done && std::chrono::steady_clock::now() - t0 < std::chrono::microseconds(40)) {
     }
@@ -371,8 +372,9 @@ cudaError_t run_checked(ckv_ctx* ctx, cudaStream_t s, bool* bad, F&& launch)
 {
     volatile int* const flag = ctx->h_flag;
     flag[0] = flag[1] = 0;
-    cudaError_t e = launch(Report{ctx->h_flag, ctx->h_flag + 1, reinterpret_cast<unsigned*>(ctx->d_err + 1)});
-    if (e == cudaSuccess) e = wait_done(flag + 1, s);
+    Report report{ctx->h_flag, ctx->h_flag + 1, reinterpret_cast<unsigned*>(ctx->d_err + 1)};
+    cudaError_t e = launch(report);
+    if (e == cudaSuccess) e = wait_done(report.done, s);
     *bad = flag[0] != 0;
     return e;
 }
@@ -1402,7 +1404,7 @@ ckv_status ckv_cache_put_batch(ckv_ctx* ctx, int32_t n, const int64_t* users, co
         ckv_status st = arena_take(ctx, total_units, s, &base);
         if (st != CKV_OK) return st;
         bool bad;
-        const cudaError_t e = run_checked(ctx, s, &bad, [&](const Report& report) {
+        const cudaError_t e = run_checked(ctx, s, &bad, [&](Report& report) {
             return launch_pack(ctx->cfg.dtype, G, ctx->n_entries, ctx->idx_bytes, n,
                                n > kInlinePuts ? (const PutUser*)ctx->put_dev.p : nullptr, &inl,
                                total_units / (32 * (int64_t)G), base, (const int32_t*)sik.dev, (const int32_t*)siv.dev,
@@ -1468,16 +1470,19 @@ ckv_status ckv_cache_append(ckv_ctx* ctx, int64_t user, int32_t L_new, const int
         ckv_status st = arena_take(ctx, units, s, &base);
         if (st != CKV_OK) return st;
     }
-    auto append = [&](int32_t n_new, const Report& report) {
+    auto append = [&](int32_t n_new, Report& report) {
         return launch_append(ctx->cfg.dtype, G, ctx->n_entries, ctx->idx_bytes, old.base, old.L, old.Lpad, base, n_new,
                              Lpad_tot, (const int32_t*)sik.dev, (const int32_t*)siv.dev, suk.dev, suv.dev, view_of(ctx),
                              ctx->cfg.head_dim, report, s);
     };
     bool bad;
-    cudaError_t e = run_checked(ctx, s, &bad, [&](const Report& report) { return append(L_new, report); });
+    cudaError_t e = run_checked(ctx, s, &bad, [&](Report& report) { return append(L_new, report); });
     if (e != cudaSuccess || bad) {  // the user keeps the old history
         if (!in_place) arena_give(ctx, base, units);
-        else if (e == cudaSuccess) e = append(0, Report{ctx->h_flag});  // padding again
+        else if (e == cudaSuccess) {  // padding again
+            Report none{ctx->h_flag};
+            e = append(0, none);
+        }
         return e != cudaSuccess ? ctx->fail(e) : CKV_ERR_INDEX_RANGE;
     }
     if (!in_place) arena_give(ctx, old.base, (int64_t)G * old.Lpad);
@@ -2071,10 +2076,10 @@ ckv_status ckv_route(int32_t device, int32_t n, int32_t n_groups, int32_t d_in, 
         if (!flag.p) return CKV_ERR_OOM;
         // (a kernel's report covers what it has written to this GPU's own memory; for managed memory and a peer's the call
         // waits for the stream)
-        const int slot = out_at == device ? flag.slot() : -1;
+        int slot = out_at == device ? flag.slot() : -1;
         e = (variant == 0 && route_few(d_in, x, W, n, n_entries, n_groups) ? launch_route_few : launch_route_umma)(
-            d_in, x, W, bias, n, n_entries, n_groups, idx_out, flag.p, slot, s);
-        if (e == cudaSuccess) e = slot >= 0 ? wait_done(flag.p + 1, s) : cudaStreamSynchronize(s);
+            d_in, x, W, bias, n, n_entries, n_groups, idx_out, flag.p, &slot, s);
+        if (e == cudaSuccess) e = wait_done(slot >= 0 ? flag.p + 1 : nullptr, s);
         // a bounded wait inside the kernel ran out: the output is not valid
         if (e == cudaSuccess && *(volatile int*)flag.p) return CKV_ERR_CUDA;
     }

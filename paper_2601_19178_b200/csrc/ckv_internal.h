@@ -184,18 +184,18 @@ struct PutTable {
 };
 // Packs n users' [P][G] indices and [P][G][d_user] user parts into arena units and validates the index range.  The users
 // come from `table` (device memory) or, if that is null, from *inl; the arena arrays and the sides' widths from `cv`
-// (head_dim D).
+// (head_dim D).  report.done becomes null if the kernel does not report (here and below).
 cudaError_t launch_pack(int dtype, int G, int n_entries, int idx_bytes, int n_users, const PutUser* table,
                         const PutTable* inl, int64_t total_tiles, int64_t arena_base, const int32_t* idxK,
                         const int32_t* idxV, const void* userK, const void* userV, const CacheView& cv, int D,
-                        const Report& report, cudaStream_t s);
+                        Report& report, cudaStream_t s);
 // Writes a user's units for L_old + L_new positions at arena unit dst_base: the first L_old positions copied from
 // the units at old_base (same arena), the rest packed from the new [L_new][G] indices and [L_new][G][d_user] parts.  dst_base = old_base (and
 // Lpad_tot = Lpad_old): the new positions are written behind the old ones, in place.
 cudaError_t launch_append(int dtype, int G, int n_entries, int idx_bytes, int64_t old_base, int L_old,
                           int Lpad_old, int64_t dst_base, int L_new, int Lpad_tot, const int32_t* idxK,
                           const int32_t* idxV, const void* userK, const void* userV, const CacheView& cv, int D,
-                          const Report& report, cudaStream_t s);
+                          Report& report, cudaStream_t s);
 cudaError_t launch_materialize(int dtype, int D, const CacheView& cv, int64_t base, int L, int Lpad,
                                void* K_out, void* V_out, cudaStream_t s);
 
@@ -242,16 +242,17 @@ cudaError_t launch_route(int d_in, const void* x, const void* W, const float* bi
 
 // ---- kernels_route_umma.cu : the same router on tcgen05 (TMEM accumulators, warp-specialised)
 // flags: two host-mapped ints.  flags[0] becomes non-zero if a bounded wait inside the kernel ran out (`out` is not
-// valid then, whether written or not); flags[1] becomes 1 at its end if slot is in [0, kRouteSlots) and no other launch uses it at the time.
+// valid then, whether written or not).  If *slot is in [0, kRouteSlots), and no other launch uses it at the time, flags[1] becomes 1
+// at its end; where the kernel does not report (several rounds of blocks) *slot becomes -1.
 constexpr int kRouteSlots = 64;
 cudaError_t launch_route_umma(int d_in, const void* x, const void* W, const float* bias, int n, int n_entries, int G,
-                              int32_t* out, int* flags, int slot, cudaStream_t s);
+                              int32_t* out, int* flags, int* slot, cudaStream_t s);
 
 // kernels_route.cu, the same for few positions (route_few says which calls that is): the entries shared by the warps of a
 // cluster.  flags, slot: as above, flags[0] stays 0.
 bool route_few(int d_in, const void* x, const void* W, int n, int n_entries, int G);
 cudaError_t launch_route_few(int d_in, const void* x, const void* W, const float* bias, int n, int n_entries, int G,
-                             int32_t* out, int* flags, int slot, cudaStream_t s);
+                             int32_t* out, int* flags, int* slot, cudaStream_t s);
 
 // out[i][g][c] = x_i . W[g][c] + bias[g][c] (bf16 in and out, fp32 sums); W [G][d_out][d_in], bias [G][d_out] or null.
 bool project_supported(int d_in, int d_out, int n_groups);

@@ -219,13 +219,12 @@ constexpr int kMaxReporting = 1024;
 cudaError_t launch_pack(int dtype, int G, int n_entries, int idx_bytes, int n_users, const PutUser* table,
                         const PutTable* inl, int64_t total_tiles, int64_t arena_base, const int32_t* idxK,
                         const int32_t* idxV, const void* userK, const void* userV, const CacheView& cv, int D,
-                        const Report& to, cudaStream_t s)
+                        Report& report, cudaStream_t s)
 {
     if (total_tiles == 0) return cudaSuccess;
     // two warps per block while that leaves SMs without a block, then eight; at most 16 blocks of eight per SM
     const int block = total_tiles <= 148 * 8 ? 64 : 256, wpb = block / 32;
     const int grid = (int)std::min<int64_t>((total_tiles + wpb - 1) / wpb, 148 * 16);
-    Report report = to;
     if (grid > kMaxReporting) report.done = nullptr;
     static const PutTable none{};
     const PutTable& pt = inl ? *inl : none;
@@ -247,12 +246,11 @@ cudaError_t launch_pack(int dtype, int G, int n_entries, int idx_bytes, int n_us
 cudaError_t launch_append(int dtype, int G, int n_entries, int idx_bytes, int64_t old_base, int L_old,
                           int Lpad_old, int64_t dst_base, int L_new, int Lpad_tot, const int32_t* idxK,
                           const int32_t* idxV, const void* userK, const void* userV, const CacheView& cv, int D,
-                          const Report& to, cudaStream_t s)
+                          Report& report, cudaStream_t s)
 {
     const int64_t total = (int64_t)G * (Lpad_tot - (dst_base == old_base ? L_old : 0));
     if (total == 0) return cudaSuccess;
     const int grid = grid_for(total, 256);
-    Report report = to;
     if (grid > kMaxReporting) report.done = nullptr;
     const int es = dtype == CKV_BF16 ? 2 : 4;
     const SideDst dK = side_dst(cv.full_k, cv.idxK, cv.userK, cv.d_user, D, es, userK);

@@ -322,16 +322,18 @@ __global__ void __launch_bounds__(kFewWarps * 32, DIN == 128 ? 1 : 2)
 
 template <int DIN>
 cudaError_t launch_route_few_t(const void* x, const void* W, const float* bias, int n, int m, int G, int32_t* out, int* flags,
-                               int slot, cudaStream_t s)
+                               int* slot, cudaStream_t s)
 {
     const int64_t blocks = (int64_t)((n + kFewRows - 1) / kFewRows) * G;
     const int tiles = (m + 7) / 8;
     // a cluster's blocks share the entries as long as there are SMs for them and each warp keeps two batches
+    const int resident = DIN == 128 ? 148 : 2 * 148;
     int split = 1;
-    while (split < kFewMaxSplit && blocks * split * 2 <= (DIN == 128 ? 148 : 2 * 148) && tiles >= 2 * split * kFewWarps * 2 * kFewBatch) split *= 2;
+    while (split < kFewMaxSplit && blocks * split * 2 <= resident && tiles >= 2 * split * kFewWarps * 2 * kFewBatch) split *= 2;
     const dim3 grid((unsigned)((n + kFewRows - 1) / kFewRows * split), (unsigned)G);
+    if (blocks * split > resident) *slot = -1;
     return launch_kernel(Launch{s, nullptr, nullptr}, route_few_kernel<DIN>, grid, kFewWarps * 32, 0, split, (const uint16_t*)x,
-                         (const uint16_t*)W, bias, n, m, G, out, flags, slot, split);
+                         (const uint16_t*)W, bias, n, m, G, out, flags, *slot, split);
 }
 
 // User-specific low-dimensional projection of the prefill (Sec. 4.2): y[i][g][c] = x_i . W[g][c] + b[g][c],
@@ -392,7 +394,7 @@ bool route_few(int d_in, const void* x, const void* W, int n, int n_entries, int
 }
 
 cudaError_t launch_route_few(int d_in, const void* x, const void* W, const float* bias, int n, int n_entries, int G,
-                             int32_t* out, int* flags, int slot, cudaStream_t s)
+                             int32_t* out, int* flags, int* slot, cudaStream_t s)
 {
     switch (d_in) {
         case 32: return launch_route_few_t<32>(x, W, bias, n, n_entries, G, out, flags, slot, s);

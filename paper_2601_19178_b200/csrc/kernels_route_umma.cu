@@ -479,7 +479,7 @@ bool make_weight_map(int d_in, int64_t rows, int tile_rows, const void* W, CUten
 
 template <int DIN>
 cudaError_t launch_t(const void* x, const void* W, const float* bias, int n, int m, int G, int32_t* out, int* flags,
-                     int slot, cudaStream_t s)
+                     int* slot, cudaStream_t s)
 {
     CUtensorMap map;
     if (!make_weight_map(DIN, (int64_t)G * m, RU<DIN>::TN, W, &map)) return cudaErrorInvalidValue;
@@ -500,15 +500,15 @@ cudaError_t launch_t(const void* x, const void* W, const float* bias, int n, int
         }
     }
     const dim3 grid((unsigned)((n + kRows - 1) / kRows * split), (unsigned)G);
-    if (ctas * split > sms) slot = -1;  // several rounds: the report at the end of each CTA would delay the next
+    if (ctas * split > sms) *slot = -1;  // several rounds: the report at the end of each CTA would delay the next
     return launch_kernel(Launch{s, nullptr, nullptr}, route_umma_kernel<DIN>, grid, kThreadsRU, RU<DIN>::SMEM, split,
-                         (const uint16_t*)x, map, bias, n, m, G, out, flags, slot, split);
+                         (const uint16_t*)x, map, bias, n, m, G, out, flags, *slot, split);
 }
 
 }  // namespace
 
 cudaError_t launch_route_umma(int d_in, const void* x, const void* W, const float* bias, int n, int n_entries, int G,
-                              int32_t* out, int* flags, int slot, cudaStream_t s)
+                              int32_t* out, int* flags, int* slot, cudaStream_t s)
 {
     if (n == 0) return cudaSuccess;
     switch (d_in) {

@@ -217,3 +217,30 @@ def test_tma_loader_option_leaves_the_tcgen05_kernel_its_lists(lib):
             assert attend(*call) == 0
             assert lib.ckv_last_stat(ctx, b"kernel", C.byref(kernel)) == 0 and kernel.value == family
         lib.ckv_destroy(ctx)
+
+
+def test_a_report_that_does_not_come_is_not_waited_for(lib):
+    """Kernels of several rounds of blocks do not report: their calls go to the stream at once, not behind the 40 us that they
+    watch for a report (which no kernel writes here, so that calls whose kernel reports take those 40 us)."""
+    G, d = 4, 64
+    block = device_block(lib, 1 << 20)
+    ctx, _ = context(lib, G=G)
+    user = np.zeros(1, np.int64)
+
+    def us(call):
+        best = 1e9
+        for _ in range(20):
+            t = time.perf_counter()
+            assert call() == 0
+            best = min(best, time.perf_counter() - t)
+        return best * 1e6
+
+    def route(n, m, variant):
+        return us(lambda: lib.ckv_route(0, n, G, d, m, block, block, None, block, variant, None))
+
+    assert route(200, 1024, 0) >= 40 and route(200, 1024, 2) >= 40
+    assert route(20000, 64, 2) < 30 and route(1000000, 16384, 0) < 30
+    assert route(300000, 8, 0) < 30  # (more blocks than the report's counter could tell apart)
+    assert us(lambda: put(lib, ctx, block, user, [1000])) >= 40
+    assert us(lambda: put(lib, ctx, block, user, [1100 * 8 * 32])) < 30
+    lib.ckv_destroy(ctx)
