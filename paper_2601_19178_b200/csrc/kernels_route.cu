@@ -174,6 +174,7 @@ cudaError_t launch_route_t(const void* x, const void* W, const float* bias, int 
 // the report to the host included (the tcgen05 kernel has TMEM, barriers, tensor maps and a pipeline to set up first), and
 // with more positions the weights, which every block of 32 reads from L2 for itself.
 constexpr int kFewRows = 32, kFewWarps = 8, kFewMaxSplit = 8, kFewBatch = 4;
+constexpr int kFewBlocks = 2 * 148;  // see route_few
 
 __device__ unsigned few_count[kRouteSlots];  // finished blocks of the launch that holds the slot, zero between launches
 
@@ -327,7 +328,7 @@ cudaError_t launch_route_few_t(const void* x, const void* W, const float* bias, 
     const int64_t blocks = (int64_t)((n + kFewRows - 1) / kFewRows) * G;
     const int tiles = (m + 7) / 8;
     // a cluster's blocks share the entries as long as there are SMs for them and each warp keeps two batches
-    const int resident = DIN == 128 ? 148 : 2 * 148;
+    const int resident = DIN == 128 ? 148 : kFewBlocks;
     int split = 1;
     while (split < kFewMaxSplit && blocks * split * 2 <= resident && tiles >= 2 * split * kFewWarps * 2 * kFewBatch) split *= 2;
     const dim3 grid((unsigned)((n + kFewRows - 1) / kFewRows * split), (unsigned)G);
@@ -386,11 +387,16 @@ cudaError_t launch_route(int d_in, const void* x, const void* W, const float* bi
 
 // Up to 1.1e9 products: 500 positions x 16384 entries x 2 groups (d_in 64, 1.05e9) 37 us against 42 with the tcgen05 kernel,
 // 1000 x 4096 x 4 27 / 32, 2000 x 4096 x 4 (d_in 32) 29 / 34; at 1.3e9 33 / 32 and 39 / 34, at 2.1e9 40 / 42 and 47 / 40 (a call
-// and a wait for the stream, before the report; without that wait the line lies in the same place).
+// and a wait for the stream, before the report; without that wait the line lies in the same place).  And up to 296 blocks of 32
+// positions and a group, two for each SM: a small pool leaves most warps of a block without a tile, and every further round of
+// blocks costs 1.5 to 3.5 us, where the tcgen05 kernel has 384 positions to a block.  64 entries, 4 groups (d_in 32): 2000
+// positions (252 blocks) 11.8 us against 13.7, 3000 (376) 14.9 / 13.5, 10000 20.5 / 14.1, 100000 89 / 41; 1024 entries, 2 groups
+// (d_in 64): 2000 15.9 / 17.5, 5000 (314) 23.7 / 18.4; 32 entries, 4 groups (d_in 128, one block per SM): 2000 16.0 / 18.2, 3000
+// 18.5 / 18.3, 5000 22.2 / 18.5.
 bool route_few(int d_in, const void* x, const void* W, int n, int n_entries, int G)
 {
     if (((uintptr_t)x | (uintptr_t)W) & 15) return false;  // rows are read sixteen bytes at a time
-    return (double)n * n_entries * G * d_in <= 1.1e9;
+    return (double)n * n_entries * G * d_in <= 1.1e9 && ((int64_t)n + kFewRows - 1) / kFewRows * G <= kFewBlocks;
 }
 
 cudaError_t launch_route_few(int d_in, const void* x, const void* W, const float* bias, int n, int n_entries, int G,

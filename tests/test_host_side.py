@@ -244,3 +244,15 @@ def test_a_report_that_does_not_come_is_not_waited_for(lib):
     assert us(lambda: put(lib, ctx, block, user, [1000])) >= 40
     assert us(lambda: put(lib, ctx, block, user, [1100 * 8 * 32])) < 30
     lib.ckv_destroy(ctx)
+
+
+# (d_in, positions, entries, groups, threads of a block: 256 where the entries are shared by its warps, 512 for the tcgen05 kernel)
+@pytest.mark.parametrize("d,n,m,G,threads", [(64, 1, 8, 1, 256), (64, 1072, 8000, 2, 256), (64, 1075, 8000, 2, 512),
+                                             (64, 9472, 32, 1, 256), (64, 9473, 32, 1, 512), (32, 2368, 1000, 4, 256),
+                                             (32, 2369, 1000, 4, 512), (128, 4736, 16, 2, 256), (128, 4737, 16, 2, 512),
+                                             (64, 1000000, 16, 1, 512), (64, 32, 16, 296, 256), (64, 32, 16, 297, 512)])
+def test_kernel_of_router_calls(lib, d, n, m, G, threads):
+    """The kernel for few positions takes 1.1e9 products and 296 blocks of 32 positions and a group, no more."""
+    block = device_block(lib, 1 << 20)
+    assert lib.ckv_route(0, n, G, d, m, block, block, None, block, 0, None) == 0
+    assert np.ctypeslib.as_array(lib.fake_launched(), (6,))[3] == threads

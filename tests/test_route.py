@@ -273,10 +273,12 @@ def test_gpu_router_at_the_edges_of_blocks_and_tiles(d_in, n, m):
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("d_in,n,m,G", [(32, 1, 1, 1), (32, 33, 7, 2), (64, 32, 9, 1), (64, 31, 257, 3), (128, 65, 4096, 1),
-                                        (64, 200, 16384, 1), (32, 1000, 2048, 2), (64, 1072, 8000, 2), (64, 1075, 8000, 2)])
+                                        (64, 200, 16384, 1), (32, 1000, 2048, 2), (64, 1072, 8000, 2), (64, 1075, 8000, 2),
+                                        (64, 4736, 33, 2), (64, 4737, 33, 2), (128, 4736, 16, 2), (128, 2400, 70, 2)])
 def test_gpu_router_for_few_positions(d_in, n, m, G):
     """The kernel that shares the entries among warps and clusters: blocks of 32 positions, tiles of eight entries, begun ones,
-    warps without a tile, and both sides of the line (1.1e9 products) beyond which the tcgen05 kernel takes over."""
+    warps without a tile, both sides of the lines (1.1e9 products, 296 blocks) beyond which the tcgen05 kernel takes over, and
+    more blocks than there is room for at a time (d_in 128)."""
     rng = np.random.default_rng(n + m)
     x = _bf16(rng.standard_normal((n, d_in)) / np.sqrt(d_in))
     W = rng.standard_normal((G, m, d_in)).astype(np.float32)
