@@ -69,10 +69,13 @@ __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, const vo
     }
     return false;
 }
-// Named barrier of an accumulator, for its block's four read-out warps and its issuing warp: "it has been read".  The read-out arrives
-// and runs on; once a wait has run out it takes part as the issuing warp does, so that no step is passed twice.
-__device__ __forceinline__ void acc_arrive(int acc) { asm volatile("bar.arrive %0, 160;" ::"r"(1 + acc) : "memory"); }
-__device__ __forceinline__ void acc_sync(int acc) { asm volatile("bar.sync %0, 160;" ::"r"(1 + acc) : "memory"); }
+// Named barriers of an accumulator, for its block's four read-out warps and its issuing warp: "tile t has been read".  The
+// read-out arrives and runs on; once a wait has run out it takes part as the issuing warp does.  Two barriers in turn: a warp that
+// gives up on the next tile has arrived for this one already, and on the same barrier would count for the issuing warp, which
+// then waited for good.
+__device__ __forceinline__ int read_barrier(int acc, int tile) { return 1 + 2 * acc + (tile & 1); }
+__device__ __forceinline__ void acc_arrive(int acc, int tile) { asm volatile("bar.arrive %0, 160;" ::"r"(read_barrier(acc, tile)) : "memory"); }
+__device__ __forceinline__ void acc_sync(int acc, int tile) { asm volatile("bar.sync %0, 160;" ::"r"(read_barrier(acc, tile)) : "memory"); }
 __device__ __forceinline__ void fence_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tc_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -161,7 +164,7 @@ struct RU {
                          OFF_KEPT = OFF_BEST + kRows * 8,      // [8][kRows] four scores of a position's best chunk
                          OFF_BAR = OFF_KEPT + kRows * 128, OFF_ABORT = OFF_BAR + B_COUNT * 8, SMEM = OFF_ABORT + 16;
     static_assert(STAGES <= kMaxStages && SMEM <= 226 * 1024 && BOX % 1024 == 0, "shared memory");
-    // TMEM: an accumulator per block, the inputs of each block (two per column), the ones of the bias step
+    // TMEM: the accumulators of each block, the inputs of each block (two per column), the ones of the bias step
     static constexpr uint32_t COL_A = kBlocks * TN, COL_ONES = COL_A + kBlocks * (DIN / 2);
     static_assert(COL_ONES + 8 <= 512, "TMEM columns");
 };
@@ -299,7 +302,7 @@ __global__ void __launch_bounds__(kThreadsRU, 1)
                     if (!ok) *abort_flag = 1;
                 }
                 if (!ok) {
-                    if (t + 1 < n_tiles) acc_sync(acc);
+                    if (t + 1 < n_tiles) acc_sync(acc, t);
                     continue;
                 }
                 tc_after();
@@ -310,7 +313,7 @@ __global__ void __launch_bounds__(kThreadsRU, 1)
 #pragma unroll
                 for (int c = 0; c < AN / 32; ++c) wait_ld32(v[c]);
                 tc_before();
-                if (t + 1 < n_tiles) acc_arrive(acc);
+                if (t + 1 < n_tiles) acc_arrive(acc, t);
 #pragma unroll
                 for (int c = 0; c < AN / 32; ++c) look(v[c], (tile0 + t) * TN + AN * h + 32 * c);
             }
@@ -342,7 +345,7 @@ __global__ void __launch_bounds__(kThreadsRU, 1)
             }
 #pragma unroll
             for (int h = 0; h < ACCS; ++h) {
-                if (t > 0) acc_sync(ACCS * blk + h);
+                if (t > 0) acc_sync(ACCS * blk + h, t - 1);
                 if (ok && elect_one()) {
                     tc_after();
                     // (entries AN h and up of the tile: whole groups of eight rows further on)
