@@ -219,7 +219,7 @@ def test_prefill_outputs_feed_the_decode_path():
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("variant", [0, 1])
+@pytest.mark.parametrize("variant", [0, 1, 2])
 @pytest.mark.parametrize("n,G,d,m", [(200, 2, 64, 1024), (5, 1, 32, 1000), (40000, 2, 128, 1111)])
 def test_gpu_route_biases_out_of_the_ordinary(n, G, d, m, variant):
     """A bias is an fp32 summand, whatever its size: one that is not a number never wins (also where its upper sixteen bits
@@ -232,7 +232,7 @@ def test_gpu_route_biases_out_of_the_ordinary(n, G, d, m, variant):
     nan.view(np.uint32)[:, 3] = 0x7f800001
     nan.view(np.uint32)[:, 700] = 0xff80ffff
     without = np.where(np.isnan(nan), np.float32(-np.inf), nan)
-    if variant == 0:
+    if variant != 1:
         assert np.array_equal(_gpu_route(x, W, nan, variant), _gpu_route(x, W, without, variant))
     got = _gpu_route(x, W, np.where(np.arange(m) == 700, np.float32(np.inf), bias).astype(np.float32), variant)
     assert (got == 700).all()
@@ -253,22 +253,23 @@ def test_gpu_route_biases_out_of_the_ordinary(n, G, d, m, variant):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("variant", [0, 2])
 @pytest.mark.parametrize("d_in", [32, 64, 128])
 @pytest.mark.parametrize("n,m", [(128, 64), (129, 65), (257, 96), (384, 97), (385, 128), (383, 129), (769, 193), (64, 2500)])
-def test_gpu_router_at_the_edges_of_blocks_and_tiles(d_in, n, m):
+def test_gpu_router_at_the_edges_of_blocks_and_tiles(d_in, n, m, variant):
     """Whole blocks of 128 positions and one more or less, accumulators and tiles that are full, begun or missing; every
     position's best entry planted, so that each column of a tile is the answer of some position, bit for bit."""
     rng = np.random.default_rng(n * m)
     x = _bf16(rng.standard_normal((n, d_in)) / np.sqrt(d_in))
     W = _bf16(rng.standard_normal((2, m, d_in)))
     bias = (0.1 * rng.standard_normal((2, m))).astype(np.float32)
-    _check(x, W, bias, f"d_in={d_in} n={n} m={m}")
+    _check(x, W, bias, f"d_in={d_in} n={n} m={m} variant={variant}", variant)
     # weights zero: the score is the bias, and a position's choice the largest bias, the first of two equal ones
     for j in {0, 31, 32, 63, 64, 95, 96, 127, 128, m - 1} & set(range(m)):
         b = np.zeros((2, m), np.float32)
         b[0, j] = b[1, j] = 1.0
         b[1, m - 1] = 1.0
-        assert (_gpu_route(x, np.zeros_like(W), b) == j).all(), j
+        assert (_gpu_route(x, np.zeros_like(W), b, variant) == j).all(), j
 
 
 @pytest.mark.gpu
