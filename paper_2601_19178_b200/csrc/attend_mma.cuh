@@ -44,7 +44,7 @@ namespace ckv {
 namespace {
 
 constexpr float kLog2e = 1.4426950408889634f;
-constexpr float kSumLimit = 0x1p70f;  // see `normalise`
+constexpr float kOctavesAbove = 10.f, kSumLimit = 1.f;  // see `normalise`
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src)
 {
@@ -466,12 +466,13 @@ __global__ void __launch_bounds__(128, MmaCfg<D, MT, TMA, DENSE>::MIN_BLOCKS)
                         if (pc + 1 >= e_hi) s[nt][3] = -CUDART_INF_F;
                     }
                 }
-                // A row's reference is the maximum of the first tile and stays there: fp32 sums and bf16 weights have the
-                // exponent range for scores far above it.  A lane's eight weights that add up to more than 2^70, or to no
-                // number, give away that a score has left it; then, as in the first tile, the reference goes to the
-                // maximum.  (A row that sees nothing of the first tile sees nothing of the others.)  That takes the maxima
-                // and four dependent shuffles out of every other tile (65536 users x 512 positions x 16 queries
-                // 2364 -> 2163 us, 4096 x 512 x 16 64-wide 315 -> 259, 199 ragged ones 63 -> 58).
+                // A row's reference lies ten octaves above the maximum of the first tile and stays there.  A lane's eight weights
+                // that add up to more than one, or to no number, give away that a score has come near it; then, as in the first
+                // tile, the reference goes ten octaves above the maximum.  (A row that sees nothing of the first tile sees
+                // nothing of the others.)  No weight is more than one, as with the running maximum, so that sums with
+                // values near fp32's largest stay in range.  That takes the maxima and four dependent shuffles out of every
+                // other tile (65536 users x 512 positions x 16 queries 2364 -> 2163 us, 4096 x 512 x 16 64-wide 315 -> 259, 199
+                // ragged ones 63 -> 58).
                 float ps0, ps1;
                 auto weigh = [&]() {  // the weights and this lane's share of their sums
                     const float r0 = VAR && m_run[mt][0] == -CUDART_INF_F ? 0.f : m_run[mt][0],
@@ -507,11 +508,11 @@ __global__ void __launch_bounds__(128, MmaCfg<D, MT, TMA, DENSE>::MIN_BLOCKS)
                     }
                     // a row may not see any position of this tile (or of any tile so far): its maximum is then -inf
                     // and must not enter the exponent arguments
-                    const float mn0 = fmaxf(m_run[mt][0], mx0 * sc);
-                    const float mn1 = has_hi ? fmaxf(m_run[mt][1], mx1 * sc) : 0.f;
+                    const float mn0 = fmaxf(m_run[mt][0], fmaf(mx0, sc, kOctavesAbove));
+                    const float mn1 = has_hi ? fmaxf(m_run[mt][1], fmaf(mx1, sc, kOctavesAbove)) : 0.f;
                     // (without visible lengths the first position of a tile is always attended and the maxima are finite)
                     const float ms0 = VAR && mn0 == -CUDART_INF_F ? 0.f : mn0, ms1 = VAR && mn1 == -CUDART_INF_F ? 0.f : mn1;
-                    // the running maxima settle after a few tiles: rescale only when one of them moved
+                    // rescale only when one of them moved (in the first tile, and rarely behind it)
                     const bool moved = mn0 != m_run[mt][0] || (has_hi && mn1 != m_run[mt][1]);
                     if (__any_sync(0xffffffffu, moved)) {
                         const float c0 = ex2(m_run[mt][0] - ms0), c1 = has_hi ? ex2(m_run[mt][1] - ms1) : 1.f;

@@ -289,3 +289,68 @@ def test_short_lists_under_stream_capture(queries):
     assert torch.equal(out, want)
     del graph
     s.close()
+
+
+_WIDE_LISTS = [(2, head, users, queries) for head, queries in (((30, 2), 7), ((30, 2), 33), ((60, 4), 16), ((60, 4), 20))
+               for users in (1, 900)]
+
+
+@pytest.mark.parametrize("kernel,head,users,queries", _WIDE_LISTS)
+@pytest.mark.parametrize("ramp", [(-60, 60), (60, -60), (0, 20)])
+def test_values_near_the_largest_behind_scores_above_the_first(kernel, head, users, queries, ramp):
+    """Values of 2^112 and scores that climb by up to 170 octaves along a history: weights and sums stay in fp32's range, as they
+    do with weights relative to the running maximum (at most 400 of them, each at most one: 2^121)."""
+    w = _workload(head=head, users=users, hist=(200, 400), queries=queries)
+    d = synth.generate(w)
+    for a, b in zip(d["hist_off"][:-1], d["hist_off"][1:]):
+        d["user_K"][a:b, :, 0] = synth.f32_to_bf16_bits(np.linspace(*ramp, b - a, dtype=np.float32))[:, None]
+    d["queries"][:, :, 0] = synth.f32_to_bf16_bits(np.full(d["queries"].shape[:2], 1.0, np.float32))
+    sel = np.arange(0, users, 90)
+    want = oracle_attend(w, d, scale=1.0, sel=sel)
+    for k in ("pool_V", "user_V"):  # times a power of two: exact
+        d[k] = synth.f32_to_bf16_bits(synth.bf16_bits_to_f32(d[k]) * np.float32(2.0 ** 112))
+    s = make_session(w, d, scale=1.0, kernel=kernel)
+    got = gpu_attend(w, d, session=s)
+    assert s.stat("device_errors") == 0
+    s.close()
+    rows = np.concatenate([np.arange(d["q_off"][u], d["q_off"][u + 1]) for u in sel])
+    assert_close(got[rows] * 2.0 ** -112, want, "bf16", f"{kernel} {users} {head} {queries} {ramp}")
+
+
+@pytest.mark.parametrize("kernel,head,users,queries", _WIDE_LISTS)
+@pytest.mark.parametrize("what", ["key -inf", "key +inf", "key nan", "value +inf", "value nan"])
+def test_infinities_behind_a_first_tile(kernel, head, users, queries, what):
+    """One position behind the first 64 of every other user: a key of -inf takes no weight, +inf or none at all leave no number in the
+    row, a value shows in its own column alone."""
+    w = _workload(head=head, users=users, hist=(200, 400), queries=queries)
+    d = synth.generate(w)
+    side, x = what.split()
+    bits = {"-inf": 0xff80, "+inf": 0x7f80, "nan": 0x7fc0}[x]
+    hit = np.arange(0, users, 2)
+    for u in hit:
+        d["user_K" if side == "key" else "user_V"][d["hist_off"][u] + 70 + u % 100, :, 1] = bits
+    d["queries"][:, :, 1] = synth.f32_to_bf16_bits(np.full(d["queries"].shape[:2], 1.0, np.float32))
+    sel = np.unique(np.concatenate([np.arange(0, users, 90), np.arange(0, users, 91)]))
+    clean = {k: v.copy() for k, v in d.items()}
+    for u in hit:  # the oracle's arithmetic: what such a position does to the others is known
+        p = d["hist_off"][u] + 70 + u % 100
+        if side == "key":
+            clean["user_K"][p, :, 1] = synth.f32_to_bf16_bits(np.float32(-1e30))
+        else:
+            clean["user_V"][p, :, 1] = 0
+    want = oracle_attend(w, clean, scale=1.0, sel=sel)
+    row = 0
+    for u in sel:
+        n = d["q_off"][u + 1] - d["q_off"][u]
+        if u % 2 == 0 and what != "key -inf":
+            if side == "key": want[row:row + n] = np.nan
+            else: want[row:row + n, :, 1] = np.inf if x == "+inf" else np.nan
+        row += n
+    s = make_session(w, d, scale=1.0, kernel=kernel)
+    got = gpu_attend(w, d, session=s)
+    assert s.stat("device_errors") == 0
+    s.close()
+    got = got[np.concatenate([np.arange(d["q_off"][u], d["q_off"][u + 1]) for u in sel])]
+    odd = ~np.isfinite(want)
+    assert np.array_equal(got[odd], want[odd], equal_nan=True)
+    assert_close(np.where(odd, 0, got), np.where(odd, 0, want), "bf16", f"{kernel} {users} {head} {queries} {what}")
