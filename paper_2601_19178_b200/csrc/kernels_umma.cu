@@ -38,11 +38,11 @@
 // off behind the next unit's first tile, 548 us and 3.27 ms: with the registers that takes the arithmetic no longer
 // overlaps itself.)
 //
-// Softmax bookkeeping.  The reference maximum m of a row is the largest of the first 32 scores of the unit's
-// first tile and stays fixed: later scores may exceed it by up to 2^64 (fp32 accumulators and bf16
-// P have the exponent range for that).  The row sum l is added up by the row's thread in fp32, chunk by chunk, and
-// a chunk's share of it also tells when a row has left that bound (32 weights within it sum to at most 2^69); only
-// then is the reference moved, O and the row sum rescaled (TMEM read-modify-write) and the chunk worked out again.
+// Softmax bookkeeping.  The reference m of a row lies ten octaves above the largest of the first 32 scores of the unit's
+// first tile and stays fixed.  The row sum l is added up by the row's thread in fp32, chunk by chunk, and a chunk's share of
+// it also tells when a score has come near the reference (32 weights above one, in sum); only then is the reference moved, O
+// and the row sum rescaled (TMEM read-modify-write) and the chunk worked out again.  So no weight is more than one, as with
+// the running maximum, and sums with values near fp32's largest stay in range.
 //
 // Shared-memory tiles hold rows of 64 bytes one behind the other, 16-byte chunk c of row r at chunk c ^ (r / 2 mod 4): the
 // 64-byte swizzle of the UMMA layouts, K-major for Q and K, MN-major for V.  A copied row then lies in one 64-byte
@@ -80,8 +80,8 @@ constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kColWorker = 2 * TH + D;  // worker b: S_i (and P_i over its head) at kColWorker b + 64 i, O behind them
 static_assert(kColWorker * NW <= kTmemCols, "TMEM columns");
 constexpr float kLog2e = 1.4426950408889634f;
-constexpr float kHeadroom = 64.0f;       // log2 units a score may exceed the reference maximum
-constexpr float kSumLimit = 1180591620717411303424.0f;  // 2^70: a chunk's sum beyond it gives the excess away
+constexpr float kOctavesAbove = 10.f;    // of a row's reference above the maximum it is set by
+constexpr float kSumLimit = 1.f;         // a chunk's sum beyond it gives away a score near the reference
 constexpr uint32_t kSpinLimit = 1u << 18;  // polls of a wait before the CTA gives up
 constexpr uint32_t kSuspendNs = 4000;      // how long one poll may stay suspended in hardware (longer hints wake later)
 
@@ -390,7 +390,7 @@ __device__ __noinline__ float chunk_max(const uint32_t* cur, float sc, float nm,
 // is still to be read when chunk 0's weights land on columns 0..15, and chunk 1's weights
 // land on columns 16..31, whose scores have been consumed).  The chunk's weights are added to the row sum l.  With `first`
 // (the unit's first tile) chunk 0 sets the row's reference m from its 32 scores (column 0 is the tile's position 0, always a
-// real one).  A chunk whose sum gives away that a score has left the headroom moves the reference up by a whole
+// real one).  A chunk whose sum gives away a score near the reference moves it up by a whole
 // number of octaves and is written again from its scores, read once more; what O holds so far
 // (`have_o`; wait_prev() waits for the previous step's MMAs) and, for chunk 1, the weights of chunk 0 are
 // multiplied by the same power of two.  Returns false if that wait ran out.
@@ -414,7 +414,7 @@ __device__ __forceinline__ bool softmax_chunk(const uint32_t (&cur)[32], int c, 
             t0 = max3(t0, x[0], x[1]);
             t1 = max3(t1, x[2], x[3]);
         }
-        m_ref = fmaxf(t0, t1) * sc;
+        m_ref = ceilf(fmaxf(t0, t1) * sc) + kOctavesAbove;  // (whole octaves: what moves it is exact)
     }
     float nm = -m_ref;
     float ls0 = 0.f, ls1 = 0.f;  // this chunk's share of the row sum
@@ -431,22 +431,21 @@ __device__ __forceinline__ bool softmax_chunk(const uint32_t (&cur)[32], int c, 
         add2(ls0, ls1, e0, e1);
         p[e >> 1] = pack_bf16(e0, e1);
     }
-    // Leaving the headroom shows in the chunk's sum: 32 weights of at most 2^64 add up to at most 2^69, so a sum
-    // beyond kSumLimit = 2^70 (or one that is not a number) means some weight of this row is beyond 2^65.  That
-    // costs one comparison here instead of a running maximum over the arguments.
+    // A sum beyond one (or one that is not a number) means some weight of this row is beyond 2^-5, while a sum of 32 weights
+    // ten octaves down is 2^-5 at most.  That costs one comparison here instead of a running maximum over the arguments.
     if (!__any_sync(0xffffffffu, !(ls0 + ls1 <= kSumLimit))) {
         tmem_st16(tS + 16 * c, p);
     } else {
-        // rare: some row of this warp left the headroom and its weights may have overflowed.  Nothing of this
+        // rare: some row of this warp came near its reference and its weights may have overflowed.  Nothing of this
         // chunk has been written yet, so its scores are still in TMEM: move the reference, bring what was
         // accumulated and written before into the new scale, and work the chunk out again from there.
         uint32_t again[32];
         tmem_ld32(tS + 32 * c, again);
         tmem_wait_ld32(again);
         const float mx = chunk_max<TAIL>(again, sc, nm, valid, c);
-        const float shift = mx > kHeadroom ? ceilf(mx) : 0.f;
-        const float f = ex2(-shift);
-        m_ref += shift;
+        const float moved = mx > -5.f ? m_ref + (ceilf(mx) + kOctavesAbove) : m_ref;
+        const float f = moved != m_ref ? ex2(m_ref - moved) : 1.f;  // (a row that sees nothing has no finite reference)
+        m_ref = moved;
         nm = -m_ref;
         tc_wait_st();
         l *= f;
@@ -709,7 +708,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_umma_kernel(const AttendAr
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tc_fence_after();
-                // (softmax, only taken when a row leaves the headroom) the previous step's weighted sum must have
+                // (softmax, only taken when a row's reference moves) the previous step's weighted sum must have
                 // finished before O is rescaled: it is what releases that step's stage
                 auto wait_prev = [&]() {
                     bool w = mbar_wait(bar(BAR_EMPTY + stage), sphase, abort_flag, SITE_PREV);

@@ -292,7 +292,7 @@ def test_short_lists_under_stream_capture(queries):
 
 
 _WIDE_LISTS = [(2, head, users, queries) for head, queries in (((30, 2), 7), ((30, 2), 33), ((60, 4), 16), ((60, 4), 20))
-               for users in (1, 900)]
+               for users in (1, 900)] + [(3, (30, 2), users, queries) for queries in (20, 120) for users in (1, 300)]
 
 
 @pytest.mark.parametrize("kernel,head,users,queries", _WIDE_LISTS)
@@ -354,3 +354,24 @@ def test_infinities_behind_a_first_tile(kernel, head, users, queries, what):
     odd = ~np.isfinite(want)
     assert np.array_equal(got[odd], want[odd], equal_nan=True)
     assert_close(np.where(odd, 0, got), np.where(odd, 0, want), "bf16", f"{kernel} {users} {head} {queries} {what}")
+
+
+@pytest.mark.parametrize("queries", [40, 97])
+def test_reference_moves_beside_rows_that_see_nothing(queries):
+    """Scores that climb along a history while rows of the same warp see nothing, the first tile only, or all of it."""
+    w = _workload(users=9, hist=(150, 400), queries=queries)
+    d = synth.generate(w)
+    for a, b in zip(d["hist_off"][:-1], d["hist_off"][1:]):
+        d["user_K"][a:b, :, 0] = synth.f32_to_bf16_bits(np.linspace(0, 90, b - a, dtype=np.float32))[:, None]
+    d["queries"][:, :, 0] = synth.f32_to_bf16_bits(np.full(d["queries"].shape[:2], 1.0, np.float32))
+    lens = np.diff(d["hist_off"])
+    vis = np.concatenate([np.where(np.arange(queries) % 3 == 0, 0, np.where(np.arange(queries) % 3 == 1, 40, L)) for L in lens]).astype(np.int32)
+    want = O.attend_variants(w.dtype, w.mode, 1.0, w.head_dim, d["pool_K"], d["pool_V"], d["hist_off"], d["idx_K"],
+                             d["idx_V"], d["user_K"], d["user_V"], d["q_off"], d["queries"], vis=vis)
+    for kernel in (2, 3):
+        s = make_session(w, d, scale=1.0, kernel=kernel)
+        out = s.attend_visible(d["users"], d["q_off"], torch.from_numpy(vis).cuda(), to_dev(d["queries"], w.dtype))
+        torch.cuda.synchronize()
+        assert s.stat("kernel") == kernel and s.stat("device_errors") == 0
+        s.close()
+        assert_close(out.float().cpu().numpy().astype(np.float64), want, "bf16", f"{kernel} {queries}")
