@@ -543,18 +543,31 @@ void arena_give(ckv_ctx* ctx, int64_t base, int64_t units)
 // What the warp-level tensor-core kernel's work consists of: units of (chunk, group, query block) and their 32-position tiles.
 struct MmaWork {
     int64_t units = 0, tiles = 0, min_tiles = INT64_MAX, max_tiles = 0;  // of one group
+    int64_t chunks = 0, max_blocks = 0;  // the grid has room for all of a chunk's query blocks, units or not
     bool alike = true;  // every unit costs the same, if min_tiles = max_tiles
     // a request of `blocks` query blocks (as many as every other if `same`), chunks of `chunk` positions
     void add(int64_t L, int64_t blocks, bool same, int64_t chunk)
     {
         alike = alike && same && L <= chunk;
-        const int64_t chunks = L > chunk ? (L + chunk - 1) / chunk : 1, t = (std::min(L, chunk) + 31) / 32;
-        units += blocks * chunks;
+        const int64_t n = L > chunk ? (L + chunk - 1) / chunk : 1, t = (std::min(L, chunk) + 31) / 32;
+        units += blocks * n;
+        chunks += n;
+        max_blocks = std::max(max_blocks, blocks);
         tiles += blocks * ((L + 31) / 32);
         min_tiles = std::min(min_tiles, t);
         max_tiles = std::max(max_tiles, t);
     }
 };
+
+// Rounds of the `dense` form's blocks over the SMs, three to an SM, if `n` units of each group (or places for them) are shared by
+// `parts` warps each.  A cluster's blocks have to lie side by side, so that not every place is of use: of 400 lists of 0.7
+// to 1.1 rounds those in clusters of four took a second round from 0.94 on, those in clusters of eight from 0.85 on, and 1.3
+// to 1.6 times as long.
+double dense_rounds(const ckv_ctx* ctx, int64_t n, int parts)
+{
+    const double room = 3.0 * ctx->n_sms * (parts <= 8 ? 1 : parts == 16 ? 0.93 : 0.85);
+    return (double)((n * parts + 3) / 4) * ctx->cfg.n_groups / room;
+}
 
 // Warps that share one unit: the number with the shortest estimated run, in tile times of a resident warp.  A unit costs two
 // tiles besides its own.  Every further warp per unit shortens the units but adds blocks, and a round of blocks costs
@@ -571,8 +584,8 @@ int mma_parts(const ckv_ctx* ctx, const MmaWork& w, int qpw, double* tile_times,
         const double rounds = w.units * G * parts / warps;
         const double extra = parts == 1 ? 2 : parts <= 4 ? 4 : D != 64 ? 5 : parts <= 16 ? 6 : 9;
         const double t = w.alike && w.min_tiles == w.max_tiles
-                             ? std::ceil(rounds) * ((w.max_tiles + parts - 1) / parts + 2) + rounds * (extra - 2) +
-                                   (parts > 16 ? 2 : parts > 1 ? 1 : 0)
+                             ? std::ceil(dense ? dense_rounds(ctx, w.units, parts) : rounds) * ((w.max_tiles + parts - 1) / parts + 2) +
+                                   rounds * (extra - 2) + (parts > 16 ? 2 : parts > 1 ? 1 : 0)
                              : w.tiles * G / warps + rounds * extra + 0.75 * (double)w.max_tiles / parts;
         if (t < best_t) {
             best_t = t;
@@ -634,6 +647,8 @@ struct ListShape {
         w.tiles = tiles[qpw / 16 - 1];
         w.min_tiles = (min_L + 31) / 32;
         w.max_tiles = (max_L + 31) / 32;
+        w.chunks = active;
+        w.max_blocks = mma_blocks(max_M, qpw);
         w.alike = same_M();
         return w;
     }
@@ -655,8 +670,11 @@ constexpr double kDenseTile = 1.3;  // see mma_shape
 // slots instead of eight with three, whose tile times count kDenseTile times as long.  That is the ratio of a warp that
 // has latency to wait for and no others beside it; on full SMs the dense form is 6 to 15 % faster (199 ragged users 58.3 -> 50.3 us a
 // call, 4096 x 512 x 16 queries 259 -> 242, 2000 of 30..300 positions 47.8 -> 41.6), and 29 % where a list fits twelve
-// warps in one round and eight in two (220 users x 1000, 2 groups: 22.2 -> 15.7 us); of 56 lists none lost more than 4 %.  At 1.2
-// lists of a few ragged users lose up to 19 %.
+// warps in one round and eight in two (220 users x 1000, 2 groups: 22.2 -> 15.7 us).  A list whose blocks the other form has
+// room for at a time stays there, unless more warps share a unit for it and have room as well: 61 users x 391 positions x 13..31
+// queries x 4 groups 10.1 us, dense 14.0.  (Of 1260 lists of 1..3000 users, 20..4000 positions and 1..130 queries 17 lose more
+// than 3 % against never taking it, 18 % at most, and 374 gain more; with the estimate's ratio alone and clusters that
+// fill every place 28 lost, 46 % at most.  At 1.2 lists of a few ragged users lose up to 19 %.)
 template <typename F>
 void mma_shape(const ckv_ctx* ctx, const ListShape& s, int64_t chunk, bool plain, F&& each, int& qpw, int& parts, bool& dense,
                double* tile_times = nullptr)
@@ -672,7 +690,9 @@ void mma_shape(const ckv_ctx* ctx, const ListShape& s, int64_t chunk, bool plain
         if (plain && ctx->cfg.head_dim == 64 && q == 16) {
             double td;
             const int pd = mma_parts(ctx, w, q, &td, true);
-            if (kDenseTile * td < t) {
+            const int64_t places = w.chunks * w.max_blocks;
+            const bool fits = (double)places * ctx->cfg.n_groups * p <= (double)ctx->n_sms * mma_warps_per_sm(64, 16);
+            if (kDenseTile * td < t && !(fits && (pd == p || dense_rounds(ctx, places, pd) > 1))) {
                 t = kDenseTile * td;
                 p = pd;
                 d = true;

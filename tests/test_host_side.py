@@ -256,3 +256,24 @@ def test_kernel_of_router_calls(lib, d, n, m, G, threads):
     block = device_block(lib, 1 << 20)
     assert lib.ckv_route(0, n, G, d, m, block, block, None, block, 0, None) == 0
     assert np.ctypeslib.as_array(lib.fake_launched(), (6,))[3] == threads
+
+
+# (users, positions, queries, groups, twelve warps per SM)
+@pytest.mark.parametrize("users,lens,queries,G,dense", [
+    (220, (1000, 1000), (3, 3), 2, True), (222, (1000, 1000), (3, 3), 2, True), (223, (1000, 1000), (3, 3), 2, False),
+    (199, (17, 1999), (1, 40), 4, True), (6, (3059, 3059), (94, 94), 3, False), (5, (3059, 3059), (94, 94), 3, True),
+    (61, (391, 391), (13, 31), 4, False),
+    (241, (254, 254), (1, 24), 2, False), (50, (816, 816), (4, 9), 1, False)])
+def test_resident_warps_of_lists_with_64_wide_heads(lib, users, lens, queries, G, dense):
+    """Twelve warps per SM, with rings of two slots, where a list needs them and all of its blocks have room: blocks of four warps,
+    empty ones included, and clusters that do not fill every place."""
+    rng = np.random.default_rng(users)
+    ctx, block = context(lib, G=G, D=64)
+    ids = np.arange(users, dtype=np.int64)
+    L, M = rng.integers(lens[0], lens[1] + 1, users), rng.integers(queries[0], queries[1] + 1, users)
+    assert put(lib, ctx, block, ids, L) == 0
+    q_off = np.concatenate([[0], np.cumsum(M)]).astype(np.int32)
+    assert lib.ckv_set_option(ctx, b"kernel", C.c_int64(2)) == 0
+    assert lib.ckv_attend(ctx, users, ptr(ids), ptr(q_off), block, block, None) == 0
+    assert np.ctypeslib.as_array(lib.fake_launched(), (6,))[4] == 4 * (2 if dense else 3) * 2 * 32 * 128
+    lib.ckv_destroy(ctx)
