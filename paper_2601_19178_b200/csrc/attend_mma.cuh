@@ -536,6 +536,16 @@ __global__ void __launch_bounds__(128, MmaCfg<D, MT, TMA, DENSE>::MIN_BLOCKS)
                         if (moves || !left()) break;
                         moves = true;
                     }
+                } else if constexpr (D == 32 && MT != 2) {
+                    // (what a first tile goes through lies in a row: one-tile histories otherwise wait for instructions.  1890
+                    // users x 18..56 positions x 7..73 queries x 8 groups 121 -> 111 us, 861 x 32 x 18 x 3 12.2 -> 10.7, 65536 x 512 x
+                    // 16 x 4 2192 -> 2184; the others, with more registers, lose 1 % on full SMs.)
+                    if (step == 0) move();
+                    weigh();
+                    if (step != 0 && left()) {
+                        move();
+                        weigh();
+                    }
                 } else {
                     if (step != 0) weigh();
                     if (step == 0 || left()) {
