@@ -390,10 +390,10 @@ __device__ __noinline__ float chunk_max(const uint32_t* cur, float sc, float nm,
 // is still to be read when chunk 0's weights land on columns 0..15, and chunk 1's weights
 // land on columns 16..31, whose scores have been consumed).  The chunk's weights are added to the row sum l.  With `first`
 // (the unit's first tile) chunk 0 sets the row's reference m from its 32 scores (column 0 is the tile's position 0, always a
-// real one).  A chunk whose sum gives away a score near the reference moves it up by a whole
-// number of octaves and is written again from its scores, read once more; what O holds so far
+// real one).  A chunk whose sum gives away a score near the reference moves it up by some
+// octaves and is written again from its scores, read once more; what O holds so far
 // (`have_o`; wait_prev() waits for the previous step's MMAs) and, for chunk 1, the weights of chunk 0 are
-// multiplied by the same power of two.  Returns false if that wait ran out.
+// multiplied by the same factor.  Returns false if that wait ran out.
 // `valid` counts the real positions of the tile (1..64); column e of chunk c holds position
 // pos_of_col(c, e) of the tile.  TAIL = true (the last tile of a history, at most once per unit) masks the
 // columns beyond.
@@ -414,7 +414,7 @@ __device__ __forceinline__ bool softmax_chunk(const uint32_t (&cur)[32], int c, 
             t0 = max3(t0, x[0], x[1]);
             t1 = max3(t1, x[2], x[3]);
         }
-        m_ref = ceilf(fmaxf(t0, t1) * sc) + kOctavesAbove;  // (whole octaves: what moves it is exact)
+        m_ref = fmaf(fmaxf(t0, t1), sc, kOctavesAbove);
     }
     float nm = -m_ref;
     float ls0 = 0.f, ls1 = 0.f;  // this chunk's share of the row sum
@@ -444,7 +444,8 @@ __device__ __forceinline__ bool softmax_chunk(const uint32_t (&cur)[32], int c, 
         tmem_wait_ld32(again);
         const float mx = chunk_max<TAIL>(again, sc, nm, valid, c);
         const float moved = mx > -5.f ? m_ref + (ceilf(mx) + kOctavesAbove) : m_ref;
-        const float f = moved != m_ref ? ex2(m_ref - moved) : 1.f;  // (a row that sees nothing has no finite reference)
+        // (by what the reference moved, rounding included; a row that sees nothing has no finite one)
+        const float f = moved != m_ref ? ex2(m_ref - moved) : 1.f;
         m_ref = moved;
         nm = -m_ref;
         tc_wait_st();
