@@ -277,3 +277,13 @@ def test_resident_warps_of_lists_with_64_wide_heads(lib, users, lens, queries, G
     assert lib.ckv_attend(ctx, users, ptr(ids), ptr(q_off), block, block, None) == 0
     assert np.ctypeslib.as_array(lib.fake_launched(), (6,))[4] == 4 * (2 if dense else 3) * 2 * 32 * 128
     lib.ckv_destroy(ctx)
+
+
+@pytest.mark.parametrize("d,n,m,G,cluster", [(64, 3359, 1424, 2, 4), (64, 1506, 1058, 4, 4), (32, 686, 1261, 8, 4), (128, 2179, 3901, 3, 4),
+                                             (64, 2129, 300, 2, 2), (128, 2153, 14000, 2, 8), (128, 400, 13857, 8, 8),
+                                             (128, 7159, 2786, 8, 1), (64, 131072, 16384, 4, 1)])
+def test_clusters_of_router_calls(lib, d, n, m, G, cluster):
+    """CTAs that share positions lie in a cluster, and clusters of four and eight leave SMs without one."""
+    block = device_block(lib, 1 << 20)
+    assert lib.ckv_route(0, n, G, d, m, block, block, None, block, 2, None) == 0
+    assert np.ctypeslib.as_array(lib.fake_launched(), (6,))[5] == cluster
