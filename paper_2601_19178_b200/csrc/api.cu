@@ -786,7 +786,9 @@ int choose_family(const ckv_ctx* ctx, bool with_vis, const ListShape& s)
     // us and a cost per tile time of its resident warps, by the queries a warp holds.  Of the 244 lists that umma_chunk is
     // fitted to, most get the faster kernel; they lose 1.2 % in the mean, 36 % at most (with the tcgen05 kernel from 48
     // queries on alone 3.8 and 74).  24 queries, 3643 users of 531 positions, 2 groups: 142 / 131 us; 40 queries, 1500 x 1000, 8
-    // groups: 567 / 470.
+    // groups: 567 / 470.  (Of 1300 others of up to 4000 users and 96 queries 1.7 and 61 %.  Of 525 of them with 17 to 47 queries and
+    // more than 224 users 28 run more than 3 % longer than in the warp-level kernel, 37 % at most, all of them 3 % shorter in
+    // the mean; costs that count how unevenly the workers share mixed histories make as many lists slower as faster.)
     // A list that can travel as a kernel argument to the warp-level kernel is one launch there, under stream capture too; the
     // tcgen05 kernel has to have it planned, 15 us and 0.16 per user of the host, which bound a caller with a new list
     // on every call (199 users of 17..1999 positions, 1..40 queries: 47 us a call, the kernel 28, the warp-level one 35).  Such a
