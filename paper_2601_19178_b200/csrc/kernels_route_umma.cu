@@ -12,7 +12,7 @@
 // leaves the SM.
 // What bounds it: the turn of an accumulator, products -> commit -> read-out -> release -> products, some 800 to 1000
 // clocks of latency of which the products are 160, and TMEM, which holds 384 columns of accumulators in turn; with that the
-// tensor core is 83 % busy with bias and products at d_in = 64 (51 % before).  So the turn is kept short: the release is a named
+// tensor core is 82 % busy with bias and products at d_in = 64 (51 % before).  So the turn is kept short: the release is a named
 // barrier of five warps (an mbarrier cost 340 clocks next to running products), the issuing warp waits for its tile
 // before it, the products are issued under elect.sync from values known to be uniform (under "lane 0" the five of them
 // took 380 clocks, now 200).  131072 positions x 16384 entries x 4 groups, d_in 64: 1250 us -> 880 (1250 TFLOP/s; 1197 with
